@@ -608,19 +608,21 @@ static int launch_sum_errors_decode(const Dims& dm, const void* q, const void* K
   }
 }
 
-// Shapes the tensor-core prefill kernels cover.
+// Shapes the tensor-core row-block kernels take: bf16, whatever the single-query kernels do not. The any-shape kernels
+// (fp32 on the CUDA cores, 5 - 7 TFLOP/s) are left with fp32 inputs. Steps measured on both: blocks of 128 with the last
+// query's weights, 16 units of 6128 tokens: 7.07 -> 0.256 ms; with carried weights, 32 units of about 7.3 k: 8.67 -> 0.237
+// ms; one query, head_dim 64, 128 units of about 3.6 k: 0.276 -> 0.168 ms; blocks of a few queries, 2 - 7 times faster.
 static bool prefill_shape_ok(const caote_params_t* p) {
-  const int G = p->n_q_heads / p->n_kv_heads;
-  return p->dtype == CAOTE_BF16 && p->head_dim == 128 && p->base_mode == CAOTE_BASE_CHUNK_SUM && p->n_new >= 16 && p->scale > 0.f &&
-         (long long)G * p->n_new >= 64 && (long long)p->batch * p->n_kv_heads * p->capacity < (1LL << 31) &&
+  return !decode_shape_ok(p) && p->dtype == CAOTE_BF16 && p->scale > 0.f && (long long)p->batch * p->n_kv_heads * p->capacity < (1LL << 31) &&
          (long long)p->batch * p->n_q_heads * p->n_new < (1LL << 31);
 }
 
-static int encode_rows_map(CUtensorMap* tm, const void* ptr, unsigned long long rows, TensorMapEncodeFn encode,
-                           unsigned box_rows = 128) {
-  const cuuint64_t gdim[2] = {128, (cuuint64_t)rows};
-  const cuuint64_t gstride[1] = {256};
-  const cuuint32_t box[2] = {64, box_rows};
+// Rows of D bf16 channels, `pitch` bytes apart, in boxes of 64 channels x 128 rows.
+static int encode_rows_map(CUtensorMap* tm, const void* ptr, int D, unsigned long long rows, unsigned long long pitch,
+                           TensorMapEncodeFn encode) {
+  const cuuint64_t gdim[2] = {(cuuint64_t)D, (cuuint64_t)rows};
+  const cuuint64_t gstride[1] = {(cuuint64_t)pitch};
+  const cuuint32_t box[2] = {64, 128};
   const cuuint32_t estride[2] = {1, 1};
   CUresult r = encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), gdim, gstride, box, estride,
                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -632,49 +634,62 @@ static int encode_rows_map(CUtensorMap* tm, const void* ptr, unsigned long long 
   return CAOTE_OK;
 }
 
-static int launch_prefill_score(const Dims& dm, const void* q, const void* K, const void* V, const int* len, float* o,
-                                float* scores, char* ws, cudaStream_t st, bool* used, const float* vsum) {
+template <int D, bool kFew>
+static int launch_prefill_kernels(const Dims& dm, const prefill::Scratch& sc, const void* q, const void* K, const void* V,
+                                  const int* len, float* base, float* o, float* scores, char* ws, cudaStream_t st,
+                                  const float* vsum, TensorMapEncodeFn encode) {
+  int* status = reinterpret_cast<int*>(ws);
+  const unsigned long long row = (unsigned long long)D * 2, heads = (unsigned long long)dm.B * dm.Hq;
+  const bool last_only = dm.base_mode == CAOTE_BASE_LAST_QUERY;
+  CUtensorMap tmQ, tmQs, tmK, tmV;
+  int rc = encode_rows_map(&tmQ, q, D, heads * dm.m, row, encode);
+  // the score pass reads the counted rows only: the last one of every head is a map of its own with a pitch of m rows
+  if (!rc) rc = last_only ? encode_rows_map(&tmQs, (const char*)q + (size_t)(dm.m - 1) * row, D, heads, row * dm.m, encode)
+                          : (tmQs = tmQ, CAOTE_OK);
+  if (!rc) rc = encode_rows_map(&tmK, K, D, (unsigned long long)dm.units * dm.cap, row, encode);
+  if (!rc) rc = encode_rows_map(&tmV, V, D, (unsigned long long)dm.units * dm.cap, row, encode);
+  const auto score = dm.base_mode == CAOTE_BASE_ACCUM ? prefill::score_kernel<D, kFew, true> : prefill::score_kernel<D, kFew, false>;
+  if (!rc) rc = allow_smem(prefill::attn_kernel<D, kFew>, prefill::attn_smem_bytes<D>());
+  if (!rc) rc = allow_smem(score, prefill::score_smem_bytes<D>());
+  if (rc) return rc;
+  {
+    dim3 grid((dm.R + prefill::kTile - 1) / prefill::kTile, dm.units, sc.nsplit);
+    CAOTE_LAUNCH("prefill_attn_kernel", st,
+                 launch_pdl(prefill::attn_kernel<D, kFew>, grid, dim3(prefill::kAttnThreads), prefill::attn_smem_bytes<D>(), st,
+                            tmQ, tmK, tmV, dm, len, sc, o, status));
+  }
+  {
+    const bool plain = !kFew && dm.base_mode == CAOTE_BASE_CHUNK_SUM && !vsum;
+    dim3 grid(dm.units, D / 16);
+    CAOTE_LAUNCH("prefill_combine_xsum_kernel", st,
+                 launch_pdl(plain ? prefill::attn_combine_xsum_kernel<D, true> : prefill::attn_combine_xsum_kernel<D, false>, grid,
+                            dim3(prefill::kCxThreads), 0, st, dm, len, sc, o, (const float*)base, (const __nv_bfloat16*)V, vsum));
+  }
+  if (dm.base_mode == CAOTE_BASE_EXTERNAL) {
+    dim3 grid((dm.cap + 63) / 64, dm.units);
+    CAOTE_LAUNCH("prefill_score_external_kernel", st,
+                 launch_pdl(prefill::score_external_kernel<D>, grid, dim3(256), 0, st, dm, (const __nv_bfloat16*)V, len, sc,
+                            (const float*)base, scores));
+  } else {
+    dim3 grid((dm.cap + prefill::kScoreKeys - 1) / prefill::kScoreKeys, dm.units);
+    CAOTE_LAUNCH("prefill_score_kernel", st,
+                 launch_pdl(score, grid, dim3(prefill::kScoreThreads), prefill::score_smem_bytes<D>(), st, tmQs, tmK, tmV, dm, len, sc,
+                            base, scores, status));
+  }
+  return CAOTE_OK;
+}
+
+static int launch_prefill_score(const Dims& dm, const void* q, const void* K, const void* V, const int* len, float* base,
+                                float* o, float* scores, char* ws, cudaStream_t st, bool* used, const float* vsum) {
   *used = false;
   TensorMapEncodeFn encode = tensor_map_encoder();
   if (!encode) return CAOTE_OK;
   prefill::Scratch sc;
   prefill::carve(dm, ws + kHeaderBytes, &sc);
-  int* status = reinterpret_cast<int*>(ws);
-  CUtensorMap tmQ, tmK, tmK64, tmV64;
-  int rc = encode_rows_map(&tmQ, q, (unsigned long long)dm.B * dm.Hq * dm.m, encode);
-  if (!rc) rc = encode_rows_map(&tmK, K, (unsigned long long)dm.units * dm.cap, encode);
-  if (!rc) rc = encode_rows_map(&tmK64, K, (unsigned long long)dm.units * dm.cap, encode, prefill::kKeys);
-  if (!rc) rc = encode_rows_map(&tmV64, V, (unsigned long long)dm.units * dm.cap, encode, prefill::kKeys);
-  if (rc) return rc;
-  rc = allow_smem(prefill::attn_kernel, prefill::attn_smem_bytes());
-  if (!rc) rc = allow_smem(prefill::score_kernel, prefill::score_smem_bytes());
-  if (rc) return rc;
-  {
-    dim3 grid((dm.R + prefill::kTile - 1) / prefill::kTile, dm.units, sc.nsplit);
-    CAOTE_LAUNCH("prefill_attn_kernel", st,
-                 launch_pdl(prefill::attn_kernel, dim3(grid), dim3(prefill::kAttnThreads), prefill::attn_smem_bytes(), st, tmQ, tmK64, tmV64, dm, len,
-                                                                                                    sc, o, status));
-  }
-  const bool merged_with_mean = !vsum;  // the splits' merge (if there are splits) and the column mean in one launch
-  if (merged_with_mean) {
-    dim3 grid(dm.units, prefill::kD / 16);
-    CAOTE_LAUNCH("prefill_combine_xsum_kernel", st,
-                 launch_pdl(prefill::attn_combine_xsum_kernel, dim3(grid), dim3(prefill::kCxThreads), 0, st, dm, len, sc, o));
-  } else if (sc.nsplit > 1) {
-    dim3 grid((dm.R + 3) / 4, dm.units);
-    CAOTE_LAUNCH("prefill_attn_combine_kernel", st, launch_pdl(prefill::attn_combine_kernel, dim3(grid), dim3(4 * prefill::kD), 0, st, dm, len, sc, o));
-  }
-  if (vsum) {
-    CAOTE_LAUNCH("fast_mean_kernel", st, fast::mean_kernel<<<dm.units, prefill::kD, 0, st>>>(dm.Hkv, dm.cap, prefill::kD, len, vsum, sc.X));
-  }
-  {
-    dim3 grid((dm.cap + prefill::kScoreKeys - 1) / prefill::kScoreKeys, dm.units);
-    CAOTE_LAUNCH("prefill_score_kernel", st,
-                 launch_pdl(prefill::score_kernel, dim3(grid), dim3(prefill::kScoreThreads), prefill::score_smem_bytes(), st, 
-                     tmQ, tmK, tmV64, dm, len, sc, scores, status));
-  }
   *used = true;
-  return CAOTE_OK;
+  auto run = dm.D == 128 ? (sc.few ? launch_prefill_kernels<128, true> : launch_prefill_kernels<128, false>)
+                         : (sc.few ? launch_prefill_kernels<64, true> : launch_prefill_kernels<64, false>);
+  return run(dm, sc, q, K, V, len, base, o, scores, ws, st, vsum, encode);
 }
 
 // The split heuristics of the prefill and any-shape paths look at the SM count: keep it current for this device
@@ -697,7 +712,8 @@ static void refresh_sm_count() {
   g_sm_count = n;
 }
 
-static size_t workspace_bytes(const caote_params_t* p) {
+// row_blocks: with room for the tensor-core row-block kernels where they cover the shape.
+static size_t workspace_bytes(const caote_params_t* p, bool row_blocks = true) {
   refresh_sm_count();
   const Dims dm = make_dims(p);
   size_t need = generic::carve(dm, nullptr, nullptr);
@@ -705,7 +721,7 @@ static size_t workspace_bytes(const caote_params_t* p) {
     const size_t need2 = rowstat_bytes(dm) + decode::carve(dm, nullptr, nullptr, 0);
     if (need2 > need) need = need2;
   }
-  if (prefill_shape_ok(p)) {
+  if (row_blocks && prefill_shape_ok(p)) {
     const size_t need3 = prefill::carve(dm, nullptr, nullptr);
     if (need3 > need) need = need3;
   }
@@ -884,8 +900,9 @@ static int score_args_check(const caote_params_t* p, const void* q, const void* 
   if (!aligned(q, 16) || !aligned(K, 16) || !aligned(V, 16) || !aligned(o, 16)) return CAOTE_ERR_INVALID_ARG;
   return CAOTE_OK;
 }
-static int score_workspace_check(const caote_params_t* p, const void* workspace, size_t workspace_bytes_) {
-  if (!workspace || workspace_bytes_ < workspace_bytes(p) || !aligned(workspace, 256)) return CAOTE_ERR_INVALID_ARG;
+static int score_workspace_check(const caote_params_t* p, const void* workspace, size_t workspace_bytes_,
+                                 bool row_blocks = true) {
+  if (!workspace || workspace_bytes_ < workspace_bytes(p, row_blocks) || !aligned(workspace, 256)) return CAOTE_ERR_INVALID_ARG;
   return CAOTE_OK;
 }
 
@@ -933,9 +950,9 @@ int caote_append(const caote_params_t* p, void* K, void* V, float* base, int32_t
 // caote_score (vsum == NULL) and caote_score_fast (vsum: the per-unit sums of the cached value rows).
 static int score_impl(const caote_params_t* p, const void* q, const void* K, const void* V, const int32_t* len,
                       float* base, const float* vsum, float* o, float* scores, void* workspace, size_t workspace_bytes_,
-                      caote_stream_t stream, bool allow_side_stream = true) {
+                      caote_stream_t stream, bool allow_side_stream = true, bool row_blocks = true) {
   int rc = score_args_check(p, q, K, V, len, base, o, scores);
-  if (!rc) rc = score_workspace_check(p, workspace, workspace_bytes_);
+  if (!rc) rc = score_workspace_check(p, workspace, workspace_bytes_, row_blocks);
   if (!rc) rc = check_device();
   if (rc) return rc;
   const Dims dm = make_dims(p);
@@ -989,9 +1006,9 @@ static int score_impl(const caote_params_t* p, const void* q, const void* K, con
     rc = launch_decode_score(dm, q, K, V, len, base, o, scores, status, scratch, rowstat, kStatPerHead, 0, st, &used, vsum);
     if (rc || used) return rc;
   }
-  if (prefill_shape_ok(p)) {
+  if (row_blocks && prefill_shape_ok(p)) {
     bool used = false;
-    rc = launch_prefill_score(dm, q, K, V, len, o, scores, ws, st, &used, vsum);
+    rc = launch_prefill_score(dm, q, K, V, len, base, o, scores, ws, st, &used, vsum);
     if (rc || used) return rc;
   }
   if (p->dtype == CAOTE_BF16) {
@@ -1063,7 +1080,9 @@ int caote_score_static(const caote_params_t* p, const void* q, const void* K, co
   // everything caote_score would refuse is refused here, before anything touches the stream or the array
   int rc = score_args_check(p, q, K, V, len, base, o, scores);
   if (rc) return rc;
-  if (workspace_bytes(p) > kStaticScratchBytes) return CAOTE_ERR_TOO_LARGE;
+  // (a shape whose key splits do not fit the array may still fit it on the any-shape kernels)
+  const bool row_blocks = workspace_bytes(p) <= kStaticScratchBytes;
+  if (!row_blocks && workspace_bytes(p, false) > kStaticScratchBytes) return CAOTE_ERR_TOO_LARGE;
   rc = check_device();
   if (rc) return rc;
   char* scratch = nullptr;
@@ -1073,7 +1092,7 @@ int caote_score_static(const caote_params_t* p, const void* q, const void* K, co
   // the array keeps whatever the previous call left: the status word has to start at zero
   CAOTE_CUDA(cudaMemsetAsync(scratch, 0, kHeaderBytes, st));
   // (no second stream here: making one allocates)
-  rc = score_impl(p, q, K, V, len, base, nullptr, o, scores, scratch, kStaticScratchBytes, stream, false);
+  rc = score_impl(p, q, K, V, len, base, nullptr, o, scores, scratch, kStaticScratchBytes, stream, false, row_blocks);
   if (rc) return rc;
   if (status_out) CAOTE_CUDA(cudaMemcpyAsync(status_out, scratch, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
   return CAOTE_OK;

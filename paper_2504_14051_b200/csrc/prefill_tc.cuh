@@ -1,6 +1,7 @@
-// Chunked-prefill scoring path on the 5th-generation tensor cores (tcgen05 + TMEM) for bf16,
-// head_dim 128, base mode CHUNK_SUM: a block of m new queries per sequence, M = G * m query rows per
-// (sequence, KV head) unit against its n cached keys.
+// Tensor-core scoring path (tcgen05 + TMEM) for bf16, head_dim 64 or 128, any base mode: M = G * m query rows per
+// (sequence, KV head) unit against its n cached keys. Blocks of a prompt are what it is built for; it also takes the
+// single-query shapes that the cluster kernel has no form for (see decode_shape_ok): a row block is then mostly
+// padding, but a pass over K and V at this kernel's pace per tile still keeps up with HBM.
 //
 //   attn_kernel   rows x keys. One CTA owns 128 query rows of a unit and walks the unit's keys in
 //                 tiles of 128: S = Q K^T (tcgen05.mma, fp32 accumulator in TMEM), per-row online
@@ -10,14 +11,20 @@
 //                 softmax statistics (reference, 1 / sum). One lane each of three extra warps issues
 //                 the products, the K copies and the V copies, so the tensor pipe always has the
 //                 next S queued while the rows are busy with the current one.
-//   attn_combine_xsum_kernel   merges the key splits of small grids (attn_combine_kernel does only that, for
-//                 FastCAOTE) and forms X = mean of the unit's M output rows (the weights of CHUNK_SUM are the
-//                 column sums of the attention matrix divided by M, so sum_j w_j v_j is the mean output row).
-//   score_kernel  keys x rows. One CTA owns 256 keys of a unit (two key tiles) and walks the unit's
-//                 rows in blocks of 128: S^T = K Q^T lands in TMEM with one key per lane, so each
+//   attn_combine_xsum_kernel   merges the key splits of small grids and forms X = sum_j w_j v_j = (sum of the counted
+//                 output rows + sum_j base_j v_j) / (counted rows + sum_j base_j). Counted are the rows whose
+//                 attention defines the base score: all (CHUNK_SUM, ACCUM), the last of every head (LAST_QUERY) or
+//                 none (EXTERNAL). The carried scores' share, a pass over V, runs here because V has just been read
+//                 by the attention pass and mostly comes from L2.
+//   score_kernel  keys x counted rows. One CTA owns 256 keys of a unit (two key tiles) and walks the unit's
+//                 counted rows in blocks of 128: S^T = K Q^T lands in TMEM with one key per lane, so each
 //                 thread sums exp2(s - ref_r) / sum_r over the rows of its own key without any
-//                 exchange: h_j = sum_r alpha_{r,j}. Then c_j = w_j / (1 - w_j) * ||X - v_j||,
-//                 w_j = h_j / M.
+//                 exchange: h_j = sum_r alpha_{r,j} (+ base_j). Then c_j = w_j / (1 - w_j) * ||X - v_j||.
+//
+// 1 - w_j. With 64 counted rows or more it is formed as the difference (rows - h_j) (exact to 6e-8 of the row count).
+// A few rows may well agree on one token, so for fewer than 64 (`few`) the attention pass keeps the largest numerator
+// of every counted row apart from the sum of the others, and the complement of the row's top token is that sum's
+// share, everybody else's 1 - alpha with alpha <= 1/2: no cancellation.
 //
 // Operands are staged by TMA as 64-channel boxes with the 128-byte swizzle, which is the canonical
 // K-major UMMA layout (8-row groups 1024 bytes apart); V in the second product is read through an
@@ -34,21 +41,28 @@
 namespace caote {
 namespace prefill {
 
-constexpr int kD = 128;
 constexpr int kTile = 128;                  // rows / keys per tile
-constexpr int kHalfBytes = kTile * 128;     // one 64-channel box
-constexpr int kTileBytes = 2 * kHalfBytes;  // 32 KB
+constexpr int kHalfBytes = kTile * 128;     // one 64-channel box of 128 rows: 16 KB
+template <int D>
+constexpr int kTileBytesOf = (D / 64) * kHalfBytes;  // a tile of 128 rows
 constexpr int kThreads = 128;
 constexpr long long kWaitCycles = 2000000000LL;
 
 struct Scratch {
   float* stats;  // [units][Mpad]: log2-domain softmax reference + log2(sum of 2^(s - ref)): alpha = 2^(s - stats)
-  float* X;      // [units][kD]
+  float* X;      // [units][D]
+  float* hb;     // [units] sum of the carried base scores
+  float* sstat;  // [units][kTile] LAST_QUERY: the counted rows' statistics side by side (else null)
+  float* crest;  // [units][kTile] few: share of all tokens but the counted row's top one (else null)
+  float2* ptop;  // [units][nsplit][kTile] few, nsplit > 1: per split (largest logit, share of the split's other tokens)
   int Mpad;      // M rounded up to a multiple of kTile
   int nsplit;    // key splits of the attention pass (1: none)
-  float* po;     // [units][nsplit][Mpad][kD] per-split outputs, normalised by their own sums (nsplit > 1)
+  int Ms;        // counted rows per unit
+  bool few;      // 0 < Ms < kFewRows: complements without cancellation (see the file comment)
+  float* po;     // [units][nsplit][M][D] per-split outputs, normalised by their own sums (nsplit > 1)
   float* pstat;  // [units][nsplit][Mpad] per-split statistics
 };
+constexpr int kFewRows = 64;
 
 // Few units and few query rows leave most SMs idle: the keys of a unit are then cut into up to 8 splits
 // that run as CTAs of their own; attn_combine_kernel merges them. A function of the shape only.
@@ -77,21 +91,35 @@ __host__ __device__ inline void split_plan(int n, int m, int nsplit, int& ts, in
 inline size_t carve(const Dims& dm, char* base, Scratch* out) {
   Scratch s;
   s.Mpad = (dm.R + kTile - 1) / kTile * kTile;
-  size_t off = 0;
-  s.stats = reinterpret_cast<float*>(base + off);
-  off = align_up(off + sizeof(float) * (size_t)dm.units * s.Mpad, 256);
-  s.X = reinterpret_cast<float*>(base + off);
-  off = align_up(off + sizeof(float) * (size_t)dm.units * kD, 256);
   s.nsplit = attn_splits(dm);
-  s.po = s.pstat = nullptr;
-  if (s.nsplit > 1) {
-    s.po = reinterpret_cast<float*>(base + off);
-    off = align_up(off + sizeof(float) * (size_t)dm.units * s.nsplit * s.Mpad * kD, 256);
-    s.pstat = reinterpret_cast<float*>(base + off);
-    off = align_up(off + sizeof(float) * (size_t)dm.units * s.nsplit * s.Mpad, 256);
-  }
+  s.Ms = dm.base_mode == CAOTE_BASE_LAST_QUERY ? dm.G : (dm.base_mode == CAOTE_BASE_EXTERNAL ? 0 : dm.R);
+  s.few = s.Ms > 0 && s.Ms < kFewRows;
+  size_t off = 0;
+  auto take = [&](bool wanted, size_t n_floats) {
+    if (!wanted) return static_cast<float*>(nullptr);
+    float* p = reinterpret_cast<float*>(base + off);
+    off = align_up(off + sizeof(float) * n_floats, 256);
+    return p;
+  };
+  const size_t units = (size_t)dm.units;
+  s.stats = take(true, units * s.Mpad);  // (first: caote_post_evict_output_ws finds it right behind the header)
+  s.X = take(true, units * dm.D);
+  s.hb = take(true, units);
+  s.sstat = take(dm.base_mode == CAOTE_BASE_LAST_QUERY, units * kTile);
+  s.crest = take(s.few, units * kTile);
+  s.ptop = reinterpret_cast<float2*>(take(s.few && s.nsplit > 1, units * s.nsplit * kTile * 2));
+  s.po = take(s.nsplit > 1, units * s.nsplit * dm.R * dm.D);
+  s.pstat = take(s.nsplit > 1, units * s.nsplit * s.Mpad);
   if (out) *out = s;
   return off;
+}
+// Is row R of a unit one of the rows whose attention defines the base score, and which counted row is it?
+__device__ __forceinline__ bool row_counted(const Dims& dm, int R) {
+  if (dm.base_mode == CAOTE_BASE_LAST_QUERY) return R % dm.m == dm.m - 1;
+  return dm.base_mode != CAOTE_BASE_EXTERNAL;
+}
+__device__ __forceinline__ int counted_index(const Dims& dm, int R) {
+  return dm.base_mode == CAOTE_BASE_LAST_QUERY ? R / dm.m : R;
 }
 
 // ---- PTX wrappers (ptx.cuh), the waits built on them, and the tcgen05 wrappers ----------------------------
@@ -288,35 +316,33 @@ __device__ __forceinline__ uint64_t desc_mn_major(uint32_t tile_addr, int ks) {
 //   threads:      softmax(t) ............ softmax(t+1) ...
 constexpr int kKeys = 128;                   // keys per tile of the attention pass
 constexpr int kKvHalf = kKeys * 128;         // one 64-channel box of 128 keys: 16 KB
-constexpr int kKvTile = 2 * kKvHalf;         // K or V tile: 32 KB
 constexpr int kKStages = 3;                  // a K stage is free as soon as S is formed
 constexpr int kVStages = 2;
 constexpr int kRowThreads = 2 * kThreads;    // two threads per query row: each owns 64 of the tile's 128 keys
 constexpr int kAttnThreads = kRowThreads + 96;  // + MMA, K-load and V-load warps
 
+constexpr int kXchFloats = 5 * kRowThreads;     // half-row maxima and sums in turn, and the few-rows form's three closing values
+
+template <int D>
 inline size_t attn_smem_bytes() {
-  return 1024 + kTileBytes + (size_t)(kKStages + kVStages) * kKvTile + 2 * kRowThreads * sizeof(float) + 256;
+  return 1024 + (size_t)(1 + kKStages + kVStages) * kTileBytesOf<D> + kXchFloats * sizeof(float) + 256;
 }
 
-// K-major / MN-major descriptors of k-step ks of a key tile (boxes of kKeys rows x 64 channels: kKvHalf apart).
-__device__ __forceinline__ uint64_t desc_k_major64(uint32_t tile_addr, int ks) {
-  return smem_desc(tile_addr + (ks >> 2) * kKvHalf + (ks & 3) * 32, 16, 1024);
-}
-__device__ __forceinline__ uint64_t desc_mn_major64(uint32_t tile_addr, int ks) {
-  return smem_desc(tile_addr + ks * 2048, kKvHalf, 1024);
-}
 __host__ __device__ constexpr uint32_t instr_desc_n(bool b_mn_major, uint32_t n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((b_mn_major ? 1u : 0u) << 16) | ((n >> 3) << 17) | ((128u >> 4) << 24);
 }
 
-// o and row statistics of 128 query rows of one unit. grid = (row blocks, units), 352 threads:
+// o and row statistics of 128 query rows of one unit. grid = (row blocks, units, splits), 352 threads:
 // warps 0..7 are the row threads (two per row); one lane each of warps 8, 9, 10 issues the products,
 // the K copies and the V copies.
-// tmK64 / tmV64: tensor maps of K and V with boxes of 64 channels x kKeys rows.
+// tmK / tmV: tensor maps of K and V with boxes of 64 channels x kKeys rows. kFew: the counted rows' largest numerators
+// are kept apart (see the file comment).
+template <int D, bool kFew>
 __global__ void __launch_bounds__(kAttnThreads, 1)
-attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK64,
-            const __grid_constant__ CUtensorMap tmV64, Dims dm, const int* __restrict__ len, Scratch sc,
+attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+            const __grid_constant__ CUtensorMap tmV, Dims dm, const int* __restrict__ len, Scratch sc,
             float* __restrict__ o, int* status) {
+  constexpr int kTB = kTileBytesOf<D>, kBoxes = D / 64, kSteps = D / 16;  // k-steps of the first product
   ptx::pdl_wait();
   ptx::pdl_trigger();
   extern __shared__ char smem_raw[];
@@ -324,10 +350,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   // read and written through it compiles to shared-memory accesses, not generic ones)
   char* sm = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
   char* Qs = sm;
-  char* Ksm = Qs + kTileBytes;                 // [kKStages]
-  char* Vsm = Ksm + kKStages * kKvTile;        // [kVStages]
-  float* xch = reinterpret_cast<float*>(Vsm + kVStages * kKvTile);  // [2][kRowThreads] half-row maxima / sums
-  uint64_t* bars = reinterpret_cast<uint64_t*>(xch + 2 * kRowThreads);
+  char* Ksm = Qs + kTB;                    // [kKStages]
+  char* Vsm = Ksm + kKStages * kTB;        // [kVStages]
+  float* xch = reinterpret_cast<float*>(Vsm + kVStages * kTB);  // [kXchFloats]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(xch + kXchFloats);
   uint64_t *q_bar = &bars[0], *k_bar = &bars[1], *v_bar = k_bar + kKStages, *s_bar = v_bar + kVStages, *o_bar = s_bar + 2,
            *p_bar = o_bar + 2, *k_free = p_bar + 2, *v_free = k_free + kKStages;
   constexpr int kBars = 1 + 2 * (kKStages + kVStages) + 6;
@@ -369,15 +395,15 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   if (warp == 9) {
     // =============================== K loads (one lane) ===============================
     if (tid == kRowThreads + 32) {
-      mbar_expect_tx(q_bar, kTileBytes);
-      tma_load_2d(Qs, &tmQ, 0, unit * M + row0, q_bar);
-      tma_load_2d(Qs + kHalfBytes, &tmQ, 64, unit * M + row0, q_bar);
+      mbar_expect_tx(q_bar, kTB);
+#pragma unroll
+      for (int x = 0; x < kBoxes; ++x) tma_load_2d(Qs + x * kHalfBytes, &tmQ, 64 * x, unit * M + row0, q_bar);
       for (int kt = 0; kt < ntiles; ++kt) {
         const int st = kt % kKStages, row = unit * dm.cap + (kt0 + kt) * kKeys;
         if (kt >= kKStages) mbar_wait_idle(&k_free[st], ((kt / kKStages) - 1) & 1, status);  // S of tile kt - 3 is formed
-        mbar_expect_tx(&k_bar[st], kKvTile);
-        tma_load_2d(Ksm + st * kKvTile, &tmK64, 0, row, &k_bar[st]);
-        tma_load_2d(Ksm + st * kKvTile + kKvHalf, &tmK64, 64, row, &k_bar[st]);
+        mbar_expect_tx(&k_bar[st], kTB);
+#pragma unroll
+        for (int x = 0; x < kBoxes; ++x) tma_load_2d(Ksm + st * kTB + x * kKvHalf, &tmK, 64 * x, row, &k_bar[st]);
       }
     }
   } else if (warp == 10) {
@@ -386,30 +412,30 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       for (int kt = 0; kt < ntiles; ++kt) {
         const int st = kt % kVStages, row = unit * dm.cap + (kt0 + kt) * kKeys;
         if (kt >= kVStages) mbar_wait_idle(&v_free[st], ((kt / kVStages) - 1) & 1, status);  // O += P V of tile kt - 2 is done
-        mbar_expect_tx(&v_bar[st], kKvTile);
-        tma_load_2d(Vsm + st * kKvTile, &tmV64, 0, row, &v_bar[st]);
-        tma_load_2d(Vsm + st * kKvTile + kKvHalf, &tmV64, 64, row, &v_bar[st]);
+        mbar_expect_tx(&v_bar[st], kTB);
+#pragma unroll
+        for (int x = 0; x < kBoxes; ++x) tma_load_2d(Vsm + st * kTB + x * kKvHalf, &tmV, 64 * x, row, &v_bar[st]);
       }
     }
   } else if (warp == 8) {
     // =============================== products (one lane) ===============================
     if (tid == kRowThreads) {
-      constexpr uint32_t kIdescS = instr_desc_n(false, kKeys), kIdescO = instr_desc_n(true, kD);
+      constexpr uint32_t kIdescS = instr_desc_n(false, kKeys), kIdescO = instr_desc_n(true, D);
       const uint32_t q_addr = smem_u32(Qs);
       // Descriptors are built once; inside the loop a product costs one 64-bit add per operand (the
       // single issuing thread is bound by the latency of its own instruction stream, not by the pipe).
-      uint64_t qdesc[8];
+      uint64_t qdesc[kSteps];
 #pragma unroll
-      for (int ks = 0; ks < 8; ++ks) qdesc[ks] = desc_k_major(q_addr, ks);
+      for (int ks = 0; ks < kSteps; ++ks) qdesc[ks] = desc_k_major(q_addr, ks);
       const uint64_t kdesc0 = smem_desc(smem_u32(Ksm), 16, 1024);
       const uint64_t vdesc0 = smem_desc(smem_u32(Vsm), kKvHalf, 1024);
       auto issue_qk = [&](int kt) {
         mbar_wait_idle(&k_bar[kt % kKStages], (kt / kKStages) & 1, status);
         tc_fence_after();
-        const uint64_t kd = kdesc0 + (uint64_t)(((kt % kKStages) * kKvTile) >> 4);
+        const uint64_t kd = kdesc0 + (uint64_t)(((kt % kKStages) * kTB) >> 4);
         const uint32_t d_s = tmem + (kt & 1) * kKeys;  // S0 or S1
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks)
+        for (int ks = 0; ks < kSteps; ++ks)
           umma(d_s, qdesc[ks], kd + (uint64_t)((((ks >> 2) * kKvHalf) + (ks & 3) * 32) >> 4), kIdescS, ks > 0);
         umma_commit(&s_bar[kt & 1]);
         umma_commit(&k_free[kt % kKStages]);
@@ -424,7 +450,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         mbar_wait_idle(&p_bar[kt & 1], (kt >> 1) & 1, status);
         mbar_wait_idle(&v_bar[kt % kVStages], (kt / kVStages) & 1, status);
         tc_fence_after();
-        const uint64_t vd = vdesc0 + (uint64_t)(((kt % kVStages) * kKvTile) >> 4);
+        const uint64_t vd = vdesc0 + (uint64_t)(((kt % kVStages) * kTB) >> 4);
         const uint32_t p_tmem = tmem + (kt & 1) * kKeys;
         if (kt == 0) {
           umma_ts(tmem + 256, p_tmem, vd, kIdescO, false);
@@ -451,8 +477,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     const int nvis = (R < M) ? n - m + (R % m) + 1 : n;  // keys this row sees (causal inside the block)
     const float scale2 = dm.scale * 1.4426950408889634f;
     const uint32_t t_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t t_o = t_lane + 256 + half * 64;
+    const uint32_t t_o = t_lane + 256 + half * (D / 2);
     float m_ref = -INFINITY, l = 0.f;
+    // few counted rows (kFew): this thread's largest logit, its numerator and the sum of the other numerators; warps
+    // without a counted row skip that
+    float smax = -INFINITY, ptop = 0.f, lrest = 0.f;
+    const bool counted = kFew && R < M && row_counted(dm, R);
+    const bool keep_top = kFew && __any_sync(0xffffffffu, counted);
 
     for (int kt = 0; kt < ntiles; ++kt) {
       mbar_wait(&s_bar[kt & 1], (kt >> 1) & 1, status);
@@ -475,6 +506,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         for (int i = 8; i < 64; ++i) pm[i & 7] = fmaxf(pm[i & 7], sv[i] * scale2);
         mx = fmaxf(fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3])), fmaxf(fmaxf(pm[4], pm[5]), fmaxf(pm[6], pm[7])));
       }
+      const float mine = mx;
       // the other half of the row
       float* xm = xch + (kt & 1) * kRowThreads;
       xm[tid] = mx;
@@ -486,11 +518,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         const float corr = need ? fast_exp2(m_ref - mx) : 1.f;
         if (need) m_ref = mx;
         l *= corr;
+        if (kFew) { ptop *= corr; lrest *= corr; }
         if (kt > 0) {
           mbar_wait(&o_bar[(kt - 1) & 1], ((kt - 1) >> 1) & 1, status);  // O += P V of the previous tile is done
           tc_fence_after();
 #pragma unroll
-          for (int cc = 0; cc < 2; ++cc) {
+          for (int cc = 0; cc < D / 64; ++cc) {
             float v[32];
             tmem_ld32(t_o + cc * 32, v);
 #pragma unroll
@@ -523,15 +556,33 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         tmem_st32u(t_p + 64, lo);
         tmem_st_wait();
         l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
+        if (kFew && keep_top) {
+          // the same numerators once more, the tile's largest (every copy of it but one) left out
+          float rest[4] = {0.f, 0.f, 0.f, 0.f};
+          int copies = 0;
+#pragma unroll
+          for (int c = 0; c < 64; ++c) {
+            const bool top = sv[c] * scale2 == mine;
+            rest[c & 3] += top ? 0.f : fast_exp2(fmaf(sv[c], scale2, neg_ref));
+            copies += top ? 1 : 0;
+          }
+          const float pt = (mine == -INFINITY) ? 0.f : fast_exp2(mine + neg_ref);
+          float r = (rest[0] + rest[1]) + (rest[2] + rest[3]) + (float)(copies - 1) * pt;
+          const bool bigger = mine > smax;
+          r += bigger ? ptop : pt;
+          lrest += r;
+          ptop = bigger ? pt : ptop;
+          smax = bigger ? mine : smax;
+        }
       }
       const int n_valid = min(kKeys, n - (kt0 + kt) * kKeys);
       if (n_valid < kKeys) {
         // V rows behind the unit's length: clear them so that 0 * (stray NaN) cannot reach O
         mbar_wait(&v_bar[kt % kVStages], (kt / kVStages) & 1, status);
         if (tid < kKeys && tid >= n_valid) {
-          char* vt = Vsm + (kt % kVStages) * kKvTile;
+          char* vt = Vsm + (kt % kVStages) * kTB;
 #pragma unroll
-          for (int c = 0; c < 16; ++c)
+          for (int c = 0; c < D / 8; ++c)
             *reinterpret_cast<uint4*>(vt + (c >> 3) * kKvHalf + tid * 128 + (((c & 7) ^ (tid & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
         }
       }
@@ -547,12 +598,26 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     xl[tid] = l;
     asm volatile("bar.sync 1, %0;" ::"n"(kRowThreads) : "memory");
     l += xl[tid ^ kThreads];
+    if (kFew) {
+      // the two halves' (sum of the others, largest numerator, its logit): the larger one stays apart
+      float* xt = xch + 2 * kRowThreads;
+      xt[tid] = lrest;
+      xt[kRowThreads + tid] = ptop;
+      xt[2 * kRowThreads + tid] = smax;
+      asm volatile("bar.sync 1, %0;" ::"n"(kRowThreads) : "memory");
+      const int other = tid ^ kThreads;
+      const float op = xt[kRowThreads + other], os = xt[2 * kRowThreads + other];
+      const bool keep = smax > os || (smax == os && half == 0);
+      lrest += xt[other] + (keep ? op : ptop);
+      ptop = keep ? ptop : op;
+      smax = fmaxf(smax, os);
+    }
     const float inv_l = 1.f / l;
     // (with key splits: this split's output, normalised by its own sum, and its statistic go to scratch)
-    float* orow = (nsp > 1 ? sc.po + (((size_t)unit * sc.nsplit + split) * sc.Mpad + R) * kD
-                           : o + ((size_t)unit * M + R) * kD) + half * 64;
+    float* orow = (nsp > 1 ? sc.po + (((size_t)unit * sc.nsplit + split) * M + R) * D : o + ((size_t)unit * M + R) * D) +
+                  half * (D / 2);
 #pragma unroll
-    for (int cc = 0; cc < 2; ++cc) {
+    for (int cc = 0; cc < D / 64; ++cc) {
       float v[32];
       tmem_ld32(t_o + cc * 32, v);  // collective: every lane takes part, rows beyond M just do not store
       if (R < M) {
@@ -562,8 +627,18 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       }
     }
     if (R < M && half == 0) {
-      if (nsp > 1) sc.pstat[((size_t)unit * sc.nsplit + split) * sc.Mpad + R] = m_ref + __log2f(l);
-      else sc.stats[(size_t)unit * sc.Mpad + R] = m_ref + __log2f(l);
+      const float stat = m_ref + __log2f(l);
+      if (nsp > 1) {
+        sc.pstat[((size_t)unit * sc.nsplit + split) * sc.Mpad + R] = stat;
+        if (kFew && counted)
+          sc.ptop[((size_t)unit * sc.nsplit + split) * kTile + counted_index(dm, R)] = make_float2(smax, lrest / (lrest + ptop));
+      } else {
+        sc.stats[(size_t)unit * sc.Mpad + R] = stat;
+        if (kFew && counted) {
+          if (sc.sstat) sc.sstat[(size_t)unit * kTile + counted_index(dm, R)] = stat;
+          sc.crest[(size_t)unit * kTile + counted_index(dm, R)] = lrest / (lrest + ptop);
+        }
+      }
     }
   }
   tc_fence_before();
@@ -571,44 +646,23 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-// Merge the key splits of a unit: o = sum_s o_s 2^(stat_s - stat), stat = log2 sum_s 2^stat_s.
-// grid = (ceil(M / 4), units), 4 rows x 128 channels per CTA. Units that ran unsplit are left alone.
-__global__ void __launch_bounds__(4 * kD)
-attn_combine_kernel(Dims dm, const int* __restrict__ len, Scratch sc, float* __restrict__ o) {
-  ptx::pdl_wait();
-  ptx::pdl_trigger();
-  const int unit = blockIdx.y, c = threadIdx.x % kD, R = blockIdx.x * 4 + threadIdx.x / kD;
-  const int n = len[unit / dm.Hkv];
-  if (n == 0 || n < dm.m || n > dm.cap || R >= dm.R) return;
-  int ts, nsp;
-  split_plan(n, dm.m, sc.nsplit, ts, nsp);
-  if (nsp <= 1) return;
-  float st[8], mx = -INFINITY;
-  for (int s = 0; s < nsp; ++s) {
-    st[s] = sc.pstat[((size_t)unit * sc.nsplit + s) * sc.Mpad + R];
-    mx = fmaxf(mx, st[s]);
-  }
-  float tot = 0.f, acc = 0.f;
-  for (int s = 0; s < nsp; ++s) {
-    const float w = exp2f(st[s] - mx);
-    tot += w;
-    acc = fmaf(sc.po[(((size_t)unit * sc.nsplit + s) * sc.Mpad + R) * kD + c], w, acc);
-  }
-  o[((size_t)unit * dm.R + R) * kD + c] = acc / tot;
-  if (c == 0) sc.stats[(size_t)unit * sc.Mpad + R] = mx + log2f(tot);
-}
-
-// The merge of the key splits and the column mean X (the weights of CHUNK_SUM are the column sums of the attention
-// matrix divided by M, so sum_j w_j v_j is the mean output row) in one launch: a CTA takes 16 channels of a unit and
-// all of its rows, merges the splits row by row exactly as attn_combine_kernel does, writes o and (the CTA of channels
-// 0..15) the rows' statistics, and adds up its 16 columns in a fixed order for X. Units that ran unsplit are only
-// summed. grid = (units, kD / 16), 512 threads: a warp takes 8 rows at a time, 4 lanes per row.
+// The merge of the key splits, o = sum_s o_s 2^(stat_s - stat) with stat = log2 sum_s 2^stat_s, and
+// X = (sum of the counted output rows + sum_j base_j v_j) / (counted rows + sum_j base_j) in one launch (FastCAOTE: the
+// mean of the cached values, vsum / n): a CTA takes 16 channels of a unit and all of its rows, merges the splits row by
+// row, writes o and (the CTA of channels 0..15) the rows' statistics, and adds up its 16 columns in a fixed order for X.
+// Units that ran unsplit are only summed. grid = (units, D / 16), 512 threads: a warp takes 8 rows at a time, 4 lanes
+// per row; for the carried scores' share two lanes take a key's 16 channels.
 constexpr int kCxThreads = 512;
+// kPlain: every row counts and nothing is carried (CHUNK_SUM, not few, not FastCAOTE).
+template <int D, bool kPlain>
 __global__ void __launch_bounds__(kCxThreads, 2)
-attn_combine_xsum_kernel(Dims dm, const int* __restrict__ len, Scratch sc, float* __restrict__ o) {
+attn_combine_xsum_kernel(Dims dm, const int* __restrict__ len, Scratch sc, float* __restrict__ o,
+                         const float* __restrict__ base, const __nv_bfloat16* __restrict__ V,
+                         const float* __restrict__ vsum) {
   ptx::pdl_wait();
   ptx::pdl_trigger();
   __shared__ float4 wpart[kCxThreads / 32][4];
+  __shared__ float wy[kCxThreads / 32][17];  // the carried scores' share of the 16 channels, and their sum
   const int unit = blockIdx.x, c0 = blockIdx.y * 16;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = len[unit / dm.Hkv];
@@ -616,6 +670,7 @@ attn_combine_xsum_kernel(Dims dm, const int* __restrict__ len, Scratch sc, float
   int ts, nsp;
   split_plan(n, dm.m, sc.nsplit, ts, nsp);
   const int ch = c0 + 4 * (lane & 3);
+  const bool carried = !kPlain && (dm.base_mode == CAOTE_BASE_ACCUM || dm.base_mode == CAOTE_BASE_EXTERNAL);
   float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
   // A warp's time here is round trips to L2, not arithmetic: every load of a pass is issued before the first use.
   constexpr int kStep = (kCxThreads / 32) * 8;
@@ -630,7 +685,7 @@ attn_combine_xsum_kernel(Dims dm, const int* __restrict__ len, Scratch sc, float
         p[s] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (s < nsp) {
           st[s] = sc.pstat[((size_t)unit * sc.nsplit + s) * sc.Mpad + R];
-          p[s] = *reinterpret_cast<const float4*>(sc.po + (((size_t)unit * sc.nsplit + s) * sc.Mpad + R) * kD + ch);
+          p[s] = *reinterpret_cast<const float4*>(sc.po + (((size_t)unit * sc.nsplit + s) * dm.R + R) * D + ch);
         }
       }
       float mx = -INFINITY;
@@ -646,22 +701,81 @@ attn_combine_xsum_kernel(Dims dm, const int* __restrict__ len, Scratch sc, float
         acc.z = fmaf(p[s].z, w, acc.z); acc.w = fmaf(p[s].w, w, acc.w);
       }
       const float4 res = make_float4(acc.x / tot, acc.y / tot, acc.z / tot, acc.w / tot);
-      *reinterpret_cast<float4*>(o + ((size_t)unit * dm.R + R) * kD + ch) = res;
-      if (ch == 0) sc.stats[(size_t)unit * sc.Mpad + R] = mx + log2f(tot);
-      cs.x += res.x; cs.y += res.y; cs.z += res.z; cs.w += res.w;
+      *reinterpret_cast<float4*>(o + ((size_t)unit * dm.R + R) * D + ch) = res;
+      const bool in_x = kPlain || row_counted(dm, R);
+      if (ch == 0) {
+        const float stat = mx + log2f(tot);
+        sc.stats[(size_t)unit * sc.Mpad + R] = stat;
+        if (!kPlain && in_x && sc.sstat) sc.sstat[(size_t)unit * kTile + counted_index(dm, R)] = stat;
+        if (!kPlain && in_x && sc.few) {
+          // all tokens but the row's top one: the other splits, and the rest of the split that holds it
+          const float2* pt = sc.ptop + (size_t)unit * sc.nsplit * kTile + counted_index(dm, R);
+          float smax = -INFINITY, rest = 0.f;
+          int at = 0;
+          for (int s = 0; s < nsp; ++s) {
+            const float v = pt[s * kTile].x;
+            if (v > smax) { smax = v; at = s; }
+          }
+          for (int s = 0; s < nsp; ++s) rest += exp2f(st[s] - mx) * (s == at ? pt[s * kTile].y : 1.f);
+          sc.crest[(size_t)unit * kTile + counted_index(dm, R)] = rest / tot;
+        }
+      }
+      if (in_x) { cs.x += res.x; cs.y += res.y; cs.z += res.z; cs.w += res.w; }
     }
-  } else {
-    for (int R0 = warp * 8 + (lane >> 2); R0 < dm.R; R0 += 4 * kStep) {  // four rows in flight, summed in row order
+  } else if (kPlain || !vsum) {
+    const bool last_only = !kPlain && dm.base_mode == CAOTE_BASE_LAST_QUERY;
+    const int first = last_only ? dm.m - 1 : 0, stride = last_only ? dm.m : 1, Ms = kPlain ? dm.R : sc.Ms;
+    for (int t0 = warp * 8 + (lane >> 2); t0 < Ms; t0 += 4 * kStep) {  // four rows in flight, summed in row order
       float4 r[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int R = R0 + u * kStep;
-        r[u] = (R < dm.R) ? *reinterpret_cast<const float4*>(o + ((size_t)unit * dm.R + R) * kD + ch)
-                          : make_float4(0.f, 0.f, 0.f, 0.f);
+        const int t = t0 + u * kStep;
+        r[u] = (t < Ms) ? *reinterpret_cast<const float4*>(o + ((size_t)unit * dm.R + first + (size_t)t * stride) * D + ch)
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        if (R0 + u * kStep < dm.R) { cs.x += r[u].x; cs.y += r[u].y; cs.z += r[u].z; cs.w += r[u].w; }
+        if (t0 + u * kStep < Ms) { cs.x += r[u].x; cs.y += r[u].y; cs.z += r[u].z; cs.w += r[u].w; }
+    }
+  }
+  if (carried) {
+    // sum_j base_j v_j and sum_j base_j: lanes 2 i and 2 i + 1 take eight channels each of key i of a pass of 256
+    const float* bu = base + (size_t)unit * dm.cap;
+    const __nv_bfloat16* Vu = V + (size_t)unit * dm.cap * D + c0 + 8 * (tid & 1);
+    float y[8], hb = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) y[c] = 0.f;
+    constexpr int kPass = kCxThreads / 2, kFly = 4;
+    for (int j0 = tid >> 1; j0 < n; j0 += kFly * kPass) {
+      float bj[kFly];
+      uint4 raw[kFly];
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) {
+        const int j = j0 + u * kPass;
+        bj[u] = (j < n) ? bu[j] : 0.f;
+        raw[u] = (j < n) ? *reinterpret_cast<const uint4*>(Vu + (size_t)j * D) : make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) {
+        const uint32_t w[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
+        hb += bj[u];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          y[2 * e] = fmaf(bj[u], __uint_as_float(w[e] << 16), y[2 * e]);
+          y[2 * e + 1] = fmaf(bj[u], __uint_as_float(w[e] & 0xffff0000u), y[2 * e + 1]);
+        }
+      }
+    }
+#pragma unroll
+    for (int off = 2; off < 32; off <<= 1) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) y[c] += __shfl_xor_sync(0xffffffffu, y[c], off);
+      hb += __shfl_xor_sync(0xffffffffu, hb, off);
+    }
+    if (lane < 2) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) wy[warp][8 * lane + c] = y[c];
+      if (lane == 0) wy[warp][16] = hb;
     }
   }
   // the warp's eight row lanes of every channel quad, then the warps in order
@@ -676,12 +790,25 @@ attn_combine_xsum_kernel(Dims dm, const int* __restrict__ len, Scratch sc, float
   __syncthreads();
   if (tid < 4) {
     float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+    float hb = 0.f;
     for (int w = 0; w < kCxThreads / 32; ++w) {
       const float4 p = wpart[w][tid];
       t.x += p.x; t.y += p.y; t.z += p.z; t.w += p.w;
+      if (carried) {
+        t.x += wy[w][4 * tid]; t.y += wy[w][4 * tid + 1]; t.z += wy[w][4 * tid + 2]; t.w += wy[w][4 * tid + 3];
+        hb += wy[w][16];
+      }
     }
-    const float inv = 1.f / (float)dm.R;
-    *reinterpret_cast<float4*>(sc.X + (size_t)unit * kD + c0 + 4 * tid) = make_float4(t.x * inv, t.y * inv, t.z * inv, t.w * inv);
+    const float H = kPlain ? (float)dm.R : (float)sc.Ms + hb, inv = H > 0.f ? 1.f / H : 0.f;
+    float* x = sc.X + (size_t)unit * D + c0 + 4 * tid;
+    if (!kPlain && vsum) {
+      const float4 v = *reinterpret_cast<const float4*>(vsum + (size_t)unit * D + c0 + 4 * tid);
+      const float fn = (float)n;
+      *reinterpret_cast<float4*>(x) = make_float4(v.x / fn, v.y / fn, v.z / fn, v.w / fn);
+    } else {
+      *reinterpret_cast<float4*>(x) = make_float4(t.x * inv, t.y * inv, t.z * inv, t.w * inv);
+    }
+    if (!kPlain && c0 == 0 && tid == 0) sc.hb[unit] = hb;
   }
 }
 
@@ -692,8 +819,10 @@ constexpr int kStatBytes = kTile * 4;             // the softmax statistic of th
 constexpr int kQStages = 4;                       // Q blocks: a stage is free again once its products are done
 constexpr int kSStages = 8;                       // their rows' statistics: free once the key threads have used them
 
+template <int D>
 inline size_t score_smem_bytes() {
-  return 1024 + (2 + kQStages) * (size_t)kTileBytes + kSStages * (size_t)kStatBytes + (kD + kScoreKeys) * sizeof(float) + 256;
+  return 1024 + (2 + kQStages) * (size_t)kTileBytesOf<D> + kSStages * (size_t)kStatBytes +
+         (D + 2 * kScoreKeys + kTile) * sizeof(float) + 256;
 }
 
 // 2^x for two arguments at once on the FMA pipe instead of the special-function unit: x = i + f with i the nearest
@@ -755,26 +884,49 @@ __device__ __forceinline__ void score_piece16(const uint32_t (&v)[16], const flo
   }
 }
 
+// The same for a few counted rows: besides the weights, the complements 1 - alpha of the key; a weight above one half
+// belongs to the row's top token, whose complement the attention pass has left in crest.
+__device__ __forceinline__ void score_piece16_few(const uint32_t (&v)[16], const float4 (&st)[4], const float* crest, float scale2,
+                                                  int R0, int M, int m, int need, float& h, float& rest) {
+  if (R0 >= M) return;
+  const float stf[16] = {st[0].x, st[0].y, st[0].z, st[0].w, st[1].x, st[1].y, st[1].z, st[1].w,
+                         st[2].x, st[2].y, st[2].z, st[2].w, st[3].x, st[3].y, st[3].z, st[3].w};
+  int rm = R0 % m;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const bool row = R0 + i < M;
+    const float a = (row && rm >= need) ? fast_exp2(fmaf(__uint_as_float(v[i]), scale2, -stf[i])) : 0.f;
+    h += a;
+    rest += row ? (a > 0.5f ? crest[i] : 1.f - a) : 0.f;
+    if (++rm == m) rm = 0;
+  }
+}
+
 // CAOTE scores of 256 keys of one unit. grid = (key tile pairs, units), 576 threads: warps 0..15 are the
 // key threads, two per key (warps 0..3 and 8..11 the first key tile, 4..7 and 12..15 the second; the
 // lower eight take rows 0..63 of every Q block, the upper eight rows 64..127), one lane of warp 16 issues
-// the products, one lane of warp 17 the copies.
+// the products, one lane of warp 17 the copies. tmQ: the counted rows (LAST_QUERY: the last row of every head).
+// kFew: complements without cancellation; kAccum: carried scores are added and written back.
+template <int D, bool kFew, bool kAccum>
 __global__ void __launch_bounds__(kScoreThreads, 1)
 score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
              const __grid_constant__ CUtensorMap tmV, Dims dm, const int* __restrict__ len, Scratch sc,
-             float* __restrict__ scores, int* status) {
+             float* __restrict__ base, float* __restrict__ scores, int* status) {
+  constexpr int kTB = kTileBytesOf<D>, kBoxes = D / 64, kSteps = D / 16;
   ptx::pdl_wait();
   ptx::pdl_trigger();
   extern __shared__ char smem_raw[];
   // (aligned by an offset into the array, not through an integer: the pointer keeps its address space, and what is
   // read and written through it compiles to shared-memory accesses, not generic ones)
   char* sm = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
-  char* Ks = sm;                                                     // [2] key tiles
-  char* Qst = Ks + 2 * kTileBytes;                                   // [kQStages] Q blocks
-  float* Sst = reinterpret_cast<float*>(Qst + kQStages * kTileBytes);  // [kSStages][kTile] row statistics
-  float* Xs = Sst + kSStages * kTile;                                // [kD]
-  float* hx = Xs + kD;                                               // [kScoreKeys] upper halves' sums
-  uint64_t* bars = reinterpret_cast<uint64_t*>(hx + kScoreKeys);
+  char* Ks = sm;                                                // [2] key tiles
+  char* Qst = Ks + 2 * kTB;                                     // [kQStages] Q blocks
+  float* Sst = reinterpret_cast<float*>(Qst + kQStages * kTB);  // [kSStages][kTile] row statistics
+  float* Xs = Sst + kSStages * kTile;                           // [D]
+  float* hx = Xs + D;                                           // [kScoreKeys] upper halves' sums
+  float* rx = hx + kScoreKeys;                                  // [kScoreKeys] kFew: their complements
+  float* crs = rx + kScoreKeys;                                 // [kTile] kFew: the counted rows' crest
+  uint64_t* bars = reinterpret_cast<uint64_t*>(crs + kTile);
   uint64_t *k_bar = &bars[0], *v_bar = &bars[1], *q_bar = &bars[2], *q_done = q_bar + kQStages, *st_bar = q_done + kQStages,
            *s_bar = st_bar + kSStages, *c_bar = s_bar + 2, *st_free = c_bar + 2;
   constexpr int kBars1 = 2 + 2 * kQStages + kSStages + 2;  // single arrivals (a copy's bytes, a commit)
@@ -784,8 +936,10 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   const int tid = threadIdx.x, warp = tid >> 5;
   const int unit = blockIdx.y, j0 = blockIdx.x * kScoreKeys;
   const int b = unit / dm.Hkv;
-  const int n = len[b], M = dm.R, m = dm.m;
-  if (n == 0 || n < m || n > dm.cap || j0 >= n) return;
+  const int n = len[b];
+  const bool last_only = kFew && dm.base_mode == CAOTE_BASE_LAST_QUERY;
+  const int M = kFew ? sc.Ms : dm.R, m = last_only ? 1 : dm.m;  // counted rows, and the block they are causal in
+  if (n == 0 || n < dm.m || n > dm.cap || j0 >= n) return;
   const int nblocks = (M + kTile - 1) / kTile;
 
   if (tid == 0) {
@@ -795,42 +949,44 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(tmem_slot, 512);
-  if (tid < kD) Xs[tid] = sc.X[(size_t)unit * kD + tid];
+  if (tid < D) Xs[tid] = sc.X[(size_t)unit * D + tid];
+  if (kFew && tid >= kTile && tid < 2 * kTile) crs[tid - kTile] = (tid - kTile < M) ? sc.crest[(size_t)unit * kTile + tid - kTile] : 0.f;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;  // key tile kk, buffer buf: columns [kk * 256 + buf * 128, + 128)
-  float h = 0.f;
+  float h = 0.f, rest_few = 0.f;
   const int j = j0 + (tid & (kScoreKeys - 1));  // key threads: this thread's key
   const int rhalf = tid >> 8;                   // key threads: which 64 rows of a Q block
 
   if (warp == 17) {
     // =============================== copies (one lane) ===============================
     if (tid == kKeyThreads + 32) {
-      mbar_expect_tx(k_bar, 2 * kTileBytes);
-      for (int kk = 0; kk < 2; ++kk) {
-        tma_load_2d(Ks + kk * kTileBytes, &tmK, 0, unit * dm.cap + j0 + kk * kTile, k_bar);
-        tma_load_2d(Ks + kk * kTileBytes + kHalfBytes, &tmK, 64, unit * dm.cap + j0 + kk * kTile, k_bar);
-      }
+      auto load_pair = [&](char* dst, const CUtensorMap* tm, uint64_t* bar) {  // the two tiles of this CTA's keys
+        mbar_expect_tx(bar, 2 * kTB);
+        for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+          for (int x = 0; x < kBoxes; ++x)
+            tma_load_2d(dst + kk * kTB + x * kHalfBytes, tm, 64 * x, unit * dm.cap + j0 + kk * kTile, bar);
+      };
+      load_pair(Ks, &tmK, k_bar);
+      const float* rstat = last_only ? sc.sstat + (size_t)unit * kTile : sc.stats + (size_t)unit * sc.Mpad;
       for (int rb = 0; rb < nblocks; ++rb) {
         const int st = rb % kQStages, ss = rb % kSStages;
         if (rb >= kQStages) mbar_wait_idle(&q_done[st], ((rb / kQStages) - 1) & 1, status);  // the products of block rb - 4 are done
-        char* qd = Qst + st * kTileBytes;
-        mbar_expect_tx(&q_bar[st], kTileBytes);
-        tma_load_2d(qd, &tmQ, 0, unit * M + rb * kTile, &q_bar[st]);
-        tma_load_2d(qd + kHalfBytes, &tmQ, 64, unit * M + rb * kTile, &q_bar[st]);
+        char* qd = Qst + st * kTB;
+        mbar_expect_tx(&q_bar[st], kTB);
+#pragma unroll
+        for (int x = 0; x < kBoxes; ++x) tma_load_2d(qd + x * kHalfBytes, &tmQ, 64 * x, unit * M + rb * kTile, &q_bar[st]);
         if (rb >= kSStages) mbar_wait_idle(&st_free[ss], ((rb / kSStages) - 1) & 1, status);  // block rb - 8 is summed
         mbar_expect_tx(&st_bar[ss], kStatBytes);
-        bulk_load(Sst + ss * kTile, sc.stats + (size_t)unit * sc.Mpad + (size_t)rb * kTile, kStatBytes, &st_bar[ss]);
+        bulk_load(Sst + ss * kTile, rstat + (size_t)rb * kTile, kStatBytes, &st_bar[ss]);
       }
       // the value rows of the CTA's keys, for the distances at the end: into the first two Q stages once the last
-      // product has read its Q block (a commit covers every product before it)
-      mbar_wait_idle(&q_done[(nblocks - 1) % kQStages], ((nblocks - 1) / kQStages) & 1, status);
-      mbar_expect_tx(v_bar, 2 * kTileBytes);
-      for (int kk = 0; kk < 2; ++kk) {
-        tma_load_2d(Qst + kk * kTileBytes, &tmV, 0, unit * dm.cap + j0 + kk * kTile, v_bar);
-        tma_load_2d(Qst + kk * kTileBytes + kHalfBytes, &tmV, 64, unit * dm.cap + j0 + kk * kTile, v_bar);
-      }
+      // product has read its Q block (a commit covers every product before it); a few rows are one block, which leaves
+      // stages 2 and 3 alone
+      if (!kFew) mbar_wait_idle(&q_done[(nblocks - 1) % kQStages], ((nblocks - 1) / kQStages) & 1, status);
+      load_pair(Qst + (kFew ? 2 * kTB : 0), &tmV, v_bar);
     }
   } else if (warp == 16) {
     // =============================== products (one lane) ===============================
@@ -843,12 +999,12 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         mbar_wait_idle(&q_bar[st], (rb / kQStages) & 1, status);
         if (rb >= 2) mbar_wait_idle(&c_bar[buf], ((rb - 2) >> 1) & 1, status);  // its S buffers have been read
         tc_fence_after();
-        const uint32_t q_addr = smem_u32(Qst + st * kTileBytes);
+        const uint32_t q_addr = smem_u32(Qst + st * kTB);
 #pragma unroll
         for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
-          for (int ks = 0; ks < 8; ++ks)
-            umma(tmem + kk * 256 + buf * 128, desc_k_major(k_addr + kk * kTileBytes, ks), desc_k_major(q_addr, ks), kIdesc, ks > 0);
+          for (int ks = 0; ks < kSteps; ++ks)
+            umma(tmem + kk * 256 + buf * 128, desc_k_major(k_addr + kk * kTB, ks), desc_k_major(q_addr, ks), kIdesc, ks > 0);
         }
         umma_commit(&s_bar[buf]);
         umma_commit(&q_done[st]);
@@ -867,6 +1023,10 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     const uint32_t t_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kk * 256 + rhalf * 64;
     const int lane = tid & 31;
     const int need = j - (n - m);  // row R sees key j iff (R % m) >= need
+    auto piece = [&](const uint32_t (&v)[16], const float4 (&st)[4], bool plain, int R0, float2 (&ha)[2]) {
+      if constexpr (kFew) score_piece16_few(v, st, crs + R0, scale2, R0, M, m, need, h, rest_few);
+      else score_piece16(v, st, scale2, plain, R0, M, m, need, ha, h);
+    };
     uint32_t va[16], vb[16];
     float4 sa[4], sb[4];
     float2 hacc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -887,17 +1047,17 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       tmem_ld16_wait(va);
       tmem_ld16_issue(t_s + 16, vb);
       lds16_issue(stc + 16, sb);
-      score_piece16(va, sa, scale2, plain, R0, M, m, need, hacc, h);
+      piece(va, sa, plain, R0, hacc);
       // piece 1; piece 2 on its way
       tmem_ld16_wait(vb);
       tmem_ld16_issue(t_s + 32, va);
       lds16_issue(stc + 32, sa);
-      score_piece16(vb, sb, scale2, plain, R0 + 16, M, m, need, hacc, h);
+      piece(vb, sb, plain, R0 + 16, hacc);
       // piece 2; piece 3 on its way
       tmem_ld16_wait(va);
       tmem_ld16_issue(t_s + 48, vb);
       lds16_issue(stc + 48, sb);
-      score_piece16(va, sa, scale2, plain, R0 + 32, M, m, need, hacc, h);
+      piece(va, sa, plain, R0 + 32, hacc);
       // piece 3; the S buffer is free, the next block's piece 0 on its way
       tmem_ld16_wait(vb);
       tc_fence_before();
@@ -911,24 +1071,30 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         tmem_ld16_issue(t_lane + (buf ^ 1) * 128, va);
         lds16_issue(Sst + ss1 * kTile + rhalf * 64, sa);
       }
-      score_piece16(vb, sb, scale2, plain, R0 + 48, M, m, need, hacc, h);
+      piece(vb, sb, plain, R0 + 48, hacc);
       __syncwarp();
       if (lane == 0) mbar_arrive(&st_free[ss]);  // ... and is done with the block's statistics
     }
     h += (hacc[0].x + hacc[0].y) + (hacc[1].x + hacc[1].y);
   }
 
-  // ---- the two halves of a key add up; then c_j = w_j / (1 - w_j) * ||X - v_j||, w_j = h_j / M ----
-  if (tid >= kScoreKeys && tid < kKeyThreads) hx[tid - kScoreKeys] = h;
+  // ---- the two halves of a key add up; then c_j = w_j / (1 - w_j) * ||X - v_j||, w_j = h_j / H ----
+  if (tid >= kScoreKeys && tid < kKeyThreads) {
+    hx[tid - kScoreKeys] = h;
+    if (kFew) rx[tid - kScoreKeys] = rest_few;
+  }
   __syncthreads();
-  if (tid < kScoreKeys) h += hx[tid];
-  if (tid < kScoreKeys) mbar_wait(v_bar, 0, status);
+  if (tid < kScoreKeys) {
+    h += hx[tid];
+    if (kFew) rest_few += rx[tid];
+    mbar_wait(v_bar, 0, status);
+  }
   if (tid < kScoreKeys && j < n) {
-    // the key's value row: 16 chunks of 8 channels in the staged tile (two boxes of 64 channels, 128-byte swizzle)
-    const char* vt = Qst + (tid >> 7) * kTileBytes;
+    // the key's value row: chunks of 8 channels in the staged tile (boxes of 64 channels, 128-byte swizzle)
+    const char* vt = Qst + (kFew ? 2 * kTB : 0) + (tid >> 7) * kTB;
     float acc = 0.f;
 #pragma unroll
-    for (int c = 0; c < 16; ++c) {
+    for (int c = 0; c < D / 8; ++c) {
       const uint4 raw = *reinterpret_cast<const uint4*>(vt + tile_off(tid & (kTile - 1), c));
       const uint32_t w4[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
@@ -939,14 +1105,58 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         acc = fmaf(d1, d1, acc);
       }
     }
-    const float Htot = (float)M;
-    const float rest = Htot - h;
-    const float ratio = (rest > 0.f) ? h / rest : INFINITY;
-    scores[(size_t)unit * dm.cap + j] = (ratio == 0.f) ? 0.f : ((ratio == INFINITY) ? INFINITY : ratio * sqrtf(acc));
+    float rest = kFew ? rest_few : (float)M - h;  // (1 - w_j) H
+    const size_t slot = (size_t)unit * dm.cap + j;
+    if (kAccum) {
+      const float bj = base[slot];
+      rest += sc.hb[unit] - bj;
+      h += bj;
+      base[slot] = h;
+    }
+    float ratio = 0.f;
+    if (h > 0.f) ratio = (rest > 0.f) ? h / rest : INFINITY;
+    scores[slot] = (ratio == 0.f) ? 0.f : ((ratio == INFINITY) ? INFINITY : ratio * sqrtf(acc));
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, 512);
+}
+
+// The scores when the caller supplies the weights (EXTERNAL): h_j = base_j, one pass over V. grid = (ceil(cap / 64),
+// units), 256 threads: four threads per token, D / 4 channels each.
+template <int D>
+__global__ void __launch_bounds__(256)
+score_external_kernel(Dims dm, const __nv_bfloat16* __restrict__ V, const int* __restrict__ len, Scratch sc,
+                      const float* __restrict__ base, float* __restrict__ scores) {
+  ptx::pdl_wait();
+  ptx::pdl_trigger();
+  const int unit = blockIdx.y, n = len[unit / dm.Hkv], j = blockIdx.x * 64 + (threadIdx.x >> 2), part = threadIdx.x & 3;
+  if (n < dm.m || n > dm.cap || blockIdx.x * 64 >= n) return;
+  float acc = 0.f;
+  if (j < n) {
+    const uint4* row = reinterpret_cast<const uint4*>(V + ((size_t)unit * dm.cap + j) * D);
+    const float4* x = reinterpret_cast<const float4*>(sc.X + (size_t)unit * D);
+#pragma unroll
+    for (int i = 0; i < D / 32; ++i) {  // the four threads' chunks of 8 channels side by side
+      const int c = 4 * i + part;
+      const uint4 raw = row[c];
+      const float4 a = x[2 * c], b = x[2 * c + 1];
+      const float d0 = a.x - __uint_as_float(raw.x << 16), d1 = a.y - __uint_as_float(raw.x & 0xffff0000u);
+      const float d2 = a.z - __uint_as_float(raw.y << 16), d3 = a.w - __uint_as_float(raw.y & 0xffff0000u);
+      const float d4 = b.x - __uint_as_float(raw.z << 16), d5 = b.y - __uint_as_float(raw.z & 0xffff0000u);
+      const float d6 = b.z - __uint_as_float(raw.w << 16), d7 = b.w - __uint_as_float(raw.w & 0xffff0000u);
+      acc = fmaf(d0, d0, fmaf(d1, d1, fmaf(d2, d2, fmaf(d3, d3, acc))));
+      acc = fmaf(d4, d4, fmaf(d5, d5, fmaf(d6, d6, fmaf(d7, d7, acc))));
+    }
+  }
+  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+  if (part == 0 && j < n) {
+    const size_t slot = (size_t)unit * dm.cap + j;
+    const float h = base[slot], rest = sc.hb[unit] - h;
+    const float ratio = h > 0.f ? (rest > 0.f ? h / rest : INFINITY) : 0.f;
+    scores[slot] = (ratio == 0.f) ? 0.f : ((ratio == INFINITY) ? INFINITY : ratio * sqrtf(acc));
+  }
 }
 
 }  // namespace prefill

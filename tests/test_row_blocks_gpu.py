@@ -1,0 +1,64 @@
+"""The tensor-core row-block kernels on the shapes between the single-query kernels and long blocks of a prompt: any base
+mode, head_dim 64, groups of more than 8, blocks of a few queries."""
+import pytest
+import torch
+
+from test_gpu_parity import dominant_case, make_case, run_score
+from parity import assert_close, check_scores_and_o, f32, oracle_for
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+# B, Hq, Hkv, d, cap, m, lens: lengths at the edges of key tiles (128) and key-tile pairs (256), of the key splits, and
+# of the block itself; counted rows around the 64 below which the complements are kept apart
+SHAPES = [
+    (2, 16, 1, 128, 300, 1, [128, 129]),        # one query, 16 heads per group
+    (3, 4, 1, 64, 1040, 1, [1, 256, 1025]),     # one query, head_dim 64, a single token
+    (1, 8, 1, 128, 2064, 1, [2049]),            # one query, 8 heads and (accum, external) carried scores
+    (2, 14, 2, 128, 272, 9, [9, 257]),          # 63 rows, a sequence that is nothing but its block
+    (1, 8, 1, 64, 1600, 8, [1537]),             # 64 rows
+    (1, 2, 1, 128, 4112, 128, [4097]),          # key splits, two row blocks
+    (2, 16, 1, 64, 4112, 2, [4096, 130]),       # key splits for one of two sequences
+]
+
+
+@pytest.mark.parametrize("mode", ["last_query", "chunk_sum", "accum", "external"])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_row_block_scores_match_oracle(shape, mode):
+    B, Hq, Hkv, d, cap, m, lens = shape
+    q, K, V, lens_t = make_case(900 + SHAPES.index(shape), B, Hq, Hkv, d, cap, m, torch.bfloat16, lens)
+    base = None
+    if mode in ("accum", "external"):
+        base = (torch.rand((B, Hkv, cap), generator=torch.Generator().manual_seed(6)) * 2.0).to(DEV)
+    base_in = None if base is None else base.clone()
+    _, _, o, scores = run_score(q, K, V, lens_t, m, mode, base)
+    r = oracle_for(q, K, V, lens_t, scale=d ** -0.5, n_new=m, base_mode=mode, base=base_in)
+    check_scores_and_o(r, scores, o, lens_t, f"{shape} {mode}")
+    if mode == "accum":
+        for b, n in enumerate(lens):
+            assert_close(f32(base)[b, :, :n], r["base"][b, :, :n], "accumulated base", rtol=1e-5, atol=1e-6)
+            assert torch.equal(base[b, :, n:], base_in[b, :, n:])
+    if mode == "external":
+        assert torch.equal(base, base_in)
+
+
+@pytest.mark.parametrize("eps", [1e-1, 1e-2, 1e-3])
+@pytest.mark.parametrize("shape", [
+    (1, 16, 1, 128, 700, 1, [640], "last_query"),      # one row block
+    (1, 8, 2, 64, 5000, 1, [4900], "accum"),           # the planted token in one of several key splits
+    (2, 8, 2, 128, 2100, 128, [2048, 700], "last_query"),  # the counted rows of a long block
+    (1, 7, 1, 128, 300, 9, [290], "chunk_sum"),        # 63 rows
+])
+def test_few_rows_that_agree_on_one_token(shape, eps):
+    """One token holds all but ~eps of every counted row's weight: the complement is the others' sum, not a difference
+    (tolerance as everywhere: at eps 1e-3 a difference of fp32 weights would lose it)."""
+    B, Hq, Hkv, d, cap, m, lens, mode = shape
+    q, K, V, lens_t = dominant_case(17 + Hq, B, Hq, Hkv, d, cap, m, torch.bfloat16, lens, eps, 77)
+    base = None
+    if mode == "accum":
+        base = (torch.rand((B, Hkv, cap), generator=torch.Generator().manual_seed(3)) * 1e-9).to(DEV)
+    base_in = None if base is None else base.clone()
+    _, _, o, scores = run_score(q, K, V, lens_t, m, mode, base)
+    r = oracle_for(q, K, V, lens_t, scale=d ** -0.5, n_new=m, base_mode=mode, base=base_in)
+    assert ((1.0 - r["w"][:, :, 77]) < 8 * eps).all()
+    check_scores_and_o(r, scores, o, lens_t, f"{shape} eps {eps}")
