@@ -35,6 +35,8 @@
 
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -247,6 +249,13 @@ __device__ __forceinline__ void tmem_ld16_wait(uint32_t (&r)[16]) {
         "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
       :: "memory");
 }
+__device__ __forceinline__ void tmem_st16u(uint32_t taddr, const uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+      ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]),
+        "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
+}
 // Sixteen floats from shared memory, issued where the statement stands (the compiler may not sink it towards the
 // first use: the point is to have the loads in flight while other work is done).
 __device__ __forceinline__ void lds16_issue(const float* p, float4 (&s)[4]) {
@@ -321,6 +330,12 @@ constexpr int kVStages = 2;
 constexpr int kRowThreads = 2 * kThreads;    // two threads per query row: each owns 64 of the tile's 128 keys
 constexpr int kAttnThreads = kRowThreads + 96;  // + MMA, K-load and V-load warps
 
+// The tensor pipe adds to an fp32 accumulator without rounding to nearest: every addition loses about 2^-25 of the running
+// value, always towards zero, so o drifts with the length of the chain (2 x 8 products per tile: 3e-8 x n / 8). After
+// every kShare tiles the row threads therefore move O to a second accumulator, which they add to in fp32.
+// (n 16 896: error of o against 64 bits 6.5e-5 -> 4.7e-6, what is left is the 16 bits of P; the attention pass 3.03 ->
+// 3.01 ms: it is a wait for a product that has nearly finished, and 64 columns, every eighth tile.)
+constexpr int kShare = 8;
 constexpr int kXchFloats = 5 * kRowThreads;     // half-row maxima and sums in turn, and the few-rows form's three closing values
 
 template <int D>
@@ -387,7 +402,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  // columns: S0 [0,128), S1 [128,256), O [256,384). P of a tile takes the place of its S once the row threads have
+  // columns: S0 [0,128), S1 [128,256), O [256,384), the finished shares of O [384,512). P of a tile takes the place of its S once the row threads have
   // read that: hi part in the buffer's columns [0,64), lo part in [64,128) (two bf16 per column), so P is double-
   // buffered like S and the softmax of a tile does not wait for the previous tile's O += P V
   const uint32_t tmem = *tmem_slot;
@@ -452,7 +467,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         tc_fence_after();
         const uint64_t vd = vdesc0 + (uint64_t)(((kt % kVStages) * kTB) >> 4);
         const uint32_t p_tmem = tmem + (kt & 1) * kKeys;
-        if (kt == 0) {
+        if (kt % kShare == 0) {  // a new share
           umma_ts(tmem + 256, p_tmem, vd, kIdescO, false);
         } else {
           umma_ts(tmem + 256, p_tmem, vd, kIdescO, true);
@@ -479,8 +494,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     const uint32_t t_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t t_o = t_lane + 256 + half * (D / 2);
     float m_ref = -INFINITY, l = 0.f;
-    // few counted rows (kFew): this thread's largest logit, its numerator and the sum of the other numerators; warps
-    // without a counted row skip that
+    // few counted rows (kFew): this thread's largest product, its numerator and the sum of the other numerators; warps
+    // without a counted row skip that (summing the exponentials a second time instead: 158 us against 104 us at 16 units,
+    // 896 rows, 6 128 tokens)
     float smax = -INFINITY, ptop = 0.f, lrest = 0.f;
     const bool counted = kFew && R < M && row_counted(dm, R);
     const bool keep_top = kFew && __any_sync(0xffffffffu, counted);
@@ -497,16 +513,16 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 #pragma unroll
         for (int i = 0; i < 64; ++i) sv[i] = (j0 + i < nvis) ? sv[i] : -INFINITY;
       }
-      float mx;
+      float raw_top;  // (scale2 > 0: the largest product is the largest logit)
       {
         float pm[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) pm[i] = sv[i] * scale2;
+        for (int i = 0; i < 8; ++i) pm[i] = sv[i];
 #pragma unroll
-        for (int i = 8; i < 64; ++i) pm[i & 7] = fmaxf(pm[i & 7], sv[i] * scale2);
-        mx = fmaxf(fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3])), fmaxf(fmaxf(pm[4], pm[5]), fmaxf(pm[6], pm[7])));
+        for (int i = 8; i < 64; ++i) pm[i & 7] = fmaxf(pm[i & 7], sv[i]);
+        raw_top = fmaxf(fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3])), fmaxf(fmaxf(pm[4], pm[5]), fmaxf(pm[6], pm[7])));
       }
-      const float mine = mx;
+      float mx = raw_top * scale2;
       // the other half of the row
       float* xm = xch + (kt & 1) * kRowThreads;
       xm[tid] = mx;
@@ -514,7 +530,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       mx = fmaxf(mx, xm[tid ^ kThreads]);
       // the reference moves only when a logit exceeds it by more than 8 (p <= 256 in between)
       const bool need = mx > m_ref + 8.f;
-      if (__any_sync(0xffffffffu, need)) {
+      const bool close = kt > 0 && kt % kShare == 0;  // O holds a finished share
+      if (close || __any_sync(0xffffffffu, need)) {
         const float corr = need ? fast_exp2(m_ref - mx) : 1.f;
         if (need) m_ref = mx;
         l *= corr;
@@ -522,57 +539,68 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         if (kt > 0) {
           mbar_wait(&o_bar[(kt - 1) & 1], ((kt - 1) >> 1) & 1, status);  // O += P V of the previous tile is done
           tc_fence_after();
+          const bool shares = kt > kShare;  // there is a sum of earlier shares
 #pragma unroll
-          for (int cc = 0; cc < D / 64; ++cc) {
-            float v[32];
-            tmem_ld32(t_o + cc * 32, v);
+          for (int cc = 0; cc < D / 32; ++cc) {
+            uint32_t v[16], w[16];
+            tmem_ld16_issue(t_o + cc * 16, v);
+            if (shares) tmem_ld16_issue(t_o + 128 + cc * 16, w);
+            tmem_ld16_wait(v);
+            if (shares) tmem_ld16_wait(w);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] *= corr;
-            tmem_st32(t_o + cc * 32, v);
+            for (int i = 0; i < 16; ++i) {
+              const float x = __uint_as_float(v[i]), y = shares ? __uint_as_float(w[i]) : 0.f;
+              v[i] = __float_as_uint(x * corr);
+              w[i] = __float_as_uint((close ? x + y : y) * corr);
+            }
+            if (!close) tmem_st16u(t_o + cc * 16, v);
+            if (close || shares) tmem_st16u(t_o + 128 + cc * 16, w);
           }
           tmem_st_wait();
         }
       }
       {
         const float neg_ref = -m_ref;
-        float ls[4] = {0.f, 0.f, 0.f, 0.f};
+        float ls[4] = {0.f, 0.f, 0.f, 0.f}, rs[4] = {0.f, 0.f, 0.f, 0.f};
         uint32_t hi[32], lo[32];  // column c = keys 2c (low half) and 2c + 1
+        auto numerators = [&](auto top) {  // top: rs sums the numerators of all keys but the tile's largest
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
-          // P = hi + lo, hi truncated and lo rounded to bf16 (16 significant bits together); plain bit
-          // operations, so the conversion unit is left to the exponentials
-          const float p0 = fast_exp2(fmaf(sv[2 * c], scale2, neg_ref));
-          const float p1 = fast_exp2(fmaf(sv[2 * c + 1], scale2, neg_ref));
-          const uint32_t b0 = __float_as_uint(p0), b1 = __float_as_uint(p1);
-          hi[c] = __byte_perm(b0, b1, 0x7632);
-          const float r0 = p0 - __uint_as_float(b0 & 0xffff0000u), r1 = p1 - __uint_as_float(b1 & 0xffff0000u);
-          lo[c] = __byte_perm(__float_as_uint(r0) + 0x8000u, __float_as_uint(r1) + 0x8000u, 0x7632);  // rounded
-          ls[c & 3] += p0 + p1;
-        }
+          for (int c = 0; c < 32; ++c) {
+            // P = hi + lo, hi truncated and lo rounded to bf16 (16 significant bits together); plain bit
+            // operations, so the conversion unit is left to the exponentials
+            const float p0 = fast_exp2(fmaf(sv[2 * c], scale2, neg_ref));
+            const float p1 = fast_exp2(fmaf(sv[2 * c + 1], scale2, neg_ref));
+            const uint32_t b0 = __float_as_uint(p0), b1 = __float_as_uint(p1);
+            hi[c] = __byte_perm(b0, b1, 0x7632);
+            const float r0 = p0 - __uint_as_float(b0 & 0xffff0000u), r1 = p1 - __uint_as_float(b1 & 0xffff0000u);
+            lo[c] = __byte_perm(__float_as_uint(r0) + 0x8000u, __float_as_uint(r1) + 0x8000u, 0x7632);  // rounded
+            ls[c & 3] += p0 + p1;
+            if constexpr (decltype(top)::value) {
+              if (sv[2 * c] != raw_top) rs[c & 3] += p0;
+              if (sv[2 * c + 1] != raw_top) rs[c & 3] += p1;
+            }
+          }
+        };
+        if (kFew && keep_top) numerators(std::true_type{});
+        else numerators(std::false_type{});
         // P goes where S was: both halves of the row have read their S columns (the barrier above), and the
         // product that read the buffer's previous P was issued before the product that formed this S
         const uint32_t t_p = t_lane + (kt & 1) * kKeys + half * 32;  // this half's 64 keys = 32 packed columns
         tmem_st32u(t_p, hi);
         tmem_st32u(t_p + 64, lo);
         tmem_st_wait();
-        l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
+        const float lt = (ls[0] + ls[1]) + (ls[2] + ls[3]);
+        l += lt;
         if (kFew && keep_top) {
-          // the same numerators once more, the tile's largest (every copy of it but one) left out
-          float rest[4] = {0.f, 0.f, 0.f, 0.f};
-          int copies = 0;
-#pragma unroll
-          for (int c = 0; c < 64; ++c) {
-            const bool top = sv[c] * scale2 == mine;
-            rest[c & 3] += top ? 0.f : fast_exp2(fmaf(sv[c], scale2, neg_ref));
-            copies += top ? 1 : 0;
-          }
-          const float pt = (mine == -INFINITY) ? 0.f : fast_exp2(mine + neg_ref);
-          float r = (rest[0] + rest[1]) + (rest[2] + rest[3]) + (float)(copies - 1) * pt;
-          const bool bigger = mine > smax;
+          // one copy of the tile's largest numerator stays apart, any other copies join the rest (their number from the
+          // two sums: pt is the largest of 64 terms, so the sums' rounding is far below half of it)
+          const float pt = fast_exp2(fmaf(raw_top, scale2, neg_ref)), rt = (rs[0] + rs[1]) + (rs[2] + rs[3]);
+          float r = rt + (pt > 0.f ? rintf((lt - rt) / pt) - 1.f : 0.f) * pt;
+          const bool bigger = raw_top > smax;
           r += bigger ? ptop : pt;
           lrest += r;
           ptop = bigger ? pt : ptop;
-          smax = bigger ? mine : smax;
+          smax = bigger ? raw_top : smax;
         }
       }
       const int n_valid = min(kKeys, n - (kt0 + kt) * kKeys);
@@ -620,6 +648,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     for (int cc = 0; cc < D / 64; ++cc) {
       float v[32];
       tmem_ld32(t_o + cc * 32, v);  // collective: every lane takes part, rows beyond M just do not store
+      if (ntiles > kShare) {
+        float w[32];
+        tmem_ld32(t_o + 128 + cc * 32, w);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] += w[i];
+      }
       if (R < M) {
 #pragma unroll
         for (int i = 0; i < 32; i += 4)
