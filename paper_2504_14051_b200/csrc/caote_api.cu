@@ -762,24 +762,26 @@ static int launch_post_evict(const Dims& dm, const void* q, const void* K, const
   const int* tag = ws ? reinterpret_cast<const int*>(ws) + kStatTagIndex : nullptr;
   const float* stats = ws ? reinterpret_cast<const float*>(ws + kHeaderBytes) : nullptr;
   const int stat_stride = (dm.R + prefill::kTile - 1) / prefill::kTile * prefill::kTile;
-  // Blocks of queries in bf16 / d 128 may have per-row statistics in the workspace (only the device knows which path
+  // Blocks of queries in bf16 may have per-row statistics in the workspace (only the device knows which path
   // scored them): the kernel for that case goes first and returns at once if they are not there; the general
   // kernel after it returns at once if they are.
   int rows_kernel = 0;
-  if constexpr (std::is_same<T, __nv_bfloat16>::value && D == 128) {
+  if constexpr (std::is_same<T, __nv_bfloat16>::value) {
     if (ws && dm.m > 1 && aligned(o, 16) && aligned(o_post, 16)) {
-      rc = allow_smem(post::post_evict_rows_kernel, post::rows_smem_bytes());
+      rc = allow_smem(post::post_evict_tc_kernel<D>, post::tc_smem_bytes<D>());
       if (rc) return rc;
-      dim3 rgrid((dm.R + post::kBlockRows - 1) / post::kBlockRows, dm.units);
-      CAOTE_LAUNCH("post_evict_rows_kernel", st, post::post_evict_rows_kernel<<<rgrid, 256, post::rows_smem_bytes(), st>>>(
-          dm, (const T*)q, (const T*)K, (const T*)V, len, evict_idx, max_evict, n_evict, o, o_post, tag, stats, stat_stride));
+      dim3 rgrid((dm.R + prefill::kTile - 1) / prefill::kTile, dm.units);
+      CAOTE_LAUNCH("post_evict_tc_kernel", st,
+                   launch_pdl(post::post_evict_tc_kernel<D>, rgrid, dim3(post::kTcThreads), post::tc_smem_bytes<D>(), st, dm, (const T*)q,
+                              (const T*)K, (const T*)V, len, evict_idx, max_evict, n_evict, o, o_post, tag, stats, stat_stride,
+                              reinterpret_cast<int*>(const_cast<char*>(ws))));
       rows_kernel = 1;
     }
   }
   dim3 grid((dm.R + post::kRows - 1) / post::kRows, dm.units);
-  CAOTE_LAUNCH("post_evict_kernel", st, post::post_evict_kernel<T, D><<<grid, 32 * post::kRows, smem, st>>>(
-      dm, (const T*)q, (const T*)K, (const T*)V, len, evict_idx, max_evict, n_evict, o, o_post, tag, stats, stat_stride,
-      rows_kernel));
+  CAOTE_LAUNCH("post_evict_kernel", st,
+               launch_pdl(post::post_evict_kernel<T, D>, grid, dim3(32 * post::kRows), smem, st, dm, (const T*)q, (const T*)K,
+                          (const T*)V, len, evict_idx, max_evict, n_evict, o, o_post, tag, stats, stat_stride, rows_kernel));
   return CAOTE_OK;
 }
 
@@ -1154,7 +1156,7 @@ int caote_compact(const caote_params_t* p, void* K, void* V, float* base, int32_
   const int row_bytes = dm.D * (p->dtype == CAOTE_BF16 ? 2 : 4);
   cudaStream_t st = (cudaStream_t)stream;
   if (mode == CAOTE_COMPACT_FILL) {
-    CAOTE_LAUNCH("compact_fill_kernel", st, launch_pdl(sel::compact_fill_kernel, dim3(dm.units), dim3(256), 0, st, dm.Hkv, dm.cap, row_bytes, (char*)K, (char*)V, base, pos,
+    CAOTE_LAUNCH("compact_fill_kernel", st, launch_pdl(sel::compact_fill_kernel, dim3(dm.units), dim3(dm.m > 16 ? sel::kSelThreads : 256), 0, st, dm.Hkv, dm.cap, row_bytes, (char*)K, (char*)V, base, pos,
                                                        len, evict_idx, max_evict, n_evict));
   } else {
     dim3 grid(dm.units, 3);

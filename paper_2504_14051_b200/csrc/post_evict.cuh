@@ -9,11 +9,12 @@
 // and o; the kind of statistics present is a tag in the workspace header. Otherwise the normaliser is
 // recomputed with one pass over K (fp32 on the CUDA cores, any dtype, head_dim 64 or 128).
 // grid = (ceil(R / kRows), units), 256 threads: one warp per query row.
-// Blocks of queries with per-row statistics (the tensor-core prefill kernels) have a kernel of their own further
-// down, which shares the evicted rows among 32 query rows; this one then leaves those calls alone.
+// Blocks of queries with per-row statistics (the tensor-core row-block kernels) have a tensor-core kernel of their own
+// further down, which shares the evicted rows among 128 query rows; this one then leaves those calls alone.
 #pragma once
 
 #include "common.cuh"
+#include "prefill_tc.cuh"
 
 namespace caote {
 namespace post {
@@ -32,7 +33,9 @@ post_evict_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
                   const int* __restrict__ stat_tag, const float* __restrict__ stats, int prefill_stride,
                   int rows_kernel_ran) {
   constexpr int LD = D + 4, CPL = D / 32;  // channels per lane
-  if (rows_kernel_ran && stat_tag && *stat_tag == kStatPerRow) return;  // post_evict_rows_kernel has done the work
+  ptx::pdl_wait();
+  ptx::pdl_trigger();
+  if (rows_kernel_ran && stat_tag && *stat_tag == kStatPerRow) return;  // post_evict_tc_kernel has done the work
   extern __shared__ __align__(16) float smem[];
   float* Ks = smem;             // [kKeys][LD]
   float* Qs = Ks + kKeys * LD;  // [kRows][D]
@@ -117,131 +120,159 @@ post_evict_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
   }
 }
 
-// The same correction for blocks of queries whose rows' statistics the scoring call left behind (bf16, head_dim 128):
-// does nothing unless the workspace header says so. A CTA takes 16 query rows of a unit (two per warp) and walks
-// the unit's evicted slots 32 at a time: their K and V rows are gathered into shared memory once for all its query
-// rows; for the logits a lane is an evicted token (its K row against the warp's four query rows, both from shared
-// memory), for the weighted value sum a lane is four channels. grid = (ceil(R / 16), units), 256 threads.
-constexpr int kRowsPerWarp = 2, kBlockRows = 8 * kRowsPerWarp, kChunk = 32, kRowsD = 128, kKLd = kRowsD + 1;
-inline size_t rows_smem_bytes() {
-  return sizeof(float) * ((size_t)kBlockRows * kRowsD + (size_t)kChunk * kKLd + (size_t)kChunk * kRowsD + (size_t)kBlockRows * kChunk) +
-         sizeof(int) * kChunk;
+// The same correction for blocks of queries whose rows' statistics the scoring call left behind (bf16): does nothing
+// unless the workspace header says so. It is the attention pass over the evicted rows with a reference that is already
+// known, so a CTA takes 128 query rows of a unit (two threads per row) and walks the unit's evicted slots 128 at a time:
+// their K and V rows are gathered into swizzled tiles by plain loads, S = Q K_E^T and Y += P V_E (P as two bf16 parts) run
+// on tcgen05, and the weights 2^(s - stat) are formed in between. What bounds it is the chain of one tile (gather, product,
+// exponentials, product, write-out): 16 units x 896 rows x 128 evictions, 82 us on the CUDA cores (a CTA per 16 rows) -> 25 between events.
+// grid = (ceil(R / 128), units), 256 threads; TMEM columns: S / P [0, 128), Y [128, 128 + D).
+constexpr int kTcThreads = 256;
+template <int D>
+inline size_t tc_smem_bytes() {
+  return 1024 + 3 * (size_t)prefill::kTileBytesOf<D> + prefill::kTile * sizeof(int) + kTcThreads * sizeof(float) + 64;
 }
 
-__global__ void __launch_bounds__(256)
-post_evict_rows_kernel(Dims dm, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ K,
-                       const __nv_bfloat16* __restrict__ V, const int* __restrict__ len,
-                       const int* __restrict__ evict_idx, int max_evict, const int* __restrict__ n_evict,
-                       const float* __restrict__ o, float* __restrict__ o_post, const int* __restrict__ stat_tag,
-                       const float* __restrict__ stats, int stat_stride) {
-  constexpr int D = kRowsD;
+template <int D>
+__global__ void __launch_bounds__(kTcThreads, 2)
+post_evict_tc_kernel(Dims dm, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ K,
+                     const __nv_bfloat16* __restrict__ V, const int* __restrict__ len, const int* __restrict__ evict_idx,
+                     int max_evict, const int* __restrict__ n_evict, const float* o, float* o_post,
+                     const int* __restrict__ stat_tag, const float* __restrict__ stats, int stat_stride, int* status) {
+  using namespace prefill;
+  constexpr int kTB = kTileBytesOf<D>, kChunks = D / 8;  // 16-byte chunks of a row
+  ptx::pdl_wait();
+  ptx::pdl_trigger();
   if (*stat_tag != kStatPerRow) return;
-  extern __shared__ __align__(16) float smem[];
-  float* Qs = smem;                        // [kBlockRows][D]
-  float* Ks = Qs + kBlockRows * D;         // [kChunk][kKLd]   (odd row pitch: a lane per row, no bank conflicts)
-  float* Vs = Ks + kChunk * kKLd;          // [kChunk][D]
-  float* As = Vs + kChunk * D;             // [kBlockRows][kChunk] weights of the chunk
-  int* js = reinterpret_cast<int*>(As + kBlockRows * kChunk);  // [kChunk] slot of the evicted token, -1: none
-  const int unit = blockIdx.y, b = unit / dm.Hkv, h = unit % dm.Hkv;
-  const int n = len[b], m = dm.m;
+  extern __shared__ char smem_raw[];
+  char* sm = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
+  char *Qs = sm, *Ks = Qs + kTB, *Vs = Ks + kTB;
+  int* js = reinterpret_cast<int*>(Vs + kTB);               // [kTile] slot of the evicted token, -1: none
+  float* xa = reinterpret_cast<float*>(js + kTile);         // [kTcThreads] half rows' sums of weights
+  uint64_t* s_bar = reinterpret_cast<uint64_t*>(xa + kTcThreads);
+  uint64_t* y_bar = s_bar + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(y_bar + 1);
+
+  const int unit = blockIdx.y, b = unit / dm.Hkv;
+  const int n = len[b], m = dm.m, k = n_evict[b];
   if (n <= 0 || n < m || n > dm.cap) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int r0 = blockIdx.x * kBlockRows;
-  const float scale2 = dm.scale * 1.4426950408889634f;
-  auto row_off = [&](int r) { return (((size_t)b * dm.Hq + h * dm.G + r / m) * m + r % m) * D; };
-  for (int idx = tid; idx < kBlockRows * D; idx += 256) {
-    const int rr = idx / D, c = idx % D, r = r0 + rr;
-    Qs[idx] = (r < dm.R) ? __bfloat162float(q[row_off(r) + c]) : 0.f;
-  }
-  constexpr int RW = kRowsPerWarp;
-  int n_vis[RW];
-  float stat[RW], A[RW], Y[RW][4];
-#pragma unroll
-  for (int i = 0; i < RW; ++i) {
-    const int r = r0 + RW * warp + i;
-    n_vis[i] = (r < dm.R) ? n - m + (r % m) + 1 : 0;
-    stat[i] = (r < dm.R) ? stats[(size_t)unit * stat_stride + r] : 0.f;
-    A[i] = 0.f;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) Y[i][c] = 0.f;
-  }
-  const int k = n_evict[b];
-  const int* E = evict_idx + (size_t)unit * max_evict;
+  const int tid = threadIdx.x, warp = tid >> 5, r0 = blockIdx.x * kTile;
+  const int half = tid >> 7, r = r0 + (tid & (kTile - 1));
   const __nv_bfloat16* Ku = K + (size_t)unit * dm.cap * D;
   const __nv_bfloat16* Vu = V + (size_t)unit * dm.cap * D;
-  for (int e0 = 0; e0 < k; e0 += kChunk) {
-    __syncthreads();  // (the query rows are staged; the previous chunk is used up)
-    // gather: warp w brings tokens 4 w .. 4 w + 3 of the chunk, a lane four channels of a row
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int tok = 4 * warp + t, e = e0 + tok;
-      int j = (e < k) ? E[e] : -1;
-      if (j < 0 || j >= n) j = -1;
-      float kf[4] = {0.f, 0.f, 0.f, 0.f}, vf[4] = {0.f, 0.f, 0.f, 0.f};
-      if (j >= 0) {
-        const uint2 kr = *reinterpret_cast<const uint2*>(Ku + (size_t)j * D + 4 * lane);
-        const uint2 vr = *reinterpret_cast<const uint2*>(Vu + (size_t)j * D + 4 * lane);
-        kf[0] = __uint_as_float(kr.x << 16); kf[1] = __uint_as_float(kr.x & 0xffff0000u);
-        kf[2] = __uint_as_float(kr.y << 16); kf[3] = __uint_as_float(kr.y & 0xffff0000u);
-        vf[0] = __uint_as_float(vr.x << 16); vf[1] = __uint_as_float(vr.x & 0xffff0000u);
-        vf[2] = __uint_as_float(vr.y << 16); vf[3] = __uint_as_float(vr.y & 0xffff0000u);
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) Ks[tok * kKLd + 4 * lane + c] = kf[c];
-      *reinterpret_cast<float4*>(Vs + tok * D + 4 * lane) = make_float4(vf[0], vf[1], vf[2], vf[3]);
-      if (lane == 0) js[tok] = j;
+  const int* E = evict_idx + (size_t)unit * max_evict;
+  if (tid == 0) {
+    mbar_init(s_bar, 1);
+    mbar_init(y_bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) tmem_alloc(tmem_slot, 256);
+  for (int idx = tid; idx < kTile * kChunks; idx += kTcThreads) {
+    const int rr = idx / kChunks, c = idx % kChunks;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (r0 + rr < dm.R) v = *reinterpret_cast<const uint4*>(q + ((size_t)unit * dm.R + r0 + rr) * D + 8 * c);
+    *reinterpret_cast<uint4*>(Qs + ptx::tile_off(rr, c)) = v;
+  }
+  const float stat = (r < dm.R) ? stats[(size_t)unit * stat_stride + r] : INFINITY;  // (rows beyond R: weights 0)
+  const int n_vis = (r < dm.R) ? n - m + (r % m) + 1 : 0;
+  const float scale2 = dm.scale * 1.4426950408889634f;
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot, t_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  float A = 0.f;
+  int t = 0;
+  for (int e0 = 0; e0 < k; e0 += kTile, ++t) {
+    if (t > 0) mbar_wait(y_bar, (t - 1) & 1, status);  // the tiles of the evicted rows have been read
+    if (tid < kTile) {
+      int j = (e0 + tid < k) ? E[e0 + tid] : -1;
+      js[tid] = (j >= 0 && j < n) ? j : -1;
     }
     __syncthreads();
-    // weights: lane = evicted token of the chunk
-    {
-      const int j = js[lane];
-      float s[RW];
 #pragma unroll
-      for (int i = 0; i < RW; ++i) s[i] = 0.f;
-      const float* kp = Ks + lane * kKLd;
-#pragma unroll 8
-      for (int c = 0; c < D; c += 4) {
-        const float k0 = kp[c], k1 = kp[c + 1], k2 = kp[c + 2], k3 = kp[c + 3];
-#pragma unroll
-        for (int i = 0; i < RW; ++i) {
-          const float4 q4 = *reinterpret_cast<const float4*>(Qs + (RW * warp + i) * D + c);
-          s[i] = fmaf(q4.x, k0, fmaf(q4.y, k1, fmaf(q4.z, k2, fmaf(q4.w, k3, s[i]))));
-        }
+    for (int i = 0; i < kTile * kChunks / kTcThreads; ++i) {
+      const int idx = tid + i * kTcThreads, e = idx / kChunks, c = idx % kChunks, j = js[e];
+      uint4 kr = make_uint4(0u, 0u, 0u, 0u), vr = kr;
+      if (j >= 0) {
+        kr = *reinterpret_cast<const uint4*>(Ku + (size_t)j * D + 8 * c);
+        vr = *reinterpret_cast<const uint4*>(Vu + (size_t)j * D + 8 * c);
       }
-#pragma unroll
-      for (int i = 0; i < RW; ++i) {
-        const float a = (j >= 0 && j < n_vis[i]) ? exp2f(fmaf(s[i], scale2, -stat[i])) : 0.f;
-        A[i] += a;
-        As[(RW * warp + i) * kChunk + lane] = a;
-      }
+      *reinterpret_cast<uint4*>(Ks + ptx::tile_off(e, c)) = kr;
+      *reinterpret_cast<uint4*>(Vs + ptx::tile_off(e, c)) = vr;
     }
-    __syncwarp();  // (a warp reads only the weights it wrote)
-    // weighted values: lane = four channels
-#pragma unroll 4
-    for (int t = 0; t < kChunk; ++t) {
-      const float4 v4 = *reinterpret_cast<const float4*>(Vs + t * D + 4 * lane);
+    fence_async_smem();
+    __syncthreads();
+    if (tid == 0) {
+      tc_fence_after();
 #pragma unroll
-      for (int i = 0; i < RW; ++i) {
-        const float a = As[(RW * warp + i) * kChunk + t];
-        Y[i][0] = fmaf(a, v4.x, Y[i][0]);
-        Y[i][1] = fmaf(a, v4.y, Y[i][1]);
-        Y[i][2] = fmaf(a, v4.z, Y[i][2]);
-        Y[i][3] = fmaf(a, v4.w, Y[i][3]);
+      for (int ks = 0; ks < D / 16; ++ks)
+        umma(tmem, desc_k_major(smem_u32(Qs), ks), desc_k_major(smem_u32(Ks), ks), instr_desc_n(false, kTile), ks > 0);
+      umma_commit(s_bar);
+    }
+    mbar_wait(s_bar, t & 1, status);
+    tc_fence_after();
+    float sv[64];
+    tmem_ld32(t_lane + half * 64, *reinterpret_cast<float(*)[32]>(&sv[0]));
+    tmem_ld32(t_lane + half * 64 + 32, *reinterpret_cast<float(*)[32]>(&sv[32]));
+    uint32_t hi[32], lo[32];
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      const int2 jj = *reinterpret_cast<const int2*>(js + half * 64 + 2 * c);
+      const float p0 = (jj.x >= 0 && jj.x < n_vis) ? fast_exp2(fmaf(sv[2 * c], scale2, -stat)) : 0.f;
+      const float p1 = (jj.y >= 0 && jj.y < n_vis) ? fast_exp2(fmaf(sv[2 * c + 1], scale2, -stat)) : 0.f;
+      const uint32_t b0 = __float_as_uint(p0), b1 = __float_as_uint(p1);
+      hi[c] = __byte_perm(b0, b1, 0x7632);
+      lo[c] = pack_bf16(p0 - __uint_as_float(b0 & 0xffff0000u), p1 - __uint_as_float(b1 & 0xffff0000u));
+      A += p0 + p1;
+    }
+    tc_fence_before();
+    __syncthreads();  // both halves of every row have read their S columns
+    tc_fence_after();
+    tmem_st32u(t_lane + half * 32, hi);
+    tmem_st32u(t_lane + 64 + half * 32, lo);
+    tmem_st_wait();
+    tc_fence_before();
+    __syncthreads();
+    if (tid == 0) {
+      tc_fence_after();
+      constexpr uint32_t kIdesc = instr_desc_n(true, D);
+#pragma unroll
+      for (int ks = 0; ks < 8; ++ks) {
+        umma_ts(tmem + kTile, tmem + ks * 8, desc_mn_major(smem_u32(Vs), ks), kIdesc, t > 0 || ks > 0);
+        umma_ts(tmem + kTile, tmem + 64 + ks * 8, desc_mn_major(smem_u32(Vs), ks), kIdesc, true);
       }
+      umma_commit(y_bar);
     }
   }
+  xa[tid] = A;
+  __syncthreads();
+  const float rest = 1.f - (xa[tid] + xa[tid ^ kTile]);
+  if (t > 0) mbar_wait(y_bar, (t - 1) & 1, status);
+  tc_fence_after();
 #pragma unroll
-  for (int i = 0; i < RW; ++i) {
-    const int r = r0 + RW * warp + i;
-    const float rest = 1.f - warp_sum(A[i]);
+  for (int cc = 0; cc < D / 64; ++cc) {
+    const int c0 = half * (D / 2) + cc * 32;
+    float y[32];
+    if (t > 0) {
+      tmem_ld32(t_lane + kTile + c0, y);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) y[i] = 0.f;
+    }
     if (r < dm.R) {
-      const size_t at = row_off(r) + 4 * lane;
-      const float4 o4 = *reinterpret_cast<const float4*>(o + at);
-      float4 res = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (rest > 0.f) res = make_float4((o4.x - Y[i][0]) / rest, (o4.y - Y[i][1]) / rest, (o4.z - Y[i][2]) / rest, (o4.w - Y[i][3]) / rest);
-      *reinterpret_cast<float4*>(o_post + at) = res;
+      const size_t at = ((size_t)unit * dm.R + r) * D + c0;
+#pragma unroll
+      for (int i = 0; i < 32; i += 4) {
+        const float4 o4 = *reinterpret_cast<const float4*>(o + at + i);
+        float4 res = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (rest > 0.f) res = make_float4((o4.x - y[i]) / rest, (o4.y - y[i + 1]) / rest, (o4.z - y[i + 2]) / rest, (o4.w - y[i + 3]) / rest);
+        *reinterpret_cast<float4*>(o_post + at + i) = res;
+      }
     }
   }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, 256);
 }
 
 }  // namespace post

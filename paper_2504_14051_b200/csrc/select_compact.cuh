@@ -285,14 +285,22 @@ __device__ __forceinline__ void compact_fill_unit(int unit, int k, int Hkv, int 
   }
 }
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSelThreads)
 compact_fill_kernel(int Hkv, int cap, int row_bytes, char* __restrict__ K, char* __restrict__ V,
                     float* __restrict__ base, int* __restrict__ pos, const int* __restrict__ len,
                     const int* __restrict__ evict_idx, int max_evict, const int* __restrict__ n_evict) {
   ptx::pdl_wait();
   ptx::pdl_trigger();
-  compact_fill_unit(blockIdx.x, n_evict[blockIdx.x / Hkv], Hkv, cap, row_bytes, K, V, base, pos, len,
-                    evict_idx + (size_t)blockIdx.x * max_evict);
+  // (the searches are chains of dependent reads of the picks: from shared memory where they fit)
+  __shared__ int s_picks[kMaxSharedPicks];
+  const int k = n_evict[blockIdx.x / Hkv];
+  const int* E = evict_idx + (size_t)blockIdx.x * max_evict;
+  if (k > 1 && k <= kMaxSharedPicks) {
+    for (int i = threadIdx.x; i < k; i += blockDim.x) s_picks[i] = E[i];
+    __syncthreads();
+    E = s_picks;
+  }
+  compact_fill_unit(blockIdx.x, k, Hkv, cap, row_bytes, K, V, base, pos, len, E);
 }
 
 // A unit that evicts exactly one token, with FILL compaction: the argmin over (score bits, position) and the move of

@@ -3,6 +3,9 @@ mode, head_dim 64, groups of more than 8, blocks of a few queries."""
 import pytest
 import torch
 
+import oracle
+import paper_2504_14051_b200 as P
+
 from test_gpu_parity import dominant_case, make_case, run_score
 from parity import assert_close, check_scores_and_o, f32, oracle_for
 
@@ -62,3 +65,29 @@ def test_few_rows_that_agree_on_one_token(shape, eps):
     r = oracle_for(q, K, V, lens_t, scale=d ** -0.5, n_new=m, base_mode=mode, base=base_in)
     assert ((1.0 - r["w"][:, :, 77]) < 8 * eps).all()
     check_scores_and_o(r, scores, o, lens_t, f"{shape} eps {eps}")
+
+
+@pytest.mark.parametrize("case", [
+    # B, Hq, Hkv, d, cap, m, lens, budget, mode: evictions at the edges of a tile of 128 evicted rows, sequences that
+    # evict nothing or all that their first rows see, ragged row blocks
+    (2, 8, 2, 128, 500, 64, [500, 300], [372, 300], "last_query"),
+    (2, 4, 2, 64, 700, 33, [650, 600], [521, 473], "chunk_sum"),
+    (1, 14, 2, 128, 900, 128, [896], [512], "chunk_sum"),
+    (1, 6, 2, 64, 300, 100, [270], [13], "last_query"),
+])
+def test_corrected_output_of_query_blocks(case):
+    B, Hq, Hkv, d, cap, m, lens, budget, mode = case
+    q, K, V, lens_t = make_case(41 + m, B, Hq, Hkv, d, cap, m, torch.bfloat16, lens)
+    p, ws, o, scores = run_score(q, K, V, lens_t, m, mode)
+    ev = torch.zeros((B, Hkv, max(n - k for n, k in zip(lens, budget))), dtype=torch.int32, device=DEV)
+    ne = torch.zeros((B,), dtype=torch.int32, device=DEV)
+    P.caote_select_evict(p, scores, lens_t, torch.tensor(budget, dtype=torch.int32, device=DEV), None, ev, ne, ws)
+    o_post = torch.full_like(o, float("nan"))
+    P.caote_post_evict_output_ws(p, q, K, V, lens_t, ev, ne, o, o_post, ws)
+    assert P.caote_read_status(ws) == 0
+    evc, nec = ev.cpu().numpy(), ne.cpu().numpy()
+    ref = oracle.post_evict_output(f32(q), f32(K), f32(V), lens, [[evc[b, h, :nec[b]] for h in range(Hkv)] for b in range(B)],
+                                   scale=d ** -0.5, n_new=m)
+    # o and the evicted share both carry P's 16 bits (8e-6 of the largest value, about 4); what is left over after the
+    # subtraction is divided by the retained weight, 0.04 at the least here (13 of 270 tokens kept)
+    assert_close(f32(o_post), ref, f"{case}", atol=2e-3 if budget[0] * 4 < lens[0] else 2e-4)
