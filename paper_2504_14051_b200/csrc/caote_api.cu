@@ -13,7 +13,6 @@
 #include "decode_tc.cuh"
 #include "generic_score.cuh"
 #include "greedy.cuh"
-#include "greedy_cluster.cuh"
 #include "post_evict.cuh"
 #include "prefill_tc.cuh"
 #include "select_compact.cuh"
@@ -785,42 +784,17 @@ static int launch_post_evict(const Dims& dm, const void* q, const void* K, const
   return CAOTE_OK;
 }
 
+// Clusters of `c` CTAs of the greedy kernel, one CTA per SM, that can be resident on the current device at once.
 template <typename T, int D>
-static int launch_greedy(const Dims& dm, const void* V, const float* h, const int* len, const int* budget, const int* pos,
-                         int* evict_idx, int* order, int max_evict, int* n_evict, int* status, cudaStream_t st) {
-  const size_t smem = greedy::smem_bytes(dm.cap, D);
-  int rc = allow_smem(greedy::greedy_kernel<T, D>, smem);
-  if (rc) return rc;
-  CAOTE_LAUNCH("greedy_select_kernel", st, greedy::greedy_kernel<T, D><<<dm.units, greedy::kThreads, smem, st>>>(
-      dm.Hkv, dm.cap, (const T*)V, h, len, budget, pos, evict_idx, order, max_evict, n_evict, status));
-  return CAOTE_OK;
-}
-
-// Greedy eviction with the unit's value rows in the shared memory of a cluster (bf16, d 128; what 16 CTAs cannot
-// hold of a long unit stays in global memory and is swept from L2). *used = false: the shape does not fit (more
-// than 16 x 2048 tokens, or no cluster can run) or the one-CTA kernel is the better choice, and the caller takes that. Among the cluster sizes that hold a unit, the largest one of which the GPU can run as
-// many at once as there are units: more CTAs per unit make a pick faster, a second wave of clusters makes the call
-// twice as long.
-static int launch_greedy_cluster(const Dims& dm, const void* V, const float* h, const int* len, const int* budget,
-                                 const int* pos, int* evict_idx, int* order, int max_evict, int* n_evict, int* status,
-                                 cudaStream_t st, bool* used) {
-  *used = false;
-  if (!aligned(V, 16)) return CAOTE_OK;
-  int need = 1;  // the smallest cluster that holds the unit in shared memory, else the largest cluster
-  while (need < greedy_cl::kMaxC && (dm.cap + need - 1) / need > greedy_cl::kMaxRows) need *= 2;
-  if ((dm.cap + need - 1) / need > greedy_cl::kMaxShare) return CAOTE_OK;
-  // (the function's limits are set to the largest any launch may ask for, the same value every time: calls from
-  // several host threads then never see a limit below what they need)
-  CAOTE_CUDA(cudaFuncSetAttribute(greedy_cl::greedy_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  CAOTE_CUDA(cudaFuncSetAttribute(greedy_cl::greedy_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)greedy_cl::smem_bytes(greedy_cl::kMaxRows, greedy_cl::kMaxShare)));
-  int best_c = 0, best_rows = 0, best_got = 0;
-  for (int c = need; c <= greedy_cl::kMaxC; c *= 2) {
-    const int rows = ((dm.cap + c - 1) / c + 7) / 8 * 8;
-    const size_t smem = greedy_cl::smem_bytes(rows < greedy_cl::kMaxRows ? rows : greedy_cl::kMaxRows, rows);
+static int greedy_cluster_capacity(int c, size_t smem) {
+  static std::atomic<int> cached[64][greedy::kMaxC + 1];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int n = cached[dev][c].load(std::memory_order_acquire);
+  if (n == 0) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(c * dm.units));
-    cfg.blockDim = dim3(greedy_cl::kThreads);
+    cfg.gridDim = dim3((unsigned)c * 64u);
+    cfg.blockDim = dim3(greedy::kThreads);
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -830,51 +804,48 @@ static int launch_greedy_cluster(const Dims& dm, const void* V, const float* h, 
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int got = 0;
-    if (cudaOccupancyMaxActiveClusters(&got, greedy_cl::greedy_cluster_kernel, &cfg) != cudaSuccess || got <= 0) {
-      (void)cudaGetLastError();
-      continue;
-    }
-    if (best_c == 0 || got >= dm.units) {
-      best_c = c;
-      best_rows = rows;
-      best_got = got;
-    }
-    if (got < dm.units && best_c != c) break;  // larger clusters only fit fewer at once
+    n = -1;
+    if (cudaOccupancyMaxActiveClusters(&got, greedy::greedy_cluster_kernel<T, D>, &cfg) == cudaSuccess && got > 0) n = got;
+    (void)cudaGetLastError();
+    cached[dev][c].store(n, std::memory_order_release);
   }
-  if (best_c == 0) return CAOTE_OK;
-  {
-    // Worth it? Per pick the one-CTA kernel sweeps the unit's rows from L2 (measured: 19 us at 4224 rows, taken as
-    // 3 us + 3.8 ns per row), this one its share of them from shared memory plus a cluster barrier (measured: 5.25 us at
-    // 528 rows per CTA, 8.35 us at 768 + 288 left in global memory: about 4.2 us + 2 ns per row + 9 ns per row from
-    // L2); but the GPU runs fewer clusters at once than single CTAs, and with a handful of picks loading the rows is
-    // all there is.
-    const int in_smem = best_rows < greedy_cl::kMaxRows ? best_rows : greedy_cl::kMaxRows;
-    const double t_one = 3.0 + 0.0038 * dm.cap, t_cluster = 4.2 + 0.002 * in_smem + 0.009 * (best_rows - in_smem);
-    const double waves_one = (double)((dm.units + g_sm_count - 1) / g_sm_count);
-    const double waves_cluster = (double)((dm.units + best_got - 1) / best_got);
-    if (max_evict < 4 || t_one * waves_one < 1.2 * t_cluster * waves_cluster) return CAOTE_OK;
-  }
-  const int rows_smem = best_rows < greedy_cl::kMaxRows ? best_rows : greedy_cl::kMaxRows;
-  const size_t smem = greedy_cl::smem_bytes(rows_smem, best_rows);
+  return n > 0 ? n : 0;
+}
+
+// The largest cluster (the two sweeps over a unit's rows are shared among its CTAs; at least 256 rows each) of which the
+// GPU runs as many at once as there are units.
+template <typename T, int D>
+static int launch_greedy(const Dims& dm, const void* V, const float* h, const int* len, const int* budget, const int* pos,
+                         int* evict_idx, int* order, int max_evict, int* n_evict, int* status, cudaStream_t st) {
+  constexpr size_t kSmem = 192 * 1024;  // (with the kernel's static share below the 227 KB an SM has)
+  const size_t need = greedy::base_smem_bytes(dm.cap);
+  const size_t smem = need > kSmem ? need : kSmem;
+  // (the largest any launch may ask for, the same value every time: calls from several host threads then never see a
+  // limit below what they need)
+  CAOTE_CUDA(cudaFuncSetAttribute(greedy::greedy_cluster_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)greedy::base_smem_bytes(greedy::kMaxTokens)));
+  int c = 1;
+  while (2 * c <= greedy::kMaxC && dm.cap >= 512 * c && greedy_cluster_capacity<T, D>(2 * c, kSmem) >= dm.units) c *= 2;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(best_c * dm.units));
-  cfg.blockDim = dim3(greedy_cl::kThreads);
+  cfg.gridDim = dim3((unsigned)(c * dm.units));
+  cfg.blockDim = dim3(greedy::kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)best_c;
+  at[0].val.clusterDim.x = (unsigned)c;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // (the kernel starts with ptx::pdl_wait)
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
+  const int rows = (int)((smem - need) / (D * sizeof(T)));
   CAOTE_LAUNCH("greedy_cluster_kernel", st, {
-    cudaError_t e = cudaLaunchKernelEx(&cfg, greedy_cl::greedy_cluster_kernel, dm.Hkv, dm.cap, best_rows, rows_smem,
-                                       (const __nv_bfloat16*)V, h, len, budget, pos, evict_idx, order, max_evict, n_evict,
-                                       status);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, greedy::greedy_cluster_kernel<T, D>, dm.Hkv, dm.cap, rows, (const T*)V, h, len, budget,
+                                       pos, evict_idx, order, max_evict, n_evict, status);
     if (e != cudaSuccess) return cuda_fail(e, "greedy_cluster_kernel");
   });
-  *used = true;
   return CAOTE_OK;
 }
 
@@ -1129,12 +1100,7 @@ int caote_select_evict_greedy(const caote_params_t* p, const void* V, const floa
   cudaStream_t st = (cudaStream_t)stream;
   int* status = (int*)workspace;
   if (p->dtype == CAOTE_BF16) {
-    if (dm.D == 128) {
-      bool used = false;
-      rc = launch_greedy_cluster(dm, V, h, len, budget, pos, evict_idx, order, max_evict, n_evict, status, st, &used);
-      if (rc || used) return rc;
-      return launch_greedy<__nv_bfloat16, 128>(dm, V, h, len, budget, pos, evict_idx, order, max_evict, n_evict, status, st);
-    }
+    if (dm.D == 128) return launch_greedy<__nv_bfloat16, 128>(dm, V, h, len, budget, pos, evict_idx, order, max_evict, n_evict, status, st);
     return launch_greedy<__nv_bfloat16, 64>(dm, V, h, len, budget, pos, evict_idx, order, max_evict, n_evict, status, st);
   }
   if (dm.D == 128) return launch_greedy<float, 128>(dm, V, h, len, budget, pos, evict_idx, order, max_evict, n_evict, status, st);

@@ -1,244 +1,439 @@
-// Greedy multi-token eviction (Appendix B of the paper, the two-token derivation chained): evict the token
-// whose removal changes the current output least, renormalise the weights of the rest, update the output,
-// and score again, k times. One CTA per (sequence, KV head) unit.
+// Greedy multi-token eviction (Appendix B of the paper, the two-token derivation chained): evict the token whose removal
+// changes the current output least, renormalise the weights of the rest, update the output, and score again, k times.
 //
-// State kept on chip for the whole sequence of picks: the tokens' un-normalised weights h_j (negative once
-// evicted) and the current distances in shared memory, the un-normalised output Y = sum_j h_j v_j and the
-// normaliser H = sum_j h_j in registers / shared memory (X = Y / H). Every pick sweeps the unit's value rows
-// once (a warp per token, its lanes over the channels, || X - v_j ||^2 by plain subtraction as on the
-// scoring path): the rows come from HBM the first time and from L2 afterwards (a unit's rows are
-// cap * d * element size, 1 MB at 4224 tokens). Per pick: that sweep, a block-wide arg-min over
-// (score bits, position), and the rank-one update Y -= h_e v_e, H -= h_e.
+// A pick moves the output X = Y / H (Y = sum_j h_j v_j, H = sum_j h_j) by exactly the score of the token it evicts, and by
+// the triangle inequality no distance || X - v_j || changes by more than that. So the distances of all tokens are formed
+// once (a "build"), and from then on a token's distance is known to within the drift, the sum of the scores evicted since
+// it was last formed. A pick forms again only the distances of the tokens that can be the minimum: those whose lower bound
+// is not above the smallest upper bound, usually one to three. The pick is the same as if all distances had been formed
+// again (the same arithmetic on the same state, compared by (score bits, position, slot)); the bounds carry margins of 1e-5
+// for the rounding of scores and 5e-7 || X || per pick for that of X.
+//
+// Likewise only the tokens with small scores at the build can be picked: the `active` ones, found by a radix search, live in
+// registers (up to kReg per thread) with as many of their value rows in shared memory as fit. A pick whose score comes
+// within the drift of the others' smallest score is not taken but starts another build; the first pick after a build is
+// always safe.
+//
+// A thread-block cluster per unit: all CTAs share the two sweeps over the unit's rows (Y, and the distances of a build); the
+// picks are a chain of reductions and run on one CTA (two block barriers per pick), the others wait at the cluster barrier.
+// 8 units of 4 224 tokens, 128 picks: 708 us with every distance formed at every pick (clusters of 8, rows in shared
+// memory, a cluster barrier per pick) -> 209 us.
 #pragma once
 
 #include "common.cuh"
+#include "ptx.cuh"
 
 namespace caote {
 namespace greedy {
 
-constexpr int kThreads = 1024;
+constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
-constexpr int kMaxTokens = 24576;  // two floats per token in shared memory
+constexpr int kReg = 4;                  // active tokens per thread
+constexpr int kList = kReg * kThreads;
+constexpr int kMaxTokens = 24576;        // two floats per token in shared memory
+constexpr int kMaxC = 8;
+constexpr int kNone = 0x7fffffff;
 
-inline size_t smem_bytes(int cap, int D) {
-  return sizeof(float) * ((size_t)2 * cap + 2 * D + 2 * kWarps) + sizeof(unsigned long long) * kWarps + sizeof(int) * kWarps + 64;
+inline size_t base_smem_bytes(int cap) { return sizeof(float) * 2 * (((size_t)cap + 3) / 4 * 4) + 16; }
+
+// w / (1 - w) * dist from the un-normalised weight h and the sum H of all.
+__device__ __forceinline__ float score_of(float h, float dist, float H) {
+  if (!(H > 0.f && h > 0.f)) return 0.f;
+  const float rest = H - h;  // the others' weight (times H)
+  return rest > 0.f ? h / rest * dist : INFINITY;
 }
 
-// CPL consecutive channels of a row as floats, with one vector load (the row pointer is 16-byte aligned, CPL = 2 or 4).
-template <int CPL>
-__device__ __forceinline__ void load_channels(const __nv_bfloat16* p, float (&f)[CPL]) {
-  if constexpr (CPL == 4) {
-    const uint2 r = *reinterpret_cast<const uint2*>(p);
-    f[0] = __uint_as_float(r.x << 16); f[1] = __uint_as_float(r.x & 0xffff0000u);
-    f[2] = __uint_as_float(r.y << 16); f[3] = __uint_as_float(r.y & 0xffff0000u);
-  } else {
-    const uint32_t r = *reinterpret_cast<const uint32_t*>(p);
-    f[0] = __uint_as_float(r << 16); f[1] = __uint_as_float(r & 0xffff0000u);
+template <typename T>
+__device__ __forceinline__ float sq_dist16(uint4 raw, const float* x) {  // 16 bytes of a row against the channels x[]
+  const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+  float a = 0.f;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    if constexpr (sizeof(T) == 2) {
+      const float d0 = x[2 * c] - __uint_as_float(w[c] << 16), d1 = x[2 * c + 1] - __uint_as_float(w[c] & 0xffff0000u);
+      a = fmaf(d0, d0, fmaf(d1, d1, a));
+    } else {
+      const float d0 = x[c] - __uint_as_float(w[c]);
+      a = fmaf(d0, d0, a);
+    }
   }
-}
-template <int CPL>
-__device__ __forceinline__ void load_channels(const float* p, float (&f)[CPL]) {
-  if constexpr (CPL == 4) {
-    const float4 r = *reinterpret_cast<const float4*>(p);
-    f[0] = r.x; f[1] = r.y; f[2] = r.z; f[3] = r.w;
-  } else {
-    const float2 r = *reinterpret_cast<const float2*>(p);
-    f[0] = r.x; f[1] = r.y;
-  }
+  return a;
 }
 
+// grid = units x C CTAs in clusters of C; rows_smem: value rows that fit behind the two arrays of `cap` floats.
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads, 1)
-greedy_kernel(int Hkv, int cap, const T* __restrict__ V, const float* __restrict__ h_in, const int* __restrict__ len,
-              const int* __restrict__ budget, const int* __restrict__ pos, int* __restrict__ evict_idx,
-              int* __restrict__ order_out, int max_evict, int* __restrict__ n_evict, int* status) {
-  constexpr int CPL = D / 32;  // channels per lane: lane l owns channels [l * CPL, (l + 1) * CPL)
-  extern __shared__ __align__(16) float gsm[];
-  float* hs = gsm;                   // [cap] weight of the token, < 0 once evicted
-  float* ds = hs + cap;              // [cap] || X - v_j || of the current state
-  float* Ys = ds + cap;              // [D]   sum of h_j v_j over the tokens present
-  float* Ypart = Ys + D;             // [D]   scratch
-  float* wsum = Ypart + D;           // [2 * kWarps]
-  unsigned long long* wkey = reinterpret_cast<unsigned long long*>(wsum + 2 * kWarps);  // [kWarps]
-  int* wslot = reinterpret_cast<int*>(wkey + kWarps);                                      // [kWarps]
+greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, const float* __restrict__ h_in,
+                      const int* __restrict__ len, const int* __restrict__ budget, const int* __restrict__ pos,
+                      int* __restrict__ evict_idx, int* __restrict__ order_out, int max_evict, int* __restrict__ n_evict,
+                      int* status) {
+  constexpr int E = 16 / (int)sizeof(T);  // elements per 16-byte piece
+  constexpr int NCH = D / 8 / E;          // pieces per lane when eight lanes share a row: pieces l8, l8 + 8, ...
+  constexpr int CPL = D / 32;             // channels per lane when a warp shares a row
+  ptx::pdl_wait();
+  ptx::pdl_trigger();
+  extern __shared__ __align__(16) unsigned char gsm[];
+  float* hs = reinterpret_cast<float*>(gsm);            // [cap] weight of the token, < 0 once evicted  (rank 0)
+  float* ds = hs + (cap + 3) / 4 * 4;                   // [cap] distance at the build                 (rank 0)
+  T* rows = reinterpret_cast<T*>(ds + (cap + 3) / 4 * 4);  // [rows_smem][D] value rows of the first active tokens
+  __shared__ float Ys[D], Xs[D], part[D + 1], wpart[kWarps][D + 1];
   __shared__ float s_H;
-  __shared__ int s_pick;
+  __shared__ int s_ctl;                                 // after a round of picks: picks done, -1: all
+  __shared__ int act[kList];
+  __shared__ unsigned hist[256];
+  __shared__ int s_digit, s_below, s_incl, s_na;
+  __shared__ unsigned s_ub[kWarps], s_cb[kWarps], s_cp[kWarps], s_min[kWarps];
+  __shared__ int s_cs[kWarps], s_ci[kWarps], s_cnt[kWarps];
+  __shared__ float s_ch[kWarps];
 
-  const int unit = blockIdx.x, b = unit / Hkv, hd = unit % Hkv;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int C = (int)ptx::cluster_nctarank(), rank = (int)ptx::cluster_ctarank();
+  const int unit = (int)ptx::cluster_id_x(), b = unit / Hkv, hd = unit % Hkv;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sub = lane >> 3, l8 = lane & 7;
   const int n = len[b];
   int bud = budget[b];
   if (bud < 1) bud = 1;
   int k = n - bud;
   if (k < 0 || n > cap) k = 0;
   if (k > max_evict) {
-    if (tid == 0) set_status(status, CAOTE_ERR_OVERFLOW);
+    if (tid == 0 && rank == 0) set_status(status, CAOTE_ERR_OVERFLOW);
     k = 0;
   }
-  if (hd == 0 && tid == 0) n_evict[b] = k;
-  if (k == 0) return;
+  if (hd == 0 && rank == 0 && tid == 0) n_evict[b] = k;
+  if (k == 0) return;  // (the whole cluster leaves: no barrier is outstanding)
+  const int share = (n + C - 1) / C, r0 = min(n, rank * share), r1 = min(n, r0 + share);  // this CTA's rows in the sweeps
   const T* Vu = V + (size_t)unit * cap * D;
   const float* hu = h_in + (size_t)unit * cap;
   const int* pu = pos ? pos + (size_t)unit * cap : nullptr;
-  int* out = evict_idx + (size_t)unit * max_evict;
-  int* ord = order_out ? order_out + (size_t)unit * max_evict : nullptr;
 
-  // ---- H = sum h, Y = sum h v (one sweep; a warp per token, fixed order of the partial sums) ----
-  float hsum = 0.f;
-  for (int j = tid; j < n; j += kThreads) {
-    const float hj = fmaxf(hu[j], 0.f);
-    hs[j] = hj;
-    hsum += hj;
-  }
-  hsum = warp_sum(hsum);
-  if (lane == 0) wsum[warp] = hsum;
-  float yacc[CPL];
+  // ---- H and Y: every CTA its rows, in a fixed order of partial sums ----
+  {
+    if (rank == 0)
+      for (int j = tid; j < n; j += kThreads) hs[j] = fmaxf(hu[j], 0.f);
+    float hsum = 0.f, y[CPL];
 #pragma unroll
-  for (int c = 0; c < CPL; ++c) yacc[c] = 0.f;
-  __syncthreads();
-  for (int j = warp; j < n; j += kWarps) {
-    const float hj = hs[j];
-    float vf[CPL];
-    load_channels<CPL>(Vu + (size_t)j * D + lane * CPL, vf);
+    for (int c = 0; c < CPL; ++c) y[c] = 0.f;
+    constexpr int kFly = 8;  // rows in flight per warp
+    for (int j0 = r0 + warp; j0 < r1; j0 += kFly * kWarps) {
+      float hj[kFly], v[kFly][CPL];
 #pragma unroll
-    for (int c = 0; c < CPL; ++c) yacc[c] = fmaf(hj, vf[c], yacc[c]);
-  }
-  if (tid < D) Ys[tid] = 0.f;
-  __syncthreads();
-  for (int w = 0; w < kWarps; ++w) {  // warps add their parts one after the other: reproducible
-    if (warp == w) {
+      for (int u = 0; u < kFly; ++u) {
+        const int j = j0 + u * kWarps;
+        hj[u] = (j < r1) ? fmaxf(hu[j], 0.f) : 0.f;
+        const T* p = Vu + (size_t)min(j, r1 - 1) * D + lane * CPL;
 #pragma unroll
-      for (int c = 0; c < CPL; ++c) Ys[lane * CPL + c] += yacc[c];
+        for (int c = 0; c < CPL; ++c) v[u][c] = to_float(p[c]);
+      }
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) {
+        hsum += hj[u];
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) y[c] = fmaf(hj[u], v[u][c], y[c]);
+      }
     }
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) wpart[warp][lane * CPL + c] = y[c];
+    if (lane == 0) wpart[warp][D] = hsum;  // (every lane added the same weights)
     __syncthreads();
+    if (tid <= D) {
+      float t = 0.f;
+      for (int w = 0; w < kWarps; ++w) t += wpart[w][tid];
+      part[tid] = t;
+    }
   }
-  if (tid == 0) {
-    float H = 0.f;
-    for (int w = 0; w < kWarps; ++w) H += wsum[w];
-    s_H = H;
+  ptx::cluster_sync_all();
+  if (rank == 0 && tid <= D) {
+    float t = 0.f;
+    for (int i = 0; i < C; ++i) t += ptx::ld_dsmem_f32(ptx::map_to_rank(ptx::smem_u32(part + tid), i));
+    if (tid < D) Ys[tid] = t; else s_H = t;
   }
-  __syncthreads();
+  ptx::cluster_sync_all();
 
-  for (int t = 0; t < k; ++t) {
-    const float H = s_H;
-    const float inv_H = (H > 0.f) ? 1.f / H : 0.f;
-    // ---- distances of the tokens present to the current output: four rows per warp at a time, eight lanes per
-    //      row, each with the 16-byte pieces l, l + 8, ... of the row (a row's loads are contiguous over its lanes) and
-    //      three shuffle steps per sum; four such passes' loads in flight (a warp per row with a five-step sum kept
-    //      the SM's one shuffle per clock busy for most of the sweep) ----
+  int t = 0;
+  while (true) {
+    // ================= a build: the distances of all tokens still present to the current output =================
+    float H = ptx::ld_dsmem_f32(ptx::map_to_rank(ptx::smem_u32(&s_H), 0));
     {
-      constexpr int E = 16 / (int)sizeof(T);  // elements per 16-byte piece
-      constexpr int NCH = D / 8 / E;          // pieces per lane
-      constexpr int kPasses = 8 / NCH;  // the passes in flight hold 32 registers of row pieces
-      const int sub = lane >> 3, l8 = lane & 7;
+      const float inv_H = (H > 0.f) ? 1.f / H : 0.f;
+      if (tid < D) Xs[tid] = ptx::ld_dsmem_f32(ptx::map_to_rank(ptx::smem_u32(Ys + tid), 0)) * inv_H;
+      __syncthreads();
       float x[NCH][E];
 #pragma unroll
       for (int i = 0; i < NCH; ++i)
 #pragma unroll
-        for (int e = 0; e < E; ++e) x[i][e] = Ys[(l8 + 8 * i) * E + e] * inv_H;
-      for (int j0 = 4 * warp; j0 < n; j0 += 4 * kWarps * kPasses) {
+        for (int e = 0; e < E; ++e) x[i][e] = Xs[(l8 + 8 * i) * E + e];
+      constexpr int kPasses = 8 / NCH;  // passes of four rows per warp in flight
+      for (int j0 = r0 + 4 * warp; j0 < r1; j0 += 4 * kWarps * kPasses) {
         uint4 raw[kPasses][NCH];
-        bool live[kPasses];
+#pragma unroll
+        for (int u = 0; u < kPasses; ++u) {
+          const int j = min(j0 + u * 4 * kWarps + sub, r1 - 1);
+#pragma unroll
+          for (int i = 0; i < NCH; ++i) raw[u][i] = reinterpret_cast<const uint4*>(Vu + (size_t)j * D)[l8 + 8 * i];
+        }
 #pragma unroll
         for (int u = 0; u < kPasses; ++u) {
           const int j = j0 + u * 4 * kWarps + sub;
-          live[u] = j < n && hs[j] >= 0.f;
-          if (live[u]) {
-            const uint4* row = reinterpret_cast<const uint4*>(Vu + (size_t)j * D);
+          float a = 0.f;
 #pragma unroll
-            for (int i = 0; i < NCH; ++i) raw[u][i] = row[l8 + 8 * i];
+          for (int i = 0; i < NCH; ++i) a += sq_dist16<T>(raw[u][i], x[i]);
+          a += __shfl_xor_sync(0xffffffffu, a, 4);
+          a += __shfl_xor_sync(0xffffffffu, a, 2);
+          a += __shfl_xor_sync(0xffffffffu, a, 1);
+          if (l8 == 0 && j < r1) ptx::st_dsmem_f32(ptx::map_to_rank(ptx::smem_u32(ds + j), 0), sqrtf(a));
+        }
+      }
+    }
+    ptx::cluster_sync_all();
+
+    if (rank == 0) {
+      // ---- the active tokens: the smallest (score, position, slot) keys, `want` of them and at most 512 more ----
+      const int present = n - t, rem = k - t, want = min(present, min(rem + 32, 768));
+      unsigned kb = 0u, kp = 0u, ks = 0u;  // the largest key that is taken
+      int below = 0;
+      for (int pass = 0;; ++pass) {  // eight bits at a time: four passes over the score, four the position, two the slot
+        if (tid < 256) hist[tid] = 0u;
+        __syncthreads();
+        const int at = pass & 3, shift = pass < 8 ? 24 - 8 * at : 8 - 8 * at;
+        for (int j = tid; j < n; j += kThreads) {
+          const float h = hs[j];
+          if (h < 0.f) continue;
+          unsigned v = __float_as_uint(score_of(h, ds[j], H)), pre = kb;
+          if (pass >= 4) {
+            if (v != kb) continue;
+            v = (unsigned)(pu ? pu[j] : j);
+            pre = kp;
+          }
+          if (pass >= 8) {
+            if (v != kp) continue;
+            v = (unsigned)j;
+            pre = ks;
+          }
+          if (shift < 24 && ((v ^ pre) >> (shift + 8)) != 0u) continue;
+          atomicAdd(&hist[(v >> shift) & 255u], 1u);
+        }
+        __syncthreads();
+        if (warp == 0) {
+          unsigned c[8], sum = 0u;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) { c[q] = hist[8 * lane + q]; sum += c[q]; }
+          unsigned incl = sum;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const unsigned u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
+          }
+          const unsigned need = (unsigned)(want - below);
+          const unsigned reach = __ballot_sync(0xffffffffu, need <= incl);
+          const int f = reach ? __ffs((int)reach) - 1 : 31;
+          if (lane == f) {
+            unsigned run = incl - sum;
+            int q = 0;
+            for (; q < 7 && run + hist[8 * lane + q] < need; ++q) run += hist[8 * lane + q];
+            s_digit = 8 * lane + q;
+            s_below = below + (int)run;
+            s_incl = below + (int)(run + hist[8 * lane + q]);
           }
         }
+        __syncthreads();
+        const unsigned digit = (unsigned)s_digit << shift;
+        if (pass < 4) kb |= digit;
+        else if (pass < 8) kp |= digit;
+        else ks |= digit;
+        below = s_below;
+        if (s_incl <= want + 512 || pass == 9) {
+          const unsigned ones = (1u << shift) - 1u;
+          if (pass < 4) { kb |= ones; kp = 0xffffffffu; ks = 0xffffffffu; }
+          else if (pass < 8) { kp |= ones; ks = 0xffffffffu; }
+          else ks |= ones;
+          break;
+        }
+      }
+      if (tid == 0) s_na = 0;
+      __syncthreads();
+      float dmin = INFINITY;  // smallest distance among the other tokens
+      for (int j0 = 0; j0 < n; j0 += kThreads) {
+        const int j = j0 + tid;
+        bool in = false;
+        if (j < n && hs[j] >= 0.f) {
+          const unsigned v = __float_as_uint(score_of(hs[j], ds[j], H));
+          in = v < kb;
+          if (v == kb) {
+            const unsigned p = (unsigned)(pu ? pu[j] : j);
+            in = p < kp || (p == kp && (unsigned)j <= ks);
+          }
+          if (!in) dmin = fminf(dmin, ds[j]);
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        int at = 0;
+        if (lane == 0 && m) at = atomicAdd(&s_na, __popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+        if (in && at < kList) act[at] = j;  // (the order of the list does not matter: keys decide)
+      }
+      {
+        const unsigned m = __reduce_min_sync(0xffffffffu, __float_as_uint(dmin));
+        if (lane == 0) s_min[warp] = m;
+      }
+      __syncthreads();
+      const int na = min(s_na, kList), nu = (na + kThreads - 1) / kThreads;
+      dmin = __uint_as_float(__reduce_min_sync(0xffffffffu, s_min[lane & (kWarps - 1)]));
+      const float tau = __uint_as_float(min(kb, 0x7f800000u));
+      float hr[kReg], ar[kReg];  // weight (< 0: none, or evicted) and distance + drift at the time it was formed
+      unsigned pr[kReg];
+      int sr[kReg];
 #pragma unroll
-        for (int u = 0; u < kPasses; ++u) {
-          float acc = 0.f;
-          if (live[u]) {
+      for (int u = 0; u < kReg; ++u) {
+        const int i = tid + u * kThreads;
+        hr[u] = -1.f; ar[u] = 0.f; pr[u] = 0u; sr[u] = 0;
+        if (i < na) {
+          const int j = act[i];
+          sr[u] = j;
+          hr[u] = hs[j];
+          ar[u] = ds[j];
+          pr[u] = (unsigned)(pu ? pu[j] : j);
+        }
+      }
+      for (int idx = tid; idx < min(na, rows_smem) * (D / E); idx += kThreads)
+        reinterpret_cast<uint4*>(rows)[idx] = reinterpret_cast<const uint4*>(Vu + (size_t)act[idx / (D / E)] * D)[idx % (D / E)];
+      float xn = 0.f;
 #pragma unroll
-            for (int i = 0; i < NCH; ++i) {
-              const uint32_t w[4] = {raw[u][i].x, raw[u][i].y, raw[u][i].z, raw[u][i].w};
+      for (int c = 0; c < CPL; ++c) xn = fmaf(Xs[lane * CPL + c], Xs[lane * CPL + c], xn);
+      xn = sqrtf(warp_sum(xn));
+      __syncthreads();
+
+      // ================= picks =================
+      float drift = 0.f;
+      bool fresh = true;
+      while (t < k) {
+        // ---- the smallest upper bound ----
+        float rr[kReg], ub = INFINITY;
 #pragma unroll
-              for (int c = 0; c < 4; ++c) {
-                if constexpr (sizeof(T) == 2) {
-                  const float d0 = x[i][2 * c] - __uint_as_float(w[c] << 16);
-                  const float d1 = x[i][2 * c + 1] - __uint_as_float(w[c] & 0xffff0000u);
-                  acc = fmaf(d0, d0, fmaf(d1, d1, acc));
-                } else {
-                  const float d0 = x[i][c] - __uint_as_float(w[c]);
-                  acc = fmaf(d0, d0, acc);
-                }
-              }
+        for (int u = 0; u < kReg; ++u) {
+          rr[u] = 0.f;
+          if (u < nu && hr[u] >= 0.f) {
+            if (H > 0.f && hr[u] > 0.f) {
+              const float rest = H - hr[u];
+              rr[u] = rest > 0.f ? __fdividef(hr[u], rest) : INFINITY;
+              ub = fminf(ub, rr[u] * (ar[u] + drift) * 1.00001f);
+            } else {
+              ub = 0.f;  // a score of exactly zero
             }
           }
-          acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-          acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-          acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-          if (live[u] && l8 == 0) ds[j0 + u * 4 * kWarps + sub] = sqrtf(acc);
         }
-      }
-    }
-    __syncthreads();
-    // ---- arg-min of w_j / (1 - w_j) * dist_j over (score bits, position) ----
-    unsigned long long best = ~0ull;
-    int best_slot = -1;
-    for (int j = tid; j < n; j += kThreads) {
-      const float hj = hs[j];
-      if (hj < 0.f) continue;
-      float sc = 0.f;
-      if (H > 0.f && hj > 0.f) {
-        const float rest = H - hj;  // the others' weight (times H)
-        sc = (rest > 0.f) ? hj / rest * ds[j] : INFINITY;
-      }
-      const unsigned long long key = ((unsigned long long)__float_as_uint(sc) << 32) | (unsigned int)(pu ? pu[j] : j);
-      if (key < best) { best = key; best_slot = j; }
-    }
+        {
+          const unsigned m = __reduce_min_sync(0xffffffffu, __float_as_uint(ub));
+          if (lane == 0) s_ub[warp] = m;
+        }
+        __syncthreads();
+        ub = __uint_as_float(__reduce_min_sync(0xffffffffu, s_ub[lane & (kWarps - 1)]));
+        // ---- exact scores of the tokens that can be the minimum ----
+        unsigned cb = 0xffffffffu, cp = 0xffffffffu;
+        int cs = kNone, ci = 0;
+        float ch = 0.f;
+        const float inv_H = (H > 0.f) ? 1.f / H : 0.f;
+        auto offer = [&](int i, float h, unsigned p, int s, float sc) {
+          const unsigned v = __float_as_uint(sc);
+          if (v < cb || (v == cb && (p < cp || (p == cp && s < cs)))) { cb = v; cp = p; cs = s; ci = i; ch = h; }
+        };
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long ok = __shfl_xor_sync(0xffffffffu, best, o);
-      const int os = __shfl_xor_sync(0xffffffffu, best_slot, o);
-      if (ok < best) { best = ok; best_slot = os; }
+        for (int u = 0; u < kReg; ++u) {
+          const bool present_u = u < nu && hr[u] >= 0.f, weighs = H > 0.f && hr[u] > 0.f;
+          if (present_u && !weighs) offer(tid + u * kThreads, hr[u], pr[u], sr[u], 0.f);
+          const bool mine = present_u && weighs && !(rr[u] * fmaxf(ar[u] - drift, 0.f) * 0.99999f > ub);
+          unsigned mask = __ballot_sync(0xffffffffu, mine);
+          while (mask) {  // four tokens at a time, eight lanes each
+            const unsigned m1 = mask & (mask - 1u), m2 = m1 & (m1 - 1u), m3 = m2 & (m2 - 1u);
+            const unsigned ms = sub == 0 ? mask : (sub == 1 ? m1 : (sub == 2 ? m2 : m3));
+            const int p = ms ? __ffs((int)ms) - 1 : 0;
+            const int j = __shfl_sync(0xffffffffu, sr[u], p), idx = warp * 32 + p + u * kThreads;
+            const uint4* row = reinterpret_cast<const uint4*>(idx < rows_smem ? rows + (size_t)idx * D : Vu + (size_t)j * D);
+            float a = 0.f;
+#pragma unroll
+            for (int i = 0; i < NCH; ++i) {
+              const uint4 raw = row[l8 + 8 * i];
+              float x[E];
+#pragma unroll
+              for (int e = 0; e < E; ++e) x[e] = Ys[(l8 + 8 * i) * E + e] * inv_H;
+              a += sq_dist16<T>(raw, x);
+            }
+            a += __shfl_xor_sync(0xffffffffu, a, 4);
+            a += __shfl_xor_sync(0xffffffffu, a, 2);
+            a += __shfl_xor_sync(0xffffffffu, a, 1);
+            const int rk = __popc(mask & ((1u << lane) - 1u));
+            a = __shfl_sync(0xffffffffu, a, 8 * min(rk, 3));
+            if ((mask >> lane & 1u) && rk < 4) {
+              const float d = sqrtf(a);
+              ar[u] = d + drift;
+              offer(tid + u * kThreads, hr[u], pr[u], sr[u], score_of(hr[u], d, H));
+            }
+            mask = m3 & (m3 - 1u);
+          }
+        }
+        {
+          const unsigned b1 = __reduce_min_sync(0xffffffffu, cb);
+          const unsigned p1 = __reduce_min_sync(0xffffffffu, cb == b1 ? cp : 0xffffffffu);
+          const bool eq = cb == b1 && cp == p1;
+          const int s1 = (int)__reduce_min_sync(0xffffffffu, eq ? (unsigned)cs : (unsigned)kNone);
+          if (s1 == kNone ? lane == 0 : (eq && cs == s1)) {
+            s_cb[warp] = b1; s_cp[warp] = p1; s_cs[warp] = s1; s_ci[warp] = ci; s_ch[warp] = ch;
+          }
+        }
+        __syncthreads();
+        const int w16 = lane & (kWarps - 1);
+        const unsigned vb = s_cb[w16], vp = s_cp[w16];
+        const int vs = s_cs[w16];
+        const unsigned b1 = __reduce_min_sync(0xffffffffu, vb);
+        const unsigned p1 = __reduce_min_sync(0xffffffffu, vb == b1 ? vp : 0xffffffffu);
+        const bool eq = vb == b1 && vp == p1;
+        const int e = (int)__reduce_min_sync(0xffffffffu, eq ? (unsigned)vs : (unsigned)kNone);
+        if (e == kNone) { t = k; break; }  // (cannot happen with k < n; the same in every thread)
+        const int wi = __ffs((int)__ballot_sync(0xffffffffu, eq && vs == e)) - 1;
+        const int ei = s_ci[wi & (kWarps - 1)];
+        const float he = s_ch[wi & (kWarps - 1)], sc = __uint_as_float(b1);
+        if (!fresh && !(sc <= tau * (1.f - drift / dmin) * 0.99999f)) break;  // another token may be smaller: build again
+        // ---- evict e: Y -= h_e v_e, H -= h_e ----
+        if (tid < D) {
+          const T* row = ei < rows_smem ? rows + (size_t)ei * D : Vu + (size_t)e * D;
+          Ys[tid] -= he * to_float(row[tid]);
+        }
+        if ((ei & (kThreads - 1)) == tid) {
+#pragma unroll
+          for (int u = 0; u < kReg; ++u)
+            if (u == ei / kThreads) hr[u] = -1.f;
+          hs[e] = -1.f;
+          if (order_out) order_out[(size_t)unit * max_evict + t] = e;
+        }
+        H -= he;
+        drift += sc * 1.0001f + 5e-7f * (xn + drift);
+        fresh = false;
+        ++t;
+      }
+      __syncthreads();
+      if (tid == 0) {
+        s_H = H;
+        s_ctl = t < k ? t : -1;
+      }
     }
-    if (lane == 0) { wkey[warp] = best; wslot[warp] = best_slot; }
-    __syncthreads();
-    if (tid == 0) {
-      unsigned long long bk = wkey[0];
-      int bs = wslot[0];
-      for (int w = 1; w < kWarps; ++w)
-        if (wkey[w] < bk) { bk = wkey[w]; bs = wslot[w]; }
-      s_pick = bs;
-    }
-    __syncthreads();
-    const int e = s_pick;
-    if (e < 0) break;  // (cannot happen with k < n; keeps every index in bounds)
-    // ---- evict e: Y -= h_e v_e, H -= h_e ----
-    const float he = hs[e];
-    if (tid < D) Ys[tid] -= he * to_float(Vu[(size_t)e * D + tid]);
-    if (tid == 0) {
-      s_H = H - he;
-      if (ord) ord[t] = e;
-    }
-    __syncthreads();
-    if (tid == 0) hs[e] = -1.f;
-    __syncthreads();
+    ptx::cluster_sync_all();
+    t = ptx::ld_dsmem_s32(ptx::map_to_rank(ptx::smem_u32(&s_ctl), 0));
+    if (t < 0) break;
   }
+  ptx::cluster_sync_all();  // (nobody reads rank 0's shared memory any more)
+  if (rank != 0) return;
   // ---- the evicted slots in ascending order (the layout caote_compact expects) ----
-  __shared__ int s_count;
-  if (tid == 0) s_count = 0;
-  __syncthreads();
+  int* out = evict_idx + (size_t)unit * max_evict;
+  int run = 0;
   for (int j0 = 0; j0 < n; j0 += kThreads) {
     const int j = j0 + tid;
     const bool gone = j < n && hs[j] < 0.f;
     const unsigned m = __ballot_sync(0xffffffffu, gone);
-    if (lane == 0) wslot[warp] = __popc(m);
+    if (lane == 0) s_cnt[warp] = __popc(m);
     __syncthreads();
-    int before = s_count;
-    for (int w = 0; w < warp; ++w) before += wslot[w];
-    if (gone) out[before + __popc(m & ((1u << lane) - 1u))] = j;
-    __syncthreads();
-    if (tid == 0) {
-      int tot = s_count;
-      for (int w = 0; w < kWarps; ++w) tot += wslot[w];
-      s_count = tot;
+    int before = run;
+    for (int w = 0; w < kWarps; ++w) {
+      if (w < warp) before += s_cnt[w];
+      run += s_cnt[w];
     }
+    if (gone) out[before + __popc(m & ((1u << lane) - 1u))] = j;
     __syncthreads();
   }
 }

@@ -126,3 +126,51 @@ def test_one_greedy_pick_is_the_plain_selection_and_k0_evicts_nothing():
     assert ne1.tolist() == ne2.tolist() == [1, 1]
     P.caote_select_evict_greedy(p, V, h, lens, lens.clone(), None, ev2, None, ne2, ws)
     assert ne2.tolist() == [0, 0] and P.caote_read_status(ws) == 0
+
+
+@pytest.mark.parametrize("case", [
+    # n, k, weights: what makes the bounds of the pruned search fail or tie
+    (700, 300, "equal"),      # equal weights: every pick moves the output by as much as the scores differ
+    (3000, 40, "zeros"),      # most weights zero: their scores tie at 0, the position decides
+    (2600, 60, "same_rows"),  # equal weights and equal rows: all scores tie
+    (900, 890, "heavy"),      # two tokens hold nearly all the weight, picks go on until little else is left
+    (4500, 1600, "tail"),     # more picks than one search of candidates covers
+])
+@pytest.mark.parametrize("dtype,d", [(torch.bfloat16, 128), (torch.float32, 64)])
+def test_greedy_when_bounds_are_loose_or_tie(case, dtype, d):
+    n, k, kind = case
+    g = torch.Generator(device="cpu").manual_seed(n + k)
+    cap = n + 5
+    V = torch.randn((1, 1, cap, d), generator=g).to(dtype)
+    h = (torch.rand((1, 1, cap), generator=g) + 0.1).float()
+    if kind in ("equal", "same_rows"):
+        h[:] = 0.5
+    if kind == "same_rows":
+        V[:] = V[:, :, :1].clone()
+    if kind == "zeros":
+        h[:, :, torch.randperm(n, generator=g)[:n - 200]] = 0.0
+    if kind == "heavy":
+        h[:, :, 10], h[:, :, 700] = 3e3, 5e3
+    if kind == "tail":
+        h = torch.randn((1, 1, cap), generator=g).exp()
+    pos = torch.randperm(cap, generator=g).to(torch.int32).view(1, 1, cap)
+    p = P.make_params(1, 1, 1, d, cap, 1, dtype, 1.0, "external")
+    ws = P.alloc_workspace(p, DEV)
+    ev = torch.full((1, 1, k), -1, dtype=torch.int32, device=DEV)
+    order, ne = torch.full_like(ev, -1), torch.zeros((1,), dtype=torch.int32, device=DEV)
+    lens = torch.tensor([n], dtype=torch.int32)
+    P.caote_select_evict_greedy(p, V.to(DEV), h.to(DEV), lens.to(DEV), (lens - k).to(DEV), pos.to(DEV), ev, order, ne, ws)
+    assert P.caote_read_status(ws) == 0 and ne.item() == k
+    og = order[0, 0].cpu().tolist()
+    assert sorted(og) == ev[0, 0].cpu().tolist() and len(set(og)) == k and 0 <= min(og) and max(og) < n
+    if kind == "zeros":  # exact ties: smallest position first, no band
+        assert og == sorted([j for j in range(n) if h[0, 0, j] == 0], key=lambda j: int(pos[0, 0, j]))[:k]
+    if kind in ("zeros", "same_rows"):
+        return  # (same rows: every distance is the rounding of X alone, any order is right)
+    # the first picks in lock-step with the oracle, in its band (the whole sequence costs minutes on the host)
+    follow(og[:24], h[0, 0, :n].numpy(), f32(V)[0, 0, :n], pos[0, 0, :n].numpy(), 24)
+    if k > 200:  # ... and picks late in the sequence, from the state the first ones leave
+        gone = set(og[:k - 12])
+        rem = [j for j in range(n) if j not in gone]
+        hr, Vr, pr = h[0, 0, rem].numpy(), f32(V)[0, 0][rem], pos[0, 0, rem].numpy()
+        follow([rem.index(j) for j in og[k - 12:]], hr, Vr, pr, 12)
