@@ -9,15 +9,16 @@
 // again (the same arithmetic on the same state, compared by (score bits, position, slot)); the bounds carry margins of 1e-5
 // for the rounding of scores and 5e-7 || X || per pick for that of X.
 //
-// Likewise only the tokens with small scores at the build can be picked: the `active` ones, found by a radix search, live in
-// registers (up to kReg per thread) with as many of their value rows in shared memory as fit. A pick whose score comes
-// within the drift of the others' smallest score is not taken but starts another build; the first pick after a build is
-// always safe.
+// Likewise only the tokens with small scores at the build can be picked: the `active` ones, found by a radix search, with as
+// many of their value rows in shared memory as fit. A pick whose score comes within the drift of the others' smallest score
+// is not taken but starts another build; the first pick after a build is always safe.
 //
 // A thread-block cluster per unit: all CTAs share the two sweeps over the unit's rows (Y, and the distances of a build); the
-// picks are a chain of reductions and run on one CTA (two block barriers per pick), the others wait at the cluster barrier.
-// 8 units of 4 224 tokens, 128 picks: 708 us with every distance formed at every pick (clusters of 8, rows in shared
-// memory, a cluster barrier per pick) -> 209 us.
+// picks are a chain of reductions and run on eight warps of one CTA (two barriers per pick), the others wait at the cluster
+// barrier. 8 units of 4 224 tokens, 128 picks: 709 us with every distance formed at every pick (clusters of 8, rows in shared
+// memory, a cluster barrier per pick) -> 146 us, 22 of them the sweeps and the search. What is left is the latency of a
+// few hundred dependent instructions per pick. Measured for the picks: sixteen warps, active tokens in registers (up to
+// four per thread, loops unrolled) 175; four warps 181; every warp with its own bound and one barrier per pick 200 - 211.
 #pragma once
 
 #include "common.cuh"
@@ -28,36 +29,74 @@ namespace greedy {
 
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
-constexpr int kReg = 4;                  // active tokens per thread
-constexpr int kList = kReg * kThreads;
+constexpr int kPickWarps = 8;            // warps that run the picks (a pick is a few hundred instructions on every one of them)
+constexpr int kPickThreads = 32 * kPickWarps;
+constexpr int kList = 3 * kPickThreads;  // active tokens
 constexpr int kMaxTokens = 24576;        // two floats per token in shared memory
 constexpr int kMaxC = 8;
-constexpr int kNone = 0x7fffffff;
 
 inline size_t base_smem_bytes(int cap) { return sizeof(float) * 2 * (((size_t)cap + 3) / 4 * 4) + 16; }
 
-// w / (1 - w) * dist from the un-normalised weight h and the sum H of all.
-__device__ __forceinline__ float score_of(float h, float dist, float H) {
-  if (!(H > 0.f && h > 0.f)) return 0.f;
+// w / (1 - w) from the un-normalised weight h and the sum H of all.
+__device__ __forceinline__ float ratio_of(float h, float H) {
   const float rest = H - h;  // the others' weight (times H)
-  return rest > 0.f ? h / rest * dist : INFINITY;
+  const float r = rest > 0.f ? __fdividef(h, rest) : INFINITY;
+  return (H > 0.f && h > 0.f) ? r : 0.f;
+}
+__device__ __forceinline__ float score_of(float h, float dist, float H) {
+  const float r = ratio_of(h, H);
+  return r == 0.f ? 0.f : r * dist;
+}
+__device__ __forceinline__ float approx_sqrt(float x) {  // 1 ulp
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
-template <typename T>
-__device__ __forceinline__ float sq_dist16(uint4 raw, const float* x) {  // 16 bytes of a row against the channels x[]
-  const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-  float a = 0.f;
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    if constexpr (sizeof(T) == 2) {
-      const float d0 = x[2 * c] - __uint_as_float(w[c] << 16), d1 = x[2 * c + 1] - __uint_as_float(w[c] & 0xffff0000u);
-      a = fmaf(d0, d0, fmaf(d1, d1, a));
-    } else {
-      const float d0 = x[c] - __uint_as_float(w[c]);
-      a = fmaf(d0, d0, a);
-    }
+// A candidate of a pick: score bits, position, slot and number in the list of active tokens, weight (as bits).
+struct __align__(16) Cand {
+  unsigned v, p, si, h;
+};
+constexpr unsigned kNoCand = 0x7fffu;  // slot of no token (slots are below kMaxTokens)
+__device__ __forceinline__ bool before(const Cand& a, const Cand& b) {
+  return a.v < b.v || (a.v == b.v && (a.p < b.p || (a.p == b.p && (a.si & 0x7fffu) < (b.si & 0x7fffu))));
+}
+
+// The lane that holds the warp's first candidate.
+__device__ __forceinline__ int first_of(const Cand& c) {
+  const unsigned v1 = __reduce_min_sync(0xffffffffu, c.v);
+  unsigned m = __ballot_sync(0xffffffffu, c.v == v1);
+  if (m & (m - 1u)) {  // a tie, or no candidate at all
+    const unsigned p1 = __reduce_min_sync(0xffffffffu, c.v == v1 ? c.p : 0xffffffffu);
+    const bool eq = c.v == v1 && c.p == p1;
+    const unsigned s1 = __reduce_min_sync(0xffffffffu, eq ? c.si & 0x7fffu : 0xffffu);
+    m = __ballot_sync(0xffffffffu, eq && (c.si & 0x7fffu) == s1);
   }
-  return a;
+  return __ffs((int)m) - 1;
+}
+
+// 16 bytes of a row against the same channels of -X (nx: 16-byte aligned), packed fp32 pairs.
+template <typename T>
+__device__ __forceinline__ float sq_dist16(uint4 raw, const float4* nx) {
+  float2 a = make_float2(0.f, 0.f);
+  const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+  if constexpr (sizeof(T) == 2) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const float4 x = nx[c];
+      const float2 d0 = __fadd2_rn(make_float2(__uint_as_float(w[2 * c] << 16), __uint_as_float(w[2 * c] & 0xffff0000u)), make_float2(x.x, x.y));
+      const float2 d1 = __fadd2_rn(make_float2(__uint_as_float(w[2 * c + 1] << 16), __uint_as_float(w[2 * c + 1] & 0xffff0000u)), make_float2(x.z, x.w));
+      a = __ffma2_rn(d0, d0, a);
+      a = __ffma2_rn(d1, d1, a);
+    }
+  } else {
+    const float4 x = nx[0];
+    const float2 d0 = __fadd2_rn(make_float2(__uint_as_float(w[0]), __uint_as_float(w[1])), make_float2(x.x, x.y));
+    const float2 d1 = __fadd2_rn(make_float2(__uint_as_float(w[2]), __uint_as_float(w[3])), make_float2(x.z, x.w));
+    a = __ffma2_rn(d0, d0, a);
+    a = __ffma2_rn(d1, d1, a);
+  }
+  return a.x + a.y;
 }
 
 // grid = units x C CTAs in clusters of C; rows_smem: value rows that fit behind the two arrays of `cap` floats.
@@ -76,15 +115,18 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
   float* hs = reinterpret_cast<float*>(gsm);            // [cap] weight of the token, < 0 once evicted  (rank 0)
   float* ds = hs + (cap + 3) / 4 * 4;                   // [cap] distance at the build                 (rank 0)
   T* rows = reinterpret_cast<T*>(ds + (cap + 3) / 4 * 4);  // [rows_smem][D] value rows of the first active tokens
-  __shared__ float Ys[D], Xs[D], part[D + 1], wpart[kWarps][D + 1];
+  __shared__ float Ys[D], part[D + 1], wpart[kWarps][D + 1];
+  __shared__ __align__(16) float nX[D];                 // -X
   __shared__ float s_H;
   __shared__ int s_ctl;                                 // after a round of picks: picks done, -1: all
-  __shared__ int act[kList];
+  __shared__ int act[kList];                            // the active tokens: slot,
+  __shared__ float th[kList], ta[kList], tr[kList];     // weight (< 0 once evicted), distance + drift when it was formed, w / (1 - w),
+  __shared__ unsigned tp[kList];                        // position
   __shared__ unsigned hist[256];
   __shared__ int s_digit, s_below, s_incl, s_na;
-  __shared__ unsigned s_ub[kWarps], s_cb[kWarps], s_cp[kWarps], s_min[kWarps];
-  __shared__ int s_cs[kWarps], s_ci[kWarps], s_cnt[kWarps];
-  __shared__ float s_ch[kWarps];
+  __shared__ unsigned s_min[kWarps], s_ub[kPickWarps];
+  __shared__ int s_cnt[kWarps];
+  __shared__ Cand s_cand[kPickWarps];
 
   const int C = (int)ptx::cluster_nctarank(), rank = (int)ptx::cluster_ctarank();
   const int unit = (int)ptx::cluster_id_x(), b = unit / Hkv, hd = unit % Hkv;
@@ -153,14 +195,14 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
     // ================= a build: the distances of all tokens still present to the current output =================
     float H = ptx::ld_dsmem_f32(ptx::map_to_rank(ptx::smem_u32(&s_H), 0));
     {
-      const float inv_H = (H > 0.f) ? 1.f / H : 0.f;
-      if (tid < D) Xs[tid] = ptx::ld_dsmem_f32(ptx::map_to_rank(ptx::smem_u32(Ys + tid), 0)) * inv_H;
+      const float inv_H = (H > 0.f) ? __fdividef(1.f, H) : 0.f;
+      if (tid < D) nX[tid] = -(ptx::ld_dsmem_f32(ptx::map_to_rank(ptx::smem_u32(Ys + tid), 0)) * inv_H);
       __syncthreads();
-      float x[NCH][E];
+      float4 x[NCH][E / 4];
 #pragma unroll
       for (int i = 0; i < NCH; ++i)
 #pragma unroll
-        for (int e = 0; e < E; ++e) x[i][e] = Xs[(l8 + 8 * i) * E + e];
+        for (int e = 0; e < E / 4; ++e) x[i][e] = reinterpret_cast<const float4*>(nX)[(l8 + 8 * i) * (E / 4) + e];
       constexpr int kPasses = 8 / NCH;  // passes of four rows per warp in flight
       for (int j0 = r0 + 4 * warp; j0 < r1; j0 += 4 * kWarps * kPasses) {
         uint4 raw[kPasses][NCH];
@@ -179,15 +221,17 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
           a += __shfl_xor_sync(0xffffffffu, a, 4);
           a += __shfl_xor_sync(0xffffffffu, a, 2);
           a += __shfl_xor_sync(0xffffffffu, a, 1);
-          if (l8 == 0 && j < r1) ptx::st_dsmem_f32(ptx::map_to_rank(ptx::smem_u32(ds + j), 0), sqrtf(a));
+          if (l8 == 0 && j < r1) ptx::st_dsmem_f32(ptx::map_to_rank(ptx::smem_u32(ds + j), 0), approx_sqrt(a));
         }
       }
     }
     ptx::cluster_sync_all();
 
     if (rank == 0) {
-      // ---- the active tokens: the smallest (score, position, slot) keys, `want` of them and at most 512 more ----
-      const int present = n - t, rem = k - t, want = min(present, min(rem + 32, 768));
+      // ---- the active tokens: the smallest (score, position, slot) keys, `want` of them and at most what fills up the
+      //      threads' last round ----
+      const int present = n - t, rem = k - t, want = min(present, min(rem + 32, kList - kPickThreads)),
+                most = (want + kPickThreads - 1) / kPickThreads * kPickThreads;
       unsigned kb = 0u, kp = 0u, ks = 0u;  // the largest key that is taken
       int below = 0;
       for (int pass = 0;; ++pass) {  // eight bits at a time: four passes over the score, four the position, two the slot
@@ -240,7 +284,7 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
         else if (pass < 8) kp |= digit;
         else ks |= digit;
         below = s_below;
-        if (s_incl <= want + 512 || pass == 9) {
+        if (s_incl <= most || pass == 9) {
           const unsigned ones = (1u << shift) - 1u;
           if (pass < 4) { kb |= ones; kp = 0xffffffffu; ks = 0xffffffffu; }
           else if (pass < 8) { kp |= ones; ks = 0xffffffffu; }
@@ -274,135 +318,102 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
         if (lane == 0) s_min[warp] = m;
       }
       __syncthreads();
-      const int na = min(s_na, kList), nu = (na + kThreads - 1) / kThreads;
+      const int na = min(s_na, kList), nu = (na + kPickThreads - 1) / kPickThreads;
       dmin = __uint_as_float(__reduce_min_sync(0xffffffffu, s_min[lane & (kWarps - 1)]));
-      const float tau = __uint_as_float(min(kb, 0x7f800000u));
-      float hr[kReg], ar[kReg];  // weight (< 0: none, or evicted) and distance + drift at the time it was formed
-      unsigned pr[kReg];
-      int sr[kReg];
-#pragma unroll
-      for (int u = 0; u < kReg; ++u) {
-        const int i = tid + u * kThreads;
-        hr[u] = -1.f; ar[u] = 0.f; pr[u] = 0u; sr[u] = 0;
-        if (i < na) {
-          const int j = act[i];
-          sr[u] = j;
-          hr[u] = hs[j];
-          ar[u] = ds[j];
-          pr[u] = (unsigned)(pu ? pu[j] : j);
-        }
+      const float tau = __uint_as_float(min(kb, 0x7f800000u)), inv_dmin = 1.f / dmin;  // (0 where there are no others)
+      for (int i = tid; i < na; i += kThreads) {
+        const int j = act[i];
+        th[i] = hs[j];
+        ta[i] = ds[j];
+        tp[i] = (unsigned)(pu ? pu[j] : j);
       }
       for (int idx = tid; idx < min(na, rows_smem) * (D / E); idx += kThreads)
         reinterpret_cast<uint4*>(rows)[idx] = reinterpret_cast<const uint4*>(Vu + (size_t)act[idx / (D / E)] * D)[idx % (D / E)];
       float xn = 0.f;
 #pragma unroll
-      for (int c = 0; c < CPL; ++c) xn = fmaf(Xs[lane * CPL + c], Xs[lane * CPL + c], xn);
+      for (int c = 0; c < CPL; ++c) xn = fmaf(nX[lane * CPL + c], nX[lane * CPL + c], xn);
       xn = sqrtf(warp_sum(xn));
       __syncthreads();
 
       // ================= picks =================
+      // (the loops over a thread's tokens stay rolled: almost always there is one round, and a few warps run straight-line
+      // code no faster than it is fetched)
       float drift = 0.f;
       bool fresh = true;
-      while (t < k) {
+      while (warp < kPickWarps && t < k) {
         // ---- the smallest upper bound ----
-        float rr[kReg], ub = INFINITY;
-#pragma unroll
-        for (int u = 0; u < kReg; ++u) {
-          rr[u] = 0.f;
-          if (u < nu && hr[u] >= 0.f) {
-            if (H > 0.f && hr[u] > 0.f) {
-              const float rest = H - hr[u];
-              rr[u] = rest > 0.f ? __fdividef(hr[u], rest) : INFINITY;
-              ub = fminf(ub, rr[u] * (ar[u] + drift) * 1.00001f);
-            } else {
-              ub = 0.f;  // a score of exactly zero
-            }
-          }
+        float ub = INFINITY;
+#pragma unroll 1
+        for (int i = tid; i < na; i += kPickThreads) {
+          const float h = th[i], r = ratio_of(h, H);
+          tr[i] = r;
+          if (h >= 0.f) ub = fminf(ub, r * (ta[i] + drift) * 1.00001f);
         }
-        {
-          const unsigned m = __reduce_min_sync(0xffffffffu, __float_as_uint(ub));
-          if (lane == 0) s_ub[warp] = m;
-        }
-        __syncthreads();
-        ub = __uint_as_float(__reduce_min_sync(0xffffffffu, s_ub[lane & (kWarps - 1)]));
+        ub = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(ub)));
+        if (lane == 0) s_ub[warp] = __float_as_uint(ub);
+        asm volatile("bar.sync 1, %0;" ::"n"(kPickThreads) : "memory");
+        ub = __uint_as_float(__reduce_min_sync(0xffffffffu, s_ub[lane & (kPickWarps - 1)]));
         // ---- exact scores of the tokens that can be the minimum ----
-        unsigned cb = 0xffffffffu, cp = 0xffffffffu;
-        int cs = kNone, ci = 0;
-        float ch = 0.f;
-        const float inv_H = (H > 0.f) ? 1.f / H : 0.f;
-        auto offer = [&](int i, float h, unsigned p, int s, float sc) {
-          const unsigned v = __float_as_uint(sc);
-          if (v < cb || (v == cb && (p < cp || (p == cp && s < cs)))) { cb = v; cp = p; cs = s; ci = i; ch = h; }
-        };
-#pragma unroll
-        for (int u = 0; u < kReg; ++u) {
-          const bool present_u = u < nu && hr[u] >= 0.f, weighs = H > 0.f && hr[u] > 0.f;
-          if (present_u && !weighs) offer(tid + u * kThreads, hr[u], pr[u], sr[u], 0.f);
-          const bool mine = present_u && weighs && !(rr[u] * fmaxf(ar[u] - drift, 0.f) * 0.99999f > ub);
+        Cand best{0xffffffffu, 0xffffffffu, kNoCand, 0u};
+#pragma unroll 1
+        for (int u = 0; u < nu; ++u) {
+          const int i0 = warp * 32 + u * kPickThreads, mi = i0 + lane;
+          const bool mine = mi < na && th[mi] >= 0.f && !(tr[mi] * fmaxf(ta[mi] - drift, 0.f) * 0.99999f > ub);
           unsigned mask = __ballot_sync(0xffffffffu, mine);
+#pragma unroll 1
           while (mask) {  // four tokens at a time, eight lanes each
             const unsigned m1 = mask & (mask - 1u), m2 = m1 & (m1 - 1u), m3 = m2 & (m2 - 1u);
             const unsigned ms = sub == 0 ? mask : (sub == 1 ? m1 : (sub == 2 ? m2 : m3));
-            const int p = ms ? __ffs((int)ms) - 1 : 0;
-            const int j = __shfl_sync(0xffffffffu, sr[u], p), idx = warp * 32 + p + u * kThreads;
+            const int idx = i0 + (ms ? __ffs((int)ms) - 1 : 0), j = act[idx];
+            const float r = tr[idx], h = th[idx];
+            const unsigned p = tp[idx];
             const uint4* row = reinterpret_cast<const uint4*>(idx < rows_smem ? rows + (size_t)idx * D : Vu + (size_t)j * D);
-            float a = 0.f;
+            float a[NCH];
 #pragma unroll
-            for (int i = 0; i < NCH; ++i) {
-              const uint4 raw = row[l8 + 8 * i];
-              float x[E];
+            for (int i = 0; i < NCH; ++i)
+              a[i] = sq_dist16<T>(row[l8 + 8 * i], reinterpret_cast<const float4*>(nX) + (l8 + 8 * i) * (E / 4));
 #pragma unroll
-              for (int e = 0; e < E; ++e) x[e] = Ys[(l8 + 8 * i) * E + e] * inv_H;
-              a += sq_dist16<T>(raw, x);
-            }
-            a += __shfl_xor_sync(0xffffffffu, a, 4);
-            a += __shfl_xor_sync(0xffffffffu, a, 2);
-            a += __shfl_xor_sync(0xffffffffu, a, 1);
-            const int rk = __popc(mask & ((1u << lane) - 1u));
-            a = __shfl_sync(0xffffffffu, a, 8 * min(rk, 3));
-            if ((mask >> lane & 1u) && rk < 4) {
-              const float d = sqrtf(a);
-              ar[u] = d + drift;
-              offer(tid + u * kThreads, hr[u], pr[u], sr[u], score_of(hr[u], d, H));
+            for (int i = 1; i < NCH; ++i) a[0] += a[i];
+            a[0] += __shfl_xor_sync(0xffffffffu, a[0], 4);
+            a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
+            a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+            if (ms && l8 == 0) {
+              const float d = approx_sqrt(a[0]);
+              const Cand c{__float_as_uint(r == 0.f ? 0.f : r * d), p, (unsigned)j | ((unsigned)idx << 16), __float_as_uint(h)};
+              if (before(c, best)) best = c;
+              ta[idx] = d + drift;
             }
             mask = m3 & (m3 - 1u);
           }
         }
+        if (lane == first_of(best)) s_cand[warp] = best;
+        asm volatile("bar.sync 1, %0;" ::"n"(kPickThreads) : "memory");
+        Cand win = s_cand[lane & (kPickWarps - 1)];
         {
-          const unsigned b1 = __reduce_min_sync(0xffffffffu, cb);
-          const unsigned p1 = __reduce_min_sync(0xffffffffu, cb == b1 ? cp : 0xffffffffu);
-          const bool eq = cb == b1 && cp == p1;
-          const int s1 = (int)__reduce_min_sync(0xffffffffu, eq ? (unsigned)cs : (unsigned)kNone);
-          if (s1 == kNone ? lane == 0 : (eq && cs == s1)) {
-            s_cb[warp] = b1; s_cp[warp] = p1; s_cs[warp] = s1; s_ci[warp] = ci; s_ch[warp] = ch;
-          }
+          Cand mineonly = win;
+          if (lane >= kPickWarps) mineonly = Cand{0xffffffffu, 0xffffffffu, kNoCand, 0u};
+          const int wl = first_of(mineonly);
+          win.v = __shfl_sync(0xffffffffu, win.v, wl);
+          win.si = __shfl_sync(0xffffffffu, win.si, wl);
+          win.h = __shfl_sync(0xffffffffu, win.h, wl);
         }
-        __syncthreads();
-        const int w16 = lane & (kWarps - 1);
-        const unsigned vb = s_cb[w16], vp = s_cp[w16];
-        const int vs = s_cs[w16];
-        const unsigned b1 = __reduce_min_sync(0xffffffffu, vb);
-        const unsigned p1 = __reduce_min_sync(0xffffffffu, vb == b1 ? vp : 0xffffffffu);
-        const bool eq = vb == b1 && vp == p1;
-        const int e = (int)__reduce_min_sync(0xffffffffu, eq ? (unsigned)vs : (unsigned)kNone);
-        if (e == kNone) { t = k; break; }  // (cannot happen with k < n; the same in every thread)
-        const int wi = __ffs((int)__ballot_sync(0xffffffffu, eq && vs == e)) - 1;
-        const int ei = s_ci[wi & (kWarps - 1)];
-        const float he = s_ch[wi & (kWarps - 1)], sc = __uint_as_float(b1);
-        if (!fresh && !(sc <= tau * (1.f - drift / dmin) * 0.99999f)) break;  // another token may be smaller: build again
-        // ---- evict e: Y -= h_e v_e, H -= h_e ----
+        const int e = (int)(win.si & 0x7fffu), ei = (int)(win.si >> 16);
+        const float he = __uint_as_float(win.h), sc = __uint_as_float(win.v);
+        if (e == (int)kNoCand) { t = k; break; }  // (cannot happen with k < n; the same in every thread)
+        if (!fresh && !(sc <= tau * (1.f - drift * inv_dmin) * 0.99999f)) break;  // another token may be smaller: build again
+        // ---- evict e: Y -= h_e v_e, H -= h_e (X is read again after the next barrier) ----
+        H -= he;
         if (tid < D) {
           const T* row = ei < rows_smem ? rows + (size_t)ei * D : Vu + (size_t)e * D;
-          Ys[tid] -= he * to_float(row[tid]);
+          const float y = Ys[tid] - he * to_float(row[tid]);
+          Ys[tid] = y;
+          nX[tid] = -(y * ((H > 0.f) ? __fdividef(1.f, H) : 0.f));
         }
-        if ((ei & (kThreads - 1)) == tid) {
-#pragma unroll
-          for (int u = 0; u < kReg; ++u)
-            if (u == ei / kThreads) hr[u] = -1.f;
+        if (ei % kPickThreads == tid) {
+          th[ei] = -1.f;
           hs[e] = -1.f;
           if (order_out) order_out[(size_t)unit * max_evict + t] = e;
         }
-        H -= he;
         drift += sc * 1.0001f + 5e-7f * (xn + drift);
         fresh = false;
         ++t;
