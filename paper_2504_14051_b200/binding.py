@@ -126,14 +126,17 @@ def make_params(batch, n_q_heads, n_kv_heads, head_dim, capacity, n_new, dtype, 
     return Params(batch, n_q_heads, n_kv_heads, head_dim, capacity, n_new, dtype, float(scale), base_mode, 0)
 
 
+# A step of a small cache takes the GPU some 15 us, so what is done here per call counts: addresses go to ctypes as plain
+# integers (the declared argument types convert them) and the library's functions are looked up once. One caote_step call:
+# 6.4 us with c_void_p objects made for every pointer, 3.8 us so.
 def _p(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+def _stream(stream) -> int:
     if stream is None:
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _check(fn: str, rc: int):
@@ -141,8 +144,20 @@ def _check(fn: str, rc: int):
         raise CaoteError(fn, rc)
 
 
+class _Functions:
+    """The library's entry points as attributes; loads the library at the first use of one."""
+
+    def __getattr__(self, name):
+        f = getattr(lib(), name)
+        setattr(self, name, f)
+        return f
+
+
+_fn = _Functions()
+
+
 def caote_workspace_bytes(p: Params) -> int:
-    return int(lib().caote_workspace_bytes(ctypes.byref(p)))
+    return int(_fn.caote_workspace_bytes(ctypes.byref(p)))
 
 
 def alloc_workspace(p: Params, device) -> torch.Tensor:
@@ -154,33 +169,33 @@ def alloc_workspace(p: Params, device) -> torch.Tensor:
 
 
 def caote_append(p, K, V, base, pos, lens, n_seen, k_new, v_new, workspace, stream=None):
-    _check("caote_append", lib().caote_append(ctypes.byref(p), _p(K), _p(V), _p(base), _p(pos), _p(lens),
-                                              _p(n_seen), _p(k_new), _p(v_new), _p(workspace),
-                                              workspace.numel(), _stream(stream)))
+    _check("caote_append", _fn.caote_append(ctypes.byref(p), _p(K), _p(V), _p(base), _p(pos), _p(lens),
+                                            _p(n_seen), _p(k_new), _p(v_new), _p(workspace),
+                                            workspace.numel(), _stream(stream)))
 
 
 def caote_score(p, q, K, V, lens, base, o, scores, workspace, stream=None):
-    _check("caote_score", lib().caote_score(ctypes.byref(p), _p(q), _p(K), _p(V), _p(lens), _p(base), _p(o),
-                                            _p(scores), _p(workspace), workspace.numel(), _stream(stream)))
+    _check("caote_score", _fn.caote_score(ctypes.byref(p), _p(q), _p(K), _p(V), _p(lens), _p(base), _p(o),
+                                          _p(scores), _p(workspace), workspace.numel(), _stream(stream)))
 
 
 def caote_score_static(p, q, K, V, lens, base, o, scores, status_out=None, stream=None):
     """caote_score on the library's built-in scratch array: for callers that may not allocate device
     memory (no workspace argument). ``status_out``: optional int32 device tensor of one element."""
     _check("caote_score_static",
-           lib().caote_score_static(ctypes.byref(p), _p(q), _p(K), _p(V), _p(lens), _p(base), _p(o), _p(scores),
-                                    _p(status_out), _stream(stream)))
+           _fn.caote_score_static(ctypes.byref(p), _p(q), _p(K), _p(V), _p(lens), _p(base), _p(o), _p(scores),
+                                  _p(status_out), _stream(stream)))
 
 
 def caote_select_evict(p, scores, lens, budget, pos, evict_idx, n_evict, workspace, stream=None):
     _check("caote_select_evict",
-           lib().caote_select_evict(ctypes.byref(p), _p(scores), _p(lens), _p(budget), _p(pos), _p(evict_idx),
-                                    evict_idx.shape[-1], _p(n_evict), _p(workspace), workspace.numel(),
-                                    _stream(stream)))
+           _fn.caote_select_evict(ctypes.byref(p), _p(scores), _p(lens), _p(budget), _p(pos), _p(evict_idx),
+                                  evict_idx.shape[-1], _p(n_evict), _p(workspace), workspace.numel(),
+                                  _stream(stream)))
 
 
 def caote_select_evict_greedy(p, V, h, lens, budget, pos, evict_idx, order, n_evict, workspace, stream=None):
-    _check("caote_select_evict_greedy", lib().caote_select_evict_greedy(
+    _check("caote_select_evict_greedy", _fn.caote_select_evict_greedy(
         ctypes.byref(p), _p(V), _p(h), _p(lens), _p(budget), _p(pos), _p(evict_idx), _p(order), evict_idx.shape[-1],
         _p(n_evict), _p(workspace), workspace.numel() * workspace.element_size(), _stream(stream)))
 
@@ -189,9 +204,9 @@ def caote_compact(p, K, V, base, pos, lens, evict_idx, n_evict, mode, workspace,
     if isinstance(mode, str):
         mode = COMPACT_MODES[mode]
     _check("caote_compact",
-           lib().caote_compact(ctypes.byref(p), _p(K), _p(V), _p(base), _p(pos), _p(lens), _p(evict_idx),
-                               evict_idx.shape[-1], _p(n_evict), mode, _p(workspace), workspace.numel(),
-                               _stream(stream)))
+           _fn.caote_compact(ctypes.byref(p), _p(K), _p(V), _p(base), _p(pos), _p(lens), _p(evict_idx),
+                             evict_idx.shape[-1], _p(n_evict), mode, _p(workspace), workspace.numel(),
+                             _stream(stream)))
 
 
 def caote_step(p, q, k_new, v_new, K, V, base, pos, lens, n_seen, budget, o, scores, evict_idx, n_evict, mode,
@@ -199,21 +214,21 @@ def caote_step(p, q, k_new, v_new, K, V, base, pos, lens, n_seen, budget, o, sco
     if isinstance(mode, str):
         mode = COMPACT_MODES[mode]
     _check("caote_step",
-           lib().caote_step(ctypes.byref(p), _p(q), _p(k_new), _p(v_new), _p(K), _p(V), _p(base), _p(pos),
-                            _p(lens), _p(n_seen), _p(budget), _p(o), _p(scores), _p(evict_idx),
-                            evict_idx.shape[-1], _p(n_evict), mode, _p(workspace), workspace.numel(),
-                            _stream(stream)))
+           _fn.caote_step(ctypes.byref(p), _p(q), _p(k_new), _p(v_new), _p(K), _p(V), _p(base), _p(pos),
+                          _p(lens), _p(n_seen), _p(budget), _p(o), _p(scores), _p(evict_idx),
+                          evict_idx.shape[-1], _p(n_evict), mode, _p(workspace), workspace.numel(),
+                          _stream(stream)))
 
 
 def caote_vsum(p, V, lens, vsum, stream=None):
     """vsum[u, :] = sum of the unit's valid V rows (FastCAOTE, Sec. 3.3)."""
-    _check("caote_vsum", lib().caote_vsum(ctypes.byref(p), _p(V), _p(lens), _p(vsum), _stream(stream)))
+    _check("caote_vsum", _fn.caote_vsum(ctypes.byref(p), _p(V), _p(lens), _p(vsum), _stream(stream)))
 
 
 def caote_score_fast(p, q, K, V, lens, base, vsum, o, scores, workspace, stream=None):
     _check("caote_score_fast",
-           lib().caote_score_fast(ctypes.byref(p), _p(q), _p(K), _p(V), _p(lens), _p(base), _p(vsum), _p(o),
-                                  _p(scores), _p(workspace), workspace.numel(), _stream(stream)))
+           _fn.caote_score_fast(ctypes.byref(p), _p(q), _p(K), _p(V), _p(lens), _p(base), _p(vsum), _p(o),
+                                _p(scores), _p(workspace), workspace.numel(), _stream(stream)))
 
 
 def caote_step_fast(p, q, k_new, v_new, K, V, base, pos, lens, n_seen, budget, vsum, o, scores, evict_idx, n_evict,
@@ -221,53 +236,53 @@ def caote_step_fast(p, q, k_new, v_new, K, V, base, pos, lens, n_seen, budget, v
     if isinstance(mode, str):
         mode = COMPACT_MODES[mode]
     _check("caote_step_fast",
-           lib().caote_step_fast(ctypes.byref(p), _p(q), _p(k_new), _p(v_new), _p(K), _p(V), _p(base), _p(pos),
-                                 _p(lens), _p(n_seen), _p(budget), _p(vsum), _p(o), _p(scores), _p(evict_idx),
-                                 evict_idx.shape[-1], _p(n_evict), mode, _p(workspace), workspace.numel(),
-                                 _stream(stream)))
+           _fn.caote_step_fast(ctypes.byref(p), _p(q), _p(k_new), _p(v_new), _p(K), _p(V), _p(base), _p(pos),
+                               _p(lens), _p(n_seen), _p(budget), _p(vsum), _p(o), _p(scores), _p(evict_idx),
+                               evict_idx.shape[-1], _p(n_evict), mode, _p(workspace), workspace.numel(),
+                               _stream(stream)))
 
 
 def caote_score_sum_errors(p, q, K, V, lens, o, scores, workspace, stream=None):
     """Scores as the sum over the counted query rows of the exact single-query eviction errors."""
     _check("caote_score_sum_errors",
-           lib().caote_score_sum_errors(ctypes.byref(p), _p(q), _p(K), _p(V), _p(lens), _p(o), _p(scores),
-                                        _p(workspace), workspace.numel(), _stream(stream)))
+           _fn.caote_score_sum_errors(ctypes.byref(p), _p(q), _p(K), _p(V), _p(lens), _p(o), _p(scores),
+                                      _p(workspace), workspace.numel(), _stream(stream)))
 
 
 def caote_post_evict_output(p, q, K, V, lens, evict_idx, n_evict, o, o_post, stream=None):
     """Attention output over the retained tokens (call between caote_select_evict and caote_compact)."""
     _check("caote_post_evict_output",
-           lib().caote_post_evict_output(ctypes.byref(p), _p(q), _p(K), _p(V), _p(lens), _p(evict_idx),
-                                         evict_idx.shape[-1], _p(n_evict), _p(o), _p(o_post), _stream(stream)))
+           _fn.caote_post_evict_output(ctypes.byref(p), _p(q), _p(K), _p(V), _p(lens), _p(evict_idx),
+                                       evict_idx.shape[-1], _p(n_evict), _p(o), _p(o_post), _stream(stream)))
 
 
 def caote_post_evict_output_ws(p, q, K, V, lens, evict_idx, n_evict, o, o_post, workspace, stream=None):
     """The same from the softmax statistics the scoring call left in `workspace`, where it left any."""
     _check("caote_post_evict_output_ws",
-           lib().caote_post_evict_output_ws(ctypes.byref(p), _p(q), _p(K), _p(V), _p(lens), _p(evict_idx),
-                                            evict_idx.shape[-1], _p(n_evict), _p(o), _p(o_post), _p(workspace),
-                                            workspace.numel(), _stream(stream)))
+           _fn.caote_post_evict_output_ws(ctypes.byref(p), _p(q), _p(K), _p(V), _p(lens), _p(evict_idx),
+                                          evict_idx.shape[-1], _p(n_evict), _p(o), _p(o_post), _p(workspace),
+                                          workspace.numel(), _stream(stream)))
 
 
 def caote_read_status(workspace, stream=None) -> int:
     out = ctypes.c_int32(0)
-    _check("caote_read_status", lib().caote_read_status(_p(workspace), _stream(stream), ctypes.byref(out)))
+    _check("caote_read_status", _fn.caote_read_status(_p(workspace), _stream(stream), ctypes.byref(out)))
     return int(out.value)
 
 
 def caote_status_string(code: int) -> str:
-    return lib().caote_status_string(code).decode()
+    return _fn.caote_status_string(code).decode()
 
 
 def caote_trace_enable(on: bool) -> None:
-    _check("caote_trace_enable", lib().caote_trace_enable(1 if on else 0))
+    _check("caote_trace_enable", _fn.caote_trace_enable(1 if on else 0))
 
 
 def caote_trace_collect(max_entries: int = 32) -> dict:
     """{kernel name: (launches, total_ms)} since the last collect."""
     buf = (TraceEntry * max_entries)()
     n = ctypes.c_int32(0)
-    _check("caote_trace_collect", lib().caote_trace_collect(buf, max_entries, ctypes.byref(n)))
+    _check("caote_trace_collect", _fn.caote_trace_collect(buf, max_entries, ctypes.byref(n)))
     return {buf[i].name.decode(): (int(buf[i].launches), float(buf[i].total_ms)) for i in range(n.value)}
 
 
@@ -275,8 +290,8 @@ OPT_WAIT_CYCLES, OPT_DECODE_CLUSTER, OPT_SIDE_BY_SIDE = 1, 2, 3
 
 
 def caote_set_option(option: int, value: int) -> None:
-    _check("caote_set_option", lib().caote_set_option(int(option), int(value)))
+    _check("caote_set_option", _fn.caote_set_option(int(option), int(value)))
 
 
 def caote_launch_count() -> int:
-    return int(lib().caote_launch_count())
+    return int(_fn.caote_launch_count())
