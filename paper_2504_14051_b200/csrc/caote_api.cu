@@ -98,19 +98,29 @@ struct TraceScope {
 
 // Launch with the programmatic-serialization attribute: the kernel may be scheduled while its predecessor in the
 // stream is still running and waits for it in its first statement (ptx::pdl_wait). Only for kernels that do so.
+// cluster > 1: in clusters of that many CTAs along x.
 template <typename... KArgs, typename... Args>
-static void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+static void launch_pdl_clusters(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, int cluster, cudaStream_t st,
+                                Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);  // (errors are picked up by after_launch)
+}
+template <typename... KArgs, typename... Args>
+static void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  launch_pdl_clusters(kernel, grid, block, smem, 1, st, std::forward<Args>(args)...);
 }
 
 static bool params_ok(const caote_params_t* p) {
@@ -182,20 +192,22 @@ static int launch_generic_score(const Dims& dm, const void* q, const void* K, co
     int rc = allow_smem(generic::attn_partial_kernel<T, D>, smem);
     if (rc) return rc;
     dim3 grid(row_tiles, sc.splits, dm.units);
-    CAOTE_LAUNCH("attn_partial_kernel", st, generic::attn_partial_kernel<T, D><<<grid, generic::kThreads, smem, st>>>(
-        dm, (const T*)q, (const T*)K, (const T*)V, len, base, sc, status));
+    CAOTE_LAUNCH("attn_partial_kernel", st,
+                 launch_pdl(generic::attn_partial_kernel<T, D>, grid, dim3(generic::kThreads), smem, st, dm, (const T*)q, (const T*)K,
+                            (const T*)V, len, (const float*)base, sc, status));
   }
   {
     dim3 grid(sc.chunks, dm.units);
-    CAOTE_LAUNCH("attn_combine_kernel", st, generic::attn_combine_kernel<T, D><<<grid, D, 0, st>>>(dm, len, sc, o));
+    CAOTE_LAUNCH("attn_combine_kernel", st, launch_pdl(generic::attn_combine_kernel<T, D>, grid, dim3(generic::kCombineThreads), 0, st, dm, len, sc, o));
   }
   if (sum_errors) {
     const size_t smem = generic::sum_errors_smem(D);
     int rc = allow_smem(generic::sum_errors_kernel<T, D>, smem);
     if (rc) return rc;
     dim3 grid((dm.cap + generic::kKT - 1) / generic::kKT, dm.units);
-    CAOTE_LAUNCH("sum_errors_kernel", st, generic::sum_errors_kernel<T, D><<<grid, generic::kThreads, smem, st>>>(
-        dm, (const T*)q, (const T*)K, (const T*)V, len, o, sc, scores));
+    CAOTE_LAUNCH("sum_errors_kernel", st,
+                 launch_pdl(generic::sum_errors_kernel<T, D>, grid, dim3(generic::kThreads), smem, st, dm, (const T*)q, (const T*)K,
+                            (const T*)V, len, (const float*)o, sc, scores));
     return CAOTE_OK;
   }
   {
@@ -203,8 +215,9 @@ static int launch_generic_score(const Dims& dm, const void* q, const void* K, co
     int rc = allow_smem(generic::score_pass_kernel<T, D>, smem);
     if (rc) return rc;
     dim3 grid((dm.cap + generic::kKT - 1) / generic::kKT, dm.units);
-    CAOTE_LAUNCH("score_pass_kernel", st, generic::score_pass_kernel<T, D><<<grid, generic::kThreads, smem, st>>>(
-        dm, (const T*)q, (const T*)K, (const T*)V, len, base, sc, scores, vsum));
+    CAOTE_LAUNCH("score_pass_kernel", st,
+                 launch_pdl(generic::score_pass_kernel<T, D>, grid, dim3(generic::kThreads), smem, st, dm, (const T*)q, (const T*)K,
+                            (const T*)V, len, base, sc, scores, vsum));
   }
   return CAOTE_OK;
 }
@@ -285,10 +298,9 @@ static ClusterKernel cluster_kernel(int g, int base_mode) {
 }
 
 // Clusters of `c` CTAs of the cluster kernel that can be resident on the current device at once; 0 if none.
-static int cluster_capacity(int c, ClusterKernel kernel) {
+static int cluster_capacity(int dev, int c, ClusterKernel kernel) {
   static std::atomic<int> cached[64][dcl::kMaxC + 1];
-  int dev = 0;
-  if (c < 1 || c > dcl::kMaxC || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (c < 1 || c > dcl::kMaxC) return 0;
   int n = cached[dev][c].load(std::memory_order_acquire);
   if (n == 0) {
     const size_t smem = dcl::smem_bytes();
@@ -321,13 +333,14 @@ static int cluster_capacity(int c, ClusterKernel kernel) {
 static int choose_cluster(const Dims& dm, ClusterKernel kernel, int* clusters_out) {
   const int cap_tiles = (dm.cap + decode::kT - 1) / decode::kT;
   const int forced = g_decode_cluster.load(std::memory_order_relaxed);
-  if (forced < 0) return 0;
+  int dev = 0;
+  if (forced < 0 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   int best = 0, best_n = 0;
   double best_cost = 0.0;
   for (int c = 1; c <= dcl::kMaxC; ++c) {
     if (forced > 0 && c != forced) continue;
     if ((cap_tiles + c - 1) / c > dcl::kMaxT) continue;
-    const int n = cluster_capacity(c, kernel);
+    const int n = cluster_capacity(dev, c, kernel);
     if (n <= 0) continue;
     const long long rounds = ((long long)dm.units + n - 1) / n;
     const double cost = (double)rounds * ((double)cap_tiles / c + 2.0 + 0.05 * c);
@@ -1039,12 +1052,19 @@ int caote_vsum(const caote_params_t* p, const void* V, const int32_t* len, float
   if (rc) return rc;
   const Dims dm = make_dims(p);
   cudaStream_t st = (cudaStream_t)stream;
-  if (p->dtype == CAOTE_BF16) {
-    CAOTE_LAUNCH("fast_vsum_kernel", st, fast::vsum_kernel<__nv_bfloat16><<<dm.units, 256, 0, st>>>(
-        dm.Hkv, dm.cap, dm.D, (const __nv_bfloat16*)V, len, vsum));
-  } else {
-    CAOTE_LAUNCH("fast_vsum_kernel", st, fast::vsum_kernel<float><<<dm.units, 256, 0, st>>>(dm.Hkv, dm.cap, dm.D, (const float*)V, len, vsum));
-  }
+  const dim3 grid(dm.units * fast::kSumCtas);
+  auto launch = [&](auto kernel, auto v) {
+    launch_pdl_clusters(kernel, grid, dim3(256), 0, fast::kSumCtas, st, dm.Hkv, dm.cap, v, len, vsum);
+  };
+  CAOTE_LAUNCH("fast_vsum_kernel", st, {
+    if (p->dtype == CAOTE_BF16) {
+      if (dm.D == 128) launch(fast::vsum_kernel<__nv_bfloat16, 128>, (const __nv_bfloat16*)V);
+      else launch(fast::vsum_kernel<__nv_bfloat16, 64>, (const __nv_bfloat16*)V);
+    } else {
+      if (dm.D == 128) launch(fast::vsum_kernel<float, 128>, (const float*)V);
+      else launch(fast::vsum_kernel<float, 64>, (const float*)V);
+    }
+  });
   return CAOTE_OK;
 }
 
@@ -1125,9 +1145,15 @@ int caote_compact(const caote_params_t* p, void* K, void* V, float* base, int32_
     CAOTE_LAUNCH("compact_fill_kernel", st, launch_pdl(sel::compact_fill_kernel, dim3(dm.units), dim3(dm.m > 16 ? sel::kSelThreads : 256), 0, st, dm.Hkv, dm.cap, row_bytes, (char*)K, (char*)V, base, pos,
                                                        len, evict_idx, max_evict, n_evict));
   } else {
-    dim3 grid(dm.units, 3);
-    CAOTE_LAUNCH("compact_stable_kernel", st, sel::compact_stable_kernel<<<grid, 256, (size_t)sel::kStableTile * row_bytes, st>>>(
-        dm.Hkv, dm.cap, row_bytes, (char*)K, (char*)V, base, pos, len, evict_idx, max_evict, n_evict));
+    rc = allow_smem(sel::compact_stable_kernel, 2 * sel::kStableTileBytes);
+    if (rc) return rc;
+    int c = 1;  // (three CTAs fit an SM)
+    while (2 * c <= sel::kStableMaxCtas && dm.units * 3 * 2 * c <= 3 * g_sm_count) c *= 2;
+    dim3 grid(dm.units * c, 3);
+    CAOTE_LAUNCH("compact_stable_kernel", st,
+                 launch_pdl_clusters(sel::compact_stable_kernel, grid, dim3(sel::kStableThreads), 2 * sel::kStableTileBytes,
+                                     c, st, dm.Hkv, dm.cap, row_bytes, (char*)K, (char*)V, base, pos, (const int*)len,
+                                     evict_idx, max_evict, n_evict));
   }
   CAOTE_LAUNCH("update_len_kernel", st, launch_pdl(sel::update_len_kernel, dim3((dm.B + 127) / 128), dim3(128), 0, st, dm.B, len, n_evict));
   return CAOTE_OK;
@@ -1154,11 +1180,11 @@ static int step_impl(const caote_params_t* p, const void* q, const void* k_new, 
       const Dims dm = make_dims(p);
       cudaStream_t st = (cudaStream_t)stream;
       if (bf16) {
-        CAOTE_LAUNCH("fast_vsum_add_kernel", st, fast::vsum_add_kernel<__nv_bfloat16><<<dm.units, dm.D, 0, st>>>(
-            dm.Hkv, dm.cap, dm.m, dm.D, (const __nv_bfloat16*)v_new, len, vsum));
+        CAOTE_LAUNCH("fast_vsum_add_kernel", st, launch_pdl(fast::vsum_add_kernel<__nv_bfloat16>, dim3(dm.units), dim3(dm.D), 0, st,
+            dm.Hkv, dm.cap, dm.m, dm.D, (const __nv_bfloat16*)v_new, (const int*)len, vsum));
       } else {
-        CAOTE_LAUNCH("fast_vsum_add_kernel", st, fast::vsum_add_kernel<float><<<dm.units, dm.D, 0, st>>>(
-            dm.Hkv, dm.cap, dm.m, dm.D, (const float*)v_new, len, vsum));
+        CAOTE_LAUNCH("fast_vsum_add_kernel", st, launch_pdl(fast::vsum_add_kernel<float>, dim3(dm.units), dim3(dm.D), 0, st,
+            dm.Hkv, dm.cap, dm.m, dm.D, (const float*)v_new, (const int*)len, vsum));
       }
     }
     rc = append_impl(p, K, V, base, pos, len, n_seen, k_new, v_new, workspace, workspace_bytes_, stream,
@@ -1187,10 +1213,10 @@ static int step_impl(const caote_params_t* p, const void* q, const void* k_new, 
     const Dims dm = make_dims(p);
     cudaStream_t st = (cudaStream_t)stream;
     if (bf16) {
-      CAOTE_LAUNCH("fast_vsum_sub_kernel", st, fast::vsum_sub_kernel<__nv_bfloat16><<<dm.units, 128, 0, st>>>(
+      CAOTE_LAUNCH("fast_vsum_sub_kernel", st, launch_pdl(fast::vsum_sub_kernel<__nv_bfloat16>, dim3(dm.units), dim3(128), 0, st,
           dm.Hkv, dm.cap, dm.D, (const __nv_bfloat16*)V, evict_idx, max_evict, n_evict, vsum));
     } else {
-      CAOTE_LAUNCH("fast_vsum_sub_kernel", st, fast::vsum_sub_kernel<float><<<dm.units, 128, 0, st>>>(
+      CAOTE_LAUNCH("fast_vsum_sub_kernel", st, launch_pdl(fast::vsum_sub_kernel<float>, dim3(dm.units), dim3(128), 0, st,
           dm.Hkv, dm.cap, dm.D, (const float*)V, evict_idx, max_evict, n_evict, vsum));
     }
   }

@@ -18,6 +18,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "ptx.cuh"
 
 namespace caote {
 namespace generic {
@@ -25,7 +26,8 @@ namespace generic {
 constexpr int kRT = 16;          // query rows per tile
 constexpr int kKT = 64;          // keys per tile
 constexpr int kThreads = 256;
-constexpr int kCombineRows = 32; // rows per combine CTA
+constexpr int kCombineThreads = 512;
+constexpr int kCombineRows = 16; // rows per combine CTA
 
 struct Scratch {
   float* part_ml;  // [units][splits][Rpad][2]   (max logit, sum of exp(s - max) over all keys but the first one at the max)
@@ -42,12 +44,12 @@ struct Scratch {
 inline int round_up(int x, int a) { return (x + a - 1) / a * a; }
 
 // Number of key splits: enough CTAs to fill the machine a few times over, never more splits than
-// there are 2-tile spans in the cache.
+// there are key tiles in the cache (a tile is a chain of its own latency: 256 tokens, 2 units: 9 us in spans of two, 5 in one).
 inline int choose_splits(const Dims& dm) {
   const int row_tiles = (dm.R + kRT - 1) / kRT;
   const long ctas = (long)dm.units * row_tiles;
   int s = (int)(((long)g_sm_count * 4 + ctas - 1) / ctas);
-  const int max_by_cap = (dm.cap + 2 * kKT - 1) / (2 * kKT);
+  const int max_by_cap = (dm.cap + kKT - 1) / kKT;
   if (s > max_by_cap) s = max_by_cap;
   if (s > 32) s = 32;
   if (s < 1) s = 1;
@@ -78,22 +80,25 @@ inline size_t carve(const Dims& dm, char* base, Scratch* out) {
   return off;
 }
 
-// scale * <q, k> over D channels, in one fixed order, from two fp32 rows in shared memory. Both the
-// attention pass and the score pass call this, so a logit has the same bits in both.
-template <int D>
-__device__ __forceinline__ float logit(const float* __restrict__ qrow, const float* __restrict__ krow,
-                                       float scale) {
-  float acc = 0.f;
+// scale * <q, k> over D channels, in one fixed order, from fp32 rows in shared memory, for four keys 16 rows apart (the
+// query row is fetched once for all of them). All passes call this, so a logit has the same bits in all of them.
+template <int D, int LD>
+__device__ __forceinline__ void logit4(const float* __restrict__ qrow, const float* __restrict__ krow, float scale, float (&s)[4]) {
+  s[0] = s[1] = s[2] = s[3] = 0.f;
 #pragma unroll 8
   for (int c = 0; c < D; c += 4) {
     const float4 a = *reinterpret_cast<const float4*>(qrow + c);
-    const float4 b = *reinterpret_cast<const float4*>(krow + c);
-    acc = fmaf(a.x, b.x, acc);
-    acc = fmaf(a.y, b.y, acc);
-    acc = fmaf(a.z, b.z, acc);
-    acc = fmaf(a.w, b.w, acc);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float4 b = *reinterpret_cast<const float4*>(krow + i * 16 * LD + c);
+      s[i] = fmaf(a.x, b.x, s[i]);
+      s[i] = fmaf(a.y, b.y, s[i]);
+      s[i] = fmaf(a.z, b.z, s[i]);
+      s[i] = fmaf(a.w, b.w, s[i]);
+    }
   }
-  return acc * scale;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) s[i] *= scale;
 }
 
 // Stage `rows` rows of D elements (global, dtype T) into shared memory as fp32 with row stride LD;
@@ -121,6 +126,8 @@ attn_partial_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, c
                     const int* __restrict__ len, const float* __restrict__ base, Scratch sc, int* status) {
   constexpr int LD = D + 4;
   constexpr int OC = D / 16;  // output channels per thread (two float4 for D = 128, one for D = 64)
+  ptx::pdl_wait();
+  ptx::pdl_trigger();
   extern __shared__ __align__(16) float smem[];
   float* Qs = smem;
   float* Ks = Qs + kRT * LD;
@@ -175,11 +182,12 @@ attn_partial_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, c
     __syncthreads();
 
     float s[4];
+    logit4<D, LD>(Qs + r * LD, Ks + c0 * LD, dm.scale, s);  // (rows beyond the length are staged as zeros)
     float mx = -INFINITY;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int j = kt + c0 + 16 * i;
-      s[i] = (j < k_end && j < n_vis) ? logit<D>(Qs + r * LD, Ks + (c0 + 16 * i) * LD, dm.scale) : -INFINITY;
+      if (j >= k_end || j >= n_vis) s[i] = -INFINITY;
       mx = fmaxf(mx, s[i]);
     }
 #pragma unroll
@@ -267,30 +275,53 @@ __device__ __forceinline__ bool row_counted(const Dims& dm, int r) {
   return dm.base_mode != CAOTE_BASE_EXTERNAL;
 }
 
+// grid = (chunks of kCombineRows rows, units); a thread is a channel of every (kCombineThreads / D)-th row of the chunk. What
+// it costs is round trips to L2: the splits' statistics and outputs are fetched eight at a time before the first is used
+// (a thread per channel for 32 rows, one value after the other: 27 - 83 us for 28 - 96 rows in up to 32 splits).
 template <typename T, int D>
-__global__ void __launch_bounds__(D)
+__global__ void __launch_bounds__(kCombineThreads)
 attn_combine_kernel(Dims dm, const int* __restrict__ len, Scratch sc, float* __restrict__ o) {
-  const int unit = blockIdx.y, chunk = blockIdx.x, c = threadIdx.x;
+  constexpr int kGroups = kCombineThreads / D, kFly = 8;
+  ptx::pdl_wait();
+  ptx::pdl_trigger();
+  __shared__ float part[kGroups][D];
+  const int unit = blockIdx.y, chunk = blockIdx.x, c = threadIdx.x % D, grp = threadIdx.x / D;
   const int b = unit / dm.Hkv, h = unit % dm.Hkv;
   const int n = len[b];
   if (n == 0 || n < dm.m || n > dm.cap) return;
   float osum = 0.f;
   const int r_end = min(dm.R, (chunk + 1) * kCombineRows);
-  for (int r = chunk * kCombineRows; r < r_end; ++r) {
+  for (int r = chunk * kCombineRows + grp; r < r_end; r += kGroups) {
+    const float2* ml = reinterpret_cast<const float2*>(sc.part_ml) + (size_t)unit * sc.splits * sc.Rpad + r;
+    const float* po = sc.part_o + ((size_t)unit * sc.splits * sc.Rpad + r) * D + c;
     float mx = -INFINITY;
-    for (int s = 0; s < sc.splits; ++s)
-      mx = fmaxf(mx, sc.part_ml[(((size_t)unit * sc.splits + s) * sc.Rpad + r) * 2]);
+    for (int s0 = 0; s0 < sc.splits; s0 += kFly) {
+      float v[kFly];
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) v[u] = (s0 + u < sc.splits) ? ml[(size_t)(s0 + u) * sc.Rpad].x : -INFINITY;
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) mx = fmaxf(mx, v[u]);
+    }
     float l_rest = 0.f, acc = 0.f;
     bool top_seen = false;  // the first split at the overall maximum keeps its top key apart; the others' join the rest
-    for (int s = 0; s < sc.splits; ++s) {
-      const size_t idx = ((size_t)unit * sc.splits + s) * sc.Rpad + r;
-      const float ms = sc.part_ml[idx * 2];
-      if (ms == -INFINITY) continue;
-      const float f = expf(ms - mx);
-      l_rest = fmaf(sc.part_ml[idx * 2 + 1], f, l_rest);
-      if (ms == mx && !top_seen) top_seen = true;
-      else l_rest += f;
-      acc = fmaf(sc.part_o[idx * D + c], f, acc);
+    for (int s0 = 0; s0 < sc.splits; s0 += kFly) {
+      float2 st[kFly];
+      float ov[kFly];
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) {
+        const bool in = s0 + u < sc.splits;
+        st[u] = in ? ml[(size_t)(s0 + u) * sc.Rpad] : make_float2(-INFINITY, 0.f);
+        ov[u] = in ? po[(size_t)(s0 + u) * sc.Rpad * D] : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) {
+        if (st[u].x == -INFINITY) continue;  // (a split in which the row sees no key)
+        const float f = expf(st[u].x - mx);
+        l_rest = fmaf(st[u].y, f, l_rest);
+        if (st[u].x == mx && !top_seen) top_seen = true;
+        else l_rest += f;
+        acc = fmaf(ov[u], f, acc);
+      }
     }
     const float inv_l = 1.f / (l_rest + 1.f);
     const float val = acc * inv_l;
@@ -302,16 +333,33 @@ attn_combine_kernel(Dims dm, const int* __restrict__ len, Scratch sc, float* __r
       sc.stats[((size_t)unit * sc.Rpad + r) * 4 + 2] = l_rest * inv_l;
     }
   }
-  sc.osum[((size_t)unit * sc.chunks + chunk) * D + c] = osum;
-  if (chunk == 0 && (dm.base_mode == CAOTE_BASE_ACCUM || dm.base_mode == CAOTE_BASE_EXTERNAL)) {
+  part[grp][c] = osum;
+  __syncthreads();
+  if (grp == 0) {
+    for (int g = 1; g < kGroups; ++g) osum += part[g][c];
+    sc.osum[((size_t)unit * sc.chunks + chunk) * D + c] = osum;
+  }
+  if (chunk == 0 && grp == kGroups - 1 && (dm.base_mode == CAOTE_BASE_ACCUM || dm.base_mode == CAOTE_BASE_EXTERNAL)) {
     float y = 0.f;
-    for (int s = 0; s < sc.splits; ++s) y += sc.part_y[((size_t)unit * sc.splits + s) * D + c];
-    sc.ytot[(size_t)unit * D + c] = y;
-    if (c == 0) {
-      double hb = 0.0;
-      for (int s = 0; s < sc.splits; ++s) hb += (double)sc.part_hb[(size_t)unit * sc.splits + s];
-      sc.hbtot[unit] = (float)hb;
+    double hb = 0.0;
+    for (int s0 = 0; s0 < sc.splits; s0 += kFly) {
+      float yv[kFly], hv[kFly];
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) {
+        const size_t us = (size_t)unit * sc.splits + min(s0 + u, sc.splits - 1);
+        yv[u] = sc.part_y[us * D + c];
+        hv[u] = sc.part_hb[us];
+      }
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) {
+        if (s0 + u < sc.splits) {
+          y += yv[u];
+          hb += (double)hv[u];
+        }
+      }
     }
+    sc.ytot[(size_t)unit * D + c] = y;
+    if (c == 0) sc.hbtot[unit] = (float)hb;
   }
 }
 
@@ -321,6 +369,8 @@ score_pass_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
                   const int* __restrict__ len, float* __restrict__ base, Scratch sc,
                   float* __restrict__ scores, const float* __restrict__ vsum) {
   constexpr int LD = D + 4;
+  ptx::pdl_wait();
+  ptx::pdl_trigger();
   extern __shared__ __align__(16) float smem[];
   float* Qs = smem;              // kRT * LD
   float* Ks = Qs + kRT * LD;     // kKT * LD
@@ -345,6 +395,7 @@ score_pass_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
   // X = (sum of counted output rows + sum_j base_j v_j) / (counted rows + sum_j base_j)
   if (tid < D) {
     float x = 0.f;
+    #pragma unroll 8
     for (int ch = 0; ch < sc.chunks; ++ch) x += sc.osum[((size_t)unit * sc.chunks + ch) * D + tid];
     if (carried) x += sc.ytot[(size_t)unit * D + tid];
     Xs[tid] = (Htot > 0.f) ? x / Htot : 0.f;
@@ -388,11 +439,13 @@ score_pass_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
       const int row = (mode == CAOTE_BASE_LAST_QUERY) ? t * dm.m + dm.m - 1 : t;
       const int n_vis = n - dm.m + (row % dm.m) + 1;
       const float mx = st[r * 4], il = st[r * 4 + 1], cr = st[r * 4 + 2];
+      float sl4[4];
+      logit4<D, LD>(Qs + r * LD, Ks + c0 * LD, dm.scale, sl4);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int j = j0 + c0 + 16 * i;
         if (j < n_vis) {
-          const float sl = logit<D>(Qs + r * LD, Ks + (c0 + 16 * i) * LD, dm.scale);
+          const float sl = sl4[i];
           const float a = expf(sl - mx) * il;
           hacc[i] += a;
           cacc[i] += (sl == mx) ? cr : 1.f - a;
@@ -478,6 +531,8 @@ __global__ void __launch_bounds__(kThreads)
 sum_errors_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, const T* __restrict__ V,
                   const int* __restrict__ len, const float* __restrict__ o, Scratch sc, float* __restrict__ scores) {
   constexpr int LD = D + 4;
+  ptx::pdl_wait();
+  ptx::pdl_trigger();
   extern __shared__ __align__(16) float smem[];
   float* Qs = smem;              // kRT * LD
   float* Os = Qs + kRT * LD;     // kRT * LD
@@ -532,11 +587,13 @@ sum_errors_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
       const int row = (mode == CAOTE_BASE_LAST_QUERY) ? t * dm.m + dm.m - 1 : t;
       const int n_vis = n - dm.m + (row % dm.m) + 1;
       const float mx = st[r * 4], il = st[r * 4 + 1], cr = st[r * 4 + 2];
+      float sl4[4];
+      logit4<D, LD>(Qs + r * LD, Ks + c0 * LD, dm.scale, sl4);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int jj = c0 + 16 * i, j = j0 + jj;
         if (j < n_vis) {
-          const float sl = logit<D>(Qs + r * LD, Ks + jj * LD, dm.scale);
+          const float sl = sl4[i];
           const float e = expf(sl - mx) * il;              // alpha
           const float rest = (sl == mx) ? cr : 1.f - e;    // 1 - alpha: the others' share, without cancellation
           float d2 = 0.f;

@@ -91,3 +91,29 @@ def test_corrected_output_of_query_blocks(case):
     # o and the evicted share both carry P's 16 bits (8e-6 of the largest value, about 4); what is left over after the
     # subtraction is divided by the retained weight, 0.04 at the least here (13 of 270 tokens kept)
     assert_close(f32(o_post), ref, f"{case}", atol=2e-3 if budget[0] * 4 < lens[0] else 2e-4)
+
+
+@pytest.mark.parametrize("dtype,d", [(torch.bfloat16, 128), (torch.float32, 128), (torch.bfloat16, 64)])
+@pytest.mark.parametrize("n,first,k", [(4100, 0, 1), (4100, 3000, 2), (3071, 5, 2500), (1025, 1024, 1)])
+def test_stable_compaction_over_several_rounds(n, first, k, dtype, d):
+    """More slots than a round of the cluster's tiles holds (512 at the least, 2048 at the most), the first evicted slot at
+    either end, and more picks than shared memory keeps."""
+    g = torch.Generator().manual_seed(n + first)
+    B, Hkv, cap = 1, 2, n + 7
+    K, V = (torch.randn((B, Hkv, cap, d), generator=g).to(dtype).to(DEV) for _ in range(2))
+    base, pos = torch.rand((B, Hkv, cap), generator=g).to(DEV), torch.arange(cap, dtype=torch.int32, device=DEV).expand(B, Hkv, cap).contiguous()
+    ev = torch.stack([torch.cat([torch.tensor([first]), first + 1 + torch.randperm(n - first - 1, generator=g)[:k - 1].sort().values])
+                      for _ in range(Hkv)]).to(torch.int32).view(B, Hkv, k)
+    lens = torch.tensor([n], dtype=torch.int32, device=DEV)
+    p = P.make_params(B, Hkv, Hkv, d, cap, 1, dtype, 1.0, "last_query")
+    K0, V0, b0 = K.clone(), V.clone(), base.clone()
+    P.caote_compact(p, K, V, base, pos, lens, ev.to(DEV), torch.tensor([k], dtype=torch.int32, device=DEV), "stable", P.alloc_workspace(p, DEV))
+    assert lens.item() == n - k
+    for h in range(Hkv):
+        keep = torch.ones(n, dtype=torch.bool)
+        keep[ev[0, h].long()] = False
+        idx = keep.nonzero().flatten().to(DEV)
+        assert torch.equal(pos[0, h, :n - k].long(), idx)
+        assert torch.equal(K[0, h, :n - k], K0[0, h, idx]) and torch.equal(V[0, h, :n - k], V0[0, h, idx])
+        assert torch.equal(base[0, h, :n - k], b0[0, h, idx])
+        assert torch.equal(K[0, h, n:], K0[0, h, n:]) and torch.equal(V[0, h, n:], V0[0, h, n:])
