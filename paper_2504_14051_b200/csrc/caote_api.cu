@@ -264,46 +264,54 @@ static int decode_grid_limit() {
 
 static inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
-// Shapes the persistent decode kernel covers; everything else takes the generic path.
-static bool decode_shape_ok(const caote_params_t* p) {
+// Shapes the single-query cluster kernel covers, as long as its clusters hold a unit.
+static bool cluster_shape_ok(const caote_params_t* p) {
   const int G = p->n_q_heads / p->n_kv_heads;
   const bool carried = p->base_mode == CAOTE_BASE_ACCUM || p->base_mode == CAOTE_BASE_EXTERNAL;
   // a carried base score rides in row 7 of the P operand (G <= 7) and is staged by 16-byte bulk copies
-  return p->dtype == CAOTE_BF16 && p->head_dim == 128 && p->n_new == 1 && G <= 8 &&
-         !(carried && (G > 7 || p->capacity % 4 != 0)) &&
+  return p->dtype == CAOTE_BF16 && p->n_new == 1 && G <= 8 && !(carried && (G > 7 || p->capacity % 4 != 0)) &&
          (long long)p->batch * p->n_kv_heads * p->capacity < (1LL << 31);
 }
+// ... and, at head_dim 128, the streaming kernel whatever the unit's length. (At head_dim 64 longer units take the row-block
+// kernels.)
+static bool decode_shape_ok(const caote_params_t* p) { return p->head_dim == 128 && cluster_shape_ok(p); }
 
 // ---- single-query path on thread-block clusters ---------------------------------------------------------
 typedef void (*ClusterKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, Dims, const int*, float*, float*,
                               float*, int*, long long, const float*);
-template <int kMode>
+template <int kMode, int D>
 static ClusterKernel cluster_kernel_for_g(int g) {
   switch (g) {
-    case 1: return dcl::decode_cluster_kernel<1, kMode>;
-    case 2: return dcl::decode_cluster_kernel<2, kMode>;
-    case 3: return dcl::decode_cluster_kernel<3, kMode>;
-    case 4: return dcl::decode_cluster_kernel<4, kMode>;
-    case 5: return dcl::decode_cluster_kernel<5, kMode>;
-    case 6: return dcl::decode_cluster_kernel<6, kMode>;
-    case 7: return dcl::decode_cluster_kernel<7, kMode>;
-    default: return dcl::decode_cluster_kernel<8, kMode>;
+    case 1: return dcl::decode_cluster_kernel<1, kMode, D>;
+    case 2: return dcl::decode_cluster_kernel<2, kMode, D>;
+    case 3: return dcl::decode_cluster_kernel<3, kMode, D>;
+    case 4: return dcl::decode_cluster_kernel<4, kMode, D>;
+    case 5: return dcl::decode_cluster_kernel<5, kMode, D>;
+    case 6: return dcl::decode_cluster_kernel<6, kMode, D>;
+    case 7: return dcl::decode_cluster_kernel<7, kMode, D>;
+    default: return dcl::decode_cluster_kernel<8, kMode, D>;
   }
 }
-// The instantiation for a group size and a base mode (LAST_QUERY and CHUNK_SUM coincide for one query).
-static ClusterKernel cluster_kernel(int g, int base_mode) {
-  if (base_mode == CAOTE_BASE_ACCUM) return cluster_kernel_for_g<CAOTE_BASE_ACCUM>(g > 7 ? 7 : g);
-  if (base_mode == CAOTE_BASE_EXTERNAL) return cluster_kernel_for_g<CAOTE_BASE_EXTERNAL>(g > 7 ? 7 : g);
-  return cluster_kernel_for_g<CAOTE_BASE_LAST_QUERY>(g);
+template <int D>
+static ClusterKernel cluster_kernel_for(int g, int base_mode) {
+  if (base_mode == CAOTE_BASE_ACCUM) return cluster_kernel_for_g<CAOTE_BASE_ACCUM, D>(g > 7 ? 7 : g);
+  if (base_mode == CAOTE_BASE_EXTERNAL) return cluster_kernel_for_g<CAOTE_BASE_EXTERNAL, D>(g > 7 ? 7 : g);
+  return cluster_kernel_for_g<CAOTE_BASE_LAST_QUERY, D>(g);
 }
+// The instantiation for a group size, a base mode (LAST_QUERY and CHUNK_SUM coincide for one query) and a head dimension.
+static ClusterKernel cluster_kernel(const Dims& dm) {
+  return dm.D == 128 ? cluster_kernel_for<128>(dm.G, dm.base_mode) : cluster_kernel_for<64>(dm.G, dm.base_mode);
+}
+static size_t cluster_smem_bytes(int D) { return D == 128 ? dcl::smem_bytes<128>() : dcl::smem_bytes<64>(); }
 
 // Clusters of `c` CTAs of the cluster kernel that can be resident on the current device at once; 0 if none.
-static int cluster_capacity(int dev, int c, ClusterKernel kernel) {
-  static std::atomic<int> cached[64][dcl::kMaxC + 1];
+static int cluster_capacity(int dev, int c, ClusterKernel kernel, int D) {
+  static std::atomic<int> cached_by_d[2][64][dcl::kMaxC + 1];
+  auto& cached = cached_by_d[D == 128];
   if (c < 1 || c > dcl::kMaxC) return 0;
   int n = cached[dev][c].load(std::memory_order_acquire);
   if (n == 0) {
-    const size_t smem = dcl::smem_bytes();
+    const size_t smem = cluster_smem_bytes(D);
     n = -1;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
         cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
@@ -340,7 +348,7 @@ static int choose_cluster(const Dims& dm, ClusterKernel kernel, int* clusters_ou
   for (int c = 1; c <= dcl::kMaxC; ++c) {
     if (forced > 0 && c != forced) continue;
     if ((cap_tiles + c - 1) / c > dcl::kMaxT) continue;
-    const int n = cluster_capacity(dev, c, kernel);
+    const int n = cluster_capacity(dev, c, kernel, dm.D);
     if (n <= 0) continue;
     const long long rounds = ((long long)dm.units + n - 1) / n;
     const double cost = (double)rounds * ((double)cap_tiles / c + 2.0 + 0.05 * c);
@@ -384,7 +392,7 @@ static int launch_decode_cluster(const Dims& dm, const void* q, const void* K, c
   TensorMapEncodeFn encode = tensor_map_encoder();
   const bool carried = dm.base_mode == CAOTE_BASE_ACCUM || dm.base_mode == CAOTE_BASE_EXTERNAL;
   if (!encode || (carried && !aligned(base, 16)) || !aligned(q, 16)) return CAOTE_OK;
-  const ClusterKernel kernel = cluster_kernel(dm.G, dm.base_mode);
+  const ClusterKernel kernel = cluster_kernel(dm);
   // (the attributes below are per function: every instantiation gets them the first time it is used)
   static std::mutex attr_mu;
   static std::vector<std::pair<int, ClusterKernel>> attr_done;
@@ -395,7 +403,7 @@ static int launch_decode_cluster(const Dims& dm, const void* q, const void* K, c
     bool done = false;
     for (auto& e : attr_done) done |= (e.first == dev && e.second == kernel);
     if (!done) {
-      CAOTE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dcl::smem_bytes()));
+      CAOTE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem_bytes(dm.D)));
       CAOTE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
       attr_done.push_back({dev, kernel});
     }
@@ -410,7 +418,7 @@ static int launch_decode_cluster(const Dims& dm, const void* q, const void* K, c
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(clusters * c));
   cfg.blockDim = dim3(dcl::kThreads);
-  cfg.dynamicSmemBytes = dcl::smem_bytes();
+  cfg.dynamicSmemBytes = cluster_smem_bytes(dm.D);
   cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -509,9 +517,9 @@ static Dims sub_dims(const Dims& dm, int count) {
 }
 
 // SMs the cluster kernel occupies on these dimensions.
-static int side_clusters_sms(const Dims& d, int base_mode) {
+static int side_clusters_sms(const Dims& d) {
   int n = 0;
-  const int c = choose_cluster(d, cluster_kernel(d.G, base_mode), &n);
+  const int c = choose_cluster(d, cluster_kernel(d), &n);
   if (n > d.units) n = d.units;
   return c * n;
 }
@@ -523,12 +531,12 @@ static int side_clusters_sms(const Dims& d, int base_mode) {
 // to the streaming kernel instead, on a second stream and on as many CTAs as there are SMs outside the clusters, at
 // the same time as the cluster kernel works on the others. Returns the number of tail sequences (0: one kernel).
 // The estimates only rank the options; rates in bytes per second per SM and per cluster round are measured ones.
-static int plan_side_by_side(const Dims& dm, int base_mode) {
+static int plan_side_by_side(const Dims& dm) {
   const int mode = g_side_by_side.load(std::memory_order_relaxed);
   if (mode == 0 || dm.B < 2) return 0;
   if (mode >= 2) {  // forced: the last mode - 1 sequences, if the cluster kernel can take the others
     const int tail = mode - 1 < dm.B ? mode - 1 : dm.B - 1;
-    return side_clusters_sms(sub_dims(dm, dm.B - tail), base_mode) > 0 ? tail : 0;
+    return side_clusters_sms(sub_dims(dm, dm.B - tail)) > 0 ? tail : 0;
   }
   const double unit_bytes = (double)dm.cap * dm.D * 4.0;  // K and V rows, bf16
   // measured: the cluster kernel moves about 33 GB/s of K and V per SM it occupies (3.7 TB/s on 112 SMs, 4.5 on 135);
@@ -538,7 +546,7 @@ static int plan_side_by_side(const Dims& dm, int base_mode) {
   auto cluster_time = [&](int seqs, int* idle) {
     const Dims d = sub_dims(dm, seqs);
     int n = 0;
-    const int c = choose_cluster(d, cluster_kernel(dm.G, base_mode), &n);
+    const int c = choose_cluster(d, cluster_kernel(d), &n);
     if (c == 0 || n == 0) return -1.0;
     if (n > d.units) n = d.units;
     *idle = g_sm_count - n * c;
@@ -952,7 +960,7 @@ static int score_impl(const caote_params_t* p, const void* q, const void* K, con
     if (!vsum) {
       const bool carried = dm.base_mode == CAOTE_BASE_ACCUM || dm.base_mode == CAOTE_BASE_EXTERNAL;
       const int tail = (allow_side_stream && decode_grid_limit() > 0 && tensor_map_encoder() && aligned(q, 16) &&
-                        (!carried || aligned(base, 16))) ? plan_side_by_side(dm, dm.base_mode) : 0;
+                        (!carried || aligned(base, 16))) ? plan_side_by_side(dm) : 0;
       if (tail > 0) {
         // the first B - tail sequences on the cluster kernel, the last `tail` on the streaming kernel beside it
         const int head = dm.B - tail;
@@ -972,7 +980,7 @@ static int score_impl(const caote_params_t* p, const void* q, const void* K, con
           rc = launch_decode_score(dt, (const __nv_bfloat16*)q + qo, (const __nv_bfloat16*)K + uo * dm.cap * dm.D,
                                    (const __nv_bfloat16*)V + uo * dm.cap * dm.D, len + head, base ? base + uo * dm.cap : nullptr,
                                    o + qo, scores + uo * dm.cap, status, scratch, rowstat + uo * kHeadStatFloats, -1,
-                                   g_sm_count - side_clusters_sms(dh, dm.base_mode), ss.stream, &used_t, nullptr);
+                                   g_sm_count - side_clusters_sms(dh), ss.stream, &used_t, nullptr);
           if (!rc && !used_t) rc = CAOTE_ERR_CUDA;  // (its preconditions were checked above)
           const cudaError_t e1 = cudaEventRecord(ss.join, ss.stream);
           const cudaError_t e2 = cudaStreamWaitEvent(st, ss.join, 0);
@@ -990,6 +998,11 @@ static int score_impl(const caote_params_t* p, const void* q, const void* K, con
       if (rc || used) return rc;
     }
     rc = launch_decode_score(dm, q, K, V, len, base, o, scores, status, scratch, rowstat, kStatPerHead, 0, st, &used, vsum);
+    if (rc || used) return rc;
+  }
+  if (cluster_shape_ok(p) && dm.D == 64) {
+    bool used = false;
+    rc = launch_decode_cluster(dm, q, K, V, len, base, o, scores, ws, st, &used, vsum);
     if (rc || used) return rc;
   }
   if (row_blocks && prefill_shape_ok(p)) {

@@ -1,4 +1,4 @@
-// Single-query (decode) scoring path, bf16, head_dim 128, group size <= 8: one thread-block cluster per
+// Single-query (decode) scoring path, bf16, head_dim 64 or 128, group size <= 8: one thread-block cluster per
 // (sequence, KV head) unit, K and V read from HBM exactly once.
 //
 // Why a cluster. The score c_j = w_j / (1 - w_j) * ||X - v_j|| needs every value row twice: once for
@@ -9,8 +9,8 @@
 //     O^T += V_tile^T P^T run on tcgen05 with the tile's tokens on the M side (a token owns one TMEM
 //     lane); the softmax group turns S^T into P^T; the keeper group copies every token's value row (256
 //     bytes) from the landed V tile into a TMEM stash slot (64 columns per tile, 7 slots beside the
-//     accumulators; a CTA's tiles beyond the 7th stay in their V ring slot instead) and keeps the
-//     token's logits in registers;
+//     accumulators; a CTA's tiles beyond the 7th stay in their V ring slot instead; at head_dim 64 half of
+//     that, and all tiles fit) and keeps the token's logits in registers;
 //   * merge: the softmax group pushes its (reference, sums, partial output) record to the peers through
 //     distributed shared memory (st.async, completion counted by an mbarrier of the receiver): the
 //     softmax statistics go to everyone, the partial outputs to the CTA that owns the channel slice;
@@ -54,10 +54,8 @@ using decode::bulk_load;
 using decode::fast_exp2;
 using decode::fence_async_smem;
 using decode::idesc_n16;
-using decode::kD;
 using decode::kHalfBytes;
 using decode::kT;
-using decode::kTileBytes;
 using decode::mbar_arrive;
 using decode::mbar_expect_tx;
 using decode::mbar_init;
@@ -70,11 +68,16 @@ using decode::tmem_ld16;
 using decode::tmem_ld8;
 using decode::tmem_st16;
 
-constexpr int kKS = 2;                    // K ring slots (a slot is free as soon as S^T is formed)
-constexpr int kVS = 4;                    // V ring slots (free after O^T += and the stash copy)
+template <int D>
+constexpr int kTileBytesOf = (D / 64) * kHalfBytes;
+template <int D>
+constexpr int kKSlots = 2 * (128 / D);    // K ring slots, 64 KB of them (a slot is free as soon as S^T is formed)
+template <int D>
+constexpr int kVSlots = 4 * (128 / D);    // V ring slots, 128 KB of them (free after O^T += and the stash copy)
 constexpr int kSB = 3;                    // S^T buffers in TMEM (free once both groups have read them)
-constexpr int kStash = 7;                 // value tiles a CTA keeps in TMEM
-constexpr int kMaxT = 9;                  // tiles of one unit per CTA: the stash + 2 held in the V ring
+template <int D>
+constexpr int kStashTiles = 7 * (128 / D);  // value tiles a CTA can keep in TMEM (D / 2 columns each)
+constexpr int kMaxT = 9;                  // tiles of one unit per CTA: the stash + 2 held in the V ring (head_dim 64: the stash)
 constexpr int kMaxC = 16;                 // largest cluster
 constexpr int kGroup = 128;               // threads of a token group
 constexpr int kNB = 2;                    // keeper groups
@@ -84,7 +87,7 @@ constexpr int kMaxKeep = (kMaxT + kNB - 1) / kNB;   // tiles of one unit per kee
 constexpr int kQBufBytes = 2048;          // 8 query rows x 128 channels as two 64-channel boxes
 constexpr int kPBytes = 4096;             // 16 rows x 128 tokens as two 64-token boxes
 constexpr int kStatFloats = 36;           // per CTA: ref[8] lrest[8] pmax[8] smax[8] brest bmax pad pad
-constexpr int kXoFloats = 8 * (kD + kMaxC);  // partial outputs received: [C][slice][8], slice = ceil(128 / C)
+constexpr int kXoFloats = 8 * (128 + kMaxC);  // partial outputs received: [C][slice][8], slice = ceil(128 / C)
 constexpr int kLenTab = 512;              // unit lengths of this cluster kept in shared memory
 constexpr uint32_t kTmemCols = 512;       // S^T x 3, O^T (16 columns each), 7 stash slots of 64 columns
 constexpr long long kDrainCycles = 4000000000LL;  // waits for hardware to finish what was already issued
@@ -101,9 +104,10 @@ struct Fin {        // per unit, every CTA computes its own copy
   float brest;      // sum of the other carried base scores
 };
 
+template <int D>
 inline size_t smem_bytes() {
-  return 1024 + (size_t)(kKS + kVS) * kTileBytes + 2 * kQBufBytes + kPBytes + kVS * (kT * 4) +
-         kMaxC * kStatFloats * 4 + kXoFloats * 4 + 2 * kD * 4 + kNB * sizeof(Fin) + kNB * kMaxC * 8 * 4 /* fac */ +
+  return 1024 + (size_t)(kKSlots<D> + kVSlots<D>) * kTileBytesOf<D> + 2 * kQBufBytes + kPBytes + kVSlots<D> * (kT * 4) +
+         kMaxC * kStatFloats * 4 + kXoFloats * 4 + 2 * D * 4 + kNB * sizeof(Fin) + kNB * kMaxC * 8 * 4 /* fac */ +
          2 * 32 * 4 /* red */ + 4 * 28 * 4 /* gred */ + kStatFloats * 4 /* mystat */ + kLenTab * 4 + 64 * 8 /* barriers, control words */ + 64;
 }
 
@@ -238,27 +242,31 @@ struct Sched {
 
 // kG: query heads per KV head; kMode: the base mode. Compile-time so that the per-head loops carry no
 // predicates and the paths of the other modes are not in the instruction stream.
-template <int kG, int kMode>
+template <int kG, int kMode, int D>
 __global__ void __launch_bounds__(kThreads, 1)
 decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                       const __grid_constant__ CUtensorMap tmQ, Dims dm, const int* __restrict__ len,
                       float* __restrict__ base, float* __restrict__ o, float* __restrict__ scores, int* status,
                       long long wait_cycles, const float* __restrict__ vsum) {
+  constexpr int kTileBytes = kTileBytesOf<D>, kKS = kKSlots<D>, kVS = kVSlots<D>, kStash = kStashTiles<D>;
+  constexpr int kBoxes = D / 64, kRowCols = D / 2;  // 64-channel boxes of a tile; TMEM columns of a stashed row
   ptx::pdl_wait();
   ptx::pdl_trigger();
   extern __shared__ char smem_raw[];
   // (aligned by an offset into the array, not through an integer: the pointer keeps its address space, and what is
   // read and written through it compiles to shared-memory accesses, not generic ones)
   char* sm = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
-  char* tilesK = sm;                                                   // [kKS][kTileBytes]
-  char* tilesV = tilesK + kKS * kTileBytes;                            // [kVS][kTileBytes]
-  char* qbuf = tilesV + kVS * kTileBytes;                              // [2][kQBufBytes]
+  // (at head_dim 64 the K ring lies behind the V ring: the O^T products, M 128, read their rows 64..127, which nobody uses,
+  // from the 16 KB behind the V tile)
+  char* tilesK = sm + (D == 64 ? kVS * kTileBytes : 0);                // [kKS][kTileBytes]
+  char* tilesV = sm + (D == 64 ? 0 : kKS * kTileBytes);                // [kVS][kTileBytes]
+  char* qbuf = sm + (kKS + kVS) * kTileBytes;                          // [2][kQBufBytes]
   char* pbuf = qbuf + 2 * kQBufBytes;                                  // [kPBytes]
   float* baseV = reinterpret_cast<float*>(pbuf + kPBytes);             // [kVS][kT] carried base scores of a V slot's tile
   float* xstats = baseV + kVS * kT;                                    // [C][kStatFloats]    written by the peers
   float* xo = xstats + kMaxC * kStatFloats;                            // [C][slice][8]       written by the peers
-  float* xnX = xo + kXoFloats;                                         // [2][kD]  -X         written by the owners
-  Fin* fins = reinterpret_cast<Fin*>(xnX + 2 * kD);                    // [kNB] one copy per keeper group
+  float* xnX = xo + kXoFloats;                                         // [2][D]  -X         written by the owners
+  Fin* fins = reinterpret_cast<Fin*>(xnX + 2 * D);                    // [kNB] one copy per keeper group
   float* facs = reinterpret_cast<float*>(fins + kNB);                  // [kNB][C][8] 2^(ref_c - m) / l per record and head
   float* red = facs + kNB * kMaxC * 8;                                       // [2][4][8] warp maxima of the softmax group
   float* gred = red + 2 * 32;                                          // [4 warps][28] closing sums of the softmax group
@@ -299,10 +307,10 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   sch.slen = slen;
   const int C = sch.C, rank = sch.rank;
   const int nk = sch.count();
-  const int slice = (kD + C - 1) / C;                                   // channels per owner
-  const int my_ch0 = min(rank * slice, kD), my_nch = min(slice, kD - my_ch0);
+  const int slice = (D + C - 1) / C;                                   // channels per owner
+  const int my_ch0 = min(rank * slice, D), my_nch = min(slice, D - my_ch0);
   const uint32_t r1_bytes = (uint32_t)(C * (kStatFloats * 4 + 8 * my_nch * 4));
-  const uint32_t r2_bytes = (uint32_t)(kD * 4 + kNB * C * 4);
+  const uint32_t r2_bytes = (uint32_t)(D * 4 + kNB * C * 4);
 
   if (tid == 0) {
     for (int i = 0; i < kKS; ++i) { mbar_init(&kfull[i], 1); mbar_init(&kempty[i], 1); }
@@ -350,14 +358,14 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           if (ctl[0]) break;
           const int row = w.unit * dm.cap + (w.t0 + j) * kT;
           char* tl = tilesK + s * kTileBytes;
-          mbar_expect_tx(&kfull[s], kTileBytes + (j == 0 ? (uint32_t)kQBufBytes : 0u));
-          tma_load_2d(tl, &tmK, 0, row, &kfull[s], pol);
-          tma_load_2d(tl + kHalfBytes, &tmK, 64, row, &kfull[s], pol);
+          mbar_expect_tx(&kfull[s], kTileBytes + (j == 0 ? (uint32_t)(kBoxes * (kQBufBytes / 2)) : 0u));
+#pragma unroll
+          for (int x = 0; x < kBoxes; ++x) tma_load_2d(tl + x * kHalfBytes, &tmK, 64 * x, row, &kfull[s], pol);
           if (j == 0) {
             char* qb = qbuf + (us & 1) * kQBufBytes;
             const int qrow = b * dm.Hq + h * G;
-            tma_load_2d(qb, &tmQ, 0, qrow, &kfull[s], pol);
-            tma_load_2d(qb + kQBufBytes / 2, &tmQ, 64, qrow, &kfull[s], pol);
+#pragma unroll
+            for (int x = 0; x < kBoxes; ++x) tma_load_2d(qb + x * (kQBufBytes / 2), &tmQ, 64 * x, qrow, &kfull[s], pol);
           }
           ctl[1] = ++ki;
         }
@@ -381,8 +389,8 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           const uint32_t base_bytes = use_base ? (uint32_t)min(kT, dm.cap - t * kT) * 4u : 0u;
           char* tl = tilesV + s * kTileBytes;
           mbar_expect_tx(&vfull[s], kTileBytes + base_bytes);
-          tma_load_2d(tl, &tmV, 0, row, &vfull[s], pol);
-          tma_load_2d(tl + kHalfBytes, &tmV, 64, row, &vfull[s], pol);
+#pragma unroll
+          for (int x = 0; x < kBoxes; ++x) tma_load_2d(tl + x * kHalfBytes, &tmV, 64 * x, row, &vfull[s], pol);
           if (use_base) bulk_load(baseV + s * kT, base + (size_t)w.unit * dm.cap + (size_t)t * kT, base_bytes, &vfull[s]);
           ctl[2] = ++vi;
         }
@@ -405,7 +413,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           prefill::tc_fence_after();
           const uint32_t ka = smem_u32(tilesK + s * kTileBytes);
 #pragma unroll
-          for (int ks = 0; ks < 8; ++ks)
+          for (int ks = 0; ks < D / 16; ++ks)
             prefill::umma(tS + sb * 16, prefill::desc_k_major(ka, ks), desc_q(qa, ks), kIdQK, ks > 0);
           prefill::umma_commit(&sfull[sb]);
           prefill::umma_commit(&kempty[s]);
@@ -567,7 +575,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           if (!valid) {
             char* vt = tilesV + vs * kTileBytes;
 #pragma unroll
-            for (int c = 0; c < 16; ++c) *reinterpret_cast<uint4*>(vt + tile_off(tok, c)) = make_uint4(0u, 0u, 0u, 0u);
+            for (int c = 0; c < D / 8; ++c) *reinterpret_cast<uint4*>(vt + tile_off(tok, c)) = make_uint4(0u, 0u, 0u, 0u);
           }
         }
         fence_async_smem();
@@ -683,12 +691,14 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           push_f32x4(map_to_rank(st_local, peer) + piece * 16, v.x, v.y, v.z, v.w, map_to_rank(bar_local, peer));
         }
         // partial outputs (thread = channel) to the owner of the channel: xo[record][channel in slice][head]
-        const int owner = tok / slice, cl = tok - owner * slice;
-        const int own_nch = min(slice, kD - owner * slice);
-        const uint32_t ra = map_to_rank(smem_u32(xo), owner) + (uint32_t)(((rank * own_nch + cl) * 8) * 4);
-        const uint32_t rb = map_to_rank(bar_local, owner);
-        push_f32x4(ra, osum[0], osum[1], osum[2], osum[3], rb);
-        push_f32x4(ra + 16, osum[4], osum[5], osum[6], osum[7], rb);
+        if (D == 128 || tok < D) {
+          const int owner = tok / slice, cl = tok - owner * slice;
+          const int own_nch = min(slice, D - owner * slice);
+          const uint32_t ra = map_to_rank(smem_u32(xo), owner) + (uint32_t)(((rank * own_nch + cl) * 8) * 4);
+          const uint32_t rb = map_to_rank(bar_local, owner);
+          push_f32x4(ra, osum[0], osum[1], osum[2], osum[3], rb);
+          push_f32x4(ra + 16, osum[4], osum[5], osum[6], osum[7], rb);
+        }
       }
       ++mu;
     }
@@ -741,14 +751,14 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         if (j < kStash) {
           const char* vt = tilesV + vs * kTileBytes;
 #pragma unroll
-          for (int half = 0; half < 2; ++half) {
+          for (int half = 0; half < kBoxes; ++half) {
             uint32_t rw[32];
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
               const uint4 raw = *reinterpret_cast<const uint4*>(vt + tile_off(tok, half * 8 + c));
               rw[4 * c] = raw.x; rw[4 * c + 1] = raw.y; rw[4 * c + 2] = raw.z; rw[4 * c + 3] = raw.w;
             }
-            prefill::tmem_st32u(tStash + lane_base + j * 64 + half * 32, rw);
+            prefill::tmem_st32u(tStash + lane_base + j * kRowCols + half * 32, rw);
           }
           prefill::tmem_st_wait();
           __syncwarp();
@@ -807,7 +817,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       {
         // owners: o and -X of this CTA's channels of this group's parity; 8 lanes per channel, lane = head
         const float inv_H = (fin->Htot > 0.f) ? 1.f / fin->Htot : 0.f;
-        float* xdst = xnX + (mu & 1) * kD;
+        float* xdst = xnX + (mu & 1) * D;
         const int r = tok & 7;
         const int nq = (my_nch - bg + kNB - 1) / kNB;  // channels dealt to this group
         for (int q0 = 0; q0 < nq; q0 += kGroup / 8) {
@@ -824,12 +834,12 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           }
           const float val = v0 + v1;
           const bool is_head = act && r < G;
-          if (is_head) o[((size_t)b * dm.Hq + h * G + r) * kD + my_ch0 + cl] = val;
+          if (is_head) o[((size_t)b * dm.Hq + h * G + r) * D + my_ch0 + cl] = val;
           float xs = (is_head && counted) ? val : ((act && use_base && r == 7) ? val : 0.f);
 #pragma unroll
           for (int off = 4; off > 0; off >>= 1) xs += __shfl_xor_sync(0xffffffffu, xs, off);
           // FastCAOTE (Sec. 3.3): the distances are taken to the mean of the unit's value rows instead of X
-          const float nxv = vsum ? -(act ? __ldg(vsum + (size_t)w.unit * kD + my_ch0 + cl) / (float)w.n : 0.f) : -(xs * inv_H);
+          const float nxv = vsum ? -(act ? __ldg(vsum + (size_t)w.unit * D + my_ch0 + cl) / (float)w.n : 0.f) : -(xs * inv_H);
           if (act && !ctl[0]) {
             for (int peer = r; peer < C; peer += 8)
               push_f32(map_to_rank(smem_u32(xdst + my_ch0 + cl), peer), nxv, map_to_rank(smem_u32(r2), peer));
@@ -850,7 +860,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       // ===================== score pass (a held tile first: its V slot is wanted back) =====================
       {
         const float Htot = fin->Htot, hbsum = fin->hbsum, fbmax = fin->bmax, fbrest = fin->brest;
-        const float* nX = xnX + (mu & 1) * kD;
+        const float* nX = xnX + (mu & 1) * D;
         const int mine = (w.T + kNB - 1 - bg) / kNB;                     // tiles this group kept
         const int first_held = (kStash + kNB - 1 - bg) / kNB;            // smallest jj with kNB jj + bg >= kStash
         const int nheld = max(mine - first_held, 0);
@@ -891,16 +901,16 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           for (int i = 0; i < 4; ++i) acc[i] = make_float2(0.f, 0.f);
           const int vs = (ti + j) % kVS;
           if (j < kStash) {
-            // the row comes back from TMEM in four pieces of 32 channels; the next piece is in flight while
+            // the row comes back from TMEM in pieces of 32 channels; the next piece is in flight while
             // this one is used
             uint32_t ra[16], rb[16];
-            tmem_ld16u(tStash + lane_base + j * 64, ra);
+            tmem_ld16u(tStash + lane_base + j * kRowCols, ra);
 #pragma unroll
-            for (int piece = 0; piece < 4; ++piece) {
+            for (int piece = 0; piece < D / 32; ++piece) {
               tmem_ld_wait();
-              if (piece < 3) {
-                if (piece & 1) tmem_ld16u(tStash + lane_base + j * 64 + (piece + 1) * 16, ra);
-                else tmem_ld16u(tStash + lane_base + j * 64 + (piece + 1) * 16, rb);
+              if (piece < D / 32 - 1) {
+                if (piece & 1) tmem_ld16u(tStash + lane_base + j * kRowCols + (piece + 1) * 16, ra);
+                else tmem_ld16u(tStash + lane_base + j * kRowCols + (piece + 1) * 16, rb);
               }
               const uint32_t* rw = (piece & 1) ? rb : ra;
 #pragma unroll
@@ -915,7 +925,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           } else {
             const char* vt = tilesV + vs * kTileBytes;
 #pragma unroll
-            for (int c = 0; c < 16; ++c) {
+            for (int c = 0; c < D / 8; ++c) {
               const uint4 raw = *reinterpret_cast<const uint4*>(vt + tile_off(tok, c));
               const float4 x0 = *reinterpret_cast<const float4*>(nX + 8 * c);
               const float4 x1 = *reinterpret_cast<const float4*>(nX + 8 * c + 4);

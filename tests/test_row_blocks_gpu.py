@@ -22,6 +22,11 @@ SHAPES = [
     (1, 8, 1, 64, 1600, 8, [1537]),             # 64 rows
     (1, 2, 1, 128, 4112, 128, [4097]),          # key splits, two row blocks
     (2, 16, 1, 64, 4112, 2, [4096, 130]),       # key splits for one of two sequences
+    # one query at head_dim 64: the cluster kernel with many units per cluster, with nine tiles per CTA on its largest
+    # cluster, and one tile more than that holds
+    (40, 14, 2, 64, 1300, 1, [1300 - 37 * (i % 9) for i in range(40)]),
+    (1, 8, 1, 64, 18432, 1, [18432]),
+    (1, 4, 1, 64, 18448, 1, [18433]),
 ]
 
 
