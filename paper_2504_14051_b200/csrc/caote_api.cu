@@ -691,7 +691,8 @@ static int launch_prefill_kernels(const Dims& dm, const prefill::Scratch& sc, co
                  launch_pdl(prefill::score_external_kernel<D>, grid, dim3(256), 0, st, dm, (const __nv_bfloat16*)V, len, sc,
                             (const float*)base, scores));
   } else {
-    dim3 grid((dm.cap + prefill::kScoreKeys - 1) / prefill::kScoreKeys, dm.units);
+    const long long items = (long long)dm.units * ((dm.cap + prefill::kScoreKeys - 1) / prefill::kScoreKeys);
+    dim3 grid((unsigned)(items < g_sm_count ? items : g_sm_count));
     CAOTE_LAUNCH("prefill_score_kernel", st,
                  launch_pdl(score, grid, dim3(prefill::kScoreThreads), prefill::score_smem_bytes<D>(), st, tmQs, tmK, tmV, dm, len, sc,
                             base, scores, status));

@@ -846,17 +846,17 @@ attn_combine_xsum_kernel(Dims dm, const int* __restrict__ len, Scratch sc, float
   }
 }
 
-constexpr int kScoreKeys = 2 * kTile;            // keys per CTA: two key tiles share every Q block
+constexpr int kScoreKeys = 2 * kTile;            // keys per work item: two key tiles share every Q block
 constexpr int kKeyThreads = 2 * kScoreKeys;       // two threads per key: each owns 64 of a block's 128 rows
-constexpr int kScoreThreads = kKeyThreads + 64;   // + a warp for the products + a warp for the copies
-constexpr int kStatBytes = kTile * 4;             // the softmax statistic of the 128 rows of a block
-constexpr int kQStages = 4;                       // Q blocks: a stage is free again once its products are done
+constexpr int kScoreThreads = kKeyThreads + 96;   // + a warp for the products, one for K and V, one for Q and the statistics
+constexpr int kQStages = 2;                       // Q blocks: a stage is free again once its products are done
 constexpr int kSStages = 8;                       // their rows' statistics: free once the key threads have used them
+template <bool kFew>
+constexpr int kStatFloatsOf = kFew ? 2 * kTile : kTile;  // the statistics of a block's 128 rows (few: and their crest)
 
 template <int D>
 inline size_t score_smem_bytes() {
-  return 1024 + (2 + kQStages) * (size_t)kTileBytesOf<D> + kSStages * (size_t)kStatBytes +
-         (D + 2 * kScoreKeys + kTile) * sizeof(float) + 256;
+  return 1024 + (4 + kQStages) * (size_t)kTileBytesOf<D> + (kSStages * 2 * kTile + 2 * D + 6 * kScoreKeys) * sizeof(float) + 320;
 }
 
 // 2^x for two arguments at once on the FMA pipe instead of the special-function unit: x = i + f with i the nearest
@@ -936,115 +936,150 @@ __device__ __forceinline__ void score_piece16_few(const uint32_t (&v)[16], const
   }
 }
 
-// CAOTE scores of 256 keys of one unit. grid = (key tile pairs, units), 576 threads: warps 0..15 are the
-// key threads, two per key (warps 0..3 and 8..11 the first key tile, 4..7 and 12..15 the second; the
-// lower eight take rows 0..63 of every Q block, the upper eight rows 64..127), one lane of warp 16 issues
-// the products, one lane of warp 17 the copies. tmQ: the counted rows (LAST_QUERY: the last row of every head).
-// kFew: complements without cancellation; kAccum: carried scores are added and written back.
+// CAOTE scores, 256 keys of a unit at a time (an item). The grid is one CTA per SM and walks the items with a stride of its
+// size, so that an item's K tiles are fetched while the one before it is summed, its value rows while its own last blocks
+// are, and the products of the next item start before the scores of this one are written. (A CTA per item: 32 units of 7.3 k
+// keys x 512 rows 82 us, of which every CTA spent 4 of 10.5 us on set-up, the first copies and the value rows; now 71.)
+// 608 threads: warps 0..15 are the key threads, two per key (warps 0..3 and 8..11 the first key tile, 4..7 and 12..15 the
+// second; the lower eight take rows 0..63 of every Q block and the lower half of the channels, the upper eight the others),
+// one lane each of warps 16, 17, 18 issues the products, the copies of K and V, and those of Q and the statistics.
+// Two buffers of two tiles take turns: K of item i, then its V once the last product has read K, then K of item i + 2.
+// tmQ: the counted rows (LAST_QUERY: the last row of every head). kFew: complements without cancellation; kAccum: carried
+// scores are added and written back.
 template <int D, bool kFew, bool kAccum>
 __global__ void __launch_bounds__(kScoreThreads, 1)
 score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
              const __grid_constant__ CUtensorMap tmV, Dims dm, const int* __restrict__ len, Scratch sc,
              float* __restrict__ base, float* __restrict__ scores, int* status) {
-  constexpr int kTB = kTileBytesOf<D>, kBoxes = D / 64, kSteps = D / 16;
+  constexpr int kTB = kTileBytesOf<D>, kBoxes = D / 64, kSteps = D / 16, kSF = kStatFloatsOf<kFew>;
   ptx::pdl_wait();
   ptx::pdl_trigger();
   extern __shared__ char smem_raw[];
   // (aligned by an offset into the array, not through an integer: the pointer keeps its address space, and what is
   // read and written through it compiles to shared-memory accesses, not generic ones)
   char* sm = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
-  char* Ks = sm;                                                // [2] key tiles
-  char* Qst = Ks + 2 * kTB;                                     // [kQStages] Q blocks
-  float* Sst = reinterpret_cast<float*>(Qst + kQStages * kTB);  // [kSStages][kTile] row statistics
-  float* Xs = Sst + kSStages * kTile;                           // [D]
-  float* hx = Xs + D;                                           // [kScoreKeys] upper halves' sums
-  float* rx = hx + kScoreKeys;                                  // [kScoreKeys] kFew: their complements
-  float* crs = rx + kScoreKeys;                                 // [kTile] kFew: the counted rows' crest
-  uint64_t* bars = reinterpret_cast<uint64_t*>(crs + kTile);
-  uint64_t *k_bar = &bars[0], *v_bar = &bars[1], *q_bar = &bars[2], *q_done = q_bar + kQStages, *st_bar = q_done + kQStages,
-           *s_bar = st_bar + kSStages, *c_bar = s_bar + 2, *st_free = c_bar + 2;
-  constexpr int kBars1 = 2 + 2 * kQStages + kSStages + 2;  // single arrivals (a copy's bytes, a commit)
-  constexpr int kBars = kBars1 + 2 + kSStages;
+  char* KVs = sm;                                               // [2][2] tiles: K, later V, of an item
+  char* Qst = KVs + 4 * kTB;                                    // [kQStages] Q blocks
+  float* Sst = reinterpret_cast<float*>(Qst + kQStages * kTB);  // [kSStages][kSF] row statistics (few: then their crest)
+  float* Xs = Sst + kSStages * 2 * kTile;                       // [2][D]
+  float* hx = Xs + 2 * D;                                       // [2][kScoreKeys] upper halves' sums,
+  float* ax = hx + 2 * kScoreKeys;                              // [2][kScoreKeys] squared distances,
+  float* rx = ax + 2 * kScoreKeys;                              // [2][kScoreKeys] few: complements
+  uint64_t* bars = reinterpret_cast<uint64_t*>(rx + 2 * kScoreKeys);
+  uint64_t *k_full = &bars[0], *k_done = k_full + 2, *v_full = k_done + 2, *q_full = v_full + 2, *q_done = q_full + kQStages,
+           *st_full = q_done + kQStages, *s_bar = st_full + kSStages, *v_free = s_bar + 2, *c_bar = v_free + 2, *st_free = c_bar + 2;
+  constexpr int kBars1 = 6 + 2 * kQStages + kSStages + 2;  // single arrivals (a copy's bytes, a commit)
+  constexpr int kBars = kBars1 + 4 + kSStages;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kBars);
 
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int unit = blockIdx.y, j0 = blockIdx.x * kScoreKeys;
-  const int b = unit / dm.Hkv;
-  const int n = len[b];
   const bool last_only = kFew && dm.base_mode == CAOTE_BASE_LAST_QUERY;
   const int M = kFew ? sc.Ms : dm.R, m = last_only ? 1 : dm.m;  // counted rows, and the block they are causal in
-  if (n == 0 || n < dm.m || n > dm.cap || j0 >= n) return;
   const int nblocks = (M + kTile - 1) / kTile;
+  const int per_unit = (dm.cap + kScoreKeys - 1) / kScoreKeys, items = dm.units * per_unit;
+  // the next item at or behind `it` that holds keys (its unit, first key and the unit's length); false: no more
+  int it = blockIdx.x, unit = 0, j0 = 0, n = 0;
+  auto next = [&]() {
+    for (; it < items; it += gridDim.x) {
+      unit = it / per_unit;
+      j0 = (it - unit * per_unit) * kScoreKeys;
+      n = __ldg(len + unit / dm.Hkv);
+      if (n >= dm.m && n <= dm.cap && j0 < n) {
+        it += gridDim.x;
+        return true;
+      }
+    }
+    return false;
+  };
 
   if (tid == 0) {
     for (int i = 0; i < kBars1; ++i) mbar_init(&bars[i], 1);
-    for (int i = 0; i < 2; ++i) mbar_init(&c_bar[i], kKeyThreads / 32);  // one arrival per key warp
-    for (int i = 0; i < kSStages; ++i) mbar_init(&st_free[i], kKeyThreads / 32);
+    for (int i = kBars1; i < kBars; ++i) mbar_init(&bars[i], kKeyThreads / 32);  // one arrival per key warp
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(tmem_slot, 512);
-  if (tid < D) Xs[tid] = sc.X[(size_t)unit * D + tid];
-  if (kFew && tid >= kTile && tid < 2 * kTile) crs[tid - kTile] = (tid - kTile < M) ? sc.crest[(size_t)unit * kTile + tid - kTile] : 0.f;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;  // key tile kk, buffer buf: columns [kk * 256 + buf * 128, + 128)
-  float h = 0.f, rest_few = 0.f;
-  const int j = j0 + (tid & (kScoreKeys - 1));  // key threads: this thread's key
-  const int rhalf = tid >> 8;                   // key threads: which 64 rows of a Q block
 
   if (warp == 17) {
-    // =============================== copies (one lane) ===============================
+    // =============================== copies of K and V (one lane) ===============================
     if (tid == kKeyThreads + 32) {
-      auto load_pair = [&](char* dst, const CUtensorMap* tm, uint64_t* bar) {  // the two tiles of this CTA's keys
-        mbar_expect_tx(bar, 2 * kTB);
+      auto load_pair = [&](int buf, const CUtensorMap* tm, uint64_t* bar, int u, int first) {
+#pragma unroll
         for (int kk = 0; kk < 2; ++kk)
 #pragma unroll
           for (int x = 0; x < kBoxes; ++x)
-            tma_load_2d(dst + kk * kTB + x * kHalfBytes, tm, 64 * x, unit * dm.cap + j0 + kk * kTile, bar);
+            tma_load_2d(KVs + (2 * buf + kk) * kTB + x * kHalfBytes, tm, 64 * x, u * dm.cap + first + kk * kTile, bar);
       };
-      load_pair(Ks, &tmK, k_bar);
-      const float* rstat = last_only ? sc.sstat + (size_t)unit * kTile : sc.stats + (size_t)unit * sc.Mpad;
-      for (int rb = 0; rb < nblocks; ++rb) {
-        const int st = rb % kQStages, ss = rb % kSStages;
-        if (rb >= kQStages) mbar_wait_idle(&q_done[st], ((rb / kQStages) - 1) & 1, status);  // the products of block rb - 4 are done
-        char* qd = Qst + st * kTB;
-        mbar_expect_tx(&q_bar[st], kTB);
-#pragma unroll
-        for (int x = 0; x < kBoxes; ++x) tma_load_2d(qd + x * kHalfBytes, &tmQ, 64 * x, unit * M + rb * kTile, &q_bar[st]);
-        if (rb >= kSStages) mbar_wait_idle(&st_free[ss], ((rb / kSStages) - 1) & 1, status);  // block rb - 8 is summed
-        mbar_expect_tx(&st_bar[ss], kStatBytes);
-        bulk_load(Sst + ss * kTile, rstat + (size_t)rb * kTile, kStatBytes, &st_bar[ss]);
+      bool more = next();
+      if (more) {
+        mbar_expect_tx(&k_full[0], 2 * kTB);
+        load_pair(0, &tmK, &k_full[0], unit, j0);
       }
-      // the value rows of the CTA's keys, for the distances at the end: into the first two Q stages once the last
-      // product has read its Q block (a commit covers every product before it); a few rows are one block, which leaves
-      // stages 2 and 3 alone
-      if (!kFew) mbar_wait_idle(&q_done[(nblocks - 1) % kQStages], ((nblocks - 1) / kQStages) & 1, status);
-      load_pair(Qst + (kFew ? 2 * kTB : 0), &tmV, v_bar);
+      for (int c = 0; more; ++c) {
+        const int buf = c & 1, u = unit, first = j0;
+        more = next();
+        if (more) {  // K of the next item, once the value rows of the one before this have been read
+          if (c >= 1) mbar_wait_idle(&v_free[buf ^ 1], ((c - 1) >> 1) & 1, status);
+          mbar_expect_tx(&k_full[buf ^ 1], 2 * kTB);
+          load_pair(buf ^ 1, &tmK, &k_full[buf ^ 1], unit, j0);
+        }
+        mbar_wait_idle(&k_done[buf], (c >> 1) & 1, status);  // every product of this item has read its K tiles
+        mbar_expect_tx(&v_full[buf], 2 * kTB + D * 4);
+        load_pair(buf, &tmV, &v_full[buf], u, first);
+        bulk_load(Xs + buf * D, sc.X + (size_t)u * D, D * 4, &v_full[buf]);
+      }
+    }
+  } else if (warp == 18) {
+    // =============================== copies of Q and the statistics (one lane) ===============================
+    if (tid == kKeyThreads + 64) {
+      int qb = 0;
+      while (next()) {
+        const float* rstat = last_only ? sc.sstat + (size_t)unit * kTile : sc.stats + (size_t)unit * sc.Mpad;
+        for (int rb = 0; rb < nblocks; ++rb, ++qb) {
+          const int st = qb % kQStages, ss = qb % kSStages;
+          if (qb >= kQStages) mbar_wait_idle(&q_done[st], ((qb / kQStages) - 1) & 1, status);  // the products that read the stage are done
+          char* qd = Qst + st * kTB;
+          mbar_expect_tx(&q_full[st], kTB);
+#pragma unroll
+          for (int x = 0; x < kBoxes; ++x) tma_load_2d(qd + x * kHalfBytes, &tmQ, 64 * x, unit * M + rb * kTile, &q_full[st]);
+          if (qb >= kSStages) mbar_wait_idle(&st_free[ss], ((qb / kSStages) - 1) & 1, status);  // the stage's last block is summed
+          mbar_expect_tx(&st_full[ss], kSF * 4);
+          bulk_load(Sst + ss * kSF, rstat + (size_t)rb * kTile, kTile * 4, &st_full[ss]);
+          if (kFew) bulk_load(Sst + ss * kSF + kTile, sc.crest + (size_t)unit * kTile, kTile * 4, &st_full[ss]);
+        }
+      }
     }
   } else if (warp == 16) {
     // =============================== products (one lane) ===============================
     if (tid == kKeyThreads) {
       constexpr uint32_t kIdesc = instr_desc(false);
-      const uint32_t k_addr = smem_u32(Ks);
-      mbar_wait_idle(k_bar, 0, status);
-      for (int rb = 0; rb < nblocks; ++rb) {
-        const int buf = rb & 1, st = rb % kQStages;
-        mbar_wait_idle(&q_bar[st], (rb / kQStages) & 1, status);
-        if (rb >= 2) mbar_wait_idle(&c_bar[buf], ((rb - 2) >> 1) & 1, status);  // its S buffers have been read
-        tc_fence_after();
-        const uint32_t q_addr = smem_u32(Qst + st * kTB);
+      int qb = 0;
+      for (int c = 0; next(); ++c) {
+        const int kb = c & 1;
+        const uint32_t k_addr = smem_u32(KVs + 2 * kb * kTB);
+        mbar_wait_idle(&k_full[kb], (c >> 1) & 1, status);
+        for (int rb = 0; rb < nblocks; ++rb, ++qb) {
+          const int buf = qb & 1, st = qb % kQStages;
+          mbar_wait_idle(&q_full[st], (qb / kQStages) & 1, status);
+          if (qb >= 2) mbar_wait_idle(&c_bar[buf], ((qb - 2) >> 1) & 1, status);  // its S buffers have been read
+          tc_fence_after();
+          const uint32_t q_addr = smem_u32(Qst + st * kTB);
 #pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
+          for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
-          for (int ks = 0; ks < kSteps; ++ks)
-            umma(tmem + kk * 256 + buf * 128, desc_k_major(k_addr + kk * kTB, ks), desc_k_major(q_addr, ks), kIdesc, ks > 0);
+            for (int ks = 0; ks < kSteps; ++ks)
+              umma(tmem + kk * 256 + buf * 128, desc_k_major(k_addr + kk * kTB, ks), desc_k_major(q_addr, ks), kIdesc, ks > 0);
+          }
+          umma_commit(&s_bar[buf]);
+          umma_commit(&q_done[st]);
         }
-        umma_commit(&s_bar[buf]);
-        umma_commit(&q_done[st]);
+        umma_commit(&k_done[kb]);
       }
       // (no arrival may still be on its way to this CTA's barriers when the CTA ends)
-      if (nblocks > 0) mbar_wait_idle(&q_done[(nblocks - 1) % kQStages], ((nblocks - 1) / kQStages) & 1, status);
+      if (qb > 0) mbar_wait_idle(&q_done[(qb - 1) % kQStages], ((qb - 1) / kQStages) & 1, status);
     }
   } else {
     // =============================== one key per thread ===============================
@@ -1053,103 +1088,112 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     // neither latency is waited for. The S buffer is handed back to the products as soon as its last piece is in
     // registers, not when it has been summed.
     const float scale2 = dm.scale * 1.4426950408889634f;
-    const int kk = (warp >> 2) & 1;
+    const int kk = (warp >> 2) & 1, rhalf = tid >> 8, lane = tid & 31, key = tid & (kScoreKeys - 1);
     const uint32_t t_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kk * 256 + rhalf * 64;
-    const int lane = tid & 31;
-    const int need = j - (n - m);  // row R sees key j iff (R % m) >= need
-    auto piece = [&](const uint32_t (&v)[16], const float4 (&st)[4], bool plain, int R0, float2 (&ha)[2]) {
-      if constexpr (kFew) score_piece16_few(v, st, crs + R0, scale2, R0, M, m, need, h, rest_few);
-      else score_piece16(v, st, scale2, plain, R0, M, m, need, ha, h);
-    };
     uint32_t va[16], vb[16];
     float4 sa[4], sb[4];
-    float2 hacc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    mbar_wait(&s_bar[0], 0, status);
-    mbar_wait(&st_bar[0], 0, status);
-    tc_fence_after();
-    tmem_ld16_issue(t_lane, va);
-    lds16_issue(Sst + rhalf * 64, sa);
-    for (int rb = 0; rb < nblocks; ++rb) {
-      const int buf = rb & 1, ss = rb % kSStages;
-      // only the keys of the new block itself are masked (causal inside the block), and only the last
-      // row block can have columns beyond M
-      const bool plain = (j0 + kScoreKeys - 1 < n - m + 1) && (rb * kTile + kTile <= M);
-      const int R0 = rb * kTile + rhalf * 64;
-      const uint32_t t_s = t_lane + buf * 128;
-      const float* stc = Sst + ss * kTile + rhalf * 64;
-      // piece 0 (in va / sa); piece 1 on its way
-      tmem_ld16_wait(va);
-      tmem_ld16_issue(t_s + 16, vb);
-      lds16_issue(stc + 16, sb);
-      piece(va, sa, plain, R0, hacc);
-      // piece 1; piece 2 on its way
-      tmem_ld16_wait(vb);
-      tmem_ld16_issue(t_s + 32, va);
-      lds16_issue(stc + 32, sa);
-      piece(vb, sb, plain, R0 + 16, hacc);
-      // piece 2; piece 3 on its way
-      tmem_ld16_wait(va);
-      tmem_ld16_issue(t_s + 48, vb);
-      lds16_issue(stc + 48, sb);
-      piece(va, sa, plain, R0 + 32, hacc);
-      // piece 3; the S buffer is free, the next block's piece 0 on its way
-      tmem_ld16_wait(vb);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&c_bar[buf]);  // this warp holds its part of the S buffer in registers
-      if (rb + 1 < nblocks) {
-        const int ss1 = (rb + 1) % kSStages;
-        mbar_wait(&s_bar[buf ^ 1], ((rb + 1) >> 1) & 1, status);
-        mbar_wait(&st_bar[ss1], ((rb + 1) / kSStages) & 1, status);  // the next block's row statistics have landed
-        tc_fence_after();
-        tmem_ld16_issue(t_lane + (buf ^ 1) * 128, va);
-        lds16_issue(Sst + ss1 * kTile + rhalf * 64, sa);
+    int qb = 0;
+    for (int c = 0; next(); ++c) {
+      const int j = j0 + key, need = j - (n - m);  // row R sees key j iff (R % m) >= need
+      float h = 0.f, rest_few = 0.f;
+      float2 hacc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      auto piece = [&](const uint32_t (&v)[16], const float4 (&st)[4], const float* crest, bool plain, int R0) {
+        if constexpr (kFew) score_piece16_few(v, st, crest, scale2, R0, M, m, need, h, rest_few);
+        else score_piece16(v, st, scale2, plain, R0, M, m, need, hacc, h);
+      };
+      mbar_wait(&s_bar[qb & 1], (qb >> 1) & 1, status);
+      mbar_wait(&st_full[qb % kSStages], (qb / kSStages) & 1, status);
+      tc_fence_after();
+      tmem_ld16_issue(t_lane + (qb & 1) * 128, va);
+      lds16_issue(Sst + (qb % kSStages) * kSF + rhalf * 64, sa);
+      for (int rb = 0; rb < nblocks; ++rb, ++qb) {
+        const int buf = qb & 1, ss = qb % kSStages;
+        // only the keys of the new block itself are masked (causal inside the block), and only the last
+        // row block can have columns beyond M
+        const bool plain = (j0 + kScoreKeys - 1 < n - m + 1) && (rb * kTile + kTile <= M);
+        const int R0 = rb * kTile + rhalf * 64;
+        const uint32_t t_s = t_lane + buf * 128;
+        const float* stc = Sst + ss * kSF + rhalf * 64;
+        const float* crs = stc + kTile;  // (few only)
+        // piece 0 (in va / sa); piece 1 on its way
+        tmem_ld16_wait(va);
+        tmem_ld16_issue(t_s + 16, vb);
+        lds16_issue(stc + 16, sb);
+        piece(va, sa, crs, plain, R0);
+        // piece 1; piece 2 on its way
+        tmem_ld16_wait(vb);
+        tmem_ld16_issue(t_s + 32, va);
+        lds16_issue(stc + 32, sa);
+        piece(vb, sb, crs + 16, plain, R0 + 16);
+        // piece 2; piece 3 on its way
+        tmem_ld16_wait(va);
+        tmem_ld16_issue(t_s + 48, vb);
+        lds16_issue(stc + 48, sb);
+        piece(va, sa, crs + 32, plain, R0 + 32);
+        // piece 3; the S buffer is free, the next block's piece 0 on its way
+        tmem_ld16_wait(vb);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&c_bar[buf]);  // this warp holds its part of the S buffer in registers
+        if (rb + 1 < nblocks) {
+          const int ss1 = (qb + 1) % kSStages;
+          mbar_wait(&s_bar[buf ^ 1], ((qb + 1) >> 1) & 1, status);
+          mbar_wait(&st_full[ss1], ((qb + 1) / kSStages) & 1, status);  // the next block's row statistics have landed
+          tc_fence_after();
+          tmem_ld16_issue(t_lane + (buf ^ 1) * 128, va);
+          lds16_issue(Sst + ss1 * kSF + rhalf * 64, sa);
+        }
+        piece(vb, sb, crs + 48, plain, R0 + 48);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&st_free[ss]);  // ... and is done with the block's statistics
       }
-      piece(vb, sb, plain, R0 + 48, hacc);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&st_free[ss]);  // ... and is done with the block's statistics
-    }
-    h += (hacc[0].x + hacc[0].y) + (hacc[1].x + hacc[1].y);
-  }
+      h += (hacc[0].x + hacc[0].y) + (hacc[1].x + hacc[1].y);
 
-  // ---- the two halves of a key add up; then c_j = w_j / (1 - w_j) * ||X - v_j||, w_j = h_j / H ----
-  if (tid >= kScoreKeys && tid < kKeyThreads) {
-    hx[tid - kScoreKeys] = h;
-    if (kFew) rx[tid - kScoreKeys] = rest_few;
-  }
-  __syncthreads();
-  if (tid < kScoreKeys) {
-    h += hx[tid];
-    if (kFew) rest_few += rx[tid];
-    mbar_wait(v_bar, 0, status);
-  }
-  if (tid < kScoreKeys && j < n) {
-    // the key's value row: chunks of 8 channels in the staged tile (boxes of 64 channels, 128-byte swizzle)
-    const char* vt = Qst + (kFew ? 2 * kTB : 0) + (tid >> 7) * kTB;
-    float acc = 0.f;
+      // ---- c_j = w_j / (1 - w_j) * ||X - v_j||, w_j = h_j / H: the two halves of a key add up ----
+      const int kb = c & 1;
+      mbar_wait(&v_full[kb], (c >> 1) & 1, status);
+      float acc = 0.f;
+      {
+        // this half's channels of the key's value row: chunks of 8 in the staged tile (boxes of 64 channels, 128-byte swizzle)
+        const char* vt = KVs + (2 * kb + (key >> 7)) * kTB;
+        const float* x = Xs + kb * D + rhalf * (D / 2);
 #pragma unroll
-    for (int c = 0; c < D / 8; ++c) {
-      const uint4 raw = *reinterpret_cast<const uint4*>(vt + tile_off(tid & (kTile - 1), c));
-      const uint32_t w4[4] = {raw.x, raw.y, raw.z, raw.w};
+        for (int i = 0; i < D / 16; ++i) {
+          const uint4 raw = *reinterpret_cast<const uint4*>(vt + tile_off(key & (kTile - 1), rhalf * (D / 16) + i));
+          const uint32_t w4[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float d0 = Xs[8 * c + 2 * e] - __uint_as_float(w4[e] << 16);
-        const float d1 = Xs[8 * c + 2 * e + 1] - __uint_as_float(w4[e] & 0xffff0000u);
-        acc = fmaf(d0, d0, acc);
-        acc = fmaf(d1, d1, acc);
+          for (int e = 0; e < 4; ++e) {
+            const float d0 = x[8 * i + 2 * e] - __uint_as_float(w4[e] << 16);
+            const float d1 = x[8 * i + 2 * e + 1] - __uint_as_float(w4[e] & 0xffff0000u);
+            acc = fmaf(d0, d0, acc);
+            acc = fmaf(d1, d1, acc);
+          }
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&v_free[kb]);
+      if (rhalf) {
+        hx[kb * kScoreKeys + key] = h;
+        ax[kb * kScoreKeys + key] = acc;
+        if (kFew) rx[kb * kScoreKeys + key] = rest_few;
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(kKeyThreads) : "memory");
+      if (!rhalf && j < n) {
+        h += hx[kb * kScoreKeys + key];
+        acc += ax[kb * kScoreKeys + key];
+        float rest = kFew ? rest_few + rx[kb * kScoreKeys + key] : (float)M - h;  // (1 - w_j) H
+        const size_t slot = (size_t)unit * dm.cap + j;
+        if (kAccum) {
+          const float bj = base[slot];
+          rest += sc.hb[unit] - bj;
+          h += bj;
+          base[slot] = h;
+        }
+        float ratio = 0.f;
+        if (h > 0.f) ratio = (rest > 0.f) ? h / rest : INFINITY;
+        scores[slot] = (ratio == 0.f) ? 0.f : ((ratio == INFINITY) ? INFINITY : ratio * sqrtf(acc));
       }
     }
-    float rest = kFew ? rest_few : (float)M - h;  // (1 - w_j) H
-    const size_t slot = (size_t)unit * dm.cap + j;
-    if (kAccum) {
-      const float bj = base[slot];
-      rest += sc.hb[unit] - bj;
-      h += bj;
-      base[slot] = h;
-    }
-    float ratio = 0.f;
-    if (h > 0.f) ratio = (rest > 0.f) ? h / rest : INFINITY;
-    scores[slot] = (ratio == 0.f) ? 0.f : ((ratio == INFINITY) ? INFINITY : ratio * sqrtf(acc));
   }
   tc_fence_before();
   __syncthreads();
