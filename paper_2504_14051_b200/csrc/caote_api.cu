@@ -654,8 +654,36 @@ static int encode_rows_map(CUtensorMap* tm, const void* ptr, int D, unsigned lon
   return CAOTE_OK;
 }
 
+// Clusters of `c` CTAs of the row-block attention kernel that can be resident on the current device at once.
 template <int D, bool kFew>
-static int launch_prefill_kernels(const Dims& dm, const prefill::Scratch& sc, const void* q, const void* K, const void* V,
+static int attn_cluster_capacity(int c) {
+  static std::atomic<int> cached[64][9];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int n = cached[dev][c].load(std::memory_order_acquire);
+  if (n == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(64, 1, (unsigned)c);
+    cfg.blockDim = dim3(prefill::kAttnThreads);
+    cfg.dynamicSmemBytes = prefill::attn_smem_bytes<D>();
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = (unsigned)c;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int got = 0;
+    n = -1;
+    if (cudaOccupancyMaxActiveClusters(&got, prefill::attn_kernel<D, kFew>, &cfg) == cudaSuccess && got > 0) n = got;
+    (void)cudaGetLastError();
+    cached[dev][c].store(n, std::memory_order_release);
+  }
+  return n > 0 ? n : 0;
+}
+
+template <int D, bool kFew, bool kCarried>
+static int launch_prefill_kernels(const Dims& dm, prefill::Scratch sc, const void* q, const void* K, const void* V,
                                   const int* len, float* base, float* o, float* scores, char* ws, cudaStream_t st,
                                   const float* vsum, TensorMapEncodeFn encode) {
   int* status = reinterpret_cast<int*>(ws);
@@ -668,34 +696,50 @@ static int launch_prefill_kernels(const Dims& dm, const prefill::Scratch& sc, co
                           : (tmQs = tmQ, CAOTE_OK);
   if (!rc) rc = encode_rows_map(&tmK, K, D, (unsigned long long)dm.units * dm.cap, row, encode);
   if (!rc) rc = encode_rows_map(&tmV, V, D, (unsigned long long)dm.units * dm.cap, row, encode);
-  const auto score = dm.base_mode == CAOTE_BASE_ACCUM ? prefill::score_kernel<D, kFew, true> : prefill::score_kernel<D, kFew, false>;
-  if (!rc) rc = allow_smem(prefill::attn_kernel<D, kFew>, prefill::attn_smem_bytes<D>());
+  const auto attn = prefill::attn_kernel<D, kFew>;
+  const auto score = prefill::score_kernel<D, kFew, kCarried>;  // (EXTERNAL has a kernel of its own)
+  if (!rc) rc = allow_smem(attn, prefill::attn_smem_bytes<D>());
   if (!rc) rc = allow_smem(score, prefill::score_smem_bytes<D>());
   if (rc) return rc;
   {
-    dim3 grid((dm.R + prefill::kTile - 1) / prefill::kTile, dm.units, sc.nsplit);
-    CAOTE_LAUNCH("prefill_attn_kernel", st,
-                 launch_pdl(prefill::attn_kernel<D, kFew>, grid, dim3(prefill::kAttnThreads), prefill::attn_smem_bytes<D>(), st,
-                            tmQ, tmK, tmV, dm, len, sc, o, status));
+    // as many splits as leave all clusters running at once (a cluster lives inside one GPC)
+    const int blocks = (dm.R + prefill::kTile - 1) / prefill::kTile;
+    while (sc.ns > 1 && attn_cluster_capacity<D, kFew>(sc.ns) < blocks * dm.units) --sc.ns;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks, dm.units, sc.ns);
+    cfg.blockDim = dim3(prefill::kAttnThreads);
+    cfg.dynamicSmemBytes = prefill::attn_smem_bytes<D>();
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // (the kernel starts with ptx::pdl_wait)
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 1;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = (unsigned)sc.ns;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    CAOTE_LAUNCH("prefill_attn_kernel", st, {
+      cudaError_t e = cudaLaunchKernelEx(&cfg, attn, tmQ, tmK, tmV, dm, len, sc, o, status);
+      if (e != cudaSuccess) return cuda_fail(e, "prefill_attn_kernel");
+    });
   }
-  {
-    const bool plain = !kFew && dm.base_mode == CAOTE_BASE_CHUNK_SUM && !vsum;
-    dim3 grid(dm.units, D / 16);
-    CAOTE_LAUNCH("prefill_combine_xsum_kernel", st,
-                 launch_pdl(plain ? prefill::attn_combine_xsum_kernel<D, true> : prefill::attn_combine_xsum_kernel<D, false>, grid,
-                            dim3(prefill::kCxThreads), 0, st, dm, len, sc, o, (const float*)base, (const __nv_bfloat16*)V, vsum));
+  if (kCarried) {
+    dim3 grid((dm.cap + prefill::kSumKeys - 1) / prefill::kSumKeys, dm.units);
+    CAOTE_LAUNCH("prefill_carried_sum_kernel", st,
+                 launch_pdl(prefill::carried_sum_kernel<D>, grid, dim3(256), 0, st, dm, len, sc, (const float*)base, (const __nv_bfloat16*)V));
   }
   if (dm.base_mode == CAOTE_BASE_EXTERNAL) {
-    dim3 grid((dm.cap + 63) / 64, dm.units);
+    dim3 grid((dm.cap + prefill::kExtKeys - 1) / prefill::kExtKeys, dm.units);
     CAOTE_LAUNCH("prefill_score_external_kernel", st,
-                 launch_pdl(prefill::score_external_kernel<D>, grid, dim3(256), 0, st, dm, (const __nv_bfloat16*)V, len, sc,
-                            (const float*)base, scores));
+                 launch_pdl(prefill::score_external_kernel<D>, grid, dim3(4 * prefill::kExtKeys), 0, st, dm, (const __nv_bfloat16*)V,
+                            len, sc, (const float*)base, scores, vsum));
   } else {
     const long long items = (long long)dm.units * ((dm.cap + prefill::kScoreKeys - 1) / prefill::kScoreKeys);
     dim3 grid((unsigned)(items < g_sm_count ? items : g_sm_count));
     CAOTE_LAUNCH("prefill_score_kernel", st,
                  launch_pdl(score, grid, dim3(prefill::kScoreThreads), prefill::score_smem_bytes<D>(), st, tmQs, tmK, tmV, dm, len, sc,
-                            base, scores, status));
+                            base, scores, vsum, status));
   }
   return CAOTE_OK;
 }
@@ -708,8 +752,13 @@ static int launch_prefill_score(const Dims& dm, const void* q, const void* K, co
   prefill::Scratch sc;
   prefill::carve(dm, ws + kHeaderBytes, &sc);
   *used = true;
-  auto run = dm.D == 128 ? (sc.few ? launch_prefill_kernels<128, true> : launch_prefill_kernels<128, false>)
-                         : (sc.few ? launch_prefill_kernels<64, true> : launch_prefill_kernels<64, false>);
+  const bool carried = dm.base_mode == CAOTE_BASE_ACCUM || dm.base_mode == CAOTE_BASE_EXTERNAL;
+  auto pick = [&](auto d) {
+    constexpr int D = decltype(d)::value;
+    if (sc.few) return carried ? launch_prefill_kernels<D, true, true> : launch_prefill_kernels<D, true, false>;
+    return carried ? launch_prefill_kernels<D, false, true> : launch_prefill_kernels<D, false, false>;
+  };
+  const auto run = dm.D == 128 ? pick(std::integral_constant<int, 128>{}) : pick(std::integral_constant<int, 64>{});
   return run(dm, sc, q, K, V, len, base, o, scores, ws, st, vsum, encode);
 }
 
@@ -733,8 +782,7 @@ static void refresh_sm_count() {
   g_sm_count = n;
 }
 
-// row_blocks: with room for the tensor-core row-block kernels where they cover the shape.
-static size_t workspace_bytes(const caote_params_t* p, bool row_blocks = true) {
+static size_t workspace_bytes(const caote_params_t* p) {
   refresh_sm_count();
   const Dims dm = make_dims(p);
   size_t need = generic::carve(dm, nullptr, nullptr);
@@ -742,7 +790,7 @@ static size_t workspace_bytes(const caote_params_t* p, bool row_blocks = true) {
     const size_t need2 = rowstat_bytes(dm) + decode::carve(dm, nullptr, nullptr, 0);
     if (need2 > need) need = need2;
   }
-  if (row_blocks && prefill_shape_ok(p)) {
+  if (prefill_shape_ok(p)) {
     const size_t need3 = prefill::carve(dm, nullptr, nullptr);
     if (need3 > need) need = need3;
   }
@@ -895,9 +943,8 @@ static int score_args_check(const caote_params_t* p, const void* q, const void* 
   if (!aligned(q, 16) || !aligned(K, 16) || !aligned(V, 16) || !aligned(o, 16)) return CAOTE_ERR_INVALID_ARG;
   return CAOTE_OK;
 }
-static int score_workspace_check(const caote_params_t* p, const void* workspace, size_t workspace_bytes_,
-                                 bool row_blocks = true) {
-  if (!workspace || workspace_bytes_ < workspace_bytes(p, row_blocks) || !aligned(workspace, 256)) return CAOTE_ERR_INVALID_ARG;
+static int score_workspace_check(const caote_params_t* p, const void* workspace, size_t workspace_bytes_) {
+  if (!workspace || workspace_bytes_ < workspace_bytes(p) || !aligned(workspace, 256)) return CAOTE_ERR_INVALID_ARG;
   return CAOTE_OK;
 }
 
@@ -945,9 +992,9 @@ int caote_append(const caote_params_t* p, void* K, void* V, float* base, int32_t
 // caote_score (vsum == NULL) and caote_score_fast (vsum: the per-unit sums of the cached value rows).
 static int score_impl(const caote_params_t* p, const void* q, const void* K, const void* V, const int32_t* len,
                       float* base, const float* vsum, float* o, float* scores, void* workspace, size_t workspace_bytes_,
-                      caote_stream_t stream, bool allow_side_stream = true, bool row_blocks = true) {
+                      caote_stream_t stream, bool allow_side_stream = true) {
   int rc = score_args_check(p, q, K, V, len, base, o, scores);
-  if (!rc) rc = score_workspace_check(p, workspace, workspace_bytes_, row_blocks);
+  if (!rc) rc = score_workspace_check(p, workspace, workspace_bytes_);
   if (!rc) rc = check_device();
   if (rc) return rc;
   const Dims dm = make_dims(p);
@@ -1006,7 +1053,7 @@ static int score_impl(const caote_params_t* p, const void* q, const void* K, con
     rc = launch_decode_cluster(dm, q, K, V, len, base, o, scores, ws, st, &used, vsum);
     if (rc || used) return rc;
   }
-  if (row_blocks && prefill_shape_ok(p)) {
+  if (prefill_shape_ok(p)) {
     bool used = false;
     rc = launch_prefill_score(dm, q, K, V, len, base, o, scores, ws, st, &used, vsum);
     if (rc || used) return rc;
@@ -1087,9 +1134,7 @@ int caote_score_static(const caote_params_t* p, const void* q, const void* K, co
   // everything caote_score would refuse is refused here, before anything touches the stream or the array
   int rc = score_args_check(p, q, K, V, len, base, o, scores);
   if (rc) return rc;
-  // (a shape whose key splits do not fit the array may still fit it on the any-shape kernels)
-  const bool row_blocks = workspace_bytes(p) <= kStaticScratchBytes;
-  if (!row_blocks && workspace_bytes(p, false) > kStaticScratchBytes) return CAOTE_ERR_TOO_LARGE;
+  if (workspace_bytes(p) > kStaticScratchBytes) return CAOTE_ERR_TOO_LARGE;
   rc = check_device();
   if (rc) return rc;
   char* scratch = nullptr;
@@ -1099,7 +1144,7 @@ int caote_score_static(const caote_params_t* p, const void* q, const void* K, co
   // the array keeps whatever the previous call left: the status word has to start at zero
   CAOTE_CUDA(cudaMemsetAsync(scratch, 0, kHeaderBytes, st));
   // (no second stream here: making one allocates)
-  rc = score_impl(p, q, K, V, len, base, nullptr, o, scores, scratch, kStaticScratchBytes, stream, false, row_blocks);
+  rc = score_impl(p, q, K, V, len, base, nullptr, o, scores, scratch, kStaticScratchBytes, stream, false);
   if (rc) return rc;
   if (status_out) CAOTE_CUDA(cudaMemcpyAsync(status_out, scratch, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
   return CAOTE_OK;

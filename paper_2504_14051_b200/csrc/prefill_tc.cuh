@@ -7,19 +7,21 @@
 //                 tiles of 128: S = Q K^T (tcgen05.mma, fp32 accumulator in TMEM), per-row online
 //                 softmax straight out of TMEM (two threads per row, 64 keys each), P back into TMEM
 //                 as two bf16 parts (hi + lo, 16 significant bits together), O += P V with P as the
-//                 TMEM-side A operand and V as the MN-major B operand. Writes o and the per-row
-//                 softmax statistics (reference, 1 / sum). One lane each of three extra warps issues
-//                 the products, the K copies and the V copies, so the tensor pipe always has the
-//                 next S queued while the rows are busy with the current one.
-//   attn_combine_xsum_kernel   merges the key splits of small grids and forms X = sum_j w_j v_j = (sum of the counted
-//                 output rows + sum_j base_j v_j) / (counted rows + sum_j base_j). Counted are the rows whose
-//                 attention defines the base score: all (CHUNK_SUM, ACCUM), the last of every head (LAST_QUERY) or
-//                 none (EXTERNAL). The carried scores' share, a pass over V, runs here because V has just been read
-//                 by the attention pass and mostly comes from L2.
+//                 TMEM-side A operand and V as the MN-major B operand. One lane each of three extra warps
+//                 issues the products, the K copies and the V copies, so the tensor pipe always has the
+//                 next S queued while the rows are busy with the current one. Few row blocks leave SMs idle: the
+//                 keys of a unit are then split among the CTAs of a thread-block cluster, which merge their
+//                 outputs and statistics through distributed shared memory. Writes o, the per-row softmax
+//                 statistics (reference + log2 of the sum) and, per CTA, the sum of its counted rows: all for
+//                 CHUNK_SUM and ACCUM, the last of every head for LAST_QUERY, none for EXTERNAL.
+//   carried_sum_kernel  (ACCUM, EXTERNAL) parts of sum_j base_j v_j and sum_j base_j. It needs nothing of the attention
+//                 pass, so as its dependent launch it does its work on the SMs that one leaves free or is done with,
+//                 and only then waits for it.
+//                 X = sum_j w_j v_j = (sum of the counted output rows + sum_j base_j v_j) / (counted rows + sum_j base_j).
 //   score_kernel  keys x counted rows. One CTA owns 256 keys of a unit (two key tiles) and walks the unit's
 //                 counted rows in blocks of 128: S^T = K Q^T lands in TMEM with one key per lane, so each
 //                 thread sums exp2(s - ref_r) / sum_r over the rows of its own key without any
-//                 exchange: h_j = sum_r alpha_{r,j} (+ base_j). Then c_j = w_j / (1 - w_j) * ||X - v_j||.
+//                 exchange: h_j = sum_r alpha_{r,j} (+ base_j). Then c_j = w_j / (1 - w_j) * ||X - v_j||, X from its parts.
 //
 // 1 - w_j. With 64 counted rows or more it is formed as the difference (rows - h_j) (exact to 6e-8 of the row count).
 // A few rows may well agree on one token, so for fewer than 64 (`few`) the attention pass keeps the largest numerator
@@ -52,22 +54,21 @@ constexpr long long kWaitCycles = 2000000000LL;
 
 struct Scratch {
   float* stats;  // [units][Mpad]: log2-domain softmax reference + log2(sum of 2^(s - ref)): alpha = 2^(s - stats)
-  float* X;      // [units][D]
-  float* hb;     // [units] sum of the carried base scores
   float* sstat;  // [units][kTile] LAST_QUERY: the counted rows' statistics side by side (else null)
   float* crest;  // [units][kTile] few: share of all tokens but the counted row's top one (else null)
-  float2* ptop;  // [units][nsplit][kTile] few, nsplit > 1: per split (largest logit, share of the split's other tokens)
+  float* xpart;  // [units][row blocks][nsplit][D] per CTA of the attention pass: the sum of its counted output rows
+  float* ypart;  // [units][cap / kSumKeys][D + 4] sum_j base_j v_j over kSumKeys keys, at [D] sum_j base_j (else null)
   int Mpad;      // M rounded up to a multiple of kTile
-  int nsplit;    // key splits of the attention pass (1: none)
+  int nsplit;    // most key splits of the attention pass (1: none)
+  int ns;        // key splits of this launch, at most nsplit
   int Ms;        // counted rows per unit
   bool few;      // 0 < Ms < kFewRows: complements without cancellation (see the file comment)
-  float* po;     // [units][nsplit][M][D] per-split outputs, normalised by their own sums (nsplit > 1)
-  float* pstat;  // [units][nsplit][Mpad] per-split statistics
 };
 constexpr int kFewRows = 64;
+constexpr int kSumKeys = 512;  // keys per CTA of carried_sum_kernel
 
 // Few units and few query rows leave most SMs idle: the keys of a unit are then cut into up to 8 splits
-// that run as CTAs of their own; attn_combine_kernel merges them. A function of the shape only.
+// that run as the CTAs of a cluster. A function of the shape only.
 inline int attn_splits(const Dims& dm) {
   const long long ctas = (long long)((dm.R + kTile - 1) / kTile) * dm.units;
   long long ns = g_sm_count / (ctas > 0 ? ctas : 1);
@@ -105,13 +106,12 @@ inline size_t carve(const Dims& dm, char* base, Scratch* out) {
   };
   const size_t units = (size_t)dm.units;
   s.stats = take(true, units * s.Mpad);  // (first: caote_post_evict_output_ws finds it right behind the header)
-  s.X = take(true, units * dm.D);
-  s.hb = take(true, units);
   s.sstat = take(dm.base_mode == CAOTE_BASE_LAST_QUERY, units * kTile);
   s.crest = take(s.few, units * kTile);
-  s.ptop = reinterpret_cast<float2*>(take(s.few && s.nsplit > 1, units * s.nsplit * kTile * 2));
-  s.po = take(s.nsplit > 1, units * s.nsplit * dm.R * dm.D);
-  s.pstat = take(s.nsplit > 1, units * s.nsplit * s.Mpad);
+  s.xpart = take(true, units * (s.Mpad / kTile) * s.nsplit * dm.D);
+  s.ypart = take(dm.base_mode == CAOTE_BASE_ACCUM || dm.base_mode == CAOTE_BASE_EXTERNAL,
+                 units * ((dm.cap + kSumKeys - 1) / kSumKeys) * (dm.D + 4));
+  s.ns = s.nsplit;
   if (out) *out = s;
   return off;
 }
@@ -336,7 +336,12 @@ constexpr int kAttnThreads = kRowThreads + 96;  // + MMA, K-load and V-load warp
 // (n 16 896: error of o against 64 bits 6.5e-5 -> 4.7e-6, what is left is the 16 bits of P; the attention pass 3.03 ->
 // 3.01 ms: it is a wait for a product that has nearly finished, and 64 columns, every eighth tile.)
 constexpr int kShare = 8;
-constexpr int kXchFloats = 5 * kRowThreads;     // half-row maxima and sums in turn, and the few-rows form's three closing values
+constexpr int kXchFloats = 7 * kRowThreads;     // half-row maxima and sums in turn, the few-rows form's three closing values, column sums
+
+// Where the splits' rows meet: [split][row of the owner][pitch] floats in the K stages.
+template <int D>
+constexpr int kMergePitch = D + 4;
+static_assert((kTile + 7) * kMergePitch<128> * 4 <= kKStages * kTileBytesOf<128> && (kTile + 7) * kMergePitch<64> * 4 <= kKStages * kTileBytesOf<64>, "");
 
 template <int D>
 inline size_t attn_smem_bytes() {
@@ -347,9 +352,9 @@ __host__ __device__ constexpr uint32_t instr_desc_n(bool b_mn_major, uint32_t n)
   return (1u << 4) | (1u << 7) | (1u << 10) | ((b_mn_major ? 1u : 0u) << 16) | ((n >> 3) << 17) | ((128u >> 4) << 24);
 }
 
-// o and row statistics of 128 query rows of one unit. grid = (row blocks, units, splits), 352 threads:
-// warps 0..7 are the row threads (two per row); one lane each of warps 8, 9, 10 issues the products,
-// the K copies and the V copies.
+// o, row statistics and counted sums of 128 query rows of one unit. grid = (row blocks, units, splits), in clusters of all
+// splits of a row block; 352 threads: warps 0..7 are the row threads (two per row); one lane each of warps 8, 9, 10 issues
+// the products, the K copies and the V copies.
 // tmK / tmV: tensor maps of K and V with boxes of 64 channels x kKeys rows. kFew: the counted rows' largest numerators
 // are kept apart (see the file comment).
 template <int D, bool kFew>
@@ -379,18 +384,25 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   const int b = unit / dm.Hkv;
   const int n = len[b], M = dm.R, m = dm.m;
   if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) status[kStatTagIndex] = kStatPerRow;
-  if (n == 0) return;
+  if (n == 0) return;  // (the same in the whole cluster)
   if (n < m || n > dm.cap) {
     if (tid == 0) set_status(status, CAOTE_ERR_BAD_LENGTH);
     return;
   }
   // this CTA's share of the unit's key tiles: [kt0, kt0 + ntiles)
   int ts, nsp;
-  split_plan(n, m, sc.nsplit, ts, nsp);
-  const int split = blockIdx.z;
-  if (split >= nsp) return;
+  split_plan(n, m, sc.ns, ts, nsp);
+  const int split = blockIdx.z;  // (the rank in the cluster)
+  if (split >= nsp) {
+    if (nsp > 1) {  // (a unit that runs unsplit has nothing to merge)
+      ptx::cluster_sync_all();
+      ptx::cluster_sync_all();
+    }
+    return;
+  }
   const int kt0 = split * ts;
   const int ntiles = min(ts, (n + kKeys - 1) / kKeys - kt0);
+  float* xpart = sc.xpart + ((size_t)unit * gridDim.x * sc.nsplit + blockIdx.x * sc.nsplit + split) * D;
 
   if (tid == 0) {
     for (int i = 0; i < kBars; ++i) mbar_init(&bars[i], 1);
@@ -640,39 +652,155 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       ptop = keep ? ptop : op;
       smax = fmaxf(smax, os);
     }
+    // this split's output, normalised by its own sum, and its statistics
     const float inv_l = 1.f / l;
-    // (with key splits: this split's output, normalised by its own sum, and its statistic go to scratch)
-    float* orow = (nsp > 1 ? sc.po + (((size_t)unit * sc.nsplit + split) * M + R) * D : o + ((size_t)unit * M + R) * D) +
-                  half * (D / 2);
+    float ov[D / 64][32];
 #pragma unroll
     for (int cc = 0; cc < D / 64; ++cc) {
-      float v[32];
-      tmem_ld32(t_o + cc * 32, v);  // collective: every lane takes part, rows beyond M just do not store
+      tmem_ld32(t_o + cc * 32, ov[cc]);
       if (ntiles > kShare) {
         float w[32];
         tmem_ld32(t_o + 128 + cc * 32, w);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] += w[i];
-      }
-      if (R < M) {
-#pragma unroll
-        for (int i = 0; i < 32; i += 4)
-          *reinterpret_cast<float4*>(orow + cc * 32 + i) = make_float4(v[i] * inv_l, v[i + 1] * inv_l, v[i + 2] * inv_l, v[i + 3] * inv_l);
+        for (int i = 0; i < 32; ++i) ov[cc][i] += w[i];
       }
     }
-    if (R < M && half == 0) {
-      const float stat = m_ref + __log2f(l);
-      if (nsp > 1) {
-        sc.pstat[((size_t)unit * sc.nsplit + split) * sc.Mpad + R] = stat;
-        if (kFew && counted)
-          sc.ptop[((size_t)unit * sc.nsplit + split) * kTile + counted_index(dm, R)] = make_float2(smax, lrest / (lrest + ptop));
-      } else {
+    const bool in_x = R < M && row_counted(dm, R);
+    if (nsp == 1) {
+      // straight out; the column sums of the counted rows by halving: after the step over lanes 16 apart a lane keeps half
+      // of its channels, and so on; in the end lane l of a warp holds D / 64 channels of its 32 rows
+#pragma unroll
+      for (int cc = 0; cc < D / 64; ++cc) {
+        float* orow = o + ((size_t)unit * M + R) * D + half * (D / 2) + cc * 32;
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) {
+          const float4 v = make_float4(ov[cc][i] * inv_l, ov[cc][i + 1] * inv_l, ov[cc][i + 2] * inv_l, ov[cc][i + 3] * inv_l);
+          if (R < M) *reinterpret_cast<float4*>(orow + i) = v;
+          ov[cc][i] = in_x ? v.x : 0.f; ov[cc][i + 1] = in_x ? v.y : 0.f; ov[cc][i + 2] = in_x ? v.z : 0.f; ov[cc][i + 3] = in_x ? v.w : 0.f;
+        }
+#pragma unroll
+        for (int w = 16; w > 0; w >>= 1) {
+          const bool up = (tid & w) != 0;
+#pragma unroll
+          for (int i = 0; i < w; ++i) {
+            const float send = up ? ov[cc][i] : ov[cc][i + w], keep = up ? ov[cc][i + w] : ov[cc][i];
+            ov[cc][i] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+          }
+        }
+        xch[5 * kRowThreads + (warp & 3) * D + half * (D / 2) + cc * 32 + (tid & 31)] = ov[cc][0];  // (lane l has channel l)
+      }
+      if (R < M && half == 0) {
+        const float stat = m_ref + __log2f(l);
         sc.stats[(size_t)unit * sc.Mpad + R] = stat;
-        if (kFew && counted) {
+        if (kFew && in_x) {
           if (sc.sstat) sc.sstat[(size_t)unit * kTile + counted_index(dm, R)] = stat;
           sc.crest[(size_t)unit * kTile + counted_index(dm, R)] = lrest / (lrest + ptop);
         }
       }
+      asm volatile("bar.sync 1, %0;" ::"n"(kRowThreads) : "memory");
+      if (tid < D) {
+        const float* part = xch + 5 * kRowThreads + tid;
+        xpart[tid] = (part[0] + part[D]) + (part[2 * D] + part[3 * D]);
+      }
+    } else {
+      // ... go to the CTA of the cluster that owns the row (its K stages; the row pitch keeps the lanes of a store on
+      // different banks), once that one is through with its tiles
+      const int rp = (kTile + nsp - 1) / nsp, owner = rowl / rp, rl = rowl - owner * rp;
+      __syncwarp();
+      ptx::cluster_sync_all();
+      const uint32_t dst = ptx::map_to_rank(smem_u32(Ksm) + (uint32_t)(((split * rp + rl) * kMergePitch<D> + half * (D / 2)) * 4), owner);
+#pragma unroll
+      for (int cc = 0; cc < D / 64; ++cc)
+#pragma unroll
+        for (int i = 0; i < 32; i += 4)
+          ptx::st_dsmem_v4(dst + (cc * 32 + i) * 4, make_uint4(__float_as_uint(ov[cc][i] * inv_l), __float_as_uint(ov[cc][i + 1] * inv_l),
+                                                               __float_as_uint(ov[cc][i + 2] * inv_l), __float_as_uint(ov[cc][i + 3] * inv_l)));
+      if (half == 0)
+        ptx::st_dsmem_v4(ptx::map_to_rank(smem_u32(xch) + (uint32_t)((split * rp + rl) * 16), owner),
+                         make_uint4(__float_as_uint(m_ref + __log2f(l)), __float_as_uint(smax), __float_as_uint(kFew ? lrest / (lrest + ptop) : 0.f), 0u));
+    }
+  }
+  if (nsp > 1) {
+    __syncwarp();
+    if (warp >= 8) ptx::cluster_sync_all();
+    ptx::cluster_sync_all();  // every split's rows have arrived; from here on the CTA reads its own shared memory only
+  }
+
+  if (nsp > 1 && warp < 8) {
+    // ---- merge: o = sum_s o_s 2^(stat_s - stat), stat = log2 sum_s 2^stat_s; a warp per row, lane = D / 32 channels ----
+    constexpr int CPL = D / 32;
+    const int rp = (kTile + nsp - 1) / nsp, lane = tid & 31;
+    const float4* rst = reinterpret_cast<const float4*>(xch);  // [split][row]: statistic, largest product, the others' share
+    float cs[CPL];
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) cs[c] = 0.f;
+    for (int rl = warp; rl < rp; rl += 8) {
+      const int R = row0 + split * rp + rl;
+      if (split * rp + rl >= kTile || R >= M) break;
+      float mx = -INFINITY, tot = 0.f, acc[CPL], wgt[8];
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) acc[c] = 0.f;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        wgt[u] = u < nsp ? rst[u * rp + rl].x : -INFINITY;
+        mx = fmaxf(mx, wgt[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (u < nsp) {
+          wgt[u] = fast_exp2(wgt[u] - mx);
+          tot += wgt[u];
+          const float* p = reinterpret_cast<const float*>(Ksm) + (u * rp + rl) * kMergePitch<D> + lane * CPL;
+          if constexpr (CPL == 4) {
+            const float4 v = *reinterpret_cast<const float4*>(p);
+            acc[0] = fmaf(v.x, wgt[u], acc[0]); acc[1] = fmaf(v.y, wgt[u], acc[1]);
+            acc[2] = fmaf(v.z, wgt[u], acc[2]); acc[3] = fmaf(v.w, wgt[u], acc[3]);
+          } else {
+            const float2 v = *reinterpret_cast<const float2*>(p);
+            acc[0] = fmaf(v.x, wgt[u], acc[0]); acc[1] = fmaf(v.y, wgt[u], acc[1]);
+          }
+        }
+      }
+      const float inv = 1.f / tot;
+      const bool in_x = row_counted(dm, R);
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) {
+        acc[c] *= inv;
+        if (in_x) cs[c] += acc[c];
+      }
+      float* orow = o + ((size_t)unit * M + R) * D + lane * CPL;
+      if constexpr (CPL == 4) *reinterpret_cast<float4*>(orow) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+      else *reinterpret_cast<float2*>(orow) = make_float2(acc[0], acc[1]);
+      if (lane == 0) {
+        const float stat = mx + __log2f(tot);
+        sc.stats[(size_t)unit * sc.Mpad + R] = stat;
+        if (kFew && in_x) {
+          const int q = counted_index(dm, R);
+          if (sc.sstat) sc.sstat[(size_t)unit * kTile + q] = stat;
+          // all tokens but the row's top one: the other splits, and the rest of the split that holds it
+          float top = -INFINITY, rest = 0.f;
+          int at = 0;
+          for (int u = 0; u < nsp; ++u) {
+            const float v = rst[u * rp + rl].y;
+            if (v > top) { top = v; at = u; }
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (u < nsp) rest += wgt[u] * (u == at ? rst[u * rp + rl].z : 1.f);
+          sc.crest[(size_t)unit * kTile + q] = rest * inv;
+        }
+      }
+    }
+    // the warps' sums, in a fixed order
+    float* wcs = reinterpret_cast<float*>(Vsm);
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) wcs[warp * D + lane * CPL + c] = cs[c];
+    asm volatile("bar.sync 1, %0;" ::"n"(kRowThreads) : "memory");
+    if (tid < D) {
+      float x = 0.f;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) x += wcs[w * D + tid];
+      xpart[tid] = x;
     }
   }
   tc_fence_before();
@@ -680,175 +808,125 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-// The merge of the key splits, o = sum_s o_s 2^(stat_s - stat) with stat = log2 sum_s 2^stat_s, and
-// X = (sum of the counted output rows + sum_j base_j v_j) / (counted rows + sum_j base_j) in one launch (FastCAOTE: the
-// mean of the cached values, vsum / n): a CTA takes 16 channels of a unit and all of its rows, merges the splits row by
-// row, writes o and (the CTA of channels 0..15) the rows' statistics, and adds up its 16 columns in a fixed order for X.
-// Units that ran unsplit are only summed. grid = (units, D / 16), 512 threads: a warp takes 8 rows at a time, 4 lanes
-// per row; for the carried scores' share two lanes take a key's 16 channels.
-constexpr int kCxThreads = 512;
-// kPlain: every row counts and nothing is carried (CHUNK_SUM, not few, not FastCAOTE).
-template <int D, bool kPlain>
-__global__ void __launch_bounds__(kCxThreads, 2)
-attn_combine_xsum_kernel(Dims dm, const int* __restrict__ len, Scratch sc, float* __restrict__ o,
-                         const float* __restrict__ base, const __nv_bfloat16* __restrict__ V,
-                         const float* __restrict__ vsum) {
-  ptx::pdl_wait();
+// Parts of sum_j base_j v_j and sum_j base_j: grid = (ceil(cap / kSumKeys), units), 256 threads. A thread takes one 16-byte
+// piece of every (256 / pieces)-th row, eight rows in flight; the rows' groups add up in shared memory in a fixed order.
+// No wait at the top: what it reads was complete before the attention pass before it got past its own wait (32 units of
+// 7.3 k tokens: 23 us in the merge of the splits -> hidden behind the attention pass; a spare warp of that kernel adding up
+// the V tiles in shared memory held them too long: attention 102 -> 194 us).
+template <int D>
+__global__ void __launch_bounds__(256)
+carried_sum_kernel(Dims dm, const int* __restrict__ len, Scratch sc, const float* __restrict__ base, const __nv_bfloat16* __restrict__ V) {
+  constexpr int P = D / 8, kGroups = 256 / P, kFly = 8;
+  __shared__ float part[kGroups][D + 1];
   ptx::pdl_trigger();
-  __shared__ float4 wpart[kCxThreads / 32][4];
-  __shared__ float wy[kCxThreads / 32][17];  // the carried scores' share of the 16 channels, and their sum
-  const int unit = blockIdx.x, c0 = blockIdx.y * 16;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n = len[unit / dm.Hkv];
-  if (n == 0 || n < dm.m || n > dm.cap) return;
-  int ts, nsp;
-  split_plan(n, dm.m, sc.nsplit, ts, nsp);
-  const int ch = c0 + 4 * (lane & 3);
-  const bool carried = !kPlain && (dm.base_mode == CAOTE_BASE_ACCUM || dm.base_mode == CAOTE_BASE_EXTERNAL);
-  float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
-  // A warp's time here is round trips to L2, not arithmetic: every load of a pass is issued before the first use.
-  constexpr int kStep = (kCxThreads / 32) * 8;
-  if (nsp > 1) {
-    // (splits beyond nsp count as weight zero, which leaves every sum as it is)
-    for (int R = warp * 8 + (lane >> 2); R < dm.R; R += kStep) {
-      float st[8];
-      float4 p[8];
-#pragma unroll
-      for (int s = 0; s < 8; ++s) {
-        st[s] = -INFINITY;
-        p[s] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (s < nsp) {
-          st[s] = sc.pstat[((size_t)unit * sc.nsplit + s) * sc.Mpad + R];
-          p[s] = *reinterpret_cast<const float4*>(sc.po + (((size_t)unit * sc.nsplit + s) * dm.R + R) * D + ch);
-        }
-      }
-      float mx = -INFINITY;
-#pragma unroll
-      for (int s = 0; s < 8; ++s) mx = fmaxf(mx, st[s]);
-      float tot = 0.f;
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int s = 0; s < 8; ++s) {
-        const float w = (s < nsp) ? exp2f(st[s] - mx) : 0.f;
-        tot += w;
-        acc.x = fmaf(p[s].x, w, acc.x); acc.y = fmaf(p[s].y, w, acc.y);
-        acc.z = fmaf(p[s].z, w, acc.z); acc.w = fmaf(p[s].w, w, acc.w);
-      }
-      const float4 res = make_float4(acc.x / tot, acc.y / tot, acc.z / tot, acc.w / tot);
-      *reinterpret_cast<float4*>(o + ((size_t)unit * dm.R + R) * D + ch) = res;
-      const bool in_x = kPlain || row_counted(dm, R);
-      if (ch == 0) {
-        const float stat = mx + log2f(tot);
-        sc.stats[(size_t)unit * sc.Mpad + R] = stat;
-        if (!kPlain && in_x && sc.sstat) sc.sstat[(size_t)unit * kTile + counted_index(dm, R)] = stat;
-        if (!kPlain && in_x && sc.few) {
-          // all tokens but the row's top one: the other splits, and the rest of the split that holds it
-          const float2* pt = sc.ptop + (size_t)unit * sc.nsplit * kTile + counted_index(dm, R);
-          float smax = -INFINITY, rest = 0.f;
-          int at = 0;
-          for (int s = 0; s < nsp; ++s) {
-            const float v = pt[s * kTile].x;
-            if (v > smax) { smax = v; at = s; }
-          }
-          for (int s = 0; s < nsp; ++s) rest += exp2f(st[s] - mx) * (s == at ? pt[s * kTile].y : 1.f);
-          sc.crest[(size_t)unit * kTile + counted_index(dm, R)] = rest / tot;
-        }
-      }
-      if (in_x) { cs.x += res.x; cs.y += res.y; cs.z += res.z; cs.w += res.w; }
-    }
-  } else if (kPlain || !vsum) {
-    const bool last_only = !kPlain && dm.base_mode == CAOTE_BASE_LAST_QUERY;
-    const int first = last_only ? dm.m - 1 : 0, stride = last_only ? dm.m : 1, Ms = kPlain ? dm.R : sc.Ms;
-    for (int t0 = warp * 8 + (lane >> 2); t0 < Ms; t0 += 4 * kStep) {  // four rows in flight, summed in row order
-      float4 r[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int t = t0 + u * kStep;
-        r[u] = (t < Ms) ? *reinterpret_cast<const float4*>(o + ((size_t)unit * dm.R + first + (size_t)t * stride) * D + ch)
-                           : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (t0 + u * kStep < Ms) { cs.x += r[u].x; cs.y += r[u].y; cs.z += r[u].z; cs.w += r[u].w; }
-    }
-  }
-  if (carried) {
-    // sum_j base_j v_j and sum_j base_j: lanes 2 i and 2 i + 1 take eight channels each of key i of a pass of 256
+  const int unit = blockIdx.y, n = len[unit / dm.Hkv], j0 = blockIdx.x * kSumKeys;
+  const int piece = threadIdx.x % P, g = threadIdx.x / P;
+  const bool work = n >= dm.m && n <= dm.cap && j0 < n;
+  if (work) {
+    const int j1 = min(n, j0 + kSumKeys);
     const float* bu = base + (size_t)unit * dm.cap;
-    const __nv_bfloat16* Vu = V + (size_t)unit * dm.cap * D + c0 + 8 * (tid & 1);
-    float y[8], hb = 0.f;
+    const uint4* src = reinterpret_cast<const uint4*>(V + (size_t)unit * dm.cap * D) + piece;
+    float2 y[4];
+    float hb = 0.f;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) y[c] = 0.f;
-    constexpr int kPass = kCxThreads / 2, kFly = 4;
-    for (int j0 = tid >> 1; j0 < n; j0 += kFly * kPass) {
-      float bj[kFly];
+    for (int e = 0; e < 4; ++e) y[e] = make_float2(0.f, 0.f);
+    for (int j = j0 + g; j < j1; j += kFly * kGroups) {
+      float b[kFly];
       uint4 raw[kFly];
 #pragma unroll
       for (int u = 0; u < kFly; ++u) {
-        const int j = j0 + u * kPass;
-        bj[u] = (j < n) ? bu[j] : 0.f;
-        raw[u] = (j < n) ? *reinterpret_cast<const uint4*>(Vu + (size_t)j * D) : make_uint4(0u, 0u, 0u, 0u);
+        const bool in = j + u * kGroups < j1;
+        b[u] = in ? bu[j + u * kGroups] : 0.f;
+        raw[u] = in ? src[(size_t)(j + u * kGroups) * P] : make_uint4(0u, 0u, 0u, 0u);
       }
 #pragma unroll
       for (int u = 0; u < kFly; ++u) {
         const uint32_t w[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
-        hb += bj[u];
+        hb += b[u];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          y[2 * e] = fmaf(bj[u], __uint_as_float(w[e] << 16), y[2 * e]);
-          y[2 * e + 1] = fmaf(bj[u], __uint_as_float(w[e] & 0xffff0000u), y[2 * e + 1]);
-        }
+        for (int e = 0; e < 4; ++e)
+          y[e] = __ffma2_rn(make_float2(b[u], b[u]), make_float2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u)), y[e]);
       }
     }
 #pragma unroll
-    for (int off = 2; off < 32; off <<= 1) {
-#pragma unroll
-      for (int c = 0; c < 8; ++c) y[c] += __shfl_xor_sync(0xffffffffu, y[c], off);
-      hb += __shfl_xor_sync(0xffffffffu, hb, off);
+    for (int e = 0; e < 4; ++e) {
+      part[g][8 * piece + 2 * e] = y[e].x;
+      part[g][8 * piece + 2 * e + 1] = y[e].y;
     }
-    if (lane < 2) {
-#pragma unroll
-      for (int c = 0; c < 8; ++c) wy[warp][8 * lane + c] = y[c];
-      if (lane == 0) wy[warp][16] = hb;
-    }
+    if (piece == 0) part[g][D] = hb;
   }
-  // the warp's eight row lanes of every channel quad, then the warps in order
-#pragma unroll
-  for (int off = 4; off < 32; off <<= 1) {
-    cs.x += __shfl_xor_sync(0xffffffffu, cs.x, off);
-    cs.y += __shfl_xor_sync(0xffffffffu, cs.y, off);
-    cs.z += __shfl_xor_sync(0xffffffffu, cs.z, off);
-    cs.w += __shfl_xor_sync(0xffffffffu, cs.w, off);
-  }
-  if (lane < 4) wpart[warp][lane] = cs;
   __syncthreads();
-  if (tid < 4) {
-    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-    float hb = 0.f;
-    for (int w = 0; w < kCxThreads / 32; ++w) {
-      const float4 p = wpart[w][tid];
-      t.x += p.x; t.y += p.y; t.z += p.z; t.w += p.w;
-      if (carried) {
-        t.x += wy[w][4 * tid]; t.y += wy[w][4 * tid + 1]; t.z += wy[w][4 * tid + 2]; t.w += wy[w][4 * tid + 3];
-        hb += wy[w][16];
-      }
-    }
-    const float H = kPlain ? (float)dm.R : (float)sc.Ms + hb, inv = H > 0.f ? 1.f / H : 0.f;
-    float* x = sc.X + (size_t)unit * D + c0 + 4 * tid;
-    if (!kPlain && vsum) {
-      const float4 v = *reinterpret_cast<const float4*>(vsum + (size_t)unit * D + c0 + 4 * tid);
-      const float fn = (float)n;
-      *reinterpret_cast<float4*>(x) = make_float4(v.x / fn, v.y / fn, v.z / fn, v.w / fn);
-    } else {
-      *reinterpret_cast<float4*>(x) = make_float4(t.x * inv, t.y * inv, t.z * inv, t.w * inv);
-    }
-    if (!kPlain && c0 == 0 && tid == 0) sc.hb[unit] = hb;
+  if (work && threadIdx.x <= D) {
+    float t = 0.f;
+#pragma unroll
+    for (int i = 0; i < kGroups; ++i) t += part[i][threadIdx.x];
+    sc.ypart[((size_t)unit * gridDim.x + blockIdx.x) * (D + 4) + threadIdx.x] = t;
   }
+  ptx::pdl_wait();  // (whoever waits for this kernel waits for the attention pass with it)
+}
+
+// X of a unit from its parts (see the file comment), by one warp: lane = D / 32 channels of x; returns sum_j base_j.
+// vsum: FastCAOTE, X is the mean of the cached values.
+template <int D>
+__device__ __forceinline__ float x_from_parts(const Dims& dm, const Scratch& sc, int unit, int n, const float* __restrict__ vsum,
+                                              int lane, float (&x)[D / 32]) {
+  constexpr int CPL = D / 32, kFly = 8;
+  float hb = 0.f;
+#pragma unroll
+  for (int c = 0; c < CPL; ++c) x[c] = vsum ? vsum[(size_t)unit * D + lane * CPL + c] : 0.f;
+  if (!vsum && sc.Ms > 0) {
+    int ts, nsp;
+    split_plan(n, dm.m, sc.ns, ts, nsp);
+    const int nrb = sc.Mpad / kTile, parts = nrb * nsp;
+    const float* xp = sc.xpart + (size_t)unit * nrb * sc.nsplit * D + lane * CPL;
+    for (int p0 = 0; p0 < parts; p0 += kFly) {
+      float v[kFly][CPL];
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) {
+        const int p = min(p0 + u, parts - 1);
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) v[u][c] = xp[(size_t)((p / nsp) * sc.nsplit + p % nsp) * D + c];
+      }
+#pragma unroll
+      for (int u = 0; u < kFly; ++u)
+        if (p0 + u < parts) {
+#pragma unroll
+          for (int c = 0; c < CPL; ++c) x[c] += v[u][c];
+        }
+    }
+  }
+  if (sc.ypart) {
+    const int parts = (n + kSumKeys - 1) / kSumKeys;
+    const float* yp = sc.ypart + (size_t)unit * ((dm.cap + kSumKeys - 1) / kSumKeys) * (D + 4);
+    for (int p0 = 0; p0 < parts; p0 += kFly) {
+      float v[kFly][CPL], h[kFly];
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) {
+        const float* at = yp + (size_t)min(p0 + u, parts - 1) * (D + 4);
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) v[u][c] = at[lane * CPL + c];
+        h[u] = at[D];
+      }
+#pragma unroll
+      for (int u = 0; u < kFly; ++u)
+        if (p0 + u < parts) {
+          hb += h[u];
+          if (!vsum) {
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) x[c] += v[u][c];
+          }
+        }
+    }
+  }
+  const float H = vsum ? (float)n : (float)sc.Ms + hb;
+#pragma unroll
+  for (int c = 0; c < CPL; ++c) x[c] = H > 0.f ? x[c] / H : 0.f;
+  return hb;
 }
 
 constexpr int kScoreKeys = 2 * kTile;            // keys per work item: two key tiles share every Q block
 constexpr int kKeyThreads = 2 * kScoreKeys;       // two threads per key: each owns 64 of a block's 128 rows
-constexpr int kScoreThreads = kKeyThreads + 96;   // + a warp for the products, one for K and V, one for Q and the statistics
+constexpr int kScoreThreads = kKeyThreads + 96;   // + a warp for the products, one for K, V and X, one for Q and the statistics
 constexpr int kQStages = 2;                       // Q blocks: a stage is free again once its products are done
 constexpr int kSStages = 8;                       // their rows' statistics: free once the key threads have used them
 template <bool kFew>
@@ -856,7 +934,7 @@ constexpr int kStatFloatsOf = kFew ? 2 * kTile : kTile;  // the statistics of a 
 
 template <int D>
 inline size_t score_smem_bytes() {
-  return 1024 + (4 + kQStages) * (size_t)kTileBytesOf<D> + (kSStages * 2 * kTile + 2 * D + 6 * kScoreKeys) * sizeof(float) + 320;
+  return 1024 + (4 + kQStages) * (size_t)kTileBytesOf<D> + (kSStages * 2 * kTile + 2 * (D + 4) + 6 * kScoreKeys) * sizeof(float) + 320;
 }
 
 // 2^x for two arguments at once on the FMA pipe instead of the special-function unit: x = i + f with i the nearest
@@ -942,7 +1020,8 @@ __device__ __forceinline__ void score_piece16_few(const uint32_t (&v)[16], const
 // keys x 512 rows 82 us, of which every CTA spent 4 of 10.5 us on set-up, the first copies and the value rows; now 71.)
 // 608 threads: warps 0..15 are the key threads, two per key (warps 0..3 and 8..11 the first key tile, 4..7 and 12..15 the
 // second; the lower eight take rows 0..63 of every Q block and the lower half of the channels, the upper eight the others),
-// one lane each of warps 16, 17, 18 issues the products, the copies of K and V, and those of Q and the statistics.
+// one lane each of warps 16, 17, 18 issues the products, the copies of K and V, and those of Q and the statistics; warp 17
+// also adds up X of the item's unit (a warp of its own for that cost 3 % on long blocks of queries).
 // Two buffers of two tiles take turns: K of item i, then its V once the last product has read K, then K of item i + 2.
 // tmQ: the counted rows (LAST_QUERY: the last row of every head). kFew: complements without cancellation; kAccum: carried
 // scores are added and written back.
@@ -950,7 +1029,7 @@ template <int D, bool kFew, bool kAccum>
 __global__ void __launch_bounds__(kScoreThreads, 1)
 score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
              const __grid_constant__ CUtensorMap tmV, Dims dm, const int* __restrict__ len, Scratch sc,
-             float* __restrict__ base, float* __restrict__ scores, int* status) {
+             float* __restrict__ base, float* __restrict__ scores, const float* __restrict__ vsum, int* status) {
   constexpr int kTB = kTileBytesOf<D>, kBoxes = D / 64, kSteps = D / 16, kSF = kStatFloatsOf<kFew>;
   ptx::pdl_wait();
   ptx::pdl_trigger();
@@ -961,8 +1040,8 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   char* KVs = sm;                                               // [2][2] tiles: K, later V, of an item
   char* Qst = KVs + 4 * kTB;                                    // [kQStages] Q blocks
   float* Sst = reinterpret_cast<float*>(Qst + kQStages * kTB);  // [kSStages][kSF] row statistics (few: then their crest)
-  float* Xs = Sst + kSStages * 2 * kTile;                       // [2][D]
-  float* hx = Xs + 2 * D;                                       // [2][kScoreKeys] upper halves' sums,
+  float* Xs = Sst + kSStages * 2 * kTile;                       // [2][D + 4]; at [D] the sum of the carried scores
+  float* hx = Xs + 2 * (D + 4);                                       // [2][kScoreKeys] upper halves' sums,
   float* ax = hx + 2 * kScoreKeys;                              // [2][kScoreKeys] squared distances,
   float* rx = ax + 2 * kScoreKeys;                              // [2][kScoreKeys] few: complements
   uint64_t* bars = reinterpret_cast<uint64_t*>(rx + 2 * kScoreKeys);
@@ -1004,33 +1083,34 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   const uint32_t tmem = *tmem_slot;  // key tile kk, buffer buf: columns [kk * 256 + buf * 128, + 128)
 
   if (warp == 17) {
-    // =============================== copies of K and V (one lane) ===============================
-    if (tid == kKeyThreads + 32) {
-      auto load_pair = [&](int buf, const CUtensorMap* tm, uint64_t* bar, int u, int first) {
+    // =============================== copies of K and V (one lane), X of the item's unit (the warp) ===============================
+    const int lane = tid & 31;
+    auto load_pair = [&](int buf, const CUtensorMap* tm, uint64_t* bar, int u, int first) {
+      mbar_expect_tx(bar, 2 * kTB);
 #pragma unroll
-        for (int kk = 0; kk < 2; ++kk)
+      for (int kk = 0; kk < 2; ++kk)
 #pragma unroll
-          for (int x = 0; x < kBoxes; ++x)
-            tma_load_2d(KVs + (2 * buf + kk) * kTB + x * kHalfBytes, tm, 64 * x, u * dm.cap + first + kk * kTile, bar);
-      };
-      bool more = next();
-      if (more) {
-        mbar_expect_tx(&k_full[0], 2 * kTB);
-        load_pair(0, &tmK, &k_full[0], unit, j0);
+        for (int x = 0; x < kBoxes; ++x)
+          tma_load_2d(KVs + (2 * buf + kk) * kTB + x * kHalfBytes, tm, 64 * x, u * dm.cap + first + kk * kTile, bar);
+    };
+    bool more = next();
+    if (more && lane == 0) load_pair(0, &tmK, &k_full[0], unit, j0);
+    for (int c = 0; more; ++c) {
+      const int buf = c & 1, u = unit, first = j0;
+      float x[D / 32];
+      const float hb = x_from_parts<D>(dm, sc, unit, n, vsum, lane, x);
+      // (K of this item went into buffer `buf` after v_free said that the item before last is done with it, and with its X)
+#pragma unroll
+      for (int i = 0; i < D / 32; ++i) Xs[buf * (D + 4) + lane * (D / 32) + i] = x[i];
+      if (lane == 0) Xs[buf * (D + 4) + D] = hb;
+      more = next();
+      if (more) {  // K of the next item, once the value rows of the one before this have been read
+        if (c >= 1) mbar_wait_idle(&v_free[buf ^ 1], ((c - 1) >> 1) & 1, status);
+        if (lane == 0) load_pair(buf ^ 1, &tmK, &k_full[buf ^ 1], unit, j0);
       }
-      for (int c = 0; more; ++c) {
-        const int buf = c & 1, u = unit, first = j0;
-        more = next();
-        if (more) {  // K of the next item, once the value rows of the one before this have been read
-          if (c >= 1) mbar_wait_idle(&v_free[buf ^ 1], ((c - 1) >> 1) & 1, status);
-          mbar_expect_tx(&k_full[buf ^ 1], 2 * kTB);
-          load_pair(buf ^ 1, &tmK, &k_full[buf ^ 1], unit, j0);
-        }
-        mbar_wait_idle(&k_done[buf], (c >> 1) & 1, status);  // every product of this item has read its K tiles
-        mbar_expect_tx(&v_full[buf], 2 * kTB + D * 4);
-        load_pair(buf, &tmV, &v_full[buf], u, first);
-        bulk_load(Xs + buf * D, sc.X + (size_t)u * D, D * 4, &v_full[buf]);
-      }
+      mbar_wait_idle(&k_done[buf], (c >> 1) & 1, status);  // every product of this item has read its K tiles
+      __syncwarp();
+      if (lane == 0) load_pair(buf, &tmV, &v_full[buf], u, first);  // (its arrival publishes X as well)
     }
   } else if (warp == 18) {
     // =============================== copies of Q and the statistics (one lane) ===============================
@@ -1156,7 +1236,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       {
         // this half's channels of the key's value row: chunks of 8 in the staged tile (boxes of 64 channels, 128-byte swizzle)
         const char* vt = KVs + (2 * kb + (key >> 7)) * kTB;
-        const float* x = Xs + kb * D + rhalf * (D / 2);
+        const float* x = Xs + kb * (D + 4) + rhalf * (D / 2);
 #pragma unroll
         for (int i = 0; i < D / 16; ++i) {
           const uint4 raw = *reinterpret_cast<const uint4*>(vt + tile_off(key & (kTile - 1), rhalf * (D / 16) + i));
@@ -1170,8 +1250,9 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           }
         }
       }
+      const float hb = kAccum ? Xs[kb * (D + 4) + D] : 0.f;
       __syncwarp();
-      if (lane == 0) mbar_arrive(&v_free[kb]);
+      if (lane == 0) mbar_arrive(&v_free[kb]);  // (and with X)
       if (rhalf) {
         hx[kb * kScoreKeys + key] = h;
         ax[kb * kScoreKeys + key] = acc;
@@ -1185,7 +1266,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         const size_t slot = (size_t)unit * dm.cap + j;
         if (kAccum) {
           const float bj = base[slot];
-          rest += sc.hb[unit] - bj;
+          rest += hb - bj;
           h += bj;
           base[slot] = h;
         }
@@ -1200,20 +1281,30 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-// The scores when the caller supplies the weights (EXTERNAL): h_j = base_j, one pass over V. grid = (ceil(cap / 64),
-// units), 256 threads: four threads per token, D / 4 channels each.
+// The scores when the caller supplies the weights (EXTERNAL): h_j = base_j, one pass over V. grid = (ceil(cap / kExtKeys),
+// units): four threads per token, D / 4 channels each.
+constexpr int kExtKeys = 128;
 template <int D>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(4 * kExtKeys)
 score_external_kernel(Dims dm, const __nv_bfloat16* __restrict__ V, const int* __restrict__ len, Scratch sc,
-                      const float* __restrict__ base, float* __restrict__ scores) {
+                      const float* __restrict__ base, float* __restrict__ scores, const float* __restrict__ vsum) {
+  __shared__ __align__(16) float Xs[D + 4];
   ptx::pdl_wait();
   ptx::pdl_trigger();
-  const int unit = blockIdx.y, n = len[unit / dm.Hkv], j = blockIdx.x * 64 + (threadIdx.x >> 2), part = threadIdx.x & 3;
-  if (n < dm.m || n > dm.cap || blockIdx.x * 64 >= n) return;
+  const int unit = blockIdx.y, n = len[unit / dm.Hkv], j = blockIdx.x * kExtKeys + (threadIdx.x >> 2), part = threadIdx.x & 3;
+  if (n < dm.m || n > dm.cap || blockIdx.x * kExtKeys >= n) return;
+  if (threadIdx.x < 32) {
+    float xr[D / 32];
+    const float hb = x_from_parts<D>(dm, sc, unit, n, vsum, threadIdx.x, xr);
+#pragma unroll
+    for (int i = 0; i < D / 32; ++i) Xs[threadIdx.x * (D / 32) + i] = xr[i];
+    if (threadIdx.x == 0) Xs[D] = hb;
+  }
+  __syncthreads();
   float acc = 0.f;
   if (j < n) {
     const uint4* row = reinterpret_cast<const uint4*>(V + ((size_t)unit * dm.cap + j) * D);
-    const float4* x = reinterpret_cast<const float4*>(sc.X + (size_t)unit * D);
+    const float4* x = reinterpret_cast<const float4*>(Xs);
 #pragma unroll
     for (int i = 0; i < D / 32; ++i) {  // the four threads' chunks of 8 channels side by side
       const int c = 4 * i + part;
@@ -1231,7 +1322,7 @@ score_external_kernel(Dims dm, const __nv_bfloat16* __restrict__ V, const int* _
   acc += __shfl_xor_sync(0xffffffffu, acc, 2);
   if (part == 0 && j < n) {
     const size_t slot = (size_t)unit * dm.cap + j;
-    const float h = base[slot], rest = sc.hb[unit] - h;
+    const float h = base[slot], rest = Xs[D] - h;
     const float ratio = h > 0.f ? (rest > 0.f ? h / rest : INFINITY) : 0.f;
     scores[slot] = (ratio == 0.f) ? 0.f : ((ratio == INFINITY) ? INFINITY : ratio * sqrtf(acc));
   }
