@@ -13,6 +13,7 @@ namespace sel {
 
 constexpr int kSelThreads = 1024;
 constexpr int kMaxSharedPicks = 2048;
+constexpr int kMaxCached = 24;  // scores per thread that a selection can keep in registers
 
 // 64-bit sort key: score bits in the high word (scores are >= +0, so the unsigned order of the bit
 // patterns is the numeric order; +inf sorts last), original position in the low word.
@@ -20,21 +21,244 @@ __device__ __forceinline__ unsigned long long make_key(float score, int pos) {
   return ((unsigned long long)__float_as_uint(score) << 32) | (unsigned int)pos;
 }
 
-// One CTA per unit. k = max(0, n - budget). Finds the k-th smallest key by 8 passes of an 8-bit
-// radix histogram (most significant digit first), then writes the slots whose key is <= that key in
-// ascending slot order with a block-wide ordered compaction. (Scores of one unit share their leading bytes, but grouping a
-// warp's lanes by digit before the shared-memory atomics, by match_any or by ballots, costs more than the atomics do.)
-// Returns k, the number of slots the unit evicts (the same value in every thread of the CTA). With e_smem (room for
+// The k smallest of n keys, 1 < k < n, by the CTA: the slots in ascending order to out (and picks, if not null). Up to kC
+// scores per thread stay in registers. The bits above the highest one in which any two scores differ are skipped (the scores
+// of one unit share their leading bits); below it, 11 bits are decided per pass of a histogram (1.1 us, of the latency of its
+// barriers and atomics), until a whole bucket is taken or no more than kRank tokens are left in it: these are then ranked
+// against one another by (score bits, position), a thread per token. Mostly that is one pass. Where more tokens than that
+// have the score at the threshold, the search goes on over their positions. (Up to eight passes of 8 bits over 64-bit keys:
+// 8 units, n 4224, k 128: 17.5 -> 15.2 us between events; n 16 896, k 512, scores read again in every pass: 53 -> 36 us.)
+template <int kC>
+__device__ __forceinline__ void select_cached(int n, int k, const float* __restrict__ sc, const int* __restrict__ ps, int* out, int* picks) {
+  constexpr int kW = kSelThreads / 32;
+  constexpr unsigned kRank = 128u, kNothing = 0xffffffffu;
+  __shared__ __align__(16) unsigned hist[2048];
+  __shared__ unsigned s_lo[kW], s_hi[kW], s_tot[kW];
+  __shared__ unsigned s_digit, s_below, s_count, s_list;
+  __shared__ unsigned long long s_kth;
+  __shared__ int s_cnt[kC * kW];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto position = [&](int j) { return (unsigned)(ps ? ps[j] : j); };
+  unsigned v[kC];  // score bits; later the positions of the tokens at the threshold, kNothing for all others
+#pragma unroll
+  for (int i = 0; i < kC; ++i) {
+    const int j = tid + i * kSelThreads;
+    v[i] = j < n ? __float_as_uint(sc[j]) : kNothing;
+  }
+  hist[tid] = 0u;
+  hist[tid + kSelThreads] = 0u;
+  if (tid == 0) s_list = 0u;
+  // thr: the threshold so far as it is known (prefix, then zeros); bits [0, top) of it are still to be decided;
+  // want: how many to take of the `left` tokens with this prefix
+  unsigned thr, want = (unsigned)k, left = (unsigned)n, taken = 0u;
+  int top;
+  auto prefix_of_all = [&]() {
+    unsigned lo = kNothing, hi = 0u;
+#pragma unroll
+    for (int i = 0; i < kC; ++i) {
+      lo = min(lo, v[i]);
+      hi = max(hi, v[i] == kNothing ? 0u : v[i]);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) { s_lo[warp] = lo; s_hi[warp] = hi; }
+    __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, s_lo[lane]);
+    hi = __reduce_max_sync(0xffffffffu, s_hi[lane]);
+    top = 32 - __clz(lo ^ hi);  // (at most 31: neither scores nor positions are negative)
+    thr = (lo >> top) << top;
+  };
+  prefix_of_all();
+  for (bool by_position = false;;) {
+    while (top > 0 && left != want && left > kRank) {
+      const int width = min(11, top), shift = top - width;
+#pragma unroll
+      for (int i = 0; i < kC; ++i)
+        if (v[i] != kNothing && ((v[i] ^ thr) >> top) == 0u) atomicAdd(&hist[(v[i] >> shift) & ((1u << width) - 1u)], 1u);
+      __syncthreads();
+      const unsigned c0 = hist[2 * tid], c1 = hist[2 * tid + 1];
+      unsigned incl = c0 + c1;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      if (lane == 31) s_tot[warp] = incl;
+      __syncthreads();
+      hist[2 * tid] = 0u;  // (for the next pass)
+      hist[2 * tid + 1] = 0u;
+      const unsigned before = __reduce_add_sync(0xffffffffu, lane < warp ? s_tot[lane] : 0u) + incl - c0 - c1;
+      if (before < want && want <= before + c0 + c1) {  // one thread
+        const bool second = want > before + c0;
+        s_digit = 2u * tid + (second ? 1u : 0u);
+        s_below = before + (second ? c0 : 0u);
+        s_count = second ? c1 : c0;
+      }
+      __syncthreads();
+      want -= s_below;
+      left = s_count;
+      thr |= s_digit << shift;
+      top = shift;
+    }
+    if (by_position || left == want || left <= kRank) break;
+    by_position = true;  // top == 0: the scores at the threshold are equal to the last bit
+#pragma unroll
+    for (int i = 0; i < kC; ++i) {
+      taken |= (v[i] < thr ? 1u : 0u) << i;
+      v[i] = v[i] == thr ? position(tid + i * kSelThreads) : kNothing;
+    }
+    __syncthreads();
+    prefix_of_all();
+  }
+  // the largest (v, position) that is taken
+  unsigned kv = thr | ((1u << top) - 1u), kp = kNothing;
+  if (left != want && left <= kRank) {
+    unsigned long long* list = reinterpret_cast<unsigned long long*>(hist);
+#pragma unroll
+    for (int i = 0; i < kC; ++i)
+      if (v[i] != kNothing && ((v[i] ^ thr) >> top) == 0u)  // (the order of the list does not matter)
+        list[atomicAdd(&s_list, 1u)] = ((unsigned long long)v[i] << 32) | position(tid + i * kSelThreads);
+    if (tid == 0 && (left & 1u)) list[left] = ~0ull;
+    __syncthreads();
+    if (tid < (int)left) {
+      const unsigned long long mine = list[tid];
+      unsigned below = 0u, same = 0u;
+#pragma unroll 4
+      for (unsigned q = 0; q < left; q += 2) {
+        const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(list + q);
+        below += (o.x < mine) + (o.y < mine);
+        same += (o.x == mine) + (o.y == mine);
+      }
+      if (below < want && want <= below + same) s_kth = mine;
+    }
+    __syncthreads();
+    kv = (unsigned)(s_kth >> 32);
+    kp = (unsigned)s_kth;
+  }
+  // one scan over the (round, warp) counts, which is the ascending order of the slots tid + round * kSelThreads
+  unsigned ballots[kC];
+#pragma unroll
+  for (int i = 0; i < kC; ++i) {
+    bool in = (taken >> i & 1u) != 0u;
+    if (v[i] != kNothing) in = v[i] < kv || (v[i] == kv && (kp == kNothing || position(tid + i * kSelThreads) <= kp));
+    ballots[i] = __ballot_sync(0xffffffffu, in);
+    if (lane == 0) s_cnt[i * kW + warp] = __popc(ballots[i]);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    int c[kC], sum = 0;
+#pragma unroll
+    for (int q = 0; q < kC; ++q) { c[q] = s_cnt[kC * lane + q]; sum += c[q]; }
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    int run = incl - sum;
+#pragma unroll
+    for (int q = 0; q < kC; ++q) { s_cnt[kC * lane + q] = run; run += c[q]; }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kC; ++i) {
+    if (ballots[i] >> lane & 1u) {
+      const int idx = s_cnt[i * kW + warp] + __popc(ballots[i] & ((1u << lane) - 1u));
+      if (idx < k) {
+        out[idx] = tid + i * kSelThreads;
+        if (picks) picks[idx] = tid + i * kSelThreads;
+      }
+    }
+  }
+}
+
+// The same for a unit of any length, on 64-bit keys read again in every pass: 8 passes of an 8-bit radix histogram at most,
+// then an ordered compaction of 1024 slots at a time.
+__device__ __noinline__ void select_long(int n, int k, const float* __restrict__ sc, const int* __restrict__ ps, int* out, int* picks) {
+  __shared__ unsigned int hist[256];
+  __shared__ unsigned long long s_prefix;
+  __shared__ int s_remaining, s_running, s_done;
+  __shared__ int s_warp_tot[kSelThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) { s_prefix = 0ull; s_remaining = k; s_done = 0; }
+  unsigned long long kth = ~0ull;
+  for (int pass = 0; pass < 8; ++pass) {
+    const int shift = 56 - 8 * pass;
+    if (tid < 256) hist[tid] = 0u;
+    __syncthreads();
+    const unsigned long long prefix = s_prefix;
+    const unsigned long long mask = (pass == 0) ? 0ull : (~0ull << (shift + 8));
+    for (int j = tid; j < n; j += kSelThreads) {
+      const unsigned long long key = make_key(sc[j], ps ? ps[j] : j);
+      if ((key & mask) == prefix) atomicAdd(&hist[(unsigned int)(key >> shift) & 255u], 1u);
+    }
+    __syncthreads();
+    if (warp == 0) {
+      // the first digit whose cumulative count reaches the number still wanted: 8 bins per lane
+      unsigned int c[8], sum = 0u;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) { c[q] = hist[8 * lane + q]; sum += c[q]; }
+      unsigned int incl = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      const unsigned int rem = (unsigned int)s_remaining;
+      const unsigned int reach = __ballot_sync(0xffffffffu, rem <= incl);
+      const int f = reach ? __ffs((int)reach) - 1 : 31;
+      if (lane == f) {
+        unsigned int r = rem - (incl - sum);
+        int q = 0;
+        for (; q < 7; ++q) {
+          if (r <= c[q]) break;
+          r -= c[q];
+        }
+        s_remaining = (int)r;
+        s_prefix = prefix | ((unsigned long long)(8 * lane + q) << shift);
+        s_done = (r == c[q]) ? 1 : 0;
+      }
+    }
+    __syncthreads();
+    if (s_done || pass == 7) {
+      kth = s_prefix | (shift ? ((1ull << shift) - 1ull) : 0ull);  // the largest key that is taken
+      break;
+    }
+  }
+  if (tid == 0) s_running = 0;
+  __syncthreads();
+  for (int j0 = 0; j0 < n; j0 += kSelThreads) {
+    const int j = j0 + tid;
+    const unsigned long long key = (j < n) ? make_key(sc[j], ps ? ps[j] : j) : ~0ull;
+    const int flag = (j < n) && (key <= kth);
+    const unsigned int ballot = __ballot_sync(0xffffffffu, flag);
+    const int in_warp = __popc(ballot & ((1u << lane) - 1u));
+    if (lane == 0) s_warp_tot[warp] = __popc(ballot);
+    __syncthreads();
+    int before = s_running;
+    for (int w = 0; w < warp; ++w) before += s_warp_tot[w];
+    const int idx = before + in_warp;
+    if (flag && idx < k) {
+      out[idx] = j;
+      if (picks) picks[idx] = j;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      int tot = s_running;
+      for (int w = 0; w < kSelThreads / 32; ++w) tot += s_warp_tot[w];
+      s_running = tot;
+    }
+    __syncthreads();
+  }
+}
+
+// One CTA per unit. k = max(0, n - budget): the k smallest keys, the slots in ascending order. Returns k, the number of slots the unit evicts (the same value in every thread of the CTA). With e_smem (room for
 // kMaxSharedPicks slots) the chosen slots are also left there when k fits, for a compaction in the same kernel.
 __device__ __forceinline__ int select_unit(int unit, int Hkv, int cap, const float* __restrict__ scores,
                                            const int* __restrict__ len, const int* __restrict__ budget,
                                            const int* __restrict__ pos, int* __restrict__ evict_idx, int max_evict,
                                            int* __restrict__ n_evict, int* status, int* e_smem = nullptr) {
-  __shared__ unsigned int hist[256];
-  __shared__ unsigned long long s_prefix;
-  __shared__ int s_remaining;
   __shared__ int s_warp_tot[kSelThreads / 32];
-  __shared__ int s_running;
   __shared__ unsigned long long s_min[kSelThreads / 32];
 
   const int b = unit / Hkv, h = unit % Hkv;
@@ -85,137 +309,10 @@ __device__ __forceinline__ int select_unit(int unit, int Hkv, int cap, const flo
     return 1;
   }
 
-  // Radix select on the 64-bit keys, 8 bits per pass, most significant first. Up to kCached keys per
-  // thread stay in registers across the passes; a pass ends the search early when the whole bucket it
-  // lands in is needed (always the case once the remaining bits only tell equal scores apart and
-  // positions are unique).
-  constexpr int kCached = 8;
-  const bool cached = n <= kSelThreads * kCached;
-  unsigned long long kreg[kCached];
-#pragma unroll
-  for (int i = 0; i < kCached; ++i) {
-    const int j = tid + i * kSelThreads;
-    kreg[i] = (cached && j < n) ? make_key(sc[j], ps ? ps[j] : j) : ~0ull;
-  }
-  __shared__ int s_done;
-  if (tid == 0) { s_prefix = 0ull; s_remaining = k; s_done = 0; }
-  unsigned long long kth = ~0ull;
-  for (int pass = 0; pass < 8; ++pass) {
-    const int shift = 56 - 8 * pass;
-    if (tid < 256) hist[tid] = 0u;
-    __syncthreads();
-    const unsigned long long prefix = s_prefix;
-    const unsigned long long mask = (pass == 0) ? 0ull : (~0ull << (shift + 8));
-    if (cached) {
-#pragma unroll
-      for (int i = 0; i < kCached; ++i) {
-        const int j = tid + i * kSelThreads;
-        if (j < n && (kreg[i] & mask) == prefix) atomicAdd(&hist[(unsigned int)(kreg[i] >> shift) & 255u], 1u);
-      }
-    } else {
-      for (int j = tid; j < n; j += kSelThreads) {
-        const unsigned long long key = make_key(sc[j], ps ? ps[j] : j);
-        if ((key & mask) == prefix) atomicAdd(&hist[(unsigned int)(key >> shift) & 255u], 1u);
-      }
-    }
-    __syncthreads();
-    if (warp == 0) {
-      // the first digit whose cumulative count reaches the number still wanted: 8 bins per lane
-      unsigned int c[8], sum = 0u;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) { c[q] = hist[8 * lane + q]; sum += c[q]; }
-      unsigned int incl = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      const unsigned int rem = (unsigned int)s_remaining;
-      const unsigned int reach = __ballot_sync(0xffffffffu, rem <= incl);
-      const int f = reach ? __ffs((int)reach) - 1 : 31;
-      if (lane == f) {
-        unsigned int r = rem - (incl - sum);
-        int q = 0;
-        for (; q < 7; ++q) {
-          if (r <= c[q]) break;
-          r -= c[q];
-        }
-        s_remaining = (int)r;
-        s_prefix = prefix | ((unsigned long long)(8 * lane + q) << shift);
-        s_done = (r == c[q]) ? 1 : 0;
-      }
-    }
-    __syncthreads();
-    if (s_done || pass == 7) {
-      kth = s_prefix | (shift ? ((1ull << shift) - 1ull) : 0ull);  // the largest key that is taken
-      break;
-    }
-  }
   int* picks = (e_smem && k <= kMaxSharedPicks) ? e_smem : nullptr;
-  if (cached) {
-    // one scan over the (round, warp) counts, which is the ascending order of the slots tid + round * kSelThreads
-    __shared__ int s_cnt[kCached * (kSelThreads / 32)];
-    unsigned int ballots[kCached];
-#pragma unroll
-    for (int i = 0; i < kCached; ++i) {
-      const int j = tid + i * kSelThreads;
-      ballots[i] = __ballot_sync(0xffffffffu, j < n && kreg[i] <= kth);
-      if (lane == 0) s_cnt[i * (kSelThreads / 32) + warp] = __popc(ballots[i]);
-    }
-    __syncthreads();
-    if (warp == 0) {
-      constexpr int kPerLane = kCached * (kSelThreads / 32) / 32;
-      int c[kPerLane], sum = 0;
-#pragma unroll
-      for (int q = 0; q < kPerLane; ++q) { c[q] = s_cnt[kPerLane * lane + q]; sum += c[q]; }
-      int incl = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      int run = incl - sum;
-#pragma unroll
-      for (int q = 0; q < kPerLane; ++q) { s_cnt[kPerLane * lane + q] = run; run += c[q]; }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < kCached; ++i) {
-      if (ballots[i] >> lane & 1u) {
-        const int idx = s_cnt[i * (kSelThreads / 32) + warp] + __popc(ballots[i] & ((1u << lane) - 1u));
-        if (idx < k) {
-          out[idx] = tid + i * kSelThreads;
-          if (picks) picks[idx] = tid + i * kSelThreads;
-        }
-      }
-    }
-    return k;
-  }
-  if (tid == 0) s_running = 0;
-  __syncthreads();
-  for (int j0 = 0; j0 < n; j0 += kSelThreads) {
-    const int j = j0 + tid;
-    const unsigned long long key = (j < n) ? make_key(sc[j], ps ? ps[j] : j) : ~0ull;
-    const int flag = (j < n) && (key <= kth);
-    const unsigned int ballot = __ballot_sync(0xffffffffu, flag);
-    const int in_warp = __popc(ballot & ((1u << lane) - 1u));
-    if (lane == 0) s_warp_tot[warp] = __popc(ballot);
-    __syncthreads();
-    int before = s_running;
-    for (int w = 0; w < warp; ++w) before += s_warp_tot[w];
-    const int idx = before + in_warp;
-    if (flag && idx < k) {
-      out[idx] = j;
-      if (picks) picks[idx] = j;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      int tot = s_running;
-      for (int w = 0; w < kSelThreads / 32; ++w) tot += s_warp_tot[w];
-      s_running = tot;
-    }
-    __syncthreads();
-  }
+  if (n <= 8 * kSelThreads) select_cached<8>(n, k, sc, ps, out, picks);
+  else if (n <= kMaxCached * kSelThreads) select_cached<kMaxCached>(n, k, sc, ps, out, picks);
+  else select_long(n, k, sc, ps, out, picks);
   return k;
 }
 
