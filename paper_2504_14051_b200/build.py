@@ -9,7 +9,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcaote.so")
-SOURCES = ["caote_api.cu"]
+SOURCES = ["caote_api.cu", "decode_step.cu"]
 
 
 def _nvcc() -> str:
@@ -34,6 +34,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         return LIB
     cmd = [
         _nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
+        "--threads", "0",
         "--shared", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
         "-cudart", "static", "-o", LIB,
     ]

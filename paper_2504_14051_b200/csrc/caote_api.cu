@@ -9,7 +9,7 @@
 #include <vector>
 
 #include "common.cuh"
-#include "decode_cluster.cuh"
+#include "decode_step.h"
 #include "decode_tc.cuh"
 #include "generic_score.cuh"
 #include "greedy.cuh"
@@ -277,19 +277,17 @@ static bool cluster_shape_ok(const caote_params_t* p) {
 static bool decode_shape_ok(const caote_params_t* p) { return p->head_dim == 128 && cluster_shape_ok(p); }
 
 // ---- single-query path on thread-block clusters ---------------------------------------------------------
-typedef void (*ClusterKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, Dims, const int*, float*, float*,
-                              float*, int*, long long, const float*);
 template <int kMode, int D>
 static ClusterKernel cluster_kernel_for_g(int g) {
   switch (g) {
-    case 1: return dcl::decode_cluster_kernel<1, kMode, D>;
-    case 2: return dcl::decode_cluster_kernel<2, kMode, D>;
-    case 3: return dcl::decode_cluster_kernel<3, kMode, D>;
-    case 4: return dcl::decode_cluster_kernel<4, kMode, D>;
-    case 5: return dcl::decode_cluster_kernel<5, kMode, D>;
-    case 6: return dcl::decode_cluster_kernel<6, kMode, D>;
-    case 7: return dcl::decode_cluster_kernel<7, kMode, D>;
-    default: return dcl::decode_cluster_kernel<8, kMode, D>;
+    case 1: return dcl::decode_cluster_kernel<1, kMode, D, false>;
+    case 2: return dcl::decode_cluster_kernel<2, kMode, D, false>;
+    case 3: return dcl::decode_cluster_kernel<3, kMode, D, false>;
+    case 4: return dcl::decode_cluster_kernel<4, kMode, D, false>;
+    case 5: return dcl::decode_cluster_kernel<5, kMode, D, false>;
+    case 6: return dcl::decode_cluster_kernel<6, kMode, D, false>;
+    case 7: return dcl::decode_cluster_kernel<7, kMode, D, false>;
+    default: return dcl::decode_cluster_kernel<8, kMode, D, false>;
   }
 }
 template <int D>
@@ -387,12 +385,13 @@ static int encode_decode_maps(const Dims& dm, const void* q, const void* K, cons
 
 static int launch_decode_cluster(const Dims& dm, const void* q, const void* K, const void* V, const int* len,
                                  float* base, float* o, float* scores, char* ws, cudaStream_t st, bool* used,
-                                 const float* vsum = nullptr) {
+                                 const float* vsum = nullptr, const dcl::StepArgs* step = nullptr) {
+  // step: the whole step in the one launch, or nothing (*used = false) where a cluster would get more than one unit
   *used = false;
   TensorMapEncodeFn encode = tensor_map_encoder();
   const bool carried = dm.base_mode == CAOTE_BASE_ACCUM || dm.base_mode == CAOTE_BASE_EXTERNAL;
   if (!encode || (carried && !aligned(base, 16)) || !aligned(q, 16)) return CAOTE_OK;
-  const ClusterKernel kernel = cluster_kernel(dm);
+  const ClusterKernel kernel = step ? step_kernel(dm) : cluster_kernel(dm);
   // (the attributes below are per function: every instantiation gets them the first time it is used)
   static std::mutex attr_mu;
   static std::vector<std::pair<int, ClusterKernel>> attr_done;
@@ -410,7 +409,7 @@ static int launch_decode_cluster(const Dims& dm, const void* q, const void* K, c
   }
   int clusters = 0;
   const int c = choose_cluster(dm, kernel, &clusters);
-  if (c == 0) return CAOTE_OK;
+  if (c == 0 || (step && clusters < dm.units)) return CAOTE_OK;
   CUtensorMap tmK, tmV, tmQ;
   int rc = encode_decode_maps(dm, q, K, V, 8, &tmK, &tmV, &tmQ, encode);
   if (rc) return rc;
@@ -431,9 +430,10 @@ static int launch_decode_cluster(const Dims& dm, const void* q, const void* K, c
   cfg.numAttrs = 2;
   int* status = reinterpret_cast<int*>(ws);
   const long long wait_cycles = g_wait_cycles.load(std::memory_order_relaxed);
-  CAOTE_LAUNCH("decode_cluster_kernel", st, {
+  const dcl::StepArgs sa = step ? *step : dcl::StepArgs{};
+  CAOTE_LAUNCH(step ? "decode_step_kernel" : "decode_cluster_kernel", st, {
     cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, tmK, tmV, tmQ, dm, len, base, o, scores, status,
-                                       wait_cycles, vsum);
+                                       wait_cycles, vsum, sa);
     if (e != cudaSuccess) return cuda_fail(e, "decode_cluster_kernel");
   });
   *used = true;
@@ -1232,6 +1232,19 @@ static int step_impl(const caote_params_t* p, const void* q, const void* k_new, 
   if (!rc) rc = check_device();
   if (rc) return rc;
   const bool bf16 = p->dtype == CAOTE_BF16;
+  if (k_new && compact_mode == CAOTE_COMPACT_FILL && max_evict == 1 && cluster_shape_ok(p)) {
+    // few single-query units: append, scoring, selection and compaction in one launch, where the scoring would be one launch
+    // of the cluster kernel with a cluster per unit
+    const Dims dm = make_dims(p);
+    if (vsum || dm.D == 64 || plan_side_by_side(dm) == 0) {
+      int* hdr = reinterpret_cast<int*>(workspace);
+      const dcl::StepArgs sa{(const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, (__nv_bfloat16*)K, (__nv_bfloat16*)V, pos, len,
+                             n_seen, budget, evict_idx, n_evict, hdr + 4, vsum};
+      bool used = false;
+      rc = launch_decode_cluster(dm, q, K, V, len, base, o, scores, (char*)workspace, (cudaStream_t)stream, &used, vsum, &sa);
+      if (rc || used) return rc;
+    }
+  }
   if (k_new || v_new) {
     const Dims dma = make_dims(p);
     const bool fold = vsum && dma.m == 1 && append_per_sequence(dma);  // the append adds the new value rows itself

@@ -37,6 +37,13 @@
 // double-buffered by unit parity. So no push can overtake a read, and no mbarrier phase can receive
 // bytes of the next one.
 //
+// The whole-step form (kStep). Where every unit has a cluster of its own and a step evicts at most one token, the step is
+// this one launch: the CTA that owns the unit's last tile first appends the new row (written with plain stores, made visible
+// to the copies by a proxy fence), the keeper warps name their smallest (score, position), rank 0 takes the smallest of
+// these after the closing cluster barrier and lets the last row fill the hole, and the cluster that finishes last moves the
+// lengths on. Append, scoring and selection as three dependent launches take 18.7 us on the device and as much on the host
+// for 8 units of 2049 tokens, so TBD.
+//
 // Every wait is bounded by a clock limit. A wait that runs out records CAOTE_ERR_TIMEOUT and raises the
 // CTA's stop flag; from then on no wait of this CTA blocks, the copy and product issuers stop, the token
 // groups run through the rest of their schedule on whatever their buffers hold (indices stay in bounds,
@@ -142,7 +149,7 @@ __device__ __forceinline__ bool mbar_try_wait_parked(uint64_t* bar, uint32_t par
 }
 
 // Wait for hardware to finish what has already been issued (copies in flight, queued products).
-__device__ __noinline__ void drain_wait(uint64_t* bar, uint32_t parity, int* status) {
+static __device__ __noinline__ void drain_wait(uint64_t* bar, uint32_t parity, int* status) {
   const long long t0 = clock64();
   while (!mbar_try_wait_parked(bar, parity, 2000u)) {
     if (clock64() - t0 > kDrainCycles) {
@@ -153,7 +160,7 @@ __device__ __noinline__ void drain_wait(uint64_t* bar, uint32_t parity, int* sta
 }
 // Bounded wait; a wait that runs out records the timeout and raises the stop flag. Never blocks once the
 // flag is up. The polling loop is kept out of line: the common case is that the phase has completed.
-__device__ __noinline__ void wait_slow(uint64_t* bar, uint32_t parity, volatile int* stop, int* status, long long limit,
+static __device__ __noinline__ void wait_slow(uint64_t* bar, uint32_t parity, volatile int* stop, int* status, long long limit,
                                        bool idle) {
   const long long t0 = clock64();
   while (!mbar_try_wait_parked(bar, parity, 2000u)) {
@@ -240,14 +247,28 @@ struct Sched {
   }
 };
 
+// What the whole-step form needs besides (pos, n_seen and vsum may be null).
+struct StepArgs {
+  const __nv_bfloat16 *k_new, *v_new;  // [units][D]
+  __nv_bfloat16 *K, *V;
+  int *pos, *len, *n_seen;
+  const int* budget;
+  int *evict_idx, *n_evict, *ticket;
+  float* vsum;
+};
+// A candidate for eviction; slot < 0: none.
+__device__ __forceinline__ void first_candidate(unsigned& v, unsigned& p, int& s, unsigned ov, unsigned op, int os) {
+  if (os >= 0 && (s < 0 || ov < v || (ov == v && (op < p || (op == p && os < s))))) { v = ov; p = op; s = os; }
+}
+
 // kG: query heads per KV head; kMode: the base mode. Compile-time so that the per-head loops carry no
 // predicates and the paths of the other modes are not in the instruction stream.
-template <int kG, int kMode, int D>
+template <int kG, int kMode, int D, bool kStep>
 __global__ void __launch_bounds__(kThreads, 1)
 decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                       const __grid_constant__ CUtensorMap tmQ, Dims dm, const int* __restrict__ len,
                       float* __restrict__ base, float* __restrict__ o, float* __restrict__ scores, int* status,
-                      long long wait_cycles, const float* __restrict__ vsum) {
+                      long long wait_cycles, const float* __restrict__ vsum, const StepArgs sa) {
   constexpr int kTileBytes = kTileBytesOf<D>, kKS = kKSlots<D>, kVS = kVSlots<D>, kStash = kStashTiles<D>;
   constexpr int kBoxes = D / 64, kRowCols = D / 2;  // 64-channel boxes of a tile; TMEM columns of a stashed row
   ptx::pdl_wait();
@@ -330,7 +351,32 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     mbar_expect_tx(r1, r1_bytes);
     mbar_expect_tx(r2, r2_bytes);
   }
-  for (int k = tid; k < min(nk, kLenTab); k += kThreads) slen[k] = __ldg(len + (sch.cid + k * sch.ncl) / dm.Hkv);
+  int step_n = 0;          // kStep: the unit's length with the new token, if there is room for it
+  bool step_fits = false;
+  if constexpr (kStep) {
+    const int u = sch.cid, b = u / dm.Hkv;
+    // the new rows are on their way while the length is
+    uint4 row = make_uint4(0u, 0u, 0u, 0u);
+    if (tid < D / 4) row = reinterpret_cast<const uint4*>((tid < D / 8 ? sa.k_new : sa.v_new) + (size_t)u * D)[tid & (D / 8 - 1)];
+    const int n0 = __ldcg(sa.len + b);
+    step_fits = n0 >= 0 && n0 < dm.cap;
+    step_n = n0 + (step_fits ? 1 : 0);
+    if (tid == 0) {
+      slen[0] = step_n;
+      if (!step_fits && rank == 0) set_status(status, CAOTE_ERR_OVERFLOW);
+    }
+    // (the deal of the tiles as in Sched::at: this CTA has the last one)
+    const int nt = step_fits ? (step_n + kT - 1) / kT : 0;
+    if (nt > 0 && rank == (nt >= C ? C : nt) - 1) {
+      const size_t slot = (size_t)u * dm.cap + n0;
+      if (tid < D / 4) reinterpret_cast<uint4*>((tid < D / 8 ? sa.K : sa.V) + slot * D)[tid & (D / 8 - 1)] = row;
+      if (tid == 96 && base) base[slot] = 0.f;
+      if (tid == 97 && sa.pos) sa.pos[slot] = sa.n_seen ? __ldcg(sa.n_seen + b) : n0;
+      ptx::fence_async_all();  // the copies below read them through the async proxy
+    }
+  } else {
+    for (int k = tid; k < min(nk, kLenTab); k += kThreads) slen[k] = __ldg(len + (sch.cid + k * sch.ncl) / dm.Hkv);
+  }
   // rows of P^T that no head writes stay zero for the whole kernel
   for (int i = tid; i < kPBytes / 16; i += kThreads) reinterpret_cast<uint4*>(pbuf)[i] = make_uint4(0u, 0u, 0u, 0u);
   fence_async_smem();
@@ -716,6 +762,8 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     float keepb[kMaxKeep];    // and their carried base scores
     int ti = 0;               // tiles this CTA has been through before the current unit
     int mu = 0;               // units merged so far (phases of r1 / r2)
+    unsigned best_v = 0xffffffffu;  // kStep: this thread's smallest score and its slot
+    int best_s = -1;
 
     for (int k = 0; k < nk; ++k) {
       const Work w = sch.at(k);
@@ -839,7 +887,16 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 #pragma unroll
           for (int off = 4; off > 0; off >>= 1) xs += __shfl_xor_sync(0xffffffffu, xs, off);
           // FastCAOTE (Sec. 3.3): the distances are taken to the mean of the unit's value rows instead of X
-          const float nxv = vsum ? -(act ? __ldg(vsum + (size_t)w.unit * D + my_ch0 + cl) / (float)w.n : 0.f) : -(xs * inv_H);
+          float nxv;
+          if constexpr (kStep) {  // (the running sum does not hold the new row yet)
+            nxv = -(xs * inv_H);
+            if (vsum && act) {
+              const size_t at = (size_t)w.unit * D + my_ch0 + cl;
+              nxv = -((__ldg(vsum + at) + (step_fits ? __bfloat162float(sa.v_new[at]) : 0.f)) / (float)w.n);
+            }
+          } else {
+            nxv = vsum ? -(act ? __ldg(vsum + (size_t)w.unit * D + my_ch0 + cl) / (float)w.n : 0.f) : -(xs * inv_H);
+          }
           if (act && !ctl[0]) {
             for (int peer = r; peer < C; peer += 8)
               push_f32(map_to_rank(smem_u32(xdst + my_ch0 + cl), peer), nxv, map_to_rank(smem_u32(r2), peer));
@@ -946,6 +1003,15 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             float sc = 0.f;
             if (Htot > 0.f && hj > 0.f) sc = (rest > 0.f) ? __fdividef(hj, rest) * fast_sqrt(n2) : INFINITY;
             scores[slot] = sc;
+            if constexpr (kStep) {
+              const unsigned v = __float_as_uint(sc);
+              const int s = t * kT + tok;
+              const int* ps = sa.pos ? sa.pos + (size_t)w.unit * dm.cap : nullptr;
+              if (best_s < 0 || v < best_v || (v == best_v && (unsigned)(ps ? __ldcg(ps + s) : s) < (unsigned)(ps ? __ldcg(ps + best_s) : best_s))) {
+                best_v = v;
+                best_s = s;
+              }
+            }
           }
           if (j >= kStash) {
             __syncwarp();
@@ -962,6 +1028,18 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       }
       ti += w.T;
       ++mu;
+    }
+    if constexpr (kStep) {
+      // the warp's candidate goes to rank 0: into its records, which every CTA was done with before anyone got here
+      const int* ps = sa.pos ? sa.pos + (size_t)sch.cid * dm.cap : nullptr;
+      const unsigned v1 = __reduce_min_sync(0xffffffffu, best_s >= 0 ? best_v : 0xffffffffu);
+      const bool eq = best_s >= 0 && best_v == v1;
+      const unsigned p = eq ? (unsigned)(ps ? __ldcg(ps + best_s) : best_s) : 0xffffffffu;
+      const unsigned p1 = __reduce_min_sync(0xffffffffu, p);
+      const int s1 = (int)__reduce_min_sync(0xffffffffu, eq && p == p1 ? (unsigned)best_s : 0x7fffffffu);
+      if (lane == 0)
+        ptx::st_dsmem_v4(map_to_rank(smem_u32(xo) + (uint32_t)((rank * 4 * kNB + warp - 4) * 16), 0),
+                         make_uint4(v1, p1, (uint32_t)(s1 == 0x7fffffff || ctl[0] ? -1 : s1), 0u));
     }
   }
 
@@ -988,6 +1066,65 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   }
   if (warp == kWarpQK) prefill::tmem_dealloc(tmem, kTmemCols);
   cluster_sync_all();
+  if constexpr (kStep) {
+    // ===================== selection and compaction: rank 0 =====================
+    if (rank != 0) return;
+    const int u = sch.cid, b = u / dm.Hkv, n = step_n;
+    int bud = __ldg(sa.budget + b);
+    if (bud < 1) bud = 1;
+    int k = (n > 0 && n <= dm.cap) ? max(n - bud, 0) : 0;
+    if (k > 1) {  // (this form is launched for calls that take one eviction at most)
+      if (tid == 0) set_status(status, CAOTE_ERR_OVERFLOW);
+      k = 0;
+    }
+    if (tid == 0 && u % dm.Hkv == 0) sa.n_evict[b] = k;
+    unsigned v = 0u, p = 0u;
+    int s = -1;
+    if (k == 1) {
+      const uint4* cand = reinterpret_cast<const uint4*>(xo);
+      for (int i = lane; i < C * 4 * kNB; i += 32) first_candidate(v, p, s, cand[i].x, cand[i].y, (int)cand[i].z);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        first_candidate(v, p, s, __shfl_xor_sync(0xffffffffu, v, o), __shfl_xor_sync(0xffffffffu, p, o), __shfl_xor_sync(0xffffffffu, s, o));
+      if (s < 0) s = n - 1;  // (every CTA gave up: the new token goes)
+    }
+    if (sa.vsum && tid >= 128 && tid < 128 + D) {  // FastCAOTE: the new row joins the running sum, the evicted one leaves it
+      const size_t at = (size_t)u * D + tid - 128;
+      float x = sa.vsum[at];
+      if (step_fits) x += __bfloat162float(sa.v_new[at]);
+      if (k == 1) x -= __bfloat162float(sa.V[((size_t)u * dm.cap + s) * D + tid - 128]);
+      sa.vsum[at] = x;
+    }
+    if (sa.vsum) __syncthreads();
+    if (k == 1) {
+      if (tid == 0) sa.evict_idx[u] = s;
+      const size_t hole = (size_t)u * dm.cap + s, tail = (size_t)u * dm.cap + n - 1;
+      if (s != n - 1) {
+        if (warp == 1 && lane < D / 8) reinterpret_cast<uint4*>(sa.K + hole * D)[lane] = __ldcg(reinterpret_cast<const uint4*>(sa.K + tail * D) + lane);
+        if (warp == 2 && lane < D / 8) reinterpret_cast<uint4*>(sa.V + hole * D)[lane] = __ldcg(reinterpret_cast<const uint4*>(sa.V + tail * D) + lane);
+        if (warp == 3 && lane == 0 && base) base[hole] = __ldcg(base + tail);
+        if (warp == 3 && lane == 1 && sa.pos) sa.pos[hole] = __ldcg(sa.pos + tail);
+      }
+    }
+    // the cluster that finishes last (a ticket, which it also resets) moves the lengths on
+    __shared__ int s_last;
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      s_last = atomicAdd(sa.ticket, 1) == dm.units - 1;
+    }
+    __syncthreads();
+    if (s_last) {
+      __threadfence();
+      for (int i = tid; i < dm.B; i += kThreads) {
+        const int n0 = __ldcg(sa.len + i);
+        const int more = (n0 >= 0 && n0 < dm.cap) ? 1 : 0;
+        sa.len[i] = n0 + more - __ldcg(sa.n_evict + i);
+        if (sa.n_seen) sa.n_seen[i] += more;
+      }
+      if (tid == 0) *sa.ticket = 0;
+    }
+  }
 }
 
 }  // namespace dcl

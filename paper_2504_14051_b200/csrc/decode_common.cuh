@@ -113,7 +113,7 @@ inline size_t carve(const Dims& dm, char* base, Plan* out, int grid) {
 }
 
 // ---- plan: items per unit, their prefix sum, and cleared counters / flags (one CTA) -------------
-__global__ void __launch_bounds__(1024)
+static __global__ void __launch_bounds__(1024)
 plan_kernel(int units, int Hkv, int cap, const int* __restrict__ len, Plan pl, int* status) {
   ptx::pdl_wait();
   ptx::pdl_trigger();

@@ -824,7 +824,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 
 // FastCAOTE, after decode_tc_kernel<true>: c_j = w_j / (1 - w_j) * || mean(v) - v_j || from the stored
 // logits, the unit's final softmax statistics and the stored distances. grid = (tiles, units), kT threads.
-__global__ void __launch_bounds__(kT)
+static __global__ void __launch_bounds__(kT)
 fast_finish_kernel(Dims dm, const int* __restrict__ len, float* __restrict__ base, float* __restrict__ scores, Plan pl) {
   ptx::pdl_wait();
   ptx::pdl_trigger();

@@ -105,3 +105,63 @@ def test_equal_lowest_scores_go_by_position(dtype, d, n):
             assert int(c.evict_idx[b, h, 0]) == want
             assert want in copies
     assert ties > 0, "the copies' scores were expected to be equal in at least one unit"
+
+
+@pytest.mark.parametrize("shape", [
+    # B, Hq, Hkv, d, cap, lengths, budgets: sequences that grow, that evict one, that have no room, that would have to
+    # evict two, a new token on a tile of its own, more CTAs in the cluster than tiles
+    (4, 8, 2, 128, 1296, [1279, 1295, 1296, 300], [1400, 1295, 1296, 299]),
+    (2, 14, 2, 128, 400, [128, 255], [128, 400]),
+    (5, 8, 8, 64, 2064, [1, 127, 128, 2047, 2063], [1, 127, 500, 2047, 2063]),
+])
+@pytest.mark.parametrize("mode", ["last_query", "accum", "external"])
+@pytest.mark.parametrize("fast", [False, True])
+def test_whole_step_kernel_equals_the_four_calls(shape, mode, fast):
+    """Steps on few units are one launch; the same calls made one after the other on a copy of the state give the same
+    cache, lengths, positions, sums and status, and scores to the rounding of the two compilations."""
+    B, Hq, Hkv, d, cap, lens, budget = shape
+    g = torch.Generator(device="cpu").manual_seed(cap + d)
+    dt = torch.bfloat16
+    mk = lambda: P.EvictionCache(B, Hq, Hkv, d, cap, 1, dt, torch.tensor(budget, dtype=torch.int32), mode, "fill", max_evict=1,
+                                 method="fast" if fast else "caote", device=DEV)
+    a, b = mk(), mk()
+    K0, V0 = (torch.randn((B, Hkv, cap, d), generator=g).to(dt) for _ in range(2))
+    base0 = torch.rand((B, Hkv, cap), generator=g) + 0.1
+    pos0 = torch.stack([torch.stack([torch.randperm(cap, generator=g) for _ in range(Hkv)]) for _ in range(B)]).to(torch.int32)
+    for c in (a, b):
+        c.load(K0, V0, torch.tensor(lens, dtype=torch.int32), base=base0, pos=pos0)
+        c.n_seen.fill_(cap + 7)
+    p = a.params
+    for step in range(3):
+        q = torch.randn((B, Hq, 1, d), generator=g).to(dt).to(DEV)
+        kn, vn = (torch.randn((B, Hkv, 1, d), generator=g).to(dt).to(DEV) for _ in range(2))
+        P.caote_trace_enable(True)
+        a.step(q, kn, vn)
+        torch.cuda.synchronize()
+        assert set(P.caote_trace_collect()) == {"decode_step_kernel"}
+        P.caote_trace_enable(False)
+        P.caote_append(p, b.K, b.V, b.base, b.pos, b.lens, b.n_seen, kn, vn, b.workspace)
+        if fast:
+            P.caote_vsum(p, b.V, b.lens, b.vsum)
+            P.caote_score_fast(p, q, b.K, b.V, b.lens, b.base, b.vsum, b.o, b.scores, b.workspace)
+        else:
+            P.caote_score(p, q, b.K, b.V, b.lens, b.base, b.o, b.scores, b.workspace)
+        P.caote_select_evict(p, b.scores, b.lens, b.budget, b.pos, b.evict_idx, b.n_evict, b.workspace)
+        P.caote_compact(p, b.K, b.V, b.base, b.pos, b.lens, b.evict_idx, b.n_evict, "fill", b.workspace)
+        torch.cuda.synchronize()
+        assert a.status() == b.status()
+        assert a.lens.tolist() == b.lens.tolist() and a.n_seen.tolist() == b.n_seen.tolist() and a.n_evict.tolist() == b.n_evict.tolist()
+        torch.testing.assert_close(a.o, b.o, rtol=1e-5, atol=1e-6)
+        for s in range(B):
+            n = int(a.lens[s])
+            if int(a.n_evict[s]):
+                assert torch.equal(a.evict_idx[s], b.evict_idx[s])
+            assert torch.equal(a.K[s, :, :n], b.K[s, :, :n]) and torch.equal(a.V[s, :, :n], b.V[s, :, :n])
+            assert torch.equal(a.pos[s, :, :n], b.pos[s, :, :n])
+            torch.testing.assert_close(a.base[s, :, :n], b.base[s, :, :n], rtol=1e-5, atol=1e-6)
+            torch.testing.assert_close(a.scores[s, :, :n], b.scores[s, :, :n], rtol=1e-4, atol=1e-6)
+        if fast:
+            ref = P.EvictionCache(B, Hq, Hkv, d, cap, 1, dt, 1, mode, "fill", method="fast", device=DEV)
+            P.caote_vsum(p, a.V, a.lens, ref.vsum)
+            # a handful of fp32 additions on sums of up to 2 k normal values (about 45): 1e-5 each
+            torch.testing.assert_close(a.vsum, ref.vsum, rtol=1e-5, atol=1e-3)
