@@ -16,6 +16,7 @@
 #include "post_evict.cuh"
 #include "prefill_tc.cuh"
 #include "select_compact.cuh"
+#include "small_step.cuh"
 #include "sum_errors_decode.cuh"
 
 namespace caote {
@@ -219,6 +220,33 @@ static int launch_generic_score(const Dims& dm, const void* q, const void* K, co
                  launch_pdl(generic::score_pass_kernel<T, D>, grid, dim3(generic::kThreads), smem, st, dm, (const T*)q, (const T*)K,
                             (const T*)V, len, base, sc, scores, vsum));
   }
+  return CAOTE_OK;
+}
+
+// The whole decode step of a short unit on the CUDA cores (small_step.cuh), for single queries that the tensor-core cluster
+// kernel does not take. Which of them, by the us of a step in several launches and in this one:
+// fp32, where the other path has the same arithmetic: up to 1 024 slots (2 units of 1 000, head_dim 64: 22.3, 20.8; 256 of
+// head_dim 128: 325, 261); from 16 units on up to 2 048, since the other path splits few long units over more SMs (4 units of
+// 2 000: 33.9, 37.3; 16: 57.9, 48.8; 256: 603, 468) and the logits of 4 096 leave one CTA per SM (256: 1159, 1373).
+// bf16, where the other path is the row-block kernels: while the step is bound by its launches, i.e. the CTAs have one tile
+// and run at once (16 heads, 2 units of 500: 28.5, 20.7; of 1 000: 28.2, 29.8; 64 units of 250, head_dim 64: 22.5, 21.4; of
+// 500, in clusters of eight: 25.7, 41.9; 128 units of 100: 25.1, 23.9).
+static bool small_step_ok(const caote_params_t* p) {
+  const long long units = (long long)p->batch * p->n_kv_heads;
+  const int nt = (p->capacity + small::kKT - 1) / small::kKT;
+  if (p->n_new != 1) return false;
+  if (p->dtype == CAOTE_F32) return units <= (1 << 20) && nt <= (units >= 16 ? 4 : 2) * small::kMaxC;
+  return nt <= small::kMaxC && units * small::cluster_size(nt) <= (nt <= 4 ? 2 : 1) * g_sm_count;
+}
+template <typename T, int D>
+static int launch_small_step(const Dims& dm, const small::Args<T>& sa, int* status, cudaStream_t st) {
+  const int nt = (dm.cap + small::kKT - 1) / small::kKT;
+  const int c = small::cluster_size(nt), tiles = (nt + c - 1) / c;
+  int rc = allow_smem(small::small_step_kernel<T, D>, small::smem_bytes(D, small::kMaxTiles));
+  if (rc) return rc;
+  CAOTE_LAUNCH("small_step_kernel", st,
+               launch_pdl_clusters(small::small_step_kernel<T, D>, dim3(dm.units * c), dim3(small::kThreads), small::smem_bytes(D, tiles), c,
+                                   st, dm, sa, tiles, status));
   return CAOTE_OK;
 }
 
@@ -1244,6 +1272,20 @@ static int step_impl(const caote_params_t* p, const void* q, const void* k_new, 
       rc = launch_decode_cluster(dm, q, K, V, len, base, o, scores, (char*)workspace, (cudaStream_t)stream, &used, vsum, &sa);
       if (rc || used) return rc;
     }
+  }
+  if (k_new && compact_mode == CAOTE_COMPACT_FILL && max_evict == 1 && !cluster_shape_ok(p) && small_step_ok(p)) {
+    const Dims dm = make_dims(p);
+    int* hdr = reinterpret_cast<int*>(workspace);
+    auto launch = [&](auto t, auto d) {
+      using T = decltype(t);
+      const small::Args<T> sa{(const T*)q, (const T*)k_new, (const T*)v_new, (T*)K, (T*)V, base, pos, len, n_seen, budget, o, scores,
+                              evict_idx, n_evict, hdr + 4, vsum};
+      return launch_small_step<T, decltype(d)::value>(dm, sa, hdr, (cudaStream_t)stream);
+    };
+    const std::integral_constant<int, 64> d64;
+    const std::integral_constant<int, 128> d128;
+    if (bf16) return dm.D == 128 ? launch(__nv_bfloat16(), d128) : launch(__nv_bfloat16(), d64);
+    return dm.D == 128 ? launch(float(), d128) : launch(float(), d64);
   }
   if (k_new || v_new) {
     const Dims dma = make_dims(p);
