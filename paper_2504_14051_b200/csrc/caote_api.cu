@@ -1230,7 +1230,7 @@ int caote_compact(const caote_params_t* p, void* K, void* V, float* base, int32_
   cudaStream_t st = (cudaStream_t)stream;
   if (mode == CAOTE_COMPACT_FILL) {
     CAOTE_LAUNCH("compact_fill_kernel", st, launch_pdl(sel::compact_fill_kernel, dim3(dm.units), dim3(dm.m > 16 ? sel::kSelThreads : 256), 0, st, dm.Hkv, dm.cap, row_bytes, (char*)K, (char*)V, base, pos,
-                                                       len, evict_idx, max_evict, n_evict));
+                                                       len, evict_idx, max_evict, n_evict, dm.B, ticket));
   } else {
     rc = allow_smem(sel::compact_stable_kernel, 2 * sel::kStableTileBytes);
     if (rc) return rc;
@@ -1239,10 +1239,9 @@ int caote_compact(const caote_params_t* p, void* K, void* V, float* base, int32_
     dim3 grid(dm.units * c, 3);
     CAOTE_LAUNCH("compact_stable_kernel", st,
                  launch_pdl_clusters(sel::compact_stable_kernel, grid, dim3(sel::kStableThreads), 2 * sel::kStableTileBytes,
-                                     c, st, dm.Hkv, dm.cap, row_bytes, (char*)K, (char*)V, base, pos, (const int*)len,
-                                     evict_idx, max_evict, n_evict));
+                                     c, st, dm.Hkv, dm.cap, row_bytes, (char*)K, (char*)V, base, pos, len, evict_idx, max_evict,
+                                     n_evict, dm.B, ticket));
   }
-  CAOTE_LAUNCH("update_len_kernel", st, launch_pdl(sel::update_len_kernel, dim3((dm.B + 127) / 128), dim3(128), 0, st, dm.B, len, n_evict));
   return CAOTE_OK;
 }
 
@@ -1250,6 +1249,7 @@ int caote_compact(const caote_params_t* p, void* K, void* V, float* base, int32_
 static int step_impl(const caote_params_t* p, const void* q, const void* k_new, const void* v_new, void* K, void* V,
                      float* base, int32_t* pos, int32_t* len, int32_t* n_seen, const int32_t* budget, float* vsum,
                      float* o, float* scores, int32_t* evict_idx, int32_t max_evict, int32_t* n_evict,
+  int* ticket = reinterpret_cast<int*>(workspace) + 4;
                      int32_t compact_mode, void* workspace, size_t workspace_bytes_, caote_stream_t stream) {
   // every host-visible check of the calls below runs before the first launch
   int rc = score_args_check(p, q, K, V, len, base, o, scores);

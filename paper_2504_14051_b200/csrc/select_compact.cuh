@@ -382,10 +382,27 @@ __device__ __forceinline__ void compact_fill_unit(int unit, int k, int Hkv, int 
   }
 }
 
+// Every CTA's last step: whichever CTA of the launch finishes last (a ticket counter in the workspace header, which that CTA
+// also resets) moves the lengths on, so that no other CTA still needs the old ones.
+__device__ __forceinline__ void finish_lengths(int B, int* __restrict__ len, const int* __restrict__ n_evict, int* ticket) {
+  __shared__ int s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = (atomicAdd(ticket, 1) == (int)(gridDim.x * gridDim.y) - 1);
+  }
+  __syncthreads();
+  if (s_last) {
+    __threadfence();
+    for (int b = threadIdx.x; b < B; b += blockDim.x) len[b] -= __ldcg(&n_evict[b]);
+    if (threadIdx.x == 0) *ticket = 0;
+  }
+}
+
 __global__ void __launch_bounds__(kSelThreads)
 compact_fill_kernel(int Hkv, int cap, int row_bytes, char* __restrict__ K, char* __restrict__ V,
-                    float* __restrict__ base, int* __restrict__ pos, const int* __restrict__ len,
-                    const int* __restrict__ evict_idx, int max_evict, const int* __restrict__ n_evict) {
+                    float* __restrict__ base, int* __restrict__ pos, int* __restrict__ len,
+                    const int* __restrict__ evict_idx, int max_evict, const int* __restrict__ n_evict, int B, int* ticket) {
   ptx::pdl_wait();
   ptx::pdl_trigger();
   // (the searches are chains of dependent reads of the picks: from shared memory where they fit)
@@ -398,6 +415,7 @@ compact_fill_kernel(int Hkv, int cap, int row_bytes, char* __restrict__ K, char*
     E = s_picks;
   }
   compact_fill_unit(blockIdx.x, k, Hkv, cap, row_bytes, K, V, base, pos, len, E);
+  finish_lengths(B, len, n_evict, ticket);
 }
 
 // A unit that evicts exactly one token, with FILL compaction: the argmin over (score bits, position) and the move of
@@ -496,25 +514,8 @@ __device__ __forceinline__ bool select_one_fill_unit(int unit, int Hkv, int cap,
   return true;
 }
 
-// The CTA that finishes last (a ticket counter, which it also resets) takes the evicted counts off the lengths.
-__device__ __forceinline__ void finish_lengths(int B, int* __restrict__ len, const int* __restrict__ n_evict, int* ticket) {
-  __shared__ int s_last;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    s_last = (atomicAdd(ticket, 1) == (int)gridDim.x - 1);
-  }
-  __syncthreads();
-  if (s_last) {
-    __threadfence();
-    for (int b = threadIdx.x; b < B; b += blockDim.x) len[b] -= __ldcg(&n_evict[b]);
-    if (threadIdx.x == 0) *ticket = 0;
-  }
-}
-
-// Selection and FILL compaction of one unit per CTA in one launch, and the length update by whichever
-// CTA finishes last (a ticket counter in the workspace header, which that CTA also resets). Same results
-// as select_kernel + compact_fill_kernel + update_len_kernel.
+// Selection, FILL compaction (one unit per CTA) and the length update in one launch. Same results as select_kernel +
+// compact_fill_kernel.
 __global__ void __launch_bounds__(kSelThreads)
 select_compact_kernel(int B, int Hkv, int cap, int row_bytes, const float* __restrict__ scores, char* __restrict__ K,
                       char* __restrict__ V, float* __restrict__ base, int* __restrict__ pos, int* __restrict__ len,
@@ -553,8 +554,8 @@ select_compact_kernel(int B, int Hkv, int cap, int row_bytes, const float* __res
 constexpr int kStableMaxCtas = 8, kStableTileBytes = 32768, kStableMaxRows = 256, kStableThreads = 256;
 __global__ void __launch_bounds__(kStableThreads)
 compact_stable_kernel(int Hkv, int cap, int row_bytes, char* __restrict__ K, char* __restrict__ V,
-                      float* __restrict__ base, int* __restrict__ pos, const int* __restrict__ len,
-                      const int* __restrict__ evict_idx, int max_evict, const int* __restrict__ n_evict) {
+                      float* __restrict__ base, int* __restrict__ pos, int* __restrict__ len,
+                      const int* __restrict__ evict_idx, int max_evict, const int* __restrict__ n_evict, int B, int* ticket) {
   ptx::pdl_wait();
   ptx::pdl_trigger();
   extern __shared__ __align__(16) char tiles[];  // [2][kStableTileBytes]
@@ -562,61 +563,55 @@ compact_stable_kernel(int Hkv, int cap, int row_bytes, char* __restrict__ K, cha
   __shared__ int s_picks[kMaxSharedPicks];
   const int C = (int)ptx::cluster_nctarank(), unit = blockIdx.x / C, rank = (int)ptx::cluster_ctarank(), b = unit / Hkv, which = blockIdx.y;
   const int tid = threadIdx.x, k = n_evict[b], n = len[b];
-  if (k <= 0 || (which == 2 && !base && !pos)) return;  // (the same in the whole cluster)
-  const int* E = evict_idx + (size_t)unit * max_evict;
-  if (k <= kMaxSharedPicks) {
-    for (int i = tid; i < k; i += kStableThreads) s_picks[i] = E[i];
-    __syncthreads();
-    E = s_picks;
-  }
-  char* arr = (which == 0 ? K : V) + (size_t)unit * cap * row_bytes;
-  float* bu = base ? base + (size_t)unit * cap : nullptr;
-  int* pu = pos ? pos + (size_t)unit * cap : nullptr;
-  const int chunks = which == 2 ? 1 : row_bytes / 16;  // pieces of a row: 16 bytes, or (base, pos)
-  const int trows = which == 2 ? kStableMaxRows : min(kStableMaxRows, kStableTileBytes / row_bytes);
-  const int first = E[0], rounds = (n - first + C * trows - 1) / (C * trows);
-  auto load = [&](int r) {
-    char* t = tiles + (r & 1) * kStableTileBytes;
-    const int s0 = first + (r * C + rank) * trows, rows = min(trows, n - s0);
-    for (int i = tid; i < rows; i += kStableThreads) {
-      const int lb = lower_bound(E, k, s0 + i);
-      s_dst[r & 1][i] = (lb < k && E[lb] == s0 + i) ? -1 : s0 + i - lb;
+  if (k > 0 && (which < 2 || base || pos)) {  // (the same in the whole cluster)
+    const int* E = evict_idx + (size_t)unit * max_evict;
+    if (k <= kMaxSharedPicks) {
+      for (int i = tid; i < k; i += kStableThreads) s_picks[i] = E[i];
+      __syncthreads();
+      E = s_picks;
     }
-    if (which == 2) {
-      for (int i = tid; i < rows; i += kStableThreads)
-        reinterpret_cast<float2*>(t)[i] = make_float2(bu ? bu[s0 + i] : 0.f, pu ? __int_as_float(pu[s0 + i]) : 0.f);
-    } else {
-      const uint4* src = reinterpret_cast<const uint4*>(arr + (size_t)s0 * row_bytes);
-#pragma unroll 8
-      for (int i = tid; i < rows * chunks; i += kStableThreads) reinterpret_cast<uint4*>(t)[i] = src[i];
-    }
-  };
-  load(0);
-  for (int r = 0; r < rounds; ++r) {
-    ptx::cluster_sync_all();  // round r has been read by everyone (and this CTA is done with the other buffer)
-    if (r + 1 < rounds) load(r + 1);
-    const char* t = tiles + (r & 1) * kStableTileBytes;
-    const int s0 = first + (r * C + rank) * trows, rows = min(trows, n - s0);
-    for (int i = tid; i < rows * chunks; i += kStableThreads) {
-      const int row = i / chunks, c = i % chunks, dst = s_dst[r & 1][row];
-      if (dst < 0) continue;
+    char* arr = (which == 0 ? K : V) + (size_t)unit * cap * row_bytes;
+    float* bu = base ? base + (size_t)unit * cap : nullptr;
+    int* pu = pos ? pos + (size_t)unit * cap : nullptr;
+    const int chunks = which == 2 ? 1 : row_bytes / 16;  // pieces of a row: 16 bytes, or (base, pos)
+    const int trows = which == 2 ? kStableMaxRows : min(kStableMaxRows, kStableTileBytes / row_bytes);
+    const int first = E[0], rounds = (n - first + C * trows - 1) / (C * trows);
+    auto load = [&](int r) {
+      char* t = tiles + (r & 1) * kStableTileBytes;
+      const int s0 = first + (r * C + rank) * trows, rows = min(trows, n - s0);
+      for (int i = tid; i < rows; i += kStableThreads) {
+        const int lb = lower_bound(E, k, s0 + i);
+        s_dst[r & 1][i] = (lb < k && E[lb] == s0 + i) ? -1 : s0 + i - lb;
+      }
       if (which == 2) {
-        const float2 v = reinterpret_cast<const float2*>(t)[row];
-        if (bu) bu[dst] = v.x;
-        if (pu) pu[dst] = __float_as_int(v.y);
+        for (int i = tid; i < rows; i += kStableThreads)
+          reinterpret_cast<float2*>(t)[i] = make_float2(bu ? bu[s0 + i] : 0.f, pu ? __int_as_float(pu[s0 + i]) : 0.f);
       } else {
-        *reinterpret_cast<uint4*>(arr + (size_t)dst * row_bytes + c * 16) = reinterpret_cast<const uint4*>(t)[i];
+        const uint4* src = reinterpret_cast<const uint4*>(arr + (size_t)s0 * row_bytes);
+  #pragma unroll 8
+        for (int i = tid; i < rows * chunks; i += kStableThreads) reinterpret_cast<uint4*>(t)[i] = src[i];
+      }
+    };
+    load(0);
+    for (int r = 0; r < rounds; ++r) {
+      ptx::cluster_sync_all();  // round r has been read by everyone (and this CTA is done with the other buffer)
+      if (r + 1 < rounds) load(r + 1);
+      const char* t = tiles + (r & 1) * kStableTileBytes;
+      const int s0 = first + (r * C + rank) * trows, rows = min(trows, n - s0);
+      for (int i = tid; i < rows * chunks; i += kStableThreads) {
+        const int row = i / chunks, c = i % chunks, dst = s_dst[r & 1][row];
+        if (dst < 0) continue;
+        if (which == 2) {
+          const float2 v = reinterpret_cast<const float2*>(t)[row];
+          if (bu) bu[dst] = v.x;
+          if (pu) pu[dst] = __float_as_int(v.y);
+        } else {
+          *reinterpret_cast<uint4*>(arr + (size_t)dst * row_bytes + c * 16) = reinterpret_cast<const uint4*>(t)[i];
+        }
       }
     }
   }
-}
-
-// len[b] -= n_evict[b], after every unit of the sequence has been compacted.
-__global__ void update_len_kernel(int B, int* __restrict__ len, const int* __restrict__ n_evict) {
-  ptx::pdl_wait();
-  ptx::pdl_trigger();
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < B) len[b] -= n_evict[b];
+  finish_lengths(B, len, n_evict, ticket);
 }
 
 // Append m new rows per unit: grid = (units, ceil(m / 8)), 8 warps per CTA, one warp per row.
