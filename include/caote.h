@@ -251,8 +251,9 @@ CAOTE_API int caote_step_fast(const caote_params_t* params, const void* q, const
  *     scores[u, j] = sum_r alpha_{r,j} / (1 - alpha_{r,j}) * || o_r - v_j ||_2 ,
  * r over the last row of every group head (LAST_QUERY) or over all rows (CHUNK_SUM); other base modes
  * return CAOTE_ERR_UNSUPPORTED. With one head and one query it equals caote_score. Arguments as in
- * caote_score (no base). Runs on the any-shape fp32 CUDA-core kernels (two dot products of length d per
- * (row, token) pair): a correctness path for comparing the two aggregations, not tuned. */
+ * caote_score (no base). Single bf16 queries of up to 8 heads per KV head read the cache twice (caote_score's cluster kernel,
+ * then a pass for the errors); everything else runs on the any-shape fp32 CUDA-core kernels (two dot products of length d
+ * per (row, token) pair), not tuned. */
 CAOTE_API int caote_score_sum_errors(const caote_params_t* params, const void* q, const void* K, const void* V,
                            const int32_t* len, float* o, float* scores, void* workspace,
                            size_t workspace_bytes, caote_stream_t stream);
@@ -285,6 +286,19 @@ CAOTE_API int caote_post_evict_output_ws(const caote_params_t* params, const voi
                                const int32_t* len, const int32_t* evict_idx, int32_t max_evict,
                                const int32_t* n_evict, const float* o, float* o_post, const void* workspace,
                                size_t workspace_bytes, caote_stream_t stream);
+
+/* Whole steps of the two variants above in one call, with the results of the separate calls: caote_append (skipped when
+ * k_new is NULL), caote_score_sum_errors, caote_select_evict, caote_compact; and caote_append, caote_score,
+ * caote_select_evict, caote_post_evict_output_ws, caote_compact. */
+CAOTE_API int caote_step_sum_errors(const caote_params_t* params, const void* q, const void* k_new, const void* v_new, void* K,
+                          void* V, float* base, int32_t* pos, int32_t* len, int32_t* n_seen, const int32_t* budget,
+                          float* o, float* scores, int32_t* evict_idx, int32_t max_evict, int32_t* n_evict,
+                          int32_t compact_mode, void* workspace, size_t workspace_bytes, caote_stream_t stream);
+CAOTE_API int caote_step_post_evict(const caote_params_t* params, const void* q, const void* k_new, const void* v_new, void* K,
+                          void* V, float* base, int32_t* pos, int32_t* len, int32_t* n_seen, const int32_t* budget,
+                          float* o, float* o_post, float* scores, int32_t* evict_idx, int32_t max_evict,
+                          int32_t* n_evict, int32_t compact_mode, void* workspace, size_t workspace_bytes,
+                          caote_stream_t stream);
 
 /* Synchronise the stream, copy the status word to *status_out (host pointer) and reset it to CAOTE_OK.
  * The word holds the first device-side error since the last reset. */

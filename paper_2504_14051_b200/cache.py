@@ -72,21 +72,16 @@ class EvictionCache:
     def step(self, q, k_new, v_new, stream=None):
         """One eviction step; returns the pre-eviction attention output o [B, Hq, m, d] (method "post_evict":
         the output over the retained tokens)."""
-        if self.method in ("sum_errors", "post_evict"):
-            p, ws = self.params, self.workspace
-            C.caote_append(p, self.K, self.V, self.base, self.pos, self.lens, self.n_seen, k_new, v_new, ws, stream)
-            if self.method == "sum_errors":
-                C.caote_score_sum_errors(p, q, self.K, self.V, self.lens, self.o, self.scores, ws, stream)
-            else:
-                C.caote_score(p, q, self.K, self.V, self.lens, self.base, self.o, self.scores, ws, stream)
-            C.caote_select_evict(p, self.scores, self.lens, self.budget, self.pos, self.evict_idx, self.n_evict, ws,
-                                 stream)
-            if self.method == "post_evict":
-                C.caote_post_evict_output_ws(p, q, self.K, self.V, self.lens, self.evict_idx, self.n_evict, self.o,
-                                             self.o_post, ws, stream)
-            C.caote_compact(p, self.K, self.V, self.base, self.pos, self.lens, self.evict_idx, self.n_evict,
-                            self.compact_mode, ws, stream)
-            return self.o_post if self.method == "post_evict" else self.o
+        if self.method == "sum_errors":
+            C.caote_step_sum_errors(self.params, q, k_new, v_new, self.K, self.V, self.base, self.pos, self.lens,
+                                    self.n_seen, self.budget, self.o, self.scores, self.evict_idx, self.n_evict,
+                                    self.compact_mode, self.workspace, stream)
+            return self.o
+        if self.method == "post_evict":
+            C.caote_step_post_evict(self.params, q, k_new, v_new, self.K, self.V, self.base, self.pos, self.lens,
+                                    self.n_seen, self.budget, self.o, self.o_post, self.scores, self.evict_idx,
+                                    self.n_evict, self.compact_mode, self.workspace, stream)
+            return self.o_post
         if self.vsum is not None:
             C.caote_step_fast(self.params, q, k_new, v_new, self.K, self.V, self.base, self.pos, self.lens,
                               self.n_seen, self.budget, self.vsum, self.o, self.scores, self.evict_idx, self.n_evict,

@@ -173,10 +173,25 @@ static int check_device() {
   return st == 1 ? CAOTE_OK : CAOTE_ERR_UNSUPPORTED;
 }
 
+// Once per device, kernel and size, not at every launch.
 template <typename KernelT>
 static int allow_smem(KernelT kernel, size_t bytes) {
-  if (bytes > 48 * 1024)
-    CAOTE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  if (bytes <= 48 * 1024) return CAOTE_OK;
+  struct Done { int dev; const void* kernel; size_t bytes; };
+  static std::mutex mu;
+  static std::vector<Done> done;
+  int dev = 0;
+  CAOTE_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lk(mu);
+  for (Done& d : done)
+    if (d.dev == dev && d.kernel == (const void*)kernel) {
+      if (d.bytes >= bytes) return CAOTE_OK;
+      CAOTE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+      d.bytes = bytes;
+      return CAOTE_OK;
+    }
+  CAOTE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  done.push_back({dev, (const void*)kernel, bytes});
   return CAOTE_OK;
 }
 
@@ -1100,14 +1115,18 @@ int caote_score(const caote_params_t* p, const void* q, const void* K, const voi
   return score_impl(p, q, K, V, len, base, nullptr, o, scores, workspace, workspace_bytes_, stream);
 }
 
-int caote_score_sum_errors(const caote_params_t* p, const void* q, const void* K, const void* V, const int32_t* len,
-                           float* o, float* scores, void* workspace, size_t workspace_bytes_, caote_stream_t stream) {
+static int sum_errors_args_check(const caote_params_t* p, const void* q, const void* K, const void* V, const int32_t* len, float* o,
+                                 float* scores, void* workspace, size_t workspace_bytes_) {
   if (!params_ok(p) || !q || !K || !V || !len || !o || !scores || !workspace) return CAOTE_ERR_INVALID_ARG;
   if (!params_supported(p)) return CAOTE_ERR_UNSUPPORTED;
   if (p->base_mode != CAOTE_BASE_LAST_QUERY && p->base_mode != CAOTE_BASE_CHUNK_SUM) return CAOTE_ERR_UNSUPPORTED;
   if (workspace_bytes_ < workspace_bytes(p) || !aligned(workspace, 256)) return CAOTE_ERR_INVALID_ARG;
   if (!aligned(q, 16) || !aligned(K, 16) || !aligned(V, 16) || !aligned(o, 16)) return CAOTE_ERR_INVALID_ARG;
-  int rc = check_device();
+  return check_device();
+}
+int caote_score_sum_errors(const caote_params_t* p, const void* q, const void* K, const void* V, const int32_t* len,
+                           float* o, float* scores, void* workspace, size_t workspace_bytes_, caote_stream_t stream) {
+  int rc = sum_errors_args_check(p, q, K, V, len, o, scores, workspace, workspace_bytes_);
   if (rc) return rc;
   const Dims dm = make_dims(p);
   cudaStream_t st = (cudaStream_t)stream;
@@ -1228,6 +1247,7 @@ int caote_compact(const caote_params_t* p, void* K, void* V, float* base, int32_
   const Dims dm = make_dims(p);
   const int row_bytes = dm.D * (p->dtype == CAOTE_BF16 ? 2 : 4);
   cudaStream_t st = (cudaStream_t)stream;
+  int* ticket = reinterpret_cast<int*>(workspace) + 4;
   if (mode == CAOTE_COMPACT_FILL) {
     CAOTE_LAUNCH("compact_fill_kernel", st, launch_pdl(sel::compact_fill_kernel, dim3(dm.units), dim3(dm.m > 16 ? sel::kSelThreads : 256), 0, st, dm.Hkv, dm.cap, row_bytes, (char*)K, (char*)V, base, pos,
                                                        len, evict_idx, max_evict, n_evict, dm.B, ticket));
@@ -1246,17 +1266,53 @@ int caote_compact(const caote_params_t* p, void* K, void* V, float* base, int32_
 }
 
 // caote_step (vsum == NULL) and caote_step_fast (vsum kept current: += appended rows, -= evicted rows).
+static int evict_args_check(const int32_t* budget, const int32_t* evict_idx, int32_t max_evict, const int32_t* n_evict, int32_t mode) {
+  if (!budget || !evict_idx || !n_evict || max_evict < 1) return CAOTE_ERR_INVALID_ARG;
+  return mode == CAOTE_COMPACT_FILL || mode == CAOTE_COMPACT_STABLE ? CAOTE_OK : CAOTE_ERR_INVALID_ARG;
+}
+// The last part of a step whose arguments have been checked: selection and compaction (and FastCAOTE's sums).
+static int select_and_compact(const caote_params_t* p, const float* scores, void* K, void* V, float* base, int32_t* pos, int32_t* len,
+                              const int32_t* budget, float* vsum, int32_t* evict_idx, int32_t max_evict, int32_t* n_evict,
+                              int32_t compact_mode, void* workspace, size_t workspace_bytes_, caote_stream_t stream) {
+  const bool bf16 = p->dtype == CAOTE_BF16;
+  if (compact_mode == CAOTE_COMPACT_FILL) {
+    // selection, compaction and the length update in one launch (same results as the two calls below)
+    const Dims dm = make_dims(p);
+    const int row_bytes = dm.D * (p->dtype == CAOTE_BF16 ? 2 : 4);
+    cudaStream_t st = (cudaStream_t)stream;
+    int* hdr = reinterpret_cast<int*>(workspace);
+    CAOTE_LAUNCH("select_compact_kernel", st,
+                 launch_pdl(sel::select_compact_kernel, dim3(dm.units), dim3(sel::kSelThreads), 0, st, 
+                     dm.B, dm.Hkv, dm.cap, row_bytes, scores, (char*)K, (char*)V, base, pos, len, budget, evict_idx,
+                     max_evict, n_evict, hdr, hdr + 4, vsum, bf16 ? 2 : 4));
+    return CAOTE_OK;
+  }
+  int rc = caote_select_evict(p, scores, len, budget, pos, evict_idx, max_evict, n_evict, workspace,
+                          workspace_bytes_, stream);
+  if (rc) return rc;
+  if (vsum) {
+    const Dims dm = make_dims(p);
+    cudaStream_t st = (cudaStream_t)stream;
+    if (bf16) {
+      CAOTE_LAUNCH("fast_vsum_sub_kernel", st, launch_pdl(fast::vsum_sub_kernel<__nv_bfloat16>, dim3(dm.units), dim3(128), 0, st,
+          dm.Hkv, dm.cap, dm.D, (const __nv_bfloat16*)V, evict_idx, max_evict, n_evict, vsum));
+    } else {
+      CAOTE_LAUNCH("fast_vsum_sub_kernel", st, launch_pdl(fast::vsum_sub_kernel<float>, dim3(dm.units), dim3(128), 0, st,
+          dm.Hkv, dm.cap, dm.D, (const float*)V, evict_idx, max_evict, n_evict, vsum));
+    }
+  }
+  return caote_compact(p, K, V, base, pos, len, evict_idx, max_evict, n_evict, compact_mode, workspace,
+                       workspace_bytes_, stream);
+}
 static int step_impl(const caote_params_t* p, const void* q, const void* k_new, const void* v_new, void* K, void* V,
                      float* base, int32_t* pos, int32_t* len, int32_t* n_seen, const int32_t* budget, float* vsum,
                      float* o, float* scores, int32_t* evict_idx, int32_t max_evict, int32_t* n_evict,
-  int* ticket = reinterpret_cast<int*>(workspace) + 4;
                      int32_t compact_mode, void* workspace, size_t workspace_bytes_, caote_stream_t stream) {
   // every host-visible check of the calls below runs before the first launch
   int rc = score_args_check(p, q, K, V, len, base, o, scores);
   if (!rc) rc = score_workspace_check(p, workspace, workspace_bytes_);
   if (!rc && (k_new || v_new)) rc = append_args_check(p, K, V, len, k_new, v_new, workspace, workspace_bytes_);
-  if (!rc && (!budget || !evict_idx || !n_evict || max_evict < 1)) rc = CAOTE_ERR_INVALID_ARG;
-  if (!rc && compact_mode != CAOTE_COMPACT_FILL && compact_mode != CAOTE_COMPACT_STABLE) rc = CAOTE_ERR_INVALID_ARG;
+  if (!rc) rc = evict_args_check(budget, evict_idx, max_evict, n_evict, compact_mode);
   if (!rc) rc = check_device();
   if (rc) return rc;
   const bool bf16 = p->dtype == CAOTE_BF16;
@@ -1307,35 +1363,8 @@ static int step_impl(const caote_params_t* p, const void* q, const void* k_new, 
   }
   rc = score_impl(p, q, K, V, len, base, vsum, o, scores, workspace, workspace_bytes_, stream);
   if (rc) return rc;
-  if (compact_mode == CAOTE_COMPACT_FILL) {
-    // selection, compaction and the length update in one launch (same results as the two calls below)
-    if (!budget || !evict_idx || !n_evict || max_evict < 1) return CAOTE_ERR_INVALID_ARG;
-    const Dims dm = make_dims(p);
-    const int row_bytes = dm.D * (p->dtype == CAOTE_BF16 ? 2 : 4);
-    cudaStream_t st = (cudaStream_t)stream;
-    int* hdr = reinterpret_cast<int*>(workspace);
-    CAOTE_LAUNCH("select_compact_kernel", st,
-                 launch_pdl(sel::select_compact_kernel, dim3(dm.units), dim3(sel::kSelThreads), 0, st, 
-                     dm.B, dm.Hkv, dm.cap, row_bytes, scores, (char*)K, (char*)V, base, pos, len, budget, evict_idx,
-                     max_evict, n_evict, hdr, hdr + 4, vsum, bf16 ? 2 : 4));
-    return CAOTE_OK;
-  }
-  rc = caote_select_evict(p, scores, len, budget, pos, evict_idx, max_evict, n_evict, workspace,
-                          workspace_bytes_, stream);
-  if (rc) return rc;
-  if (vsum) {
-    const Dims dm = make_dims(p);
-    cudaStream_t st = (cudaStream_t)stream;
-    if (bf16) {
-      CAOTE_LAUNCH("fast_vsum_sub_kernel", st, launch_pdl(fast::vsum_sub_kernel<__nv_bfloat16>, dim3(dm.units), dim3(128), 0, st,
-          dm.Hkv, dm.cap, dm.D, (const __nv_bfloat16*)V, evict_idx, max_evict, n_evict, vsum));
-    } else {
-      CAOTE_LAUNCH("fast_vsum_sub_kernel", st, launch_pdl(fast::vsum_sub_kernel<float>, dim3(dm.units), dim3(128), 0, st,
-          dm.Hkv, dm.cap, dm.D, (const float*)V, evict_idx, max_evict, n_evict, vsum));
-    }
-  }
-  return caote_compact(p, K, V, base, pos, len, evict_idx, max_evict, n_evict, compact_mode, workspace,
-                       workspace_bytes_, stream);
+  return select_and_compact(p, scores, K, V, base, pos, len, budget, vsum, evict_idx, max_evict, n_evict, compact_mode, workspace,
+                            workspace_bytes_, stream);
 }
 
 int caote_step(const caote_params_t* p, const void* q, const void* k_new, const void* v_new, void* K, void* V,
@@ -1353,6 +1382,41 @@ int caote_step_fast(const caote_params_t* p, const void* q, const void* k_new, c
   if (!vsum || !aligned(vsum, 16)) return CAOTE_ERR_INVALID_ARG;
   return step_impl(p, q, k_new, v_new, K, V, base, pos, len, n_seen, budget, vsum, o, scores, evict_idx, max_evict,
                    n_evict, compact_mode, workspace, workspace_bytes_, stream);
+}
+
+int caote_step_sum_errors(const caote_params_t* p, const void* q, const void* k_new, const void* v_new, void* K, void* V,
+                          float* base, int32_t* pos, int32_t* len, int32_t* n_seen, const int32_t* budget, float* o,
+                          float* scores, int32_t* evict_idx, int32_t max_evict, int32_t* n_evict, int32_t compact_mode,
+                          void* workspace, size_t workspace_bytes_, caote_stream_t stream) {
+  int rc = sum_errors_args_check(p, q, K, V, len, o, scores, workspace, workspace_bytes_);
+  if (!rc && (k_new || v_new)) rc = append_args_check(p, K, V, len, k_new, v_new, workspace, workspace_bytes_);
+  if (!rc) rc = evict_args_check(budget, evict_idx, max_evict, n_evict, compact_mode);
+  if (!rc && (k_new || v_new))
+    rc = append_impl(p, K, V, base, pos, len, n_seen, k_new, v_new, workspace, workspace_bytes_, stream, nullptr);
+  if (!rc) rc = caote_score_sum_errors(p, q, K, V, len, o, scores, workspace, workspace_bytes_, stream);
+  if (rc) return rc;
+  return select_and_compact(p, scores, K, V, base, pos, len, budget, nullptr, evict_idx, max_evict, n_evict, compact_mode, workspace,
+                            workspace_bytes_, stream);
+}
+
+int caote_step_post_evict(const caote_params_t* p, const void* q, const void* k_new, const void* v_new, void* K, void* V,
+                          float* base, int32_t* pos, int32_t* len, int32_t* n_seen, const int32_t* budget, float* o,
+                          float* o_post, float* scores, int32_t* evict_idx, int32_t max_evict, int32_t* n_evict,
+                          int32_t compact_mode, void* workspace, size_t workspace_bytes_, caote_stream_t stream) {
+  int rc = score_args_check(p, q, K, V, len, base, o, scores);
+  if (!rc) rc = score_workspace_check(p, workspace, workspace_bytes_);
+  if (!rc && (k_new || v_new)) rc = append_args_check(p, K, V, len, k_new, v_new, workspace, workspace_bytes_);
+  if (!rc) rc = evict_args_check(budget, evict_idx, max_evict, n_evict, compact_mode);
+  if (!rc && (!o_post || !aligned(o_post, 16))) rc = CAOTE_ERR_INVALID_ARG;
+  if (!rc) rc = check_device();
+  if (!rc && (k_new || v_new))
+    rc = append_impl(p, K, V, base, pos, len, n_seen, k_new, v_new, workspace, workspace_bytes_, stream, nullptr);
+  if (!rc) rc = score_impl(p, q, K, V, len, base, nullptr, o, scores, workspace, workspace_bytes_, stream);
+  if (!rc) rc = caote_select_evict(p, scores, len, budget, pos, evict_idx, max_evict, n_evict, workspace, workspace_bytes_, stream);
+  if (!rc)
+    rc = caote_post_evict_output_ws(p, q, K, V, len, evict_idx, max_evict, n_evict, o, o_post, workspace, workspace_bytes_, stream);
+  if (rc) return rc;
+  return caote_compact(p, K, V, base, pos, len, evict_idx, max_evict, n_evict, compact_mode, workspace, workspace_bytes_, stream);
 }
 
 static int post_evict_impl(const caote_params_t* p, const void* q, const void* K, const void* V, const int32_t* len,

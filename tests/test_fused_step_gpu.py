@@ -174,3 +174,46 @@ def test_whole_step_kernel_equals_the_four_calls(shape, mode, fast):
             P.caote_vsum(p, a.V, a.lens, ref.vsum)
             # a handful of fp32 additions on sums of up to 2 k normal values (about 45): 1e-5 each
             torch.testing.assert_close(a.vsum, ref.vsum, rtol=1e-5, atol=1e-3)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [
+    # B, Hq, Hkv, d, cap, m, budget, dtype
+    (3, 14, 2, 128, 400, 1, 390, torch.bfloat16),
+    (2, 8, 2, 64, 272, 40, 200, torch.bfloat16),
+    (2, 4, 2, 64, 100, 3, 90, torch.float32),
+])
+@pytest.mark.parametrize("compact", ["fill", "stable"])
+@pytest.mark.parametrize("method", ["sum_errors", "post_evict"])
+def test_variant_steps_equal_their_separate_calls(shape, compact, method):
+    """The whole steps of the two variants launch the kernels of the separate calls (one fused selection aside): the same
+    bits everywhere."""
+    B, Hq, Hkv, d, cap, m, budget, dt = shape
+    g = torch.Generator(device="cpu").manual_seed(cap)
+    a, b = (P.EvictionCache(B, Hq, Hkv, d, cap, m, dt, budget, "last_query", compact, method=method, device=DEV) for _ in range(2))
+    K0, V0 = (torch.randn((B, Hkv, cap, d), generator=g).to(dt) for _ in range(2))
+    for c in (a, b):
+        c.load(K0, V0, torch.tensor([budget - 5 * s for s in range(B)], dtype=torch.int32))
+    p = a.params
+    for _ in range(7):
+        q = torch.randn((B, Hq, m, d), generator=g).to(dt).to(DEV)
+        kn, vn = (torch.randn((B, Hkv, m, d), generator=g).to(dt).to(DEV) for _ in range(2))
+        a.step(q, kn, vn)
+        P.caote_append(p, b.K, b.V, b.base, b.pos, b.lens, b.n_seen, kn, vn, b.workspace)
+        if method == "sum_errors":
+            P.caote_score_sum_errors(p, q, b.K, b.V, b.lens, b.o, b.scores, b.workspace)
+        else:
+            P.caote_score(p, q, b.K, b.V, b.lens, b.base, b.o, b.scores, b.workspace)
+        P.caote_select_evict(p, b.scores, b.lens, b.budget, b.pos, b.evict_idx, b.n_evict, b.workspace)
+        if method == "post_evict":
+            P.caote_post_evict_output_ws(p, q, b.K, b.V, b.lens, b.evict_idx, b.n_evict, b.o, b.o_post, b.workspace)
+        P.caote_compact(p, b.K, b.V, b.base, b.pos, b.lens, b.evict_idx, b.n_evict, compact, b.workspace)
+        torch.cuda.synchronize()
+        assert a.status() == 0 and b.status() == 0
+        for x in ("lens", "n_evict", "n_seen", "o") + (("o_post",) if method == "post_evict" else ()):
+            assert torch.equal(getattr(a, x), getattr(b, x)), x
+        for s in range(B):
+            n = int(a.lens[s])
+            assert n <= budget
+            for x in ("K", "V", "pos", "scores"):
+                assert torch.equal(getattr(a, x)[s, :, :n], getattr(b, x)[s, :, :n]), x
