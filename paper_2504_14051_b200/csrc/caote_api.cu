@@ -404,19 +404,21 @@ static int choose_cluster(const Dims& dm, ClusterKernel kernel, int* clusters_ou
 }
 
 static int encode_decode_maps(const Dims& dm, const void* q, const void* K, const void* V, unsigned q_rows,
-                              CUtensorMap* tmK, CUtensorMap* tmV, CUtensorMap* tmQ, TensorMapEncodeFn encode) {
+                              CUtensorMap* tmK, CUtensorMap* tmV, CUtensorMap* tmQ, TensorMapEncodeFn encode,
+                              int tokens = decode::kT, int channels = 64) {
   const cuuint64_t gdim[2] = {(cuuint64_t)dm.D, (cuuint64_t)dm.units * (cuuint64_t)dm.cap};
   const cuuint64_t gstride[1] = {(cuuint64_t)dm.D * 2};
-  const cuuint32_t box[2] = {64, (cuuint32_t)decode::kT};
+  const cuuint32_t box[2] = {(cuuint32_t)channels, (cuuint32_t)tokens};
   const cuuint32_t estride[2] = {1, 1};
   for (int i = 0; i < 3; ++i) {
-    // K, V: boxes of 64 channels x 128 tokens; q: 64 channels x q_rows rows (a unit's heads, padded by its
-    // neighbours' or by zeros)
+    // K, V: boxes of `channels` channels x `tokens` tokens, swizzled over the length of their rows; q: 64 channels x q_rows
+    // rows (a unit's heads, padded by its neighbours' or by zeros)
     const cuuint64_t qdim[2] = {(cuuint64_t)dm.D, (cuuint64_t)dm.B * (cuuint64_t)dm.Hq};
     const cuuint32_t qbox[2] = {64, q_rows};
     CUresult r = encode(i == 0 ? tmK : (i == 1 ? tmV : tmQ), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
                         const_cast<void*>(i == 0 ? K : (i == 1 ? V : q)), i < 2 ? gdim : qdim, gstride, i < 2 ? box : qbox,
-                        estride, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                        estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        i < 2 && channels == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
       snprintf(g_cuda_error, sizeof(g_cuda_error), "cuTensorMapEncodeTiled failed with CUresult %d", (int)r);
@@ -639,34 +641,34 @@ static int side_stream(SideStream* out) {
 }
 
 // The sum-of-errors pass that follows the cluster kernel on single-query shapes.
-template <int G>
-static int launch_sum_errors_decode_g(const Dims& dm, const CUtensorMap& tmK, const CUtensorMap& tmV, const void* q,
-                                      const int* len, const float* o, float* scores, char* ws, cudaStream_t st) {
-  int rc = allow_smem(sed::sum_errors_decode_kernel<G>, sed::smem_bytes());
+template <int G, int D>
+static int launch_sum_errors_decode_gd(const Dims& dm, const void* q, const void* K, const void* V, const int* len, const float* o,
+                                       float* scores, char* ws, cudaStream_t st) {
+  TensorMapEncodeFn encode = tensor_map_encoder();
+  if (!encode) return CAOTE_ERR_CUDA;  // (the cluster kernel before it was launched with the same encoder)
+  CUtensorMap tmK, tmV, tmQ;
+  int rc = encode_decode_maps(dm, q, K, V, 8, &tmK, &tmV, &tmQ, encode, sed::Tile<G>::kT, sed::Tile<G>::kBoxCh);
+  if (!rc) rc = allow_smem(sed::sum_errors_decode_kernel<G, D>, (sed::smem_bytes_of<G, D>));
   if (rc) return rc;
-  dim3 grid((dm.cap + sed::kT - 1) / sed::kT, dm.units);
+  dim3 grid(sed::splits(dm.units, dm.cap, sed::Tile<G>::kT, sed::Tile<G>::kCtasPerSm), dm.units);
   CAOTE_LAUNCH("sum_errors_decode_kernel", st,
-               launch_pdl(sed::sum_errors_decode_kernel<G>, grid, dim3(sed::kThreads), sed::smem_bytes(), st, tmK, tmV, dm,
+               launch_pdl(sed::sum_errors_decode_kernel<G, D>, grid, dim3(sed::kThreads), (sed::smem_bytes_of<G, D>), st, tmK, tmV, dm,
                           (const __nv_bfloat16*)q, len, o, reinterpret_cast<const float*>(ws + kHeaderBytes), scores,
                           reinterpret_cast<int*>(ws)));
   return CAOTE_OK;
 }
+template <int D>
 static int launch_sum_errors_decode(const Dims& dm, const void* q, const void* K, const void* V, const int* len,
                                     const float* o, float* scores, char* ws, cudaStream_t st) {
-  TensorMapEncodeFn encode = tensor_map_encoder();
-  if (!encode) return CAOTE_ERR_CUDA;  // (the cluster kernel before it was launched with the same encoder)
-  CUtensorMap tmK, tmV, tmQ;
-  int rc = encode_decode_maps(dm, q, K, V, 8, &tmK, &tmV, &tmQ, encode);
-  if (rc) return rc;
   switch (dm.G) {
-    case 1: return launch_sum_errors_decode_g<1>(dm, tmK, tmV, q, len, o, scores, ws, st);
-    case 2: return launch_sum_errors_decode_g<2>(dm, tmK, tmV, q, len, o, scores, ws, st);
-    case 3: return launch_sum_errors_decode_g<3>(dm, tmK, tmV, q, len, o, scores, ws, st);
-    case 4: return launch_sum_errors_decode_g<4>(dm, tmK, tmV, q, len, o, scores, ws, st);
-    case 5: return launch_sum_errors_decode_g<5>(dm, tmK, tmV, q, len, o, scores, ws, st);
-    case 6: return launch_sum_errors_decode_g<6>(dm, tmK, tmV, q, len, o, scores, ws, st);
-    case 7: return launch_sum_errors_decode_g<7>(dm, tmK, tmV, q, len, o, scores, ws, st);
-    case 8: return launch_sum_errors_decode_g<8>(dm, tmK, tmV, q, len, o, scores, ws, st);
+    case 1: return launch_sum_errors_decode_gd<1, D>(dm, q, K, V, len, o, scores, ws, st);
+    case 2: return launch_sum_errors_decode_gd<2, D>(dm, q, K, V, len, o, scores, ws, st);
+    case 3: return launch_sum_errors_decode_gd<3, D>(dm, q, K, V, len, o, scores, ws, st);
+    case 4: return launch_sum_errors_decode_gd<4, D>(dm, q, K, V, len, o, scores, ws, st);
+    case 5: return launch_sum_errors_decode_gd<5, D>(dm, q, K, V, len, o, scores, ws, st);
+    case 6: return launch_sum_errors_decode_gd<6, D>(dm, q, K, V, len, o, scores, ws, st);
+    case 7: return launch_sum_errors_decode_gd<7, D>(dm, q, K, V, len, o, scores, ws, st);
+    case 8: return launch_sum_errors_decode_gd<8, D>(dm, q, K, V, len, o, scores, ws, st);
     default: return CAOTE_ERR_UNSUPPORTED;
   }
 }
@@ -1131,12 +1133,13 @@ int caote_score_sum_errors(const caote_params_t* p, const void* q, const void* K
   const Dims dm = make_dims(p);
   cudaStream_t st = (cudaStream_t)stream;
   char* ws = (char*)workspace;
-  if (decode_shape_ok(p)) {
+  if (cluster_shape_ok(p)) {
     // one query per head: the cluster kernel for o and the heads' statistics, then one more pass over K and V
     bool used = false;
     rc = launch_decode_cluster(dm, q, K, V, len, nullptr, o, scores, ws, st, &used);
     if (rc) return rc;
-    if (used) return launch_sum_errors_decode(dm, q, K, V, len, o, scores, ws, st);
+    if (used) return dm.D == 128 ? launch_sum_errors_decode<128>(dm, q, K, V, len, o, scores, ws, st)
+                                 : launch_sum_errors_decode<64>(dm, q, K, V, len, o, scores, ws, st);
   }
   if (p->dtype == CAOTE_BF16) {
     if (dm.D == 128) return launch_generic_score<__nv_bfloat16, 128>(dm, q, K, V, len, nullptr, o, scores, ws, st, nullptr, true);

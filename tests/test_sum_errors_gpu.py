@@ -24,6 +24,10 @@ CASES = [
     (2, 28, 4, 128, 1300, 1, [1290, 515], torch.bfloat16, "last_query"),   # 7 heads per group, ragged tiles
     (1, 64, 8, 128, 2100, 1, [2049], torch.bfloat16, "chunk_sum"),         # 8 heads per group, one token in the last tile
     (3, 2, 2, 128, 144, 1, [1, 0, 129], torch.bfloat16, "last_query"),     # a single cached token; an empty sequence
+    (3, 16, 2, 64, 1300, 1, [1290, 65, 64], torch.bfloat16, "last_query"),    # heads of 64 channels; edges of the 64-token tiles
+    (40, 8, 8, 64, 1104, 1, [1100 - 27 * b for b in range(40)], torch.bfloat16, "last_query"),  # several rounds of tiles per CTA
+    (40, 24, 8, 128, 528, 1, [1 + 13 * b for b in range(40)], torch.bfloat16, "chunk_sum"),
+    (2, 4, 2, 64, 704, 1, [700, 33], torch.bfloat16, "last_query"),           # two heads per group: the large tiles
 ]
 
 
