@@ -202,16 +202,21 @@ static int launch_generic_score(const Dims& dm, const void* q, const void* K, co
   generic::Scratch sc;
   generic::carve(dm, ws + kHeaderBytes, &sc);
   int* status = reinterpret_cast<int*>(ws);
-  const int row_tiles = (dm.R + generic::kRT - 1) / generic::kRT;
-  {
-    const size_t smem = generic::partial_smem(D);
-    int rc = allow_smem(generic::attn_partial_kernel<T, D>, smem);
+  auto attention = [&](auto rpt) {
+    constexpr int RPT = decltype(rpt)::value;
+    const size_t smem = generic::partial_smem(D, RPT);
+    int rc = allow_smem(generic::attn_partial_kernel<T, D, RPT>, smem);
     if (rc) return rc;
-    dim3 grid(row_tiles, sc.splits, dm.units);
+    dim3 grid((dm.R + generic::kRT * RPT - 1) / (generic::kRT * RPT), sc.splits, dm.units);
     CAOTE_LAUNCH("attn_partial_kernel", st,
-                 launch_pdl(generic::attn_partial_kernel<T, D>, grid, dim3(generic::kThreads), smem, st, dm, (const T*)q, (const T*)K,
-                            (const T*)V, len, (const float*)base, sc, status));
-  }
+                 launch_pdl(generic::attn_partial_kernel<T, D, RPT>, grid, dim3(generic::kThreads), smem, st, dm, (const T*)q,
+                            (const T*)K, (const T*)V, len, (const float*)base, sc, status));
+    return (int)CAOTE_OK;
+  };
+  const std::integral_constant<int, 1> one;
+  const std::integral_constant<int, generic::kManyRows> many;
+  int rc = generic::rows_per_thread(dm.R) == 1 ? attention(one) : attention(many);
+  if (rc) return rc;
   {
     dim3 grid(sc.chunks, dm.units);
     CAOTE_LAUNCH("attn_combine_kernel", st, launch_pdl(generic::attn_combine_kernel<T, D>, grid, dim3(generic::kCombineThreads), 0, st, dm, len, sc, o));
@@ -226,16 +231,19 @@ static int launch_generic_score(const Dims& dm, const void* q, const void* K, co
                             (const T*)V, len, (const float*)o, sc, scores));
     return CAOTE_OK;
   }
-  {
-    const size_t smem = generic::score_smem(D);
-    int rc = allow_smem(generic::score_pass_kernel<T, D>, smem);
+  auto scoring = [&](auto rpt) {
+    constexpr int RPT = decltype(rpt)::value;
+    const size_t smem = generic::score_smem(D, RPT);
+    int rc = allow_smem(generic::score_pass_kernel<T, D, RPT>, smem);
     if (rc) return rc;
     dim3 grid((dm.cap + generic::kKT - 1) / generic::kKT, dm.units);
     CAOTE_LAUNCH("score_pass_kernel", st,
-                 launch_pdl(generic::score_pass_kernel<T, D>, grid, dim3(generic::kThreads), smem, st, dm, (const T*)q, (const T*)K,
-                            (const T*)V, len, base, sc, scores, vsum));
-  }
-  return CAOTE_OK;
+                 launch_pdl(generic::score_pass_kernel<T, D, RPT>, grid, dim3(generic::kThreads), smem, st, dm, (const T*)q,
+                            (const T*)K, (const T*)V, len, base, sc, scores, vsum));
+    return (int)CAOTE_OK;
+  };
+  const bool all_rows = dm.base_mode == CAOTE_BASE_CHUNK_SUM || dm.base_mode == CAOTE_BASE_ACCUM;
+  return generic::rows_per_thread(all_rows ? dm.R : dm.G) == 1 ? scoring(one) : scoring(many);
 }
 
 // The whole decode step of a short unit on the CUDA cores (small_step.cuh), for single queries that the tensor-core cluster

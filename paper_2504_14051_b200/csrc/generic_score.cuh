@@ -1,7 +1,7 @@
 // Generic scoring path: any I/O dtype (bf16 / fp32), head_dim 64 or 128, any block size m, any group
 // size up to 16. Plain fp32 CUDA-core arithmetic, three launches:
 //
-//   attn_partial  split-KV flash attention over tiles of 16 query rows x 64 keys: per (unit, split,
+//   attn_partial  split-KV flash attention over tiles of 16 or 64 query rows x 64 keys: per (unit, split,
 //                 row) running max, running sum and un-normalised partial output; row tile 0 also
 //                 accumulates sum_j base_j v_j and sum_j base_j for the base modes that carry scores.
 //   attn_combine  merges the splits: final (max, 1/sum) per row, attention output o, and per 32-row
@@ -43,10 +43,17 @@ struct Scratch {
 
 inline int round_up(int x, int a) { return (x + a - 1) / a * a; }
 
+// Query rows per thread (x 16 = rows of a tile). What bounds the tiles is what shared memory delivers to registers; a thread
+// with four rows uses every K and V value four times. fp32 steps, head_dim 128, 2 048 tokens, us with one row and with four:
+// 16 units of 896 rows 2001, 969; 4 units of 896 rows 991, 355; 32 units of 64 rows 344, 218; 8 units of 45 rows 134, 116;
+// but 8 units of 32 rows 92, 98: half of the tile is empty and there are fewer tiles for the SMs.
+constexpr int kManyRows = 4;
+inline int rows_per_thread(int rows) { return rows >= 40 ? kManyRows : 1; }
+
 // Number of key splits: enough CTAs to fill the machine a few times over, never more splits than
 // there are key tiles in the cache (a tile is a chain of its own latency: 256 tokens, 2 units: 9 us in spans of two, 5 in one).
 inline int choose_splits(const Dims& dm) {
-  const int row_tiles = (dm.R + kRT - 1) / kRT;
+  const int rows = kRT * rows_per_thread(dm.R), row_tiles = (dm.R + rows - 1) / rows;
   const long ctas = (long)dm.units * row_tiles;
   int s = (int)(((long)g_sm_count * 4 + ctas - 1) / ctas);
   const int max_by_cap = (dm.cap + kKT - 1) / kKT;
@@ -80,25 +87,33 @@ inline size_t carve(const Dims& dm, char* base, Scratch* out) {
   return off;
 }
 
-// scale * <q, k> over D channels, in one fixed order, from fp32 rows in shared memory, for four keys 16 rows apart (the
-// query row is fetched once for all of them). All passes call this, so a logit has the same bits in all of them.
-template <int D, int LD>
-__device__ __forceinline__ void logit4(const float* __restrict__ qrow, const float* __restrict__ krow, float scale, float (&s)[4]) {
-  s[0] = s[1] = s[2] = s[3] = 0.f;
-#pragma unroll 8
+// scale * <q, k> over D channels, in one fixed order, from fp32 rows in shared memory, for RPT queries and four keys 16 rows
+// apart (a row is fetched once for all of them). All passes call this, so a logit has the same bits in all of them.
+template <int D, int LD, int RPT>
+__device__ __forceinline__ void logits(const float* __restrict__ qrow, const float* __restrict__ krow, float scale, float (&s)[RPT][4]) {
+#pragma unroll
+  for (int u = 0; u < RPT; ++u) s[u][0] = s[u][1] = s[u][2] = s[u][3] = 0.f;
+#pragma unroll(RPT == 1 ? 8 : 4)
   for (int c = 0; c < D; c += 4) {
-    const float4 a = *reinterpret_cast<const float4*>(qrow + c);
+    float4 a[RPT];
+#pragma unroll
+    for (int u = 0; u < RPT; ++u) a[u] = *reinterpret_cast<const float4*>(qrow + u * 16 * LD + c);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const float4 b = *reinterpret_cast<const float4*>(krow + i * 16 * LD + c);
-      s[i] = fmaf(a.x, b.x, s[i]);
-      s[i] = fmaf(a.y, b.y, s[i]);
-      s[i] = fmaf(a.z, b.z, s[i]);
-      s[i] = fmaf(a.w, b.w, s[i]);
+#pragma unroll
+      for (int u = 0; u < RPT; ++u) {
+        s[u][i] = fmaf(a[u].x, b.x, s[u][i]);
+        s[u][i] = fmaf(a[u].y, b.y, s[u][i]);
+        s[u][i] = fmaf(a[u].z, b.z, s[u][i]);
+        s[u][i] = fmaf(a[u].w, b.w, s[u][i]);
+      }
     }
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) s[i] *= scale;
+  for (int u = 0; u < RPT; ++u)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[u][i] *= scale;
 }
 
 // Stage `rows` rows of D elements (global, dtype T) into shared memory as fp32 with row stride LD;
@@ -120,20 +135,25 @@ __device__ __forceinline__ size_t q_offset(const Dims& dm, int b, int h, int r) 
   return (((size_t)b * dm.Hq + h * dm.G + g) * dm.m + i) * dm.D;
 }
 
-template <typename T, int D>
-__global__ void __launch_bounds__(kThreads)
+// Floats per key of the table of numerators (many rows: a thread's rows side by side, 16-byte columns on different banks).
+__host__ __device__ constexpr int p_pitch(int rpt) { return rpt == 1 ? kRT : kRT * rpt + 4; }
+
+// Thread (r = tid / 16, c0 = tid % 16) has rows r + 16 u of the tile, keys c0 + 16 i, channels 4 c0 + 64 x.
+template <typename T, int D, int RPT>
+__global__ void __launch_bounds__(kThreads, RPT == 1 ? 0 : 2)
 attn_partial_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, const T* __restrict__ V,
                     const int* __restrict__ len, const float* __restrict__ base, Scratch sc, int* status) {
   constexpr int LD = D + 4;
   constexpr int OC = D / 16;  // output channels per thread (two float4 for D = 128, one for D = 64)
+  constexpr int kR = kRT * RPT, kPitch = p_pitch(RPT);
   ptx::pdl_wait();
   ptx::pdl_trigger();
   extern __shared__ __align__(16) float smem[];
   float* Qs = smem;
-  float* Ks = Qs + kRT * LD;
-  float* Vs = Ks + kKT * LD;
-  float* Ps = Vs + kKT * LD;
-  float* bs = Ps + kRT * kKT;   // kKT base values
+  float* Ks = Qs + kR * LD;
+  float* Vs = RPT == 1 ? Ks + kKT * LD : Ks;  // (many rows: V takes the place of K, so that two CTAs fit an SM)
+  float* Ps = Vs + kKT * LD;                  // one row per thread: [row][key]; many: [key][kPitch], r * RPT + u in it
+  float* bs = Ps + kKT * kPitch;              // kKT base values
   float* red = bs + kKT;        // kThreads floats
 
   const int unit = blockIdx.z, split = blockIdx.y, rt = blockIdx.x;
@@ -147,15 +167,18 @@ attn_partial_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, c
   }
   const bool use_base = (dm.base_mode == CAOTE_BASE_ACCUM || dm.base_mode == CAOTE_BASE_EXTERNAL) && rt == 0;
   const int tid = threadIdx.x, r = tid >> 4, c0 = tid & 15;
-  const int r_glob = rt * kRT + r;
-  const bool row_ok = r_glob < dm.R;
-  const int n_vis = row_ok ? n - dm.m + (r_glob % dm.m) + 1 : 0;
+  int n_vis[RPT];
+#pragma unroll
+  for (int u = 0; u < RPT; ++u) {
+    const int row = rt * kR + r + 16 * u;
+    n_vis[u] = row < dm.R ? n - dm.m + (row % dm.m) + 1 : 0;
+  }
 
   // stage the query tile
-  for (int idx = tid; idx < kRT * (D / 4); idx += kThreads) {
+  for (int idx = tid; idx < kR * (D / 4); idx += kThreads) {
     const int rr = idx / (D / 4), c4 = idx % (D / 4);
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (rt * kRT + rr < dm.R) v = load4(q + q_offset(dm, b, h, rt * kRT + rr) + c4 * 4);
+    if (rt * kR + rr < dm.R) v = load4(q + q_offset(dm, b, h, rt * kR + rr) + c4 * 4);
     *reinterpret_cast<float4*>(Qs + rr * LD + c4 * 4) = v;
   }
 
@@ -167,69 +190,94 @@ attn_partial_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, c
 
   // l_rest: sum of exp(s - m_run) over the keys so far EXCEPT the first key that sits at the maximum (whose
   // term is exactly 1): the row's 1 - alpha of its top key is then l_rest / (l_rest + 1), a sum of the others
-  float m_run = -INFINITY, l_rest = 0.f;
-  float o_acc[OC];
+  float m_run[RPT], l_rest[RPT], o_acc[RPT][OC];
 #pragma unroll
-  for (int i = 0; i < OC; ++i) o_acc[i] = 0.f;
+  for (int u = 0; u < RPT; ++u) {
+    m_run[u] = -INFINITY;
+    l_rest[u] = 0.f;
+#pragma unroll
+    for (int i = 0; i < OC; ++i) o_acc[u][i] = 0.f;
+  }
   float y_acc = 0.f, hb_acc = 0.f;
   constexpr int YP = kThreads / D;  // threads per channel in the base-weighted value sum
 
   for (int kt = k_begin; kt < k_end; kt += kKT) {
     __syncthreads();
     stage_rows<T, D, LD>(Ks, Ku + (size_t)kt * D, kKT, k_end - kt);
-    stage_rows<T, D, LD>(Vs, Vu + (size_t)kt * D, kKT, k_end - kt);
+    if (RPT == 1) stage_rows<T, D, LD>(Vs, Vu + (size_t)kt * D, kKT, k_end - kt);
     if (use_base && tid < kKT) bs[tid] = (kt + tid < k_end) ? base[(size_t)unit * dm.cap + kt + tid] : 0.f;
     __syncthreads();
 
-    float s[4];
-    logit4<D, LD>(Qs + r * LD, Ks + c0 * LD, dm.scale, s);  // (rows beyond the length are staged as zeros)
-    float mx = -INFINITY;
+    float s[RPT][4];
+    logits<D, LD, RPT>(Qs + r * LD, Ks + c0 * LD, dm.scale, s);  // (rows beyond the length are staged as zeros)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int j = kt + c0 + 16 * i;
-      if (j >= k_end || j >= n_vis) s[i] = -INFINITY;
-      mx = fmaxf(mx, s[i]);
-    }
+    for (int u = 0; u < RPT; ++u) {
+      float mx = -INFINITY;
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    const float m_new = fmaxf(m_run, mx);
-    const bool new_top = mx > m_run;  // this tile holds a key above everything before it
-    // (no branch here: the two rows of a warp vote together below)
-    const float corr = (m_run == -INFINITY) ? 0.f : expf(m_run - m_new);
-    float lsum = 0.f;
-    bool found = false;  // the first key of the tile at the new maximum (smallest key index) is left out of the sum
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float p = (s[i] == -INFINITY) ? 0.f : expf(s[i] - m_new);
-      Ps[r * kKT + c0 + 16 * i] = p;
-      const unsigned at_top = (__ballot_sync(0xffffffffu, new_top && s[i] == m_new) >> (threadIdx.x & 16)) & 0xffffu;
-      const bool skip = !found && at_top != 0u && (int)(__ffs(at_top) - 1) == c0;
-      found |= at_top != 0u;
-      lsum += skip ? 0.f : p;
-    }
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-    // the old top key (term 1 before) joins the others when a new top appears
-    l_rest = l_rest * corr + ((new_top && m_run != -INFINITY) ? corr : 0.f) + lsum;
-    m_run = m_new;
-#pragma unroll
-    for (int i = 0; i < OC; ++i) o_acc[i] *= corr;
-    __syncthreads();
-
-    for (int j = 0; j < kKT; ++j) {
-      const float p = Ps[r * kKT + j];
-      const float4 v0 = *reinterpret_cast<const float4*>(Vs + j * LD + c0 * 4);
-      o_acc[0] = fmaf(p, v0.x, o_acc[0]);
-      o_acc[1] = fmaf(p, v0.y, o_acc[1]);
-      o_acc[2] = fmaf(p, v0.z, o_acc[2]);
-      o_acc[3] = fmaf(p, v0.w, o_acc[3]);
-      if (OC == 8) {
-        const float4 v1 = *reinterpret_cast<const float4*>(Vs + j * LD + 64 + c0 * 4);
-        o_acc[4] = fmaf(p, v1.x, o_acc[4]);
-        o_acc[5] = fmaf(p, v1.y, o_acc[5]);
-        o_acc[6] = fmaf(p, v1.z, o_acc[6]);
-        o_acc[7] = fmaf(p, v1.w, o_acc[7]);
+      for (int i = 0; i < 4; ++i) {
+        const int j = kt + c0 + 16 * i;
+        if (j >= k_end || j >= n_vis[u]) s[u][i] = -INFINITY;
+        mx = fmaxf(mx, s[u][i]);
       }
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      const float m_new = fmaxf(m_run[u], mx);
+      const bool new_top = mx > m_run[u];  // this tile holds a key above everything before it
+      // (no branch here: the rows of a warp vote together below)
+      const float corr = (m_run[u] == -INFINITY) ? 0.f : expf(m_run[u] - m_new);
+      float lsum = 0.f;
+      bool found = false;  // the first key of the tile at the new maximum (smallest key index) is left out of the sum
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float p = (s[u][i] == -INFINITY) ? 0.f : expf(s[u][i] - m_new);
+        if (RPT == 1) Ps[r * kKT + c0 + 16 * i] = p;
+        const unsigned at_top = (__ballot_sync(0xffffffffu, new_top && s[u][i] == m_new) >> (threadIdx.x & 16)) & 0xffffu;
+        const bool skip = !found && at_top != 0u && (int)(__ffs(at_top) - 1) == c0;
+        found |= at_top != 0u;
+        lsum += skip ? 0.f : p;
+        s[u][i] = p;
+      }
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+      // the old top key (term 1 before) joins the others when a new top appears
+      l_rest[u] = l_rest[u] * corr + ((new_top && m_run[u] != -INFINITY) ? corr : 0.f) + lsum;
+      m_run[u] = m_new;
+#pragma unroll
+      for (int i = 0; i < OC; ++i) o_acc[u][i] *= corr;
+    }
+    if constexpr (RPT == 4) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<float4*>(Ps + (c0 + 16 * i) * kPitch + r * RPT) = make_float4(s[0][i], s[1][i], s[2][i], s[3][i]);
+    }
+    __syncthreads();
+    if (RPT > 1) {
+      stage_rows<T, D, LD>(Vs, Vu + (size_t)kt * D, kKT, k_end - kt);
+      __syncthreads();
+    }
+
+    auto add_key = [&](int j) {
+      float p[RPT];
+      if constexpr (RPT == 4) *reinterpret_cast<float4*>(p) = *reinterpret_cast<const float4*>(Ps + j * kPitch + r * RPT);
+      else p[0] = Ps[r * kKT + j];
+#pragma unroll
+      for (int x = 0; x < OC / 4; ++x) {
+        const float4 v = *reinterpret_cast<const float4*>(Vs + j * LD + 64 * x + c0 * 4);
+#pragma unroll
+        for (int u = 0; u < RPT; ++u) {
+          o_acc[u][4 * x] = fmaf(p[u], v.x, o_acc[u][4 * x]);
+          o_acc[u][4 * x + 1] = fmaf(p[u], v.y, o_acc[u][4 * x + 1]);
+          o_acc[u][4 * x + 2] = fmaf(p[u], v.z, o_acc[u][4 * x + 2]);
+          o_acc[u][4 * x + 3] = fmaf(p[u], v.w, o_acc[u][4 * x + 3]);
+        }
+      }
+    };
+    // (one row per thread: unrolling and register bound are left to the compiler; larger ones cost 2 - 6 %)
+    if constexpr (RPT == 1) {
+      for (int j = 0; j < kKT; ++j) add_key(j);
+    } else {
+#pragma unroll 4
+      for (int j = 0; j < kKT; ++j) add_key(j);
     }
     if (use_base) {
       const int col = tid % D, part = tid / D;
@@ -239,15 +287,20 @@ attn_partial_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, c
   }
 
   const size_t us = (size_t)unit * sc.splits + split;
-  if (row_ok) {
-    if (c0 == 0) {
-      sc.part_ml[(us * sc.Rpad + r_glob) * 2 + 0] = m_run;
-      sc.part_ml[(us * sc.Rpad + r_glob) * 2 + 1] = l_rest;
+#pragma unroll
+  for (int u = 0; u < RPT; ++u) {
+    const int row = rt * kR + r + 16 * u;
+    if (row < dm.R) {
+      if (c0 == 0) {
+        sc.part_ml[(us * sc.Rpad + row) * 2 + 0] = m_run[u];
+        sc.part_ml[(us * sc.Rpad + row) * 2 + 1] = l_rest[u];
+      }
+      float* po = sc.part_o + (us * sc.Rpad + row) * D;
+#pragma unroll
+      for (int x = 0; x < OC / 4; ++x)
+        *reinterpret_cast<float4*>(po + 64 * x + c0 * 4) =
+            make_float4(o_acc[u][4 * x], o_acc[u][4 * x + 1], o_acc[u][4 * x + 2], o_acc[u][4 * x + 3]);
     }
-    float* po = sc.part_o + (us * sc.Rpad + r_glob) * D;
-    *reinterpret_cast<float4*>(po + c0 * 4) = make_float4(o_acc[0], o_acc[1], o_acc[2], o_acc[3]);
-    if (OC == 8)
-      *reinterpret_cast<float4*>(po + 64 + c0 * 4) = make_float4(o_acc[4], o_acc[5], o_acc[6], o_acc[7]);
   }
   if (use_base) {
     __syncthreads();
@@ -363,22 +416,22 @@ attn_combine_kernel(Dims dm, const int* __restrict__ len, Scratch sc, float* __r
   }
 }
 
-template <typename T, int D>
+template <typename T, int D, int RPT>
 __global__ void __launch_bounds__(kThreads)
 score_pass_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, const T* __restrict__ V,
                   const int* __restrict__ len, float* __restrict__ base, Scratch sc,
                   float* __restrict__ scores, const float* __restrict__ vsum) {
-  constexpr int LD = D + 4;
+  constexpr int LD = D + 4, kR = kRT * RPT;
   ptx::pdl_wait();
   ptx::pdl_trigger();
   extern __shared__ __align__(16) float smem[];
-  float* Qs = smem;              // kRT * LD
-  float* Ks = Qs + kRT * LD;     // kKT * LD
+  float* Qs = smem;              // kR * LD
+  float* Ks = Qs + kR * LD;      // kKT * LD
   float* Hred = Ks + kKT * LD;   // kRT * kKT  sums of the rows' weights of a key
   float* Cred = Hred + kRT * kKT;  // kRT * kKT  sums of the rows' complements 1 - alpha of a key
   float* Xs = Cred + kRT * kKT;  // D
-  float* st = Xs + D;            // kRT * 4
-  float* wq = st + kRT * 4;      // kKT: w_j / (1 - w_j)
+  float* st = Xs + D;            // kR * 4
+  float* wq = st + kR * 4;       // kKT: w_j / (1 - w_j)
 
   const int unit = blockIdx.y;
   const int b = unit / dm.Hkv, h = unit % dm.Hkv;
@@ -407,10 +460,10 @@ score_pass_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
   // hacc: sum over the counted rows of alpha_{r,j}; cacc: sum of 1 - alpha_{r,j}, where the row's top key takes
   // (sum of the others) / sum from the attention pass and everybody else 1 - alpha <= 1/2: no cancellation
   float hacc[4] = {0.f, 0.f, 0.f, 0.f}, cacc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int t0 = 0; t0 < n_rows; t0 += kRT) {
+  for (int t0 = 0; t0 < n_rows; t0 += kR) {
     __syncthreads();
     // counted row number t -> row of the unit
-    for (int idx = tid; idx < kRT * (D / 4); idx += kThreads) {
+    for (int idx = tid; idx < kR * (D / 4); idx += kThreads) {
       const int rr = idx / (D / 4), c4 = idx % (D / 4);
       const int t = t0 + rr;
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -420,7 +473,7 @@ score_pass_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
       }
       *reinterpret_cast<float4*>(Qs + rr * LD + c4 * 4) = v;
     }
-    if (tid < kRT) {
+    if (tid < kR) {
       const int t = t0 + tid;
       float mx = 0.f, il = 0.f, cr = 0.f;
       if (t < n_rows) {
@@ -434,23 +487,27 @@ score_pass_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
       st[tid * 4 + 2] = cr;
     }
     __syncthreads();
-    const int t = t0 + r;
-    if (t < n_rows) {
-      const int row = (mode == CAOTE_BASE_LAST_QUERY) ? t * dm.m + dm.m - 1 : t;
-      const int n_vis = n - dm.m + (row % dm.m) + 1;
-      const float mx = st[r * 4], il = st[r * 4 + 1], cr = st[r * 4 + 2];
-      float sl4[4];
-      logit4<D, LD>(Qs + r * LD, Ks + c0 * LD, dm.scale, sl4);
+    if (t0 + r < n_rows) {
+      float s[RPT][4];
+      logits<D, LD, RPT>(Qs + r * LD, Ks + c0 * LD, dm.scale, s);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int j = j0 + c0 + 16 * i;
-        if (j < n_vis) {
-          const float sl = sl4[i];
-          const float a = expf(sl - mx) * il;
-          hacc[i] += a;
-          cacc[i] += (sl == mx) ? cr : 1.f - a;
-        } else {
-          cacc[i] += 1.f;  // a row that cannot see the key gives all its weight to the others
+      for (int u = 0; u < RPT; ++u) {
+        const int t = t0 + r + 16 * u;
+        if (u > 0 && t >= n_rows) break;
+        const int row = (mode == CAOTE_BASE_LAST_QUERY) ? t * dm.m + dm.m - 1 : t;
+        const int n_vis = n - dm.m + (row % dm.m) + 1;
+        const float mx = st[(r + 16 * u) * 4], il = st[(r + 16 * u) * 4 + 1], cr = st[(r + 16 * u) * 4 + 2];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int j = j0 + c0 + 16 * i;
+          if (j < n_vis) {
+            const float sl = s[u][i];
+            const float a = expf(sl - mx) * il;
+            hacc[i] += a;
+            cacc[i] += (sl == mx) ? cr : 1.f - a;
+          } else {
+            cacc[i] += 1.f;  // a row that cannot see the key gives all its weight to the others
+          }
         }
       }
     }
@@ -517,9 +574,9 @@ score_pass_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
   }
 }
 
-inline size_t partial_smem(int D) {
+inline size_t partial_smem(int D, int rpt) {
   const int LD = D + 4;
-  return sizeof(float) * (size_t)(kRT * LD + 2 * kKT * LD + kRT * kKT + kKT + kThreads);
+  return sizeof(float) * (size_t)(kRT * rpt * LD + (rpt == 1 ? 2 : 1) * kKT * LD + kKT * p_pitch(rpt) + kKT + kThreads);
 }
 // Sum-of-errors aggregation: instead of adding the rows' weights and applying the general form once,
 // add up the exact single-query errors (Theorem 3.2, row by row) of the rows that define the base score:
@@ -587,13 +644,13 @@ sum_errors_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
       const int row = (mode == CAOTE_BASE_LAST_QUERY) ? t * dm.m + dm.m - 1 : t;
       const int n_vis = n - dm.m + (row % dm.m) + 1;
       const float mx = st[r * 4], il = st[r * 4 + 1], cr = st[r * 4 + 2];
-      float sl4[4];
-      logit4<D, LD>(Qs + r * LD, Ks + c0 * LD, dm.scale, sl4);
+      float sl4[1][4];
+      logits<D, LD, 1>(Qs + r * LD, Ks + c0 * LD, dm.scale, sl4);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int jj = c0 + 16 * i, j = j0 + jj;
         if (j < n_vis) {
-          const float sl = sl4[i];
+          const float sl = sl4[0][i];
           const float e = expf(sl - mx) * il;              // alpha
           const float rest = (sl == mx) ? cr : 1.f - e;    // 1 - alpha: the others' share, without cancellation
           float d2 = 0.f;
@@ -625,9 +682,9 @@ inline size_t sum_errors_smem(int D) {
   return sizeof(float) * (size_t)(2 * kRT * LD + 2 * kKT * LD + kRT * kKT + kRT * 4);
 }
 
-inline size_t score_smem(int D) {
+inline size_t score_smem(int D, int rpt) {
   const int LD = D + 4;
-  return sizeof(float) * (size_t)(kRT * LD + kKT * LD + 2 * kRT * kKT + D + kRT * 4 + kKT);
+  return sizeof(float) * (size_t)(kRT * rpt * LD + kKT * LD + 2 * kRT * kKT + D + kRT * rpt * 4 + kKT);
 }
 
 }  // namespace generic

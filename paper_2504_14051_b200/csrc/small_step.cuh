@@ -121,8 +121,9 @@ small_step_kernel(Dims dm, Args<T> sa, int tiles, int* status) {
     generic::stage_rows<T, D, LD>(Vs, Vu + (size_t)kt * D, kKT, n - kt);
     if (carried && tid < kKT) bs[tid] = (kt + tid < n) ? bu[kt + tid] : 0.f;
     __syncthreads();
-    float s[4], mx = -INFINITY;
-    generic::logit4<D, LD>(Qs + r * LD, Ks + c0 * LD, dm.scale, s);
+    float s1[1][4], mx = -INFINITY;
+    generic::logits<D, LD, 1>(Qs + r * LD, Ks + c0 * LD, dm.scale, s1);
+    float(&s)[4] = s1[0];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       if (r >= G || kt + c0 + 16 * i >= n) s[i] = -INFINITY;

@@ -50,6 +50,30 @@ def test_row_block_scores_match_oracle(shape, mode):
         assert torch.equal(base, base_in)
 
 
+# the any-shape fp32 kernels: rows at the edges of their tiles of 16 and, from 40 on, 64 rows; keys at those of 64
+FP32_SHAPES = [
+    (2, 3, 1, 128, 208, 13, [193, 13]),     # 39 rows
+    (2, 5, 1, 64, 272, 8, [257, 8]),        # 40
+    (1, 2, 2, 128, 528, 64, [513]),         # 64
+    (2, 5, 1, 128, 400, 13, [320, 64]),     # 65
+    (1, 2, 1, 64, 1104, 65, [1089]),        # 130
+]
+
+
+@pytest.mark.parametrize("mode", ["last_query", "chunk_sum", "accum", "external"])
+@pytest.mark.parametrize("shape", FP32_SHAPES)
+def test_fp32_row_tiles_match_oracle(shape, mode):
+    B, Hq, Hkv, d, cap, m, lens = shape
+    q, K, V, lens_t = make_case(970 + FP32_SHAPES.index(shape), B, Hq, Hkv, d, cap, m, torch.float32, lens)
+    base = None
+    if mode in ("accum", "external"):
+        base = (torch.rand((B, Hkv, cap), generator=torch.Generator().manual_seed(6)) * 2.0).to(DEV)
+    base_in = None if base is None else base.clone()
+    _, _, o, scores = run_score(q, K, V, lens_t, m, mode, base)
+    r = oracle_for(q, K, V, lens_t, scale=d ** -0.5, n_new=m, base_mode=mode, base=base_in)
+    check_scores_and_o(r, scores, o, lens_t, f"{shape} {mode}")
+
+
 @pytest.mark.parametrize("eps", [1e-1, 1e-2, 1e-3])
 @pytest.mark.parametrize("shape", [
     (1, 16, 1, 128, 700, 1, [640], "last_query"),      # one row block
