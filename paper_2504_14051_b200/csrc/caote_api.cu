@@ -200,7 +200,7 @@ static int launch_generic_score(const Dims& dm, const void* q, const void* K, co
                                 float* base, float* o, float* scores, char* ws, cudaStream_t st, const float* vsum,
                                 bool sum_errors = false) {
   generic::Scratch sc;
-  generic::carve(dm, ws + kHeaderBytes, &sc);
+  generic::carve(dm, std::is_same<T, float>::value, ws + kHeaderBytes, &sc);
   int* status = reinterpret_cast<int*>(ws);
   auto attention = [&](auto rpt) {
     constexpr int RPT = decltype(rpt)::value;
@@ -778,7 +778,7 @@ static int launch_prefill_kernels(const Dims& dm, prefill::Scratch sc, const voi
     });
   }
   if (kCarried) {
-    dim3 grid((dm.cap + prefill::kSumKeys - 1) / prefill::kSumKeys, dm.units);
+    dim3 grid((dm.cap + sc.sum_keys - 1) / sc.sum_keys, dm.units);
     CAOTE_LAUNCH("prefill_carried_sum_kernel", st,
                  launch_pdl(prefill::carried_sum_kernel<D>, grid, dim3(256), 0, st, dm, len, sc, (const float*)base, (const __nv_bfloat16*)V));
   }
@@ -838,7 +838,7 @@ static void refresh_sm_count() {
 static size_t workspace_bytes(const caote_params_t* p) {
   refresh_sm_count();
   const Dims dm = make_dims(p);
-  size_t need = generic::carve(dm, nullptr, nullptr);
+  size_t need = generic::carve(dm, p->dtype == CAOTE_F32, nullptr, nullptr);
   if (decode_shape_ok(p)) {
     const size_t need2 = rowstat_bytes(dm) + decode::carve(dm, nullptr, nullptr, 0);
     if (need2 > need) need = need2;

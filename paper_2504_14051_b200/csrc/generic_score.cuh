@@ -27,7 +27,6 @@ constexpr int kRT = 16;          // query rows per tile
 constexpr int kKT = 64;          // keys per tile
 constexpr int kThreads = 256;
 constexpr int kCombineThreads = 512;
-constexpr int kCombineRows = 16; // rows per combine CTA
 
 struct Scratch {
   float* part_ml;  // [units][splits][Rpad][2]   (max logit, sum of exp(s - max) over all keys but the first one at the max)
@@ -38,7 +37,7 @@ struct Scratch {
   float* osum;     // [units][chunks][D]
   float* ytot;     // [units][D]
   float* hbtot;    // [units]
-  int splits, Rpad, chunks;
+  int splits, Rpad, chunks, chunk_rows;  // chunk_rows: rows of a combine CTA
 };
 
 inline int round_up(int x, int a) { return (x + a - 1) / a * a; }
@@ -50,24 +49,25 @@ inline int round_up(int x, int a) { return (x + a - 1) / a * a; }
 constexpr int kManyRows = 4;
 inline int rows_per_thread(int rows) { return rows >= 40 ? kManyRows : 1; }
 
-// Number of key splits: enough CTAs to fill the machine a few times over, never more splits than
-// there are key tiles in the cache (a tile is a chain of its own latency: 256 tokens, 2 units: 9 us in spans of two, 5 in one).
-inline int choose_splits(const Dims& dm) {
-  const int rows = kRT * rows_per_thread(dm.R), row_tiles = (dm.R + rows - 1) / rows;
+// Number of key splits: enough CTAs (tiles of `rows` query rows) to fill the machine a few times over, never more splits than
+// there are spans of `span` keys in the cache.
+inline int choose_splits(const Dims& dm, int rows, int span) {
+  const int row_tiles = (dm.R + rows - 1) / rows;
   const long ctas = (long)dm.units * row_tiles;
   int s = (int)(((long)g_sm_count * 4 + ctas - 1) / ctas);
-  const int max_by_cap = (dm.cap + kKT - 1) / kKT;
+  const int max_by_cap = (dm.cap + span - 1) / span;
   if (s > max_by_cap) s = max_by_cap;
   if (s > 32) s = 32;
   if (s < 1) s = 1;
   return s;
 }
 
-inline size_t carve(const Dims& dm, char* base, Scratch* out) {
+inline size_t carve_as(const Dims& dm, char* base, Scratch* out, int splits, int chunk_rows) {
   Scratch s;
-  s.splits = choose_splits(dm);
+  s.splits = splits;
+  s.chunk_rows = chunk_rows;
   s.Rpad = round_up(dm.R, kRT);
-  s.chunks = (dm.R + kCombineRows - 1) / kCombineRows;
+  s.chunks = (dm.R + chunk_rows - 1) / chunk_rows;
   size_t off = 0;
   auto take = [&](size_t n_floats) {
     float* p = reinterpret_cast<float*>(base + off);
@@ -85,6 +85,20 @@ inline size_t carve(const Dims& dm, char* base, Scratch* out) {
   s.hbtot = take((size_t)dm.units);
   if (out) *out = s;
   return off;
+}
+
+// Splits down to single tiles (a tile is a chain of its own latency: 256 tokens, 2 units: 9 us in spans of two, 5 in one) and
+// chunks of 16 rows, as far as the scratch allows. Every split keeps a full set of partial outputs, and a thread of four rows
+// asks for up to four times as many splits, so the scratch is bounded by what tiles of 16 rows, spans of two tiles and
+// chunks of 32 rows take; for fp32, whose main path this is, by the built-in array of caote_score_static where that is more.
+// (bf16 gets here with sums of errors over blocks of queries and with the few forms that the tensor-core kernels leave;
+// without the bound a cache of 8 units, 512 rows and 4 224 slots held 21.5 MB for it instead of 8.5.)
+inline size_t carve(const Dims& dm, bool f32, char* base, Scratch* out) {
+  size_t bound = carve_as(dm, nullptr, nullptr, choose_splits(dm, kRT, 2 * kKT), 32);
+  if (f32 && bound < CAOTE_STATIC_SCRATCH_BYTES - kHeaderBytes) bound = CAOTE_STATIC_SCRATCH_BYTES - kHeaderBytes;
+  for (int splits = choose_splits(dm, kRT * rows_per_thread(dm.R), kKT); splits > 1; --splits)
+    if (carve_as(dm, nullptr, nullptr, splits, 16) <= bound) return carve_as(dm, base, out, splits, 16);
+  return carve_as(dm, base, out, 1, carve_as(dm, nullptr, nullptr, 1, 16) <= bound ? 16 : 32);
 }
 
 // scale * <q, k> over D channels, in one fixed order, from fp32 rows in shared memory, for RPT queries and four keys 16 rows
@@ -328,7 +342,7 @@ __device__ __forceinline__ bool row_counted(const Dims& dm, int r) {
   return dm.base_mode != CAOTE_BASE_EXTERNAL;
 }
 
-// grid = (chunks of kCombineRows rows, units); a thread is a channel of every (kCombineThreads / D)-th row of the chunk. What
+// grid = (chunks of rows, units); a thread is a channel of every (kCombineThreads / D)-th row of the chunk. What
 // it costs is round trips to L2: the splits' statistics and outputs are fetched eight at a time before the first is used
 // (a thread per channel for 32 rows, one value after the other: 27 - 83 us for 28 - 96 rows in up to 32 splits).
 template <typename T, int D>
@@ -343,8 +357,8 @@ attn_combine_kernel(Dims dm, const int* __restrict__ len, Scratch sc, float* __r
   const int n = len[b];
   if (n == 0 || n < dm.m || n > dm.cap) return;
   float osum = 0.f;
-  const int r_end = min(dm.R, (chunk + 1) * kCombineRows);
-  for (int r = chunk * kCombineRows + grp; r < r_end; r += kGroups) {
+  const int r_end = min(dm.R, (chunk + 1) * sc.chunk_rows);
+  for (int r = chunk * sc.chunk_rows + grp; r < r_end; r += kGroups) {
     const float2* ml = reinterpret_cast<const float2*>(sc.part_ml) + (size_t)unit * sc.splits * sc.Rpad + r;
     const float* po = sc.part_o + ((size_t)unit * sc.splits * sc.Rpad + r) * D + c;
     float mx = -INFINITY;

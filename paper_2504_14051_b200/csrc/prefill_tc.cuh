@@ -57,7 +57,8 @@ struct Scratch {
   float* sstat;  // [units][kTile] LAST_QUERY: the counted rows' statistics side by side (else null)
   float* crest;  // [units][kTile] few: share of all tokens but the counted row's top one (else null)
   float* xpart;  // [units][row blocks][nsplit][D] per CTA of the attention pass: the sum of its counted output rows
-  float* ypart;  // [units][cap / kSumKeys][D + 4] sum_j base_j v_j over kSumKeys keys, at [D] sum_j base_j (else null)
+  float* ypart;  // [units][cap / sum_keys][D + 4] sum_j base_j v_j over sum_keys keys, at [D] sum_j base_j (else null)
+  int sum_keys;  // keys per CTA of carried_sum_kernel
   int Mpad;      // M rounded up to a multiple of kTile
   int nsplit;    // most key splits of the attention pass (1: none)
   int ns;        // key splits of this launch, at most nsplit
@@ -65,7 +66,13 @@ struct Scratch {
   bool few;      // 0 < Ms < kFewRows: complements without cancellation (see the file comment)
 };
 constexpr int kFewRows = 64;
-constexpr int kSumKeys = 512;  // keys per CTA of carried_sum_kernel
+// Keys per CTA of carried_sum_kernel: 512, or more where that would be more CTAs (and parts kept in the scratch) than it takes
+// to fill the machine many times over: 512 units of 40 000 slots, 21 MB of parts -> 3.
+inline int carried_sum_keys(const Dims& dm) {
+  int keys = 512;
+  while ((long long)dm.units * ((dm.cap + keys - 1) / keys) > 8192 && keys < dm.cap) keys *= 2;
+  return keys;
+}
 
 // Few units and few query rows leave most SMs idle: the keys of a unit are then cut into up to 8 splits
 // that run as the CTAs of a cluster. A function of the shape only.
@@ -97,6 +104,7 @@ inline size_t carve(const Dims& dm, char* base, Scratch* out) {
   s.nsplit = attn_splits(dm);
   s.Ms = dm.base_mode == CAOTE_BASE_LAST_QUERY ? dm.G : (dm.base_mode == CAOTE_BASE_EXTERNAL ? 0 : dm.R);
   s.few = s.Ms > 0 && s.Ms < kFewRows;
+  s.sum_keys = carried_sum_keys(dm);
   size_t off = 0;
   auto take = [&](bool wanted, size_t n_floats) {
     if (!wanted) return static_cast<float*>(nullptr);
@@ -110,7 +118,7 @@ inline size_t carve(const Dims& dm, char* base, Scratch* out) {
   s.crest = take(s.few, units * kTile);
   s.xpart = take(true, units * (s.Mpad / kTile) * s.nsplit * dm.D);
   s.ypart = take(dm.base_mode == CAOTE_BASE_ACCUM || dm.base_mode == CAOTE_BASE_EXTERNAL,
-                 units * ((dm.cap + kSumKeys - 1) / kSumKeys) * (dm.D + 4));
+                 units * ((dm.cap + s.sum_keys - 1) / s.sum_keys) * (dm.D + 4));
   s.ns = s.nsplit;
   if (out) *out = s;
   return off;
@@ -808,7 +816,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-// Parts of sum_j base_j v_j and sum_j base_j: grid = (ceil(cap / kSumKeys), units), 256 threads. A thread takes one 16-byte
+// Parts of sum_j base_j v_j and sum_j base_j: grid = (ceil(cap / sc.sum_keys), units), 256 threads. A thread takes one 16-byte
 // piece of every (256 / pieces)-th row, eight rows in flight; the rows' groups add up in shared memory in a fixed order.
 // No wait at the top: what it reads was complete before the attention pass before it got past its own wait (32 units of
 // 7.3 k tokens: 23 us in the merge of the splits -> hidden behind the attention pass; a spare warp of that kernel adding up
@@ -819,11 +827,11 @@ carried_sum_kernel(Dims dm, const int* __restrict__ len, Scratch sc, const float
   constexpr int P = D / 8, kGroups = 256 / P, kFly = 8;
   __shared__ float part[kGroups][D + 1];
   ptx::pdl_trigger();
-  const int unit = blockIdx.y, n = len[unit / dm.Hkv], j0 = blockIdx.x * kSumKeys;
+  const int unit = blockIdx.y, n = len[unit / dm.Hkv], j0 = blockIdx.x * sc.sum_keys;
   const int piece = threadIdx.x % P, g = threadIdx.x / P;
   const bool work = n >= dm.m && n <= dm.cap && j0 < n;
   if (work) {
-    const int j1 = min(n, j0 + kSumKeys);
+    const int j1 = min(n, j0 + sc.sum_keys);
     const float* bu = base + (size_t)unit * dm.cap;
     const uint4* src = reinterpret_cast<const uint4*>(V + (size_t)unit * dm.cap * D) + piece;
     float2 y[4];
@@ -896,8 +904,8 @@ __device__ __forceinline__ float x_from_parts(const Dims& dm, const Scratch& sc,
     }
   }
   if (sc.ypart) {
-    const int parts = (n + kSumKeys - 1) / kSumKeys;
-    const float* yp = sc.ypart + (size_t)unit * ((dm.cap + kSumKeys - 1) / kSumKeys) * (D + 4);
+    const int parts = (n + sc.sum_keys - 1) / sc.sum_keys;
+    const float* yp = sc.ypart + (size_t)unit * ((dm.cap + sc.sum_keys - 1) / sc.sum_keys) * (D + 4);
     for (int p0 = 0; p0 < parts; p0 += kFly) {
       float v[kFly][CPL], h[kFly];
 #pragma unroll

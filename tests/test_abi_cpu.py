@@ -57,6 +57,21 @@ def test_status_strings_and_workspace_size():
         assert C.caote_workspace_bytes(bad) == 0
 
 
+@pytest.mark.parametrize("batch,heads,d,m,cap,dtype,mode,limit", [
+    # blocks of a prompt that caote_score_static has taken: what they asked for when a split of the any-shape path was a
+    # tile of 16 query rows, in MB, or its built-in array
+    (1, (32, 8), 128, 128, 4224, torch.bfloat16, "chunk_sum", 8.9),
+    (4, (28, 4), 128, 128, 6128, torch.bfloat16, "last_query", 8.3),
+    (2, (28, 4), 128, 45, 3056, torch.bfloat16, "chunk_sum", 9.9),
+    (4, (32, 8), 128, 128, 8320, torch.bfloat16, "accum", 9.6),
+    (64, (16, 8), 128, 16, 40000, torch.bfloat16, "accum", 10.1),   # the parts of the carried scores' sums
+    (1, (16, 1), 128, 300, 40000, torch.float32, "chunk_sum", 16.777216),
+])
+def test_blocks_of_queries_fit_the_built_in_scratch(batch, heads, d, m, cap, dtype, mode, limit):
+    p = C.make_params(batch, heads[0], heads[1], d, cap, m, dtype, 0.1, mode)
+    assert 0 < C.caote_workspace_bytes(p) <= limit * 1e6 <= C.STATIC_SCRATCH_BYTES
+
+
 def test_host_side_argument_checks_return_before_any_launch():
     lib = P.lib()
     before = C.caote_launch_count()

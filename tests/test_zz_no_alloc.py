@@ -41,6 +41,8 @@ def _inputs(seed, B, Hq, Hkv, d, cap, m, lens):
     ((2, 8, 2, 128, 700, 1, [700, 513]), "last_query"),          # single-query kernel
     ((1, 8, 2, 128, 400, 64, [390]), "chunk_sum"),               # tensor-core kernels for a block of 64 queries
     ((1, 4, 2, 64, 300, 3, [290]), "chunk_sum"),                 # any-shape kernels (head_dim 64, 3 queries)
+    ((1, 32, 8, 128, 4224, 128, [4224]), "chunk_sum"),           # the usual block of a prompt
+    ((2, 28, 4, 128, 3056, 45, [3056, 2500]), "accum"),
 ])
 def test_static_scratch_matches_workspace_call_twice(shape, mode):
     B, Hq, Hkv, d, cap, m, lens = shape
