@@ -204,7 +204,7 @@ CAOTE_API int caote_select_evict_greedy(const caote_params_t* params, const void
 /* Remove the evicted slots from K, V, base, pos in place and set len[b] -= n_evict[b], so that the
  * cache is back within budget before the next block arrives (Sec. 2, budgeted block-wise flow).
  * mode is a caote_compact_mode_t. base, pos nullable. evict_idx rows must be ascending and unique
- * (what caote_select_evict writes). */
+ * (what caote_select_evict writes). The workspace is only checked, neither read nor written. */
 CAOTE_API int caote_compact(const caote_params_t* params, void* K, void* V, float* base, int32_t* pos,
                   int32_t* len, const int32_t* evict_idx, int32_t max_evict, const int32_t* n_evict,
                   int32_t mode, void* workspace, size_t workspace_bytes, caote_stream_t stream);

@@ -1244,9 +1244,11 @@ int caote_select_evict_greedy(const caote_params_t* p, const void* V, const floa
   return launch_greedy<float, 64>(dm, V, h, len, budget, pos, evict_idx, order, max_evict, n_evict, status, st);
 }
 
-int caote_compact(const caote_params_t* p, void* K, void* V, float* base, int32_t* pos, int32_t* len,
-                  const int32_t* evict_idx, int32_t max_evict, const int32_t* n_evict, int32_t mode,
-                  void* workspace, size_t workspace_bytes_, caote_stream_t stream) {
+// own_header: the workspace header is this step's alone and was zeroed once, as every step asks for (the lengths then move by
+// its ticket); caote_compact itself leaves the workspace alone.
+static int compact_impl(const caote_params_t* p, void* K, void* V, float* base, int32_t* pos, int32_t* len,
+                        const int32_t* evict_idx, int32_t max_evict, const int32_t* n_evict, int32_t mode, void* workspace,
+                        size_t workspace_bytes_, caote_stream_t stream, bool own_header) {
   if (!params_ok(p) || !K || !V || !len || !evict_idx || !n_evict || !workspace || max_evict < 1)
     return CAOTE_ERR_INVALID_ARG;
   if (!params_supported(p)) return CAOTE_ERR_UNSUPPORTED;
@@ -1258,11 +1260,15 @@ int caote_compact(const caote_params_t* p, void* K, void* V, float* base, int32_
   const Dims dm = make_dims(p);
   const int row_bytes = dm.D * (p->dtype == CAOTE_BF16 ? 2 : 4);
   cudaStream_t st = (cudaStream_t)stream;
-  int* ticket = reinterpret_cast<int*>(workspace) + 4;
+  bool lengths_moved;
   if (mode == CAOTE_COMPACT_FILL) {
-    CAOTE_LAUNCH("compact_fill_kernel", st, launch_pdl(sel::compact_fill_kernel, dim3(dm.units), dim3(dm.m > 16 ? sel::kSelThreads : 256), 0, st, dm.Hkv, dm.cap, row_bytes, (char*)K, (char*)V, base, pos,
-                                                       len, evict_idx, max_evict, n_evict, dm.B, ticket));
+    lengths_moved = dm.Hkv <= 8;  // (the largest cluster that every device runs)
+    CAOTE_LAUNCH("compact_fill_kernel", st,
+                 launch_pdl_clusters(sel::compact_fill_kernel, dim3(dm.units), dim3(dm.m > 16 ? sel::kSelThreads : 256), 0,
+                                     lengths_moved ? dm.Hkv : 1, st, dm.Hkv, dm.cap, row_bytes, (char*)K, (char*)V, base, pos, len,
+                                     evict_idx, max_evict, n_evict, lengths_moved));
   } else {
+    lengths_moved = own_header;
     rc = allow_smem(sel::compact_stable_kernel, 2 * sel::kStableTileBytes);
     if (rc) return rc;
     int c = 1;  // (three CTAs fit an SM)
@@ -1271,9 +1277,17 @@ int caote_compact(const caote_params_t* p, void* K, void* V, float* base, int32_
     CAOTE_LAUNCH("compact_stable_kernel", st,
                  launch_pdl_clusters(sel::compact_stable_kernel, grid, dim3(sel::kStableThreads), 2 * sel::kStableTileBytes,
                                      c, st, dm.Hkv, dm.cap, row_bytes, (char*)K, (char*)V, base, pos, len, evict_idx, max_evict,
-                                     n_evict, dm.B, ticket));
+                                     n_evict, dm.B, own_header ? reinterpret_cast<int*>(workspace) + 4 : (int*)nullptr));
   }
+  if (!lengths_moved)
+    CAOTE_LAUNCH("lengths_kernel", st, launch_pdl(sel::lengths_kernel, dim3(1), dim3(256), 0, st, dm.B, len, n_evict));
   return CAOTE_OK;
+}
+
+int caote_compact(const caote_params_t* p, void* K, void* V, float* base, int32_t* pos, int32_t* len,
+                  const int32_t* evict_idx, int32_t max_evict, const int32_t* n_evict, int32_t mode,
+                  void* workspace, size_t workspace_bytes_, caote_stream_t stream) {
+  return compact_impl(p, K, V, base, pos, len, evict_idx, max_evict, n_evict, mode, workspace, workspace_bytes_, stream, false);
 }
 
 // caote_step (vsum == NULL) and caote_step_fast (vsum kept current: += appended rows, -= evicted rows).
@@ -1312,8 +1326,7 @@ static int select_and_compact(const caote_params_t* p, const float* scores, void
           dm.Hkv, dm.cap, dm.D, (const float*)V, evict_idx, max_evict, n_evict, vsum));
     }
   }
-  return caote_compact(p, K, V, base, pos, len, evict_idx, max_evict, n_evict, compact_mode, workspace,
-                       workspace_bytes_, stream);
+  return compact_impl(p, K, V, base, pos, len, evict_idx, max_evict, n_evict, compact_mode, workspace, workspace_bytes_, stream, true);
 }
 static int step_impl(const caote_params_t* p, const void* q, const void* k_new, const void* v_new, void* K, void* V,
                      float* base, int32_t* pos, int32_t* len, int32_t* n_seen, const int32_t* budget, float* vsum,
@@ -1427,7 +1440,7 @@ int caote_step_post_evict(const caote_params_t* p, const void* q, const void* k_
   if (!rc)
     rc = caote_post_evict_output_ws(p, q, K, V, len, evict_idx, max_evict, n_evict, o, o_post, workspace, workspace_bytes_, stream);
   if (rc) return rc;
-  return caote_compact(p, K, V, base, pos, len, evict_idx, max_evict, n_evict, compact_mode, workspace, workspace_bytes_, stream);
+  return compact_impl(p, K, V, base, pos, len, evict_idx, max_evict, n_evict, compact_mode, workspace, workspace_bytes_, stream, true);
 }
 
 static int post_evict_impl(const caote_params_t* p, const void* q, const void* K, const void* V, const int32_t* len,

@@ -399,15 +399,18 @@ __device__ __forceinline__ void finish_lengths(int B, int* __restrict__ len, con
   }
 }
 
+// caote_compact keeps no state of its own between or beside calls (it takes any 256 bytes as its workspace, and calls that
+// overlap may share them), so its lengths do not move by a ticket: where a sequence's units are the CTAs of one cluster
+// (`by_sequence`), its first CTA does it once all of them have read the old length; else lengths_kernel does, one launch more.
 __global__ void __launch_bounds__(kSelThreads)
 compact_fill_kernel(int Hkv, int cap, int row_bytes, char* __restrict__ K, char* __restrict__ V,
                     float* __restrict__ base, int* __restrict__ pos, int* __restrict__ len,
-                    const int* __restrict__ evict_idx, int max_evict, const int* __restrict__ n_evict, int B, int* ticket) {
+                    const int* __restrict__ evict_idx, int max_evict, const int* __restrict__ n_evict, bool by_sequence) {
   ptx::pdl_wait();
   ptx::pdl_trigger();
   // (the searches are chains of dependent reads of the picks: from shared memory where they fit)
   __shared__ int s_picks[kMaxSharedPicks];
-  const int k = n_evict[blockIdx.x / Hkv];
+  const int b = blockIdx.x / Hkv, k = n_evict[b], n = len[b];
   const int* E = evict_idx + (size_t)blockIdx.x * max_evict;
   if (k > 1 && k <= kMaxSharedPicks) {
     for (int i = threadIdx.x; i < k; i += blockDim.x) s_picks[i] = E[i];
@@ -415,7 +418,16 @@ compact_fill_kernel(int Hkv, int cap, int row_bytes, char* __restrict__ K, char*
     E = s_picks;
   }
   compact_fill_unit(blockIdx.x, k, Hkv, cap, row_bytes, K, V, base, pos, len, E);
-  finish_lengths(B, len, n_evict, ticket);
+  if (by_sequence) {
+    ptx::cluster_sync_all();
+    if (blockIdx.x % Hkv == 0 && threadIdx.x == 0) len[b] = n - k;
+  }
+}
+
+__global__ void lengths_kernel(int B, int* __restrict__ len, const int* __restrict__ n_evict) {
+  ptx::pdl_wait();
+  ptx::pdl_trigger();
+  for (int b = threadIdx.x; b < B; b += blockDim.x) len[b] -= n_evict[b];
 }
 
 // A unit that evicts exactly one token, with FILL compaction: the argmin over (score bits, position) and the move of
@@ -556,6 +568,7 @@ __global__ void __launch_bounds__(kStableThreads)
 compact_stable_kernel(int Hkv, int cap, int row_bytes, char* __restrict__ K, char* __restrict__ V,
                       float* __restrict__ base, int* __restrict__ pos, int* __restrict__ len,
                       const int* __restrict__ evict_idx, int max_evict, const int* __restrict__ n_evict, int B, int* ticket) {
+  // ticket: null where lengths_kernel follows
   ptx::pdl_wait();
   ptx::pdl_trigger();
   extern __shared__ __align__(16) char tiles[];  // [2][kStableTileBytes]
@@ -611,7 +624,7 @@ compact_stable_kernel(int Hkv, int cap, int row_bytes, char* __restrict__ K, cha
       }
     }
   }
-  finish_lengths(B, len, n_evict, ticket);
+  if (ticket) finish_lengths(B, len, n_evict, ticket);
 }
 
 // Append m new rows per unit: grid = (units, ceil(m / 8)), 8 warps per CTA, one warp per row.

@@ -146,3 +146,31 @@ def test_stable_compaction_over_several_rounds(n, first, k, dtype, d):
         assert torch.equal(K[0, h, :n - k], K0[0, h, idx]) and torch.equal(V[0, h, :n - k], V0[0, h, idx])
         assert torch.equal(base[0, h, :n - k], b0[0, h, idx])
         assert torch.equal(K[0, h, n:], K0[0, h, n:]) and torch.equal(V[0, h, n:], V0[0, h, n:])
+
+
+@pytest.mark.parametrize("mode", ["fill", "stable"])
+@pytest.mark.parametrize("Hkv", [1, 3, 8, 9])
+def test_compaction_leaves_its_workspace_alone(Hkv, mode):
+    """caote_compact takes any 256 bytes: not zeroed ones, and ones that a call on another stream is using."""
+    B, d, cap, n, k = 3, 64, 300, 290, 2
+    p = P.make_params(B, Hkv, Hkv, d, cap, 1, torch.bfloat16, 1.0, "last_query")
+    ws = torch.full((256,), 0xA5, dtype=torch.uint8, device=DEV)
+    ev = torch.tensor([3, 77], dtype=torch.int32, device=DEV).expand(B, Hkv, k).contiguous()
+    ne = torch.tensor([2, 0, 1], dtype=torch.int32, device=DEV)
+    caches, streams = [], [torch.cuda.Stream() for _ in range(2)]
+    for _ in streams:
+        K, V = (torch.randn((B, Hkv, cap, d), device=DEV).to(torch.bfloat16) for _ in range(2))
+        pos = torch.arange(cap, dtype=torch.int32, device=DEV).expand(B, Hkv, cap).contiguous()
+        caches.append((K, V, pos, torch.full((B,), n, dtype=torch.int32, device=DEV)))
+    torch.cuda.synchronize()
+    for turn in range(2):
+        for (K, V, pos, lens), st in zip(caches, streams):
+            P.caote_compact(p, K, V, None, pos, lens, ev, ne, mode, ws, stream=st)
+    torch.cuda.synchronize()
+    for _, _, pos, lens in caches:
+        assert lens.tolist() == [n - 4, n, n - 2]
+        for h in range(Hkv):
+            for b, gone in ((0, {3, 77}), (1, set()), (2, {3})):
+                left = pos[b, h, :lens[b]].tolist()
+                assert len(set(left)) == len(left) and set(left) <= set(range(n)) - gone
+    assert (ws == 0xA5).all()
