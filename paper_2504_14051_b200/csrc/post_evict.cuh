@@ -95,11 +95,13 @@ post_evict_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
   const int k = n_evict[b];
   const int* E = evict_idx + (size_t)unit * max_evict;
   float A = 0.f, Y[CPL];
+  int left = n_vis;  // tokens the row still sees: where none is left the output is 0, whatever 1 - A rounds to
 #pragma unroll
   for (int c = 0; c < CPL; ++c) Y[c] = 0.f;
   for (int e = 0; e < k; ++e) {
     const int j = E[e];
     if (j < 0 || j >= n_vis) continue;
+    --left;
     float part = 0.f, vv[CPL];
 #pragma unroll
     for (int c = 0; c < CPL; ++c) {
@@ -116,7 +118,7 @@ post_evict_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
 #pragma unroll
   for (int c = 0; c < CPL; ++c) {
     const size_t at = qoff + lane * CPL + c;
-    o_post[at] = rest > 0.f ? (o[at] - Y[c]) / rest : 0.f;
+    o_post[at] = rest > 0.f && left > 0 ? (o[at] - Y[c]) / rest : 0.f;
   }
 }
 
@@ -130,7 +132,7 @@ post_evict_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
 constexpr int kTcThreads = 256;
 template <int D>
 inline size_t tc_smem_bytes() {
-  return 1024 + 3 * (size_t)prefill::kTileBytesOf<D> + prefill::kTile * sizeof(int) + kTcThreads * sizeof(float) + 64;
+  return 1024 + 3 * (size_t)prefill::kTileBytesOf<D> + prefill::kTile * sizeof(int) + kTcThreads * (sizeof(float) + sizeof(int)) + 64;
 }
 
 template <int D>
@@ -148,8 +150,9 @@ post_evict_tc_kernel(Dims dm, const __nv_bfloat16* __restrict__ q, const __nv_bf
   char* sm = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
   char *Qs = sm, *Ks = Qs + kTB, *Vs = Ks + kTB;
   int* js = reinterpret_cast<int*>(Vs + kTB);               // [kTile] slot of the evicted token, -1: none
-  float* xa = reinterpret_cast<float*>(js + kTile);         // [kTcThreads] half rows' sums of weights
-  uint64_t* s_bar = reinterpret_cast<uint64_t*>(xa + kTcThreads);
+  float* xa = reinterpret_cast<float*>(js + kTile);         // [kTcThreads] half rows' sums of weights,
+  int* xg = reinterpret_cast<int*>(xa + kTcThreads);        // [kTcThreads] and numbers of evicted tokens
+  uint64_t* s_bar = reinterpret_cast<uint64_t*>(xg + kTcThreads);
   uint64_t* y_bar = s_bar + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(y_bar + 1);
 
@@ -181,7 +184,7 @@ post_evict_tc_kernel(Dims dm, const __nv_bfloat16* __restrict__ q, const __nv_bf
   tc_fence_after();
   const uint32_t tmem = *tmem_slot, t_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
   float A = 0.f;
-  int t = 0;
+  int gone = 0, t = 0;  // gone: evicted tokens that the row sees, in this thread's half
   for (int e0 = 0; e0 < k; e0 += kTile, ++t) {
     if (t > 0) mbar_wait(y_bar, (t - 1) & 1, status);  // the tiles of the evicted rows have been read
     if (tid < kTile) {
@@ -218,8 +221,10 @@ post_evict_tc_kernel(Dims dm, const __nv_bfloat16* __restrict__ q, const __nv_bf
 #pragma unroll
     for (int c = 0; c < 32; ++c) {
       const int2 jj = *reinterpret_cast<const int2*>(js + half * 64 + 2 * c);
-      const float p0 = (jj.x >= 0 && jj.x < n_vis) ? fast_exp2(fmaf(sv[2 * c], scale2, -stat)) : 0.f;
-      const float p1 = (jj.y >= 0 && jj.y < n_vis) ? fast_exp2(fmaf(sv[2 * c + 1], scale2, -stat)) : 0.f;
+      const bool v0 = jj.x >= 0 && jj.x < n_vis, v1 = jj.y >= 0 && jj.y < n_vis;
+      const float p0 = v0 ? fast_exp2(fmaf(sv[2 * c], scale2, -stat)) : 0.f;
+      const float p1 = v1 ? fast_exp2(fmaf(sv[2 * c + 1], scale2, -stat)) : 0.f;
+      gone += (v0 ? 1 : 0) + (v1 ? 1 : 0);
       const uint32_t b0 = __float_as_uint(p0), b1 = __float_as_uint(p1);
       hi[c] = __byte_perm(b0, b1, 0x7632);
       lo[c] = pack_bf16(p0 - __uint_as_float(b0 & 0xffff0000u), p1 - __uint_as_float(b1 & 0xffff0000u));
@@ -245,8 +250,10 @@ post_evict_tc_kernel(Dims dm, const __nv_bfloat16* __restrict__ q, const __nv_bf
     }
   }
   xa[tid] = A;
+  xg[tid] = gone;
   __syncthreads();
-  const float rest = 1.f - (xa[tid] + xa[tid ^ kTile]);
+  // (where the row sees none of the retained tokens its output is 0, whatever 1 - A rounds to)
+  const float rest = xg[tid] + xg[tid ^ kTile] < n_vis ? 1.f - (xa[tid] + xa[tid ^ kTile]) : 0.f;
   if (t > 0) mbar_wait(y_bar, (t - 1) & 1, status);
   tc_fence_after();
 #pragma unroll

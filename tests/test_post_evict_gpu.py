@@ -107,3 +107,29 @@ def test_statistics_of_another_scoring_path_are_not_used():
     ev = evict_idx.cpu().numpy()
     ref = oracle.post_evict_output(f32(q), f32(K), f32(V), lens, [[ev[0, h] for h in range(Hkv)]], scale=scale, n_new=1)
     assert_close(f32(o_post)[0], ref[0], "fallback to the pass over K")
+
+
+@pytest.mark.parametrize("d,dtype,m,stats", [(128, torch.bfloat16, 64, True), (64, torch.bfloat16, 33, True),
+                                             (128, torch.bfloat16, 64, False), (64, torch.float32, 9, False), (128, torch.bfloat16, 1, True)])
+def test_rows_that_see_none_of_the_retained_tokens_are_zero(d, dtype, m, stats):
+    """Everything that the block's first rows see is evicted: exact zeros, whatever 1 minus the sum of the weights rounds to. The
+    rows after them are left with one token or more."""
+    B, Hq, Hkv, n = 2, 8, 2, 290 if m > 1 else 3
+    empty = (m + 1) // 2 if m > 1 else 1  # rows 0 .. empty - 1 see the slots below n - m + empty
+    q, K, V, lens_t = make_case(5 + m, B, Hq, Hkv, d, 304, m, dtype, [n, n])
+    p = P.make_params(B, Hq, Hkv, d, 304, m, dtype, d ** -0.5, "last_query" if m == 1 else "chunk_sum")
+    ws = P.alloc_workspace(p, DEV)
+    o = torch.zeros(q.shape, dtype=torch.float32, device=DEV)
+    P.caote_score(p, q, K, V, lens_t, None, o, torch.zeros((B, Hkv, 304), dtype=torch.float32, device=DEV), ws)
+    k = n - m + empty
+    ev = torch.arange(k, dtype=torch.int32, device=DEV).expand(B, Hkv, k).contiguous()
+    ne = torch.tensor([k, 0], dtype=torch.int32, device=DEV)
+    o_post = torch.full_like(o, float("nan"))
+    if stats:
+        P.caote_post_evict_output_ws(p, q, K, V, lens_t, ev, ne, o, o_post, ws)
+    else:
+        P.caote_post_evict_output(p, q, K, V, lens_t, ev, ne, o, o_post)
+    assert (o_post[0, :, :empty] == 0).all()
+    assert torch.equal(o_post[1], o[1])
+    if m > 1:
+        assert (o_post[0, :, empty:] != 0).any(dim=-1).all()

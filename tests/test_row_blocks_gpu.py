@@ -98,7 +98,7 @@ def test_few_rows_that_agree_on_one_token(shape, eps):
 
 @pytest.mark.parametrize("case", [
     # B, Hq, Hkv, d, cap, m, lens, budget, mode: evictions at the edges of a tile of 128 evicted rows, sequences that
-    # evict nothing or all that their first rows see, ragged row blocks
+    # evict nothing or nearly everything, ragged row blocks
     (2, 8, 2, 128, 500, 64, [500, 300], [372, 300], "last_query"),
     (2, 4, 2, 64, 700, 33, [650, 600], [521, 473], "chunk_sum"),
     (1, 14, 2, 128, 900, 128, [896], [512], "chunk_sum"),
