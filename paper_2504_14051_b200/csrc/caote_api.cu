@@ -1175,14 +1175,18 @@ int caote_vsum(const caote_params_t* p, const void* V, const int32_t* len, float
   auto launch = [&](auto kernel, auto v) {
     launch_pdl_clusters(kernel, grid, dim3(256), 0, fast::kSumCtas, st, dm.Hkv, dm.cap, v, len, vsum);
   };
+  auto of_dim = [&](auto v, auto wide) {
+    using T = std::remove_const_t<std::remove_pointer_t<decltype(v)>>;
+    if (dm.D == 128) launch(fast::vsum_kernel<T, 128, decltype(wide)::value>, v);
+    else launch(fast::vsum_kernel<T, 64, decltype(wide)::value>, v);
+  };
+  auto of_alignment = [&](auto v) {
+    if (aligned(V, 16)) of_dim(v, std::true_type{});
+    else of_dim(v, std::false_type{});
+  };
   CAOTE_LAUNCH("fast_vsum_kernel", st, {
-    if (p->dtype == CAOTE_BF16) {
-      if (dm.D == 128) launch(fast::vsum_kernel<__nv_bfloat16, 128>, (const __nv_bfloat16*)V);
-      else launch(fast::vsum_kernel<__nv_bfloat16, 64>, (const __nv_bfloat16*)V);
-    } else {
-      if (dm.D == 128) launch(fast::vsum_kernel<float, 128>, (const float*)V);
-      else launch(fast::vsum_kernel<float, 64>, (const float*)V);
-    }
+    if (p->dtype == CAOTE_BF16) of_alignment((const __nv_bfloat16*)V);
+    else of_alignment((const float*)V);
   });
   return CAOTE_OK;
 }

@@ -15,8 +15,22 @@ namespace fast {
 // One cluster of kSumCtas CTAs per unit, every CTA a contiguous share of its rows; 256 threads, a thread sums one 16-byte
 // piece of every (256 / pieces)-th row, four rows in flight; the shares meet in rank 0 in a fixed order. (One CTA per unit
 // and two bytes per load: 286 us for 16 units of 6.3 k tokens.)
+// kWide: V is 16-byte aligned; where it is not (this call has no rule for it) a piece comes element by element.
 constexpr int kSumCtas = 8;
-template <typename T, int D>
+template <typename T, bool kWide>
+__device__ __forceinline__ uint4 load_piece(const T* p) {
+  if constexpr (kWide) return *reinterpret_cast<const uint4*>(p);
+  uint32_t w[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    if constexpr (sizeof(T) == 2)
+      w[c] = (uint32_t)__bfloat16_as_ushort(p[2 * c]) | ((uint32_t)__bfloat16_as_ushort(p[2 * c + 1]) << 16);
+    else
+      w[c] = __float_as_uint(p[c]);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+template <typename T, int D, bool kWide>
 __global__ void __launch_bounds__(256)
 vsum_kernel(int Hkv, int cap, const T* __restrict__ V, const int* __restrict__ len, float* __restrict__ vsum) {
   constexpr int E = 16 / (int)sizeof(T), P = D / E, kRowsPass = 256 / P, kFly = 4;
@@ -29,12 +43,12 @@ vsum_kernel(int Hkv, int cap, const T* __restrict__ V, const int* __restrict__ l
   float acc[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) acc[e] = 0.f;
-  const uint4* src = reinterpret_cast<const uint4*>(V + (size_t)unit * cap * D) + piece;
+  const T* src = V + (size_t)unit * cap * D + piece * E;
   for (int j0 = rank * share + g; j0 < r1; j0 += kFly * kRowsPass) {
     uint4 raw[kFly];
 #pragma unroll
     for (int u = 0; u < kFly; ++u)
-      raw[u] = (j0 + u * kRowsPass < r1) ? src[(size_t)(j0 + u * kRowsPass) * P] : make_uint4(0u, 0u, 0u, 0u);
+      raw[u] = (j0 + u * kRowsPass < r1) ? load_piece<T, kWide>(src + (size_t)(j0 + u * kRowsPass) * D) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
     for (int u = 0; u < kFly; ++u) {
       const uint32_t w[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};

@@ -228,3 +228,27 @@ def test_a_sequence_without_room_keeps_its_running_sum():
     assert torch.equal(c.vsum[1], vsum0[1]) and torch.equal(c.V[1], V1[1])
     ref = c.V[0, :, :256].double().sum(dim=1).cpu().numpy()
     assert_close(c.vsum[0].double().cpu().numpy(), ref, "running sum of the sequence that took its new row", rtol=1e-5, atol=2e-3)
+
+
+@pytest.mark.parametrize("d,dtype", [(128, torch.bfloat16), (64, torch.bfloat16), (128, torch.float32), (64, torch.float32)])
+def test_sum_of_value_rows_takes_any_alignment(d, dtype):
+    """caote_vsum has no alignment rule for V: one element past a 16-byte boundary gives the bits of the aligned sum, within
+    the rounding of fp32 sums of the sum in 64 bits."""
+    B, Hkv, cap, lens = 5, 2, 1040, [0, 1, 9, 257, 1040]
+    g = torch.Generator(device="cpu").manual_seed(d)
+    V = torch.randn((B, Hkv, cap, d), generator=g).to(dtype).to(DEV)
+    lens_t = torch.tensor(lens, dtype=torch.int32, device=DEV)
+    p = P.make_params(B, Hkv, Hkv, d, cap, 1, dtype, 1.0, "last_query")
+    sums = []
+    for shift in (0, 1):
+        buf = torch.empty(V.numel() + 16, dtype=dtype, device=DEV)
+        view = buf[shift:shift + V.numel()].view_as(V)
+        view.copy_(V)
+        assert (view.data_ptr() % 16 == 0) == (shift == 0)
+        out = torch.full((B, Hkv, d), float("nan"), device=DEV)
+        P.caote_vsum(p, view, lens_t, out)
+        sums.append(out)
+    assert torch.equal(sums[0], sums[1])
+    for b, n in enumerate(lens):
+        x = V[b, :, :n].double()
+        assert ((sums[1][b].double() - x.sum(1)).abs() <= n * 2.0 ** -24 * x.abs().sum(1)).all()
