@@ -31,7 +31,7 @@ __device__ __forceinline__ unsigned long long make_key(float score, int pos) {
 template <int kC>
 __device__ __forceinline__ void select_cached(int n, int k, const float* __restrict__ sc, const int* __restrict__ ps, int* out, int* picks) {
   constexpr int kW = kSelThreads / 32;
-  constexpr unsigned kRank = 128u, kNothing = 0xffffffffu;
+  constexpr unsigned kRank = 128u;
   __shared__ __align__(16) unsigned hist[2048];
   __shared__ unsigned s_lo[kW], s_hi[kW], s_tot[kW];
   __shared__ unsigned s_digit, s_below, s_count, s_list;
@@ -39,11 +39,12 @@ __device__ __forceinline__ void select_cached(int n, int k, const float* __restr
   __shared__ int s_cnt[kC * kW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   auto position = [&](int j) { return (unsigned)(ps ? ps[j] : j); };
-  unsigned v[kC];  // score bits; later the positions of the tokens at the threshold, kNothing for all others
+  unsigned v[kC], live = 0u;  // score bits, and which of them are there; later the positions of the tokens at the threshold
 #pragma unroll
   for (int i = 0; i < kC; ++i) {
     const int j = tid + i * kSelThreads;
-    v[i] = j < n ? __float_as_uint(sc[j]) : kNothing;
+    v[i] = j < n ? __float_as_uint(sc[j]) : 0u;
+    live |= (j < n ? 1u : 0u) << i;
   }
   hist[tid] = 0u;
   hist[tid + kSelThreads] = 0u;
@@ -51,13 +52,15 @@ __device__ __forceinline__ void select_cached(int n, int k, const float* __restr
   // thr: the threshold so far as it is known (prefix, then zeros); bits [0, top) of it are still to be decided;
   // want: how many to take of the `left` tokens with this prefix
   unsigned thr, want = (unsigned)k, left = (unsigned)n, taken = 0u;
-  int top;
+  int top;  // 0 .. 32 (a caller's own scores may have any bits)
+  auto above = [](unsigned x, int t) { return __funnelshift_rc(x, 0u, t); };  // x >> t, also for t = 32
+  auto alive = [&](int i) { return (live >> i & 1u) != 0u; };
   auto prefix_of_all = [&]() {
-    unsigned lo = kNothing, hi = 0u;
+    unsigned lo = 0xffffffffu, hi = 0u;
 #pragma unroll
     for (int i = 0; i < kC; ++i) {
-      lo = min(lo, v[i]);
-      hi = max(hi, v[i] == kNothing ? 0u : v[i]);
+      lo = min(lo, alive(i) ? v[i] : 0xffffffffu);
+      hi = max(hi, alive(i) ? v[i] : 0u);
     }
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
@@ -65,8 +68,8 @@ __device__ __forceinline__ void select_cached(int n, int k, const float* __restr
     __syncthreads();
     lo = __reduce_min_sync(0xffffffffu, s_lo[lane]);
     hi = __reduce_max_sync(0xffffffffu, s_hi[lane]);
-    top = 32 - __clz(lo ^ hi);  // (at most 31: neither scores nor positions are negative)
-    thr = (lo >> top) << top;
+    top = 32 - __clz(lo ^ hi);
+    thr = lo & ~((1ull << top) - 1ull);
   };
   prefix_of_all();
   for (bool by_position = false;;) {
@@ -74,7 +77,7 @@ __device__ __forceinline__ void select_cached(int n, int k, const float* __restr
       const int width = min(11, top), shift = top - width;
 #pragma unroll
       for (int i = 0; i < kC; ++i)
-        if (v[i] != kNothing && ((v[i] ^ thr) >> top) == 0u) atomicAdd(&hist[(v[i] >> shift) & ((1u << width) - 1u)], 1u);
+        if (alive(i) && above(v[i] ^ thr, top) == 0u) atomicAdd(&hist[(v[i] >> shift) & ((1u << width) - 1u)], 1u);
       __syncthreads();
       const unsigned c0 = hist[2 * tid], c1 = hist[2 * tid + 1];
       unsigned incl = c0 + c1;
@@ -104,19 +107,20 @@ __device__ __forceinline__ void select_cached(int n, int k, const float* __restr
     by_position = true;  // top == 0: the scores at the threshold are equal to the last bit
 #pragma unroll
     for (int i = 0; i < kC; ++i) {
-      taken |= (v[i] < thr ? 1u : 0u) << i;
-      v[i] = v[i] == thr ? position(tid + i * kSelThreads) : kNothing;
+      taken |= (alive(i) && v[i] < thr ? 1u : 0u) << i;
+      if (v[i] != thr) live &= ~(1u << i);
+      if (alive(i)) v[i] = position(tid + i * kSelThreads);
     }
     __syncthreads();
     prefix_of_all();
   }
   // the largest (v, position) that is taken
-  unsigned kv = thr | ((1u << top) - 1u), kp = kNothing;
+  unsigned kv = thr | (unsigned)((1ull << top) - 1ull), kp = 0xffffffffu;
   if (left != want && left <= kRank) {
     unsigned long long* list = reinterpret_cast<unsigned long long*>(hist);
 #pragma unroll
     for (int i = 0; i < kC; ++i)
-      if (v[i] != kNothing && ((v[i] ^ thr) >> top) == 0u)  // (the order of the list does not matter)
+      if (alive(i) && above(v[i] ^ thr, top) == 0u)  // (the order of the list does not matter)
         list[atomicAdd(&s_list, 1u)] = ((unsigned long long)v[i] << 32) | position(tid + i * kSelThreads);
     if (tid == 0 && (left & 1u)) list[left] = ~0ull;
     __syncthreads();
@@ -140,7 +144,7 @@ __device__ __forceinline__ void select_cached(int n, int k, const float* __restr
 #pragma unroll
   for (int i = 0; i < kC; ++i) {
     bool in = (taken >> i & 1u) != 0u;
-    if (v[i] != kNothing) in = v[i] < kv || (v[i] == kv && (kp == kNothing || position(tid + i * kSelThreads) <= kp));
+    if (alive(i)) in = v[i] < kv || (v[i] == kv && (kp == 0xffffffffu || position(tid + i * kSelThreads) <= kp));
     ballots[i] = __ballot_sync(0xffffffffu, in);
     if (lane == 0) s_cnt[i * kW + warp] = __popc(ballots[i]);
   }
