@@ -23,10 +23,17 @@
 //                 thread sums exp2(s - ref_r) / sum_r over the rows of its own key without any
 //                 exchange: h_j = sum_r alpha_{r,j} (+ base_j). Then c_j = w_j / (1 - w_j) * ||X - v_j||, X from its parts.
 //
-// 1 - w_j. With 64 counted rows or more it is formed as the difference (rows - h_j) (exact to 6e-8 of the row count).
-// A few rows may well agree on one token, so for fewer than 64 (`few`) the attention pass keeps the largest numerator
-// of every counted row apart from the sum of the others, and the complement of the row's top token is that sum's
-// share, everybody else's 1 - alpha with alpha <= 1/2: no cancellation.
+//   dominant_kernel  (all but EXTERNAL) scores the token that holds most of a unit's weight again, if there is one.
+//
+// 1 - w_j. With 64 counted rows or more it is formed as the difference H - h_j of the sum of all weights (rows, and carried
+// scores) and the token's own, both good to about 1e-6 of H: a weight of a few thousand exponentials, each with the rounding of
+// its statistic (|stat| 6e-8) and a quarter of them from a polynomial (3e-6, of alternating sign). For fewer rows (`few`) the
+// attention pass keeps the largest numerator of every counted row apart from the sum of the others, and the complement of
+// the row's top token is that sum's share, everybody else's 1 - alpha with alpha <= 1/2. Either is enough as long as nobody
+// holds most of the weight. For a token that does (an attention sink), || X - v_j || suffers as well: X is nearly v_j, and the
+// tensor pipe's running sums lose about 1e-6 of it towards zero, so at 1 - w_j = 1e-4 the score was 7e-3 off. There is at most one
+// token above three quarters of H; dominant_kernel forms its complement as the sum of the others' weights and its distance
+// as || sum_i w_i (v_i - v_j) || over the others: nothing cancels.
 //
 // Operands are staged by TMA as 64-channel boxes with the 128-byte swizzle, which is the canonical
 // K-major UMMA layout (8-row groups 1024 bytes apart); V in the second product is read through an
@@ -58,6 +65,7 @@ struct Scratch {
   float* crest;  // [units][kTile] few: share of all tokens but the counted row's top one (else null)
   float* xpart;  // [units][row blocks][nsplit][D] per CTA of the attention pass: the sum of its counted output rows
   float* ypart;  // [units][cap / sum_keys][D + 4] sum_j base_j v_j over sum_keys keys, at [D] sum_j base_j (else null)
+  int* dom;      // [units][2] the slot of the token that holds most of the weight, -1: none, and its h_j
   int sum_keys;  // keys per CTA of carried_sum_kernel
   int Mpad;      // M rounded up to a multiple of kTile
   int nsplit;    // most key splits of the attention pass (1: none)
@@ -119,6 +127,7 @@ inline size_t carve(const Dims& dm, char* base, Scratch* out) {
   s.xpart = take(true, units * (s.Mpad / kTile) * s.nsplit * dm.D);
   s.ypart = take(dm.base_mode == CAOTE_BASE_ACCUM || dm.base_mode == CAOTE_BASE_EXTERNAL,
                  units * ((dm.cap + s.sum_keys - 1) / s.sum_keys) * (dm.D + 4));
+  s.dom = reinterpret_cast<int*>(take(true, units * 2));
   s.ns = s.nsplit;
   if (out) *out = s;
   return off;
@@ -408,6 +417,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     }
     return;
   }
+  if (tid == 0 && split == 0 && blockIdx.x == 0) sc.dom[2 * unit] = -1;
   const int kt0 = split * ts;
   const int ntiles = min(ts, (n + kKeys - 1) / kKeys - kt0);
   float* xpart = sc.xpart + ((size_t)unit * gridDim.x * sc.nsplit + blockIdx.x * sc.nsplit + split) * D;
@@ -932,6 +942,7 @@ __device__ __forceinline__ float x_from_parts(const Dims& dm, const Scratch& sc,
   return hb;
 }
 
+constexpr float kDominant = 0.75f;  // share of a unit's weight above which a token's score is dominant_kernel's
 constexpr int kScoreKeys = 2 * kTile;            // keys per work item: two key tiles share every Q block
 constexpr int kKeyThreads = 2 * kScoreKeys;       // two threads per key: each owns 64 of a block's 128 rows
 constexpr int kScoreThreads = kKeyThreads + 96;   // + a warp for the products, one for K, V and X, one for Q and the statistics
@@ -1281,12 +1292,99 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         float ratio = 0.f;
         if (h > 0.f) ratio = (rest > 0.f) ? h / rest : INFINITY;
         scores[slot] = (ratio == 0.f) ? 0.f : ((ratio == INFINITY) ? INFINITY : ratio * sqrtf(acc));
+        if (h > kDominant * ((float)M + hb)) {
+          sc.dom[2 * unit] = j;
+          sc.dom[2 * unit + 1] = __float_as_int(h);
+        }
       }
     }
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, 512);
+}
+
+// The score of the token that holds more than kDominant of its unit's weight H (see the file comment), from the others' scores,
+// c_i = h_i / (H - h_i) d_i with d_i = || X - v_i ||, so h_i = H c_i / (d_i + c_i). A cluster of kDomCtas CTAs per unit, 256
+// threads, a thread one 16-byte piece of every (256 / pieces)-th row of its CTA's share; the shares meet in rank 0 in a fixed
+// order. Units without such a token leave at once: what the kernel costs then is its launch (block steps of 8 units,
+// 4 224 tokens 57.6 -> 58.5 us, 45 queries 46.3 -> 47.4).
+constexpr int kDomCtas = 8;
+template <int D>
+__global__ void __launch_bounds__(256)
+dominant_kernel(Dims dm, const __nv_bfloat16* __restrict__ V, const int* __restrict__ len, Scratch sc, float* __restrict__ scores,
+                const float* __restrict__ vsum) {
+  constexpr int P = D / 8, kRowsPass = 256 / P;
+  __shared__ __align__(16) float Xs[D + 4], part[kRowsPass][D + 4], mine[D + 4];
+  ptx::pdl_wait();
+  ptx::pdl_trigger();
+  const int unit = blockIdx.x / kDomCtas, rank = (int)ptx::cluster_ctarank(), n = len[unit / dm.Hkv];
+  if (n < dm.m || n > dm.cap || n == 0) return;
+  const int slot = sc.dom[2 * unit];
+  if (slot < 0) return;  // (the whole cluster)
+  const int tid = threadIdx.x, piece = tid % P, g = tid / P;
+  if (tid < 32) {
+    float x[D / 32];
+    const float hb = x_from_parts<D>(dm, sc, unit, n, vsum, tid, x);
+#pragma unroll
+    for (int i = 0; i < D / 32; ++i) Xs[tid * (D / 32) + i] = x[i];
+    if (tid == 0) Xs[D] = hb;
+  }
+  __syncthreads();
+  const float H = (float)sc.Ms + Xs[D];
+  auto load = [&](int j, float (&v)[8]) { load8(V + ((size_t)unit * dm.cap + j) * D + 8 * piece, v); };
+  float vt[8], w[8], S = 0.f;
+  load(slot, vt);
+#pragma unroll
+  for (int e = 0; e < 8; ++e) w[e] = 0.f;
+  const int share = (n + kDomCtas - 1) / kDomCtas, r0 = rank * share, r1 = min(n, r0 + share);
+#pragma unroll 2
+  for (int j0 = r0; j0 < r1; j0 += kRowsPass) {
+    const int j = j0 + g;
+    float v[8], d2 = 0.f;
+    load(min(j, n - 1), v);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const float d = Xs[8 * piece + e] - v[e];
+      d2 = fmaf(d, d, d2);
+    }
+#pragma unroll
+    for (int o = 1; o < P; o <<= 1) d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+    const float c = (j < r1 && j != slot) ? scores[(size_t)unit * dm.cap + j] : 0.f;
+    const float h = c > 0.f ? H * (c / (sqrtf(d2) + c)) : 0.f;
+    S += h;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) w[e] = fmaf(h, v[e] - vt[e], w[e]);
+  }
+#pragma unroll
+  for (int e = 0; e < 8; ++e) part[g][8 * piece + e] = w[e];
+  if (piece == 0) part[g][D] = S;
+  __syncthreads();
+  if (tid <= D) {
+    float t = 0.f;
+    for (int i = 0; i < kRowsPass; ++i) t += part[i][tid];
+    mine[tid] = t;
+  }
+  ptx::cluster_sync_all();
+  if (rank == 0 && tid <= D) {
+    float t = 0.f;
+    for (int i = 0; i < kDomCtas; ++i) t += ptx::ld_dsmem_f32(ptx::map_to_rank(ptx::smem_u32(mine + tid), i));
+    part[0][tid] = t;
+  }
+  ptx::cluster_sync_all();  // (nobody leaves while its share is read)
+  if (rank == 0 && tid < 32) {
+    float d2 = 0.f;
+#pragma unroll
+    for (int c = tid; c < D; c += 32) {
+      const float d = vsum ? Xs[c] - __bfloat162float(V[((size_t)unit * dm.cap + slot) * D + c]) : part[0][c] / H;
+      d2 = fmaf(d, d, d2);
+    }
+    d2 = warp_sum(d2);
+    if (tid == 0) {
+      const float rest = part[0][D];
+      scores[(size_t)unit * dm.cap + slot] = rest > 0.f ? __int_as_float(sc.dom[2 * unit + 1]) / rest * sqrtf(d2) : INFINITY;
+    }
+  }
 }
 
 // The scores when the caller supplies the weights (EXTERNAL): h_j = base_j, one pass over V. grid = (ceil(cap / kExtKeys),

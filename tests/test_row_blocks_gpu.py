@@ -174,3 +174,47 @@ def test_compaction_leaves_its_workspace_alone(Hkv, mode):
                 left = pos[b, h, :lens[b]].tolist()
                 assert len(set(left)) == len(left) and set(left) <= set(range(n)) - gone
     assert (ws == 0xA5).all()
+
+
+@pytest.mark.parametrize("eps", [1e-1, 1e-3, 1e-4])
+@pytest.mark.parametrize("case", [
+    # B, Hq, Hkv, d, cap, m, lens, mode, carried scores
+    (1, 8, 2, 128, 700, 64, [640], "accum", "zero"),         # one key split
+    (2, 4, 2, 128, 2100, 128, [2048, 300], "accum", "sink"),  # the same token holds nearly all of the carried scores
+    (1, 4, 2, 64, 2100, 128, [2048], "accum", "spread"),
+    (1, 8, 2, 64, 700, 64, [640], "chunk_sum", None),
+    (1, 8, 2, 128, 700, 128, [640], "chunk_sum", None),
+    (1, 8, 2, 128, 700, 128, [640], "last_query", None),     # few counted rows
+    (1, 16, 1, 128, 300, 1, [290], "accum", "sink"),         # one query
+])
+def test_token_that_holds_most_of_the_weight(case, eps):
+    """One token holds all but ~eps of the weight of every row: neither 1 - w nor || X - v || may be a difference of nearly equal
+    numbers (tolerance as everywhere; X from the tensor cores is 1e-6 off, 1e-2 of a distance of 1e-4)."""
+    B, Hq, Hkv, d, cap, m, lens, mode, carried = case
+    q, K, V, lens_t = dominant_case(31 + d + m, B, Hq, Hkv, d, cap, m, torch.bfloat16, lens, eps, 77)
+    base = None
+    if carried:
+        base = torch.rand((B, Hkv, cap), generator=torch.Generator().manual_seed(3)) * (eps / cap if carried == "sink" else 1.0)
+        if carried == "zero":
+            base.zero_()
+        if carried == "sink":
+            base[:, :, 77] = 1.0
+        base = (base * (m * Hq // Hkv if carried == "sink" else 1e-9)).to(DEV)
+    base_in = None if base is None else base.clone()
+    _, _, o, scores = run_score(q, K, V, lens_t, m, mode, base)
+    r = oracle_for(q, K, V, lens_t, scale=d ** -0.5, n_new=m, base_mode=mode, base=base_in)
+    assert ((1.0 - r["w"][:, :, 77]) < 8 * eps).all()
+    check_scores_and_o(r, scores, o, lens_t, f"{case} eps {eps}")
+
+
+def test_token_that_holds_most_of_the_weight_with_fast_scores():
+    B, Hq, Hkv, d, cap, m, lens, eps = 1, 8, 2, 128, 700, 64, [640], 1e-4
+    q, K, V, lens_t = dominant_case(8, B, Hq, Hkv, d, cap, m, torch.bfloat16, lens, eps, 77)
+    p = P.make_params(B, Hq, Hkv, d, cap, m, torch.bfloat16, d ** -0.5, "chunk_sum")
+    ws, vsum = P.alloc_workspace(p, DEV), torch.zeros((B, Hkv, d), device=DEV)
+    o, scores = torch.zeros(q.shape, device=DEV), torch.zeros((B, Hkv, cap), device=DEV)
+    P.caote_vsum(p, V, lens_t, vsum)
+    P.caote_score_fast(p, q, K, V, lens_t, None, vsum, o, scores, ws)
+    r = oracle_for(q, K, V, lens_t, scale=d ** -0.5, n_new=m, base_mode="chunk_sum")
+    for h in range(Hkv):
+        assert_close(f32(scores)[0, h, :lens[0]], oracle.fast_scores(r["w"][0, h, :lens[0]], f32(V)[0, h, :lens[0]]), f"[{h}]")
