@@ -381,7 +381,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             float* __restrict__ o, int* status) {
   constexpr int kTB = kTileBytesOf<D>, kBoxes = D / 64, kSteps = D / 16;  // k-steps of the first product
   ptx::pdl_wait();
-  ptx::pdl_trigger();
+  ptx::pdl_trigger();  // (never before the wait: carried_sum_kernel starts on it and reads what the wait is for)
   extern __shared__ char smem_raw[];
   // (aligned by an offset into the array, not through an integer: the pointer keeps its address space, and what is
   // read and written through it compiles to shared-memory accesses, not generic ones)
@@ -828,16 +828,19 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 
 // Parts of sum_j base_j v_j and sum_j base_j: grid = (ceil(cap / sc.sum_keys), units), 256 threads. A thread takes one 16-byte
 // piece of every (256 / pieces)-th row, eight rows in flight; the rows' groups add up in shared memory in a fixed order.
-// No wait at the top: what it reads was complete before the attention pass before it got past its own wait (32 units of
-// 7.3 k tokens: 23 us in the merge of the splits -> hidden behind the attention pass; a spare warp of that kernel adding up
-// the V tiles in shared memory held them too long: attention 102 -> 194 us).
+// No wait at the top (32 units of 7.3 k tokens: 23 us in the merge of the splits -> hidden behind the attention pass; a spare
+// warp of that kernel adding up the V tiles in shared memory held them too long: attention 102 -> 194 us). That is sound only
+// because the launch right before it is attn_kernel's, every CTA of which is past its own wait before it triggers this one:
+// all that came before has then completed and written back, the appended rows, the carried scores, and the last reader of
+// this scratch. A grid that has not waited for itself is promised no view of that but the one in L2, so lengths, scores and
+// rows are read there (ld.global.cg), not through a cache that may have seen them earlier.
 template <int D>
 __global__ void __launch_bounds__(256)
-carried_sum_kernel(Dims dm, const int* __restrict__ len, Scratch sc, const float* __restrict__ base, const __nv_bfloat16* __restrict__ V) {
+carried_sum_kernel(Dims dm, const int* len, Scratch sc, const float* base, const __nv_bfloat16* V) {
   constexpr int P = D / 8, kGroups = 256 / P, kFly = 8;
   __shared__ float part[kGroups][D + 1];
   ptx::pdl_trigger();
-  const int unit = blockIdx.y, n = len[unit / dm.Hkv], j0 = blockIdx.x * sc.sum_keys;
+  const int unit = blockIdx.y, n = __ldcg(len + unit / dm.Hkv), j0 = blockIdx.x * sc.sum_keys;
   const int piece = threadIdx.x % P, g = threadIdx.x / P;
   const bool work = n >= dm.m && n <= dm.cap && j0 < n;
   if (work) {
@@ -854,8 +857,8 @@ carried_sum_kernel(Dims dm, const int* __restrict__ len, Scratch sc, const float
 #pragma unroll
       for (int u = 0; u < kFly; ++u) {
         const bool in = j + u * kGroups < j1;
-        b[u] = in ? bu[j + u * kGroups] : 0.f;
-        raw[u] = in ? src[(size_t)(j + u * kGroups) * P] : make_uint4(0u, 0u, 0u, 0u);
+        b[u] = in ? __ldcg(bu + j + u * kGroups) : 0.f;
+        raw[u] = in ? __ldcg(src + (size_t)(j + u * kGroups) * P) : make_uint4(0u, 0u, 0u, 0u);
       }
 #pragma unroll
       for (int u = 0; u < kFly; ++u) {

@@ -72,9 +72,11 @@ __device__ __forceinline__ void fence_async_all() { asm volatile("fence.proxy.as
 // ---- programmatic dependent launch ------------------------------------------------------------------------
 // A kernel launched with the programmatic-serialization attribute may be scheduled while the kernel before it in
 // the stream is still running. pdl_wait() blocks until that kernel has completed and its writes are visible: it
-// is the first statement of every kernel launched that way, before any global access. pdl_trigger() lets the NEXT
-// kernel of the stream be scheduled once every CTA of this one has got this far (it then sits in its own
-// pdl_wait()): launch latency and prologue overlap the tail of this kernel. Both are no-ops in a plain launch.
+// is the first statement of every kernel launched that way, before any global access, and comes before pdl_trigger() in
+// all of them. pdl_trigger() lets the NEXT kernel of the stream be scheduled once every CTA of this one has got this far (it
+// then sits in its own pdl_wait()): launch latency and prologue overlap the tail of this kernel. Both are no-ops in a plain
+// launch. One kernel does not follow the rule: prefill::carried_sum_kernel triggers first, works, and waits last; it states
+// there what it relies on, the order of the two in prefill::attn_kernel above all.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -218,3 +218,27 @@ def test_token_that_holds_most_of_the_weight_with_fast_scores():
     r = oracle_for(q, K, V, lens_t, scale=d ** -0.5, n_new=m, base_mode="chunk_sum")
     for h in range(Hkv):
         assert_close(f32(scores)[0, h, :lens[0]], oracle.fast_scores(r["w"][0, h, :lens[0]], f32(V)[0, h, :lens[0]]), f"[{h}]")
+
+
+@pytest.mark.parametrize("d", [128, 64])
+def test_carried_sums_beside_the_attention_pass(d):
+    """Steps with accumulated scores whose launches overlap give the bits of steps whose launches are kept apart (by the
+    events that tracing records between them): the sum over the carried scores starts before the attention pass is over."""
+    B, Hq, Hkv, m, budget, steps = 2, 8, 4, 64, 4000, 5
+    def run(apart):
+        g = torch.Generator(device=DEV).manual_seed(4)
+        rn = lambda *s: torch.randn(s, generator=g, device=DEV).to(torch.bfloat16)
+        cache = P.EvictionCache(B, Hq, Hkv, d, budget + m, m, torch.bfloat16, budget, base_mode="accum")
+        lens = torch.tensor([budget, budget - 30], dtype=torch.int32, device=DEV)
+        cache.load(rn(B, Hkv, budget + m, d), rn(B, Hkv, budget + m, d), lens, base=torch.rand((B, Hkv, budget + m), generator=g, device=DEV))
+        P.caote_trace_enable(apart)
+        try:
+            outs = [cache.step(rn(B, Hq, m, d), rn(B, Hkv, m, d), rn(B, Hkv, m, d)).clone() for _ in range(steps)]
+            torch.cuda.synchronize()
+        finally:
+            P.caote_trace_enable(False)
+            traced = P.caote_trace_collect()
+        assert cache.status() == 0 and (not apart or traced["prefill_carried_sum_kernel"][0] == steps)
+        return outs + [cache.base, cache.scores, cache.K, cache.V, cache.pos, cache.lens]
+    for a, b in zip(run(False), run(True)):
+        assert torch.equal(a, b)
