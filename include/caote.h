@@ -325,7 +325,7 @@ CAOTE_API int caote_trace_collect(caote_trace_entry_t* out, int32_t max_entries,
 
 /* Process-wide settings, for tests and tuning runs. (The paper has no counterpart.)
  *   CAOTE_OPT_WAIT_CYCLES     clock cycles after which a device-side wait of the single-query cluster kernel
- *                             gives up (default 2e9, about a second). The kernel then records
+ *                             (and of the sum-of-errors pass after it) gives up (default 2e9, about a second). The kernel then records
  *                             CAOTE_ERR_TIMEOUT in the status word and still returns; its outputs are
  *                             undefined, the caches and the workspace stay usable. value >= 1.
  *   CAOTE_OPT_DECODE_CLUSTER  CTAs per thread-block cluster on the single-query path: 0 = chosen from the

@@ -662,7 +662,7 @@ static int launch_sum_errors_decode_gd(const Dims& dm, const void* q, const void
   CAOTE_LAUNCH("sum_errors_decode_kernel", st,
                launch_pdl(sed::sum_errors_decode_kernel<G, D>, grid, dim3(sed::kThreads), (sed::smem_bytes_of<G, D>), st, tmK, tmV, dm,
                           (const __nv_bfloat16*)q, len, o, reinterpret_cast<const float*>(ws + kHeaderBytes), scores,
-                          reinterpret_cast<int*>(ws)));
+                          reinterpret_cast<int*>(ws), g_wait_cycles.load(std::memory_order_relaxed)));
   return CAOTE_OK;
 }
 template <int D>

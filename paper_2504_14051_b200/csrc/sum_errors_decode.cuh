@@ -27,7 +27,7 @@ namespace sed {
 
 constexpr int kWarps = 4, kThreads = kWarps * 32;
 constexpr int kWPitch = 9;  // floats per token of the table of weights (odd: lanes on different banks)
-constexpr long long kWaitCycles = 2000000000LL;
+constexpr long long kDrainCycles = 4000000000LL;  // waits at the end for copies that are still in flight after one that ran out
 
 // Tiles by the group's size. Small copies and many warps hide latencies, large copies carry more bytes: 64 (128) units of
 // 16 000 tokens, head_dim 128: one head 164 us with large ones, 302 with small ones; 7 heads 133 and 128, 8 heads (128
@@ -56,12 +56,13 @@ inline int splits(int units, int cap, int tile, int ctas_per_sm) {
   return best;
 }
 
-// Bounded wait; the first one that runs out says so, and no later wait of the thread blocks (all indices stay in bounds).
-__device__ __forceinline__ void wait(uint64_t* bar, uint32_t parity, bool& late, int* status) {
+// Bounded wait; the first one that runs out says so, and no later wait of the thread blocks (all indices stay in bounds). A
+// lane 0 that is late starts no more copies and waits at the end for those it has started.
+__device__ __forceinline__ void wait(uint64_t* bar, uint32_t parity, bool& late, int* status, long long limit) {
   if (late || ptx::mbar_try_wait(bar, parity)) return;
   const long long t0 = clock64();
   while (!ptx::mbar_try_wait(bar, parity)) {
-    if (clock64() - t0 > kWaitCycles) {
+    if (clock64() - t0 > limit) {
       set_status(status, CAOTE_ERR_TIMEOUT);
       late = true;
       return;
@@ -88,7 +89,8 @@ template <int G, int D>
 __global__ void __launch_bounds__(kThreads, Tile<G>::kCtasPerSm)
 sum_errors_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, Dims dm,
                          const __nv_bfloat16* __restrict__ q, const int* __restrict__ len, const float* __restrict__ o,
-                         const float* __restrict__ head_stats, float* __restrict__ scores, int* status) {
+                         const float* __restrict__ head_stats, float* __restrict__ scores, int* status,
+                         long long wait_cycles) {
   constexpr int kTok = Tile<G>::kTok, kT = Tile<G>::kT, kBoxCh = Tile<G>::kBoxCh, kStageBytes = Tile<G>::kStageBytes,
                 kStages = Tile<G>::kStages;
   constexpr int kBoxes = D / kBoxCh, kSubs = 2 * kBoxes;  // stages of a tile: its K boxes, then its V boxes
@@ -140,10 +142,13 @@ sum_errors_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_c
   const float scale2 = dm.scale * 1.4426950408889634f;
   float* W = Ws + warp * kT * kWPitch;
   bool late = false;
-  int i = 0;
+  int i = 0, started = min(kStages, boxes);  // the box that is read, copies started (lane 0)
   auto next = [&]() {  // the stage has been read: the box that takes its place
     __syncwarp();
-    if (lane == 0 && i + kStages < boxes) load(i + kStages);
+    if (lane == 0 && !late && i + kStages < boxes) {
+      load(i + kStages);
+      ++started;
+    }
     ++i;
   };
   for (int t = t0 + warp; t < t1; t += kWarps) {
@@ -155,7 +160,7 @@ sum_errors_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_c
       for (int e = 0; e < 4; ++e) s[mt][e] = 0.f;
 #pragma unroll
     for (int sub = 0; sub < kBoxes; ++sub) {
-      wait(&full[i % kStages], (i / kStages) & 1, late, status);
+      wait(&full[i % kStages], (i / kStages) & 1, late, status, wait_cycles);
       const uint32_t sm = ptx::smem_u32(ring + (i % kStages) * kStageBytes);
 #pragma unroll
       for (int ks = 0; ks < kBoxCh / 16; ++ks)
@@ -186,7 +191,7 @@ sum_errors_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_c
       for (int g = 0; g < G; ++g) d2[k][g] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int sub = 0; sub < kBoxes; ++sub) {
-      wait(&full[i % kStages], (i / kStages) & 1, late, status);
+      wait(&full[i % kStages], (i / kStages) & 1, late, status, wait_cycles);
       const char* sm = ring + (i % kStages) * kStageBytes;
       const float* tab = Os + kBoxCh * sub;
 #pragma unroll 2
@@ -226,6 +231,10 @@ sum_errors_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_c
       if (j < n) scores[(size_t)unit * dm.cap + j] = cj;
     }
     __syncwarp();  // the weights have been read
+  }
+  if (lane == 0 && late) {  // (nothing may still be on its way to this CTA's shared memory when it ends)
+    bool never = false;
+    for (int k = max(0, started - kStages); k < started; ++k) wait(&full[k % kStages], (k / kStages) & 1, never, status, kDrainCycles);
   }
 }
 

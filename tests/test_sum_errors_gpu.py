@@ -84,3 +84,26 @@ def test_sum_errors_with_a_token_that_holds_almost_all_the_weight(eps):
     assert (1.0 - r["alpha_max"] < 3 * eps).all() if "alpha_max" in r else True
     for b, n in enumerate(lens):
         assert_close(f32(scores)[b, :, :n], r["scores"][b, :, :n], f"eps {eps} sum-of-errors scores[b={b}]")
+
+
+@pytest.mark.parametrize("Hq", [4, 16])  # two heads per group: large tiles; eight: small ones
+def test_a_pass_whose_waits_run_out_reports_it_and_leaves_nothing_behind(Hq):
+    """With the limit far below the latency of a copy the waits run out: the call returns with CAOTE_ERR_TIMEOUT in the status
+    word once its copies have landed, and the next call, on the same shared memory, gives the oracle's result."""
+    B, Hkv, d, cap, lens = 40, 2, 128, 1104, [1100 - 20 * b for b in range(40)]
+    q, K, V, lens_t = make_case(64, B, Hq, Hkv, d, cap, 1, torch.bfloat16, lens)
+    p = P.make_params(B, Hq, Hkv, d, cap, 1, torch.bfloat16, d ** -0.5, "last_query")
+    ws = P.alloc_workspace(p, DEV)
+    o = torch.zeros(q.shape, dtype=torch.float32, device=DEV)
+    scores = torch.zeros((B, Hkv, cap), dtype=torch.float32, device=DEV)
+    P.caote_set_option(P.binding.OPT_WAIT_CYCLES, 200)
+    try:
+        P.caote_score_sum_errors(p, q, K, V, lens_t, o, scores, ws)
+        assert P.caote_read_status(ws) == P.binding.ERR_TIMEOUT
+    finally:
+        P.caote_set_option(P.binding.OPT_WAIT_CYCLES, 2_000_000_000)
+    P.caote_score_sum_errors(p, q, K, V, lens_t, o, scores, ws)
+    assert P.caote_read_status(ws) == 0
+    r = oracle.score(f32(q), f32(K), f32(V), lens_t.cpu().numpy(), scale=d ** -0.5, n_new=1, base_mode="last_query", agg_mode="sum_errors")
+    for b, n in enumerate(lens):
+        assert_close(f32(scores)[b, :, :n], r["scores"][b, :, :n], f"[b={b}]")
