@@ -1349,9 +1349,11 @@ static int step_impl(const caote_params_t* p, const void* q, const void* k_new, 
   const bool bf16 = p->dtype == CAOTE_BF16;
   if (k_new && compact_mode == CAOTE_COMPACT_FILL && max_evict == 1 && cluster_shape_ok(p)) {
     // few single-query units: append, scoring, selection and compaction in one launch, where the scoring would be one launch
-    // of the cluster kernel with a cluster per unit
+    // of the cluster kernel with a cluster per unit (looked at first: a batch of more units is not planned twice)
     const Dims dm = make_dims(p);
-    if (vsum || dm.D == 64 || plan_side_by_side(dm) == 0) {
+    int clusters = 0;
+    if (dm.units <= g_sm_count && choose_cluster(dm, step_kernel(dm), &clusters) > 0 && clusters >= dm.units &&
+        (vsum || dm.D == 64 || plan_side_by_side(dm) == 0)) {
       int* hdr = reinterpret_cast<int*>(workspace);
       const dcl::StepArgs sa{(const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, (__nv_bfloat16*)K, (__nv_bfloat16*)V, pos, len,
                              n_seen, budget, evict_idx, n_evict, hdr + 4, vsum};
