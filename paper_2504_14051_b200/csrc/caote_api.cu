@@ -418,7 +418,7 @@ static int encode_decode_maps(const Dims& dm, const void* q, const void* K, cons
   const cuuint64_t gstride[1] = {(cuuint64_t)dm.D * 2};
   const cuuint32_t box[2] = {(cuuint32_t)channels, (cuuint32_t)tokens};
   const cuuint32_t estride[2] = {1, 1};
-  for (int i = 0; i < 3; ++i) {
+  for (int i = 0; i < (tmQ ? 3 : 2); ++i) {  // (tmQ: null if no map of q is wanted)
     // K, V: boxes of `channels` channels x `tokens` tokens, swizzled over the length of their rows; q: 64 channels x q_rows
     // rows (a unit's heads, padded by its neighbours' or by zeros)
     const cuuint64_t qdim[2] = {(cuuint64_t)dm.D, (cuuint64_t)dm.B * (cuuint64_t)dm.Hq};
@@ -654,8 +654,8 @@ static int launch_sum_errors_decode_gd(const Dims& dm, const void* q, const void
                                        float* scores, char* ws, cudaStream_t st) {
   TensorMapEncodeFn encode = tensor_map_encoder();
   if (!encode) return CAOTE_ERR_CUDA;  // (the cluster kernel before it was launched with the same encoder)
-  CUtensorMap tmK, tmV, tmQ;
-  int rc = encode_decode_maps(dm, q, K, V, 8, &tmK, &tmV, &tmQ, encode, sed::Tile<G>::kT, sed::Tile<G>::kBoxCh);
+  CUtensorMap tmK, tmV;
+  int rc = encode_decode_maps(dm, nullptr, K, V, 0, &tmK, &tmV, nullptr, encode, sed::Tile<G>::kT, sed::Tile<G>::kBoxCh);
   if (!rc) rc = allow_smem(sed::sum_errors_decode_kernel<G, D>, (sed::smem_bytes_of<G, D>));
   if (rc) return rc;
   dim3 grid(sed::splits(dm.units, dm.cap, sed::Tile<G>::kT, sed::Tile<G>::kCtasPerSm), dm.units);
