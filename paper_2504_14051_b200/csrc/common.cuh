@@ -40,6 +40,11 @@ inline int g_sm_count = 148;
 // Record the first device-side error in the status word (never overwrites an earlier one).
 __device__ inline void set_status(int* status, int code) { atomicCAS(status, 0, code); }
 
+// The first of two candidates for eviction by (score bits v, position p, slot s), left in (v, p, s); slot < 0: none.
+__device__ __forceinline__ void first_candidate(unsigned& v, unsigned& p, int& s, unsigned ov, unsigned op, int os) {
+  if (os >= 0 && (s < 0 || ov < v || (ov == v && (op < p || (op == p && os < s))))) { v = ov; p = op; s = os; }
+}
+
 // ---- element access ---------------------------------------------------------------------------
 __device__ inline float to_float(float x) { return x; }
 __device__ inline float to_float(__nv_bfloat16 x) { return __bfloat162float(x); }

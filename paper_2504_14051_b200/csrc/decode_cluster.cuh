@@ -256,10 +256,6 @@ struct StepArgs {
   int *evict_idx, *n_evict, *ticket;
   float* vsum;
 };
-// A candidate for eviction; slot < 0: none.
-__device__ __forceinline__ void first_candidate(unsigned& v, unsigned& p, int& s, unsigned ov, unsigned op, int os) {
-  if (os >= 0 && (s < 0 || ov < v || (ov == v && (op < p || (op == p && os < s))))) { v = ov; p = op; s = os; }
-}
 
 // kG: query heads per KV head; kMode: the base mode. Compile-time so that the per-head loops carry no
 // predicates and the paths of the other modes are not in the instruction stream.

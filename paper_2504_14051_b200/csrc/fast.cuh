@@ -19,16 +19,19 @@ namespace fast {
 constexpr int kSumCtas = 8;
 template <typename T, bool kWide>
 __device__ __forceinline__ uint4 load_piece(const T* p) {
-  if constexpr (kWide) return *reinterpret_cast<const uint4*>(p);
-  uint32_t w[4];
+  if constexpr (kWide) {
+    return *reinterpret_cast<const uint4*>(p);
+  } else {
+    uint32_t w[4];
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    if constexpr (sizeof(T) == 2)
-      w[c] = (uint32_t)__bfloat16_as_ushort(p[2 * c]) | ((uint32_t)__bfloat16_as_ushort(p[2 * c + 1]) << 16);
-    else
-      w[c] = __float_as_uint(p[c]);
+    for (int c = 0; c < 4; ++c) {
+      if constexpr (sizeof(T) == 2)
+        w[c] = (uint32_t)__bfloat16_as_ushort(p[2 * c]) | ((uint32_t)__bfloat16_as_ushort(p[2 * c + 1]) << 16);
+      else
+        w[c] = __float_as_uint(p[c]);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
   }
-  return make_uint4(w[0], w[1], w[2], w[3]);
 }
 template <typename T, int D, bool kWide>
 __global__ void __launch_bounds__(256)

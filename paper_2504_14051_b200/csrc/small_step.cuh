@@ -39,11 +39,6 @@ struct Args {
   float* vsum;
 };
 
-// A candidate for eviction; slot < 0: none.
-__device__ __forceinline__ void first_candidate(unsigned& v, unsigned& p, int& s, unsigned ov, unsigned op, int os) {
-  if (os >= 0 && (s < 0 || ov < v || (ov == v && (op < p || (op == p && os < s))))) { v = ov; p = op; s = os; }
-}
-
 inline size_t smem_bytes(int D, int tiles) {
   const int LD = D + 4;
   return sizeof(float) * ((size_t)kRT * LD + 2 * kKT * LD + (size_t)tiles * kRT * kKT + kRT * kKT + kRT * D + D + 8 + 2 * kRT +
