@@ -794,7 +794,7 @@ static int launch_prefill_kernels(const Dims& dm, prefill::Scratch sc, const voi
                  launch_pdl(score, grid, dim3(prefill::kScoreThreads), prefill::score_smem_bytes<D>(), st, tmQs, tmK, tmV, dm, len, sc,
                             base, scores, vsum, status));
     CAOTE_LAUNCH("prefill_dominant_kernel", st,
-                 launch_pdl_clusters(prefill::dominant_kernel<D>, dim3(dm.units * prefill::kDomCtas), dim3(256), 0, prefill::kDomCtas, st,
+                 launch_pdl_clusters(prefill::dominant_kernel<D>, dim3(dm.units * prefill::kDomCtas), dim3(prefill::kDomThreads), 0, prefill::kDomCtas, st,
                                      dm, (const __nv_bfloat16*)V, len, sc, scores, vsum));
   }
   return CAOTE_OK;

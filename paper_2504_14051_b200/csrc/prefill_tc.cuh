@@ -32,7 +32,7 @@
 // the row's top token is that sum's share, everybody else's 1 - alpha with alpha <= 1/2. Either is enough as long as nobody
 // holds most of the weight. For a token that does (an attention sink), || X - v_j || suffers as well: X is nearly v_j, and the
 // tensor pipe's running sums lose about 1e-6 of it towards zero, so at 1 - w_j = 1e-4 the score was 7e-3 off. There is at most one
-// token above three quarters of H; dominant_kernel forms its complement as the sum of the others' weights and its distance
+// token above kDominant of H; dominant_kernel forms its complement as the sum of the others' weights and its distance
 // as || sum_i w_i (v_i - v_j) || over the others: nothing cancels.
 //
 // Operands are staged by TMA as 64-channel boxes with the 128-byte swizzle, which is the canonical
@@ -911,7 +911,9 @@ __device__ __forceinline__ float x_from_parts(const Dims& dm, const Scratch& sc,
   return hb;
 }
 
-constexpr float kDominant = 0.75f;  // share of a unit's weight above which a token's score is dominant_kernel's
+// Share of a unit's weight above which a token's score is dominant_kernel's. Below it the plain differences are good to about
+// 3e-6 / (1 - w), 3e-5 of the score at the line.
+constexpr float kDominant = 0.9f;
 constexpr int kScoreKeys = 2 * kTile;            // keys per work item: two key tiles share every Q block
 constexpr int kKeyThreads = 2 * kScoreKeys;       // two threads per key: each owns 64 of a block's 128 rows
 constexpr int kScoreThreads = kKeyThreads + 96;   // + a warp for the products, one for K, V and X, one for Q and the statistics
@@ -1274,24 +1276,50 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 }
 
 // The score of the token that holds more than kDominant of its unit's weight H (see the file comment), from the others' scores,
-// c_i = h_i / (H - h_i) d_i with d_i = || X - v_i ||, so h_i = H c_i / (d_i + c_i). A cluster of kDomCtas CTAs per unit, 256
-// threads, a thread one 16-byte piece of every (256 / pieces)-th row of its CTA's share; the shares meet in rank 0 in a fixed
-// order. Units without such a token leave at once: what the kernel costs then is its launch (block steps of 8 units,
-// 4 224 tokens 57.6 -> 58.5 us, 45 queries 46.3 -> 47.4).
-constexpr int kDomCtas = 8;
+// c_i = h_i / (H - h_i) d_i with d_i = || X - v_i ||, so h_i = H c_i / (d_i + c_i). A cluster of kDomCtas CTAs per unit, 512
+// threads, a thread one 16-byte piece of every (512 / pieces)-th row of its CTA's share; the shares meet in rank 0 in a fixed
+// order. Units without such a token leave at once: what the kernel costs then is its launch, about a microsecond of a step of
+// 50 - 60. With one, it is the latency of a few round trips: up to eight rows a thread are fetched before the first is used,
+// and before X is known. Block steps without and with one in every unit: 8 units of 4 224 tokens 58.5, 70.4 us (86 with two rows
+// in flight and 256 threads); 64 units of 8 320 tokens 640, 750. (As a part of the selection, one CTA per unit and a launch
+// less: 58.0 and 95.7, and single-query steps 0.8 % slower for the selection's larger kernel.)
+constexpr int kDomCtas = 8, kDomThreads = 512;
 template <int D>
-__global__ void __launch_bounds__(256)
-dominant_kernel(Dims dm, const __nv_bfloat16* __restrict__ V, const int* __restrict__ len, Scratch sc, float* __restrict__ scores,
+__global__ void __launch_bounds__(kDomThreads)
+dominant_kernel(Dims dm, const __nv_bfloat16* __restrict__ V, const int* __restrict__ len, Scratch sc, float* scores,
                 const float* __restrict__ vsum) {
-  constexpr int P = D / 8, kRowsPass = 256 / P;
+  constexpr int P = D / 8, kRowsPass = kDomThreads / P, kFly = 8;
   __shared__ __align__(16) float Xs[D + 4], part[kRowsPass][D + 4], mine[D + 4];
   ptx::pdl_wait();
   ptx::pdl_trigger();
   const int unit = blockIdx.x / kDomCtas, rank = (int)ptx::cluster_ctarank(), n = len[unit / dm.Hkv];
-  if (n < dm.m || n > dm.cap || n == 0) return;
   const int slot = sc.dom[2 * unit];
-  if (slot < 0) return;  // (the whole cluster)
+  if (n < dm.m || n > dm.cap || n == 0 || slot < 0) return;  // (the whole cluster)
   const int tid = threadIdx.x, piece = tid % P, g = tid / P;
+  const uint4* src = reinterpret_cast<const uint4*>(V + (size_t)unit * dm.cap * D) + piece;
+  const float* cu = scores + (size_t)unit * dm.cap;
+  const int share = (n + kDomCtas - 1) / kDomCtas, r0 = rank * share, r1 = min(n, r0 + share);
+  uint4 raw[kFly];
+  float c[kFly];
+  auto fetch = [&](int j0) {
+#pragma unroll
+    for (int u = 0; u < kFly; ++u) {
+      const int j = j0 + u * kRowsPass;
+      raw[u] = j < r1 ? src[(size_t)j * P] : make_uint4(0u, 0u, 0u, 0u);
+      c[u] = j < r1 && j != slot ? cu[j] : 0.f;
+    }
+  };
+  auto unpack = [](uint4 r, float (&v)[8]) {
+    const uint32_t x[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      v[2 * e] = __uint_as_float(x[e] << 16);
+      v[2 * e + 1] = __uint_as_float(x[e] & 0xffff0000u);
+    }
+  };
+  int at = r0 + g;
+  fetch(at);
+  const uint4 top = src[(size_t)slot * P];
   if (tid < 32) {
     float x[D / 32];
     const float hb = x_from_parts<D>(dm, sc, unit, n, vsum, tid, x);
@@ -1301,29 +1329,32 @@ dominant_kernel(Dims dm, const __nv_bfloat16* __restrict__ V, const int* __restr
   }
   __syncthreads();
   const float H = (float)sc.Ms + Xs[D];
-  auto load = [&](int j, float (&v)[8]) { load8(V + ((size_t)unit * dm.cap + j) * D + 8 * piece, v); };
-  float vt[8], w[8], S = 0.f;
-  load(slot, vt);
+  float vt[8], w[8], xp[8], S = 0.f;
+  unpack(top, vt);
 #pragma unroll
-  for (int e = 0; e < 8; ++e) w[e] = 0.f;
-  const int share = (n + kDomCtas - 1) / kDomCtas, r0 = rank * share, r1 = min(n, r0 + share);
-#pragma unroll 2
-  for (int j0 = r0; j0 < r1; j0 += kRowsPass) {
-    const int j = j0 + g;
-    float v[8], d2 = 0.f;
-    load(min(j, n - 1), v);
+  for (int e = 0; e < 8; ++e) {
+    w[e] = 0.f;
+    xp[e] = Xs[8 * piece + e];
+  }
+  for (int j0 = r0; j0 < r1; j0 += kFly * kRowsPass) {  // (the same rounds for every thread: its shuffles are the warp's)
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const float d = Xs[8 * piece + e] - v[e];
-      d2 = fmaf(d, d, d2);
+    for (int u = 0; u < kFly; ++u) {
+      float v[8], d2 = 0.f;
+      unpack(raw[u], v);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const float d = xp[e] - v[e];
+        d2 = fmaf(d, d, d2);
+      }
+#pragma unroll
+      for (int o = 1; o < P; o <<= 1) d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+      const float h = c[u] > 0.f ? H * (c[u] / (sqrtf(d2) + c[u])) : 0.f;
+      S += h;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) w[e] = fmaf(h, v[e] - vt[e], w[e]);
     }
-#pragma unroll
-    for (int o = 1; o < P; o <<= 1) d2 += __shfl_xor_sync(0xffffffffu, d2, o);
-    const float c = (j < r1 && j != slot) ? scores[(size_t)unit * dm.cap + j] : 0.f;
-    const float h = c > 0.f ? H * (c / (sqrtf(d2) + c)) : 0.f;
-    S += h;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) w[e] = fmaf(h, v[e] - vt[e], w[e]);
+    at += kFly * kRowsPass;
+    fetch(at);
   }
 #pragma unroll
   for (int e = 0; e < 8; ++e) part[g][8 * piece + e] = w[e];
@@ -1331,12 +1362,14 @@ dominant_kernel(Dims dm, const __nv_bfloat16* __restrict__ V, const int* __restr
   __syncthreads();
   if (tid <= D) {
     float t = 0.f;
+#pragma unroll 8
     for (int i = 0; i < kRowsPass; ++i) t += part[i][tid];
     mine[tid] = t;
   }
   ptx::cluster_sync_all();
   if (rank == 0 && tid <= D) {
     float t = 0.f;
+#pragma unroll
     for (int i = 0; i < kDomCtas; ++i) t += ptx::ld_dsmem_f32(ptx::map_to_rank(ptx::smem_u32(mine + tid), i));
     part[0][tid] = t;
   }
@@ -1344,8 +1377,8 @@ dominant_kernel(Dims dm, const __nv_bfloat16* __restrict__ V, const int* __restr
   if (rank == 0 && tid < 32) {
     float d2 = 0.f;
 #pragma unroll
-    for (int c = tid; c < D; c += 32) {
-      const float d = vsum ? Xs[c] - __bfloat162float(V[((size_t)unit * dm.cap + slot) * D + c]) : part[0][c] / H;
+    for (int ch = tid; ch < D; ch += 32) {
+      const float d = vsum ? Xs[ch] - __bfloat162float(V[((size_t)unit * dm.cap + slot) * D + ch]) : part[0][ch] / H;
       d2 = fmaf(d, d, d2);
     }
     d2 = warp_sum(d2);
