@@ -108,7 +108,8 @@ typedef struct {
 /* Bytes of scratch that caote_score / caote_select_evict / caote_compact / caote_append need for these
  * parameters (the maximum over the four; one buffer serves all). Returns 0 if params is invalid.
  * The first 256 bytes hold the status word and the library's own counters; zero them once
- * (cudaMemsetAsync) before first use and leave them alone afterwards. */
+ * (cudaMemsetAsync) before first use and leave them alone afterwards. Calls that may overlap (streams without an
+ * ordering between them) need workspaces of their own, but for caote_compact, which does not use it. */
 CAOTE_API size_t caote_workspace_bytes(const caote_params_t* params);
 
 /* Append the m = n_new newest tokens of every sequence to its cache (Sec. 2: the block
@@ -195,7 +196,9 @@ CAOTE_API int caote_select_evict(const caote_params_t* params, const float* scor
  *   evict_idx[u, 0..k) out: the evicted slots in ascending order (what caote_compact takes);
  *   order[u, 0..k) out, nullable: the same slots in the order they were evicted;  n_evict[b] = k out.
  * capacity <= 24576 (the unit's weights and distances stay in shared memory), else CAOTE_ERR_UNSUPPORTED.
- * Cost: one sweep over the unit's value rows per eviction (from L2 after the first). */
+ * Cost: two sweeps over the unit's value rows (its output, the distances of all tokens), one more whenever the bounds on the
+ * tokens looked at no longer settle a pick (many hundreds of evictions, or weights that hold nearly all of the sum), and per
+ * eviction the rows of the few tokens that can be the minimum. */
 CAOTE_API int caote_select_evict_greedy(const caote_params_t* params, const void* V, const float* h,
                               const int32_t* len, const int32_t* budget, const int32_t* pos,
                               int32_t* evict_idx, int32_t* order, int32_t max_evict, int32_t* n_evict,
@@ -210,8 +213,10 @@ CAOTE_API int caote_compact(const caote_params_t* params, void* K, void* V, floa
                   int32_t mode, void* workspace, size_t workspace_bytes, caote_stream_t stream);
 
 /* One whole eviction step on the stream: caote_append (skipped when k_new is NULL), caote_score,
- * caote_select_evict, caote_compact, with the same arguments and the same results as the four
- * separate calls. */
+ * caote_select_evict, caote_compact, with the same arguments and the results of the four separate calls up to
+ * rounding: a kernel that does a whole step of single queries adds up in another order than the scoring call does, and
+ * takes bf16 groups of more than 8 heads (8 with ACCUM or EXTERNAL) on short caches in fp32, where caote_score has them on the
+ * tensor cores (o to about 5e-6 of its size). Tokens whose scores tie within that may be picked differently. */
 CAOTE_API int caote_step(const caote_params_t* params, const void* q, const void* k_new, const void* v_new,
                void* K, void* V, float* base, int32_t* pos, int32_t* len, int32_t* n_seen,
                const int32_t* budget, float* o, float* scores, int32_t* evict_idx, int32_t max_evict,

@@ -1,8 +1,8 @@
 """A budgeted KV cache driven through the C ABI: the call a user of the library makes per step.
 
 Holds the caller-owned device buffers (K, V, base, pos, len, scores, ...) and forwards each step to
-``caote_step`` (append the new tokens, score, select, compact), or, for the variants that have no fused entry
-point, to the same calls one after the other. No arithmetic happens here.
+``caote_step`` (append the new tokens, score, select, compact) or to the whole-step entry point of its variant. No
+arithmetic happens here.
 
 method: "caote" (Sec. 3.2 score), "fast" (FastCAOTE, Sec. 3.3), "sum_errors" (the per-row errors added up),
 "post_evict" (the "caote" step that also returns the attention output over the retained tokens, Sec. 3.1).

@@ -681,10 +681,12 @@ static int launch_sum_errors_decode(const Dims& dm, const void* q, const void* K
   }
 }
 
-// Shapes the tensor-core row-block kernels take: bf16, whatever the single-query kernels do not. The any-shape kernels
-// (fp32 on the CUDA cores, 5 - 7 TFLOP/s) are left with fp32 inputs. Steps measured on both: blocks of 128 with the last
-// query's weights, 16 units of 6128 tokens: 7.07 -> 0.256 ms; with carried weights, 32 units of about 7.3 k: 8.67 -> 0.237
-// ms; one query, head_dim 64, 128 units of about 3.6 k: 0.276 -> 0.168 ms; blocks of a few queries, 2 - 7 times faster.
+// Shapes the tensor-core row-block kernels take: bf16, whatever the single-query kernels do not. The any-shape kernels (fp32
+// on the CUDA cores, 16 TFLOP/s on blocks of rows) are left with fp32 inputs, sums of errors over blocks of queries, and
+// scales that are not positive. Scoring calls on both, us: blocks of 128 with the last query's weights, 16 units of 6 128
+// tokens 1 748, 99; with carried weights, 32 units of 7 300: 3 354, 171; head_dim 64, 64 units of 2 000: 1 052, 95; one query at
+// head_dim 64 on units longer than the largest cluster holds, 8 of 20 000: 140, 55, 32: 355, 195; blocks of 4 queries, 8 units
+// of 4 100: 83, 29, 64 at head_dim 64: 170, 71; 16 heads per group, 8 units of 4 100: 83, 29.
 static bool prefill_shape_ok(const caote_params_t* p) {
   return !decode_shape_ok(p) && p->dtype == CAOTE_BF16 && p->scale > 0.f && (long long)p->batch * p->n_kv_heads * p->capacity < (1LL << 31) &&
          (long long)p->batch * p->n_q_heads * p->n_new < (1LL << 31);
