@@ -362,7 +362,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   constexpr int kBars = 1 + 2 * (kKStages + kVStages) + 6;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kBars);
 
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = ptx::warp_index();
   const int unit = blockIdx.y, row0 = blockIdx.x * kTile;
   const int b = unit / dm.Hkv;
   const int n = len[b], M = dm.R, m = dm.m;
@@ -405,7 +405,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 
   if (warp == 9) {
     // =============================== K loads (one lane) ===============================
-    if (tid == kRowThreads + 32) {
+    if (ptx::elect_one()) {
       mbar_expect_tx(q_bar, kTB);
 #pragma unroll
       for (int x = 0; x < kBoxes; ++x) tma_load_2d(Qs + x * kHalfBytes, &tmQ, 64 * x, unit * M + row0, q_bar);
@@ -419,7 +419,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     }
   } else if (warp == 10) {
     // =============================== V loads (one lane) ===============================
-    if (tid == kRowThreads + 64) {
+    if (ptx::elect_one()) {
       for (int kt = 0; kt < ntiles; ++kt) {
         const int st = kt % kVStages, row = unit * dm.cap + (kt0 + kt) * kKeys;
         if (kt >= kVStages) mbar_wait_idle(&v_free[st], ((kt / kVStages) - 1) & 1, status);  // O += P V of tile kt - 2 is done
@@ -430,36 +430,34 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     }
   } else if (warp == 8) {
     // =============================== products (one lane) ===============================
-    if (tid == kRowThreads) {
+    if (ptx::elect_one()) {
       constexpr uint32_t kIdescS = instr_desc_n(false, kKeys), kIdescO = instr_desc_n(true, D);
       const uint32_t q_addr = smem_u32(Qs);
-      // Descriptors are built once; inside the loop a product costs one 64-bit add per operand (the
-      // single issuing thread is bound by the latency of its own instruction stream, not by the pipe).
-      uint64_t qdesc[kSteps];
-#pragma unroll
-      for (int ks = 0; ks < kSteps; ++ks) qdesc[ks] = desc_k_major(q_addr, ks);
+      const uint64_t qdesc0 = smem_desc(q_addr, 16, 1024);
       const uint64_t kdesc0 = smem_desc(smem_u32(Ksm), 16, 1024);
       const uint64_t vdesc0 = smem_desc(smem_u32(Vsm), kKvHalf, 1024);
       auto issue_qk = [&](int kt) {
-        mbar_wait_idle(&k_bar[kt % kKStages], (kt / kKStages) & 1, status);
+        mbar_wait(&k_bar[kt % kKStages], (kt / kKStages) & 1, status);
         tc_fence_after();
         const uint64_t kd = kdesc0 + (uint64_t)(((kt % kKStages) * kTB) >> 4);
         const uint32_t d_s = tmem + (kt & 1) * kKeys;  // S0 or S1
 #pragma unroll
-        for (int ks = 0; ks < kSteps; ++ks)
-          umma(d_s, qdesc[ks], kd + (uint64_t)((((ks >> 2) * kKvHalf) + (ks & 3) * 32) >> 4), kIdescS, ks > 0);
+        for (int ks = 0; ks < kSteps; ++ks) {
+          const uint64_t off = (uint64_t)((((ks >> 2) * kKvHalf) + (ks & 3) * 32) >> 4);  // (boxes of Q and K are alike)
+          umma(d_s, qdesc0 + off, kd + off, kIdescS, ks > 0);
+        }
         umma_commit(&s_bar[kt & 1]);
         umma_commit(&k_free[kt % kKStages]);
       };
-      mbar_wait_idle(q_bar, 0, status);
+      mbar_wait(q_bar, 0, status);
       issue_qk(0);
       for (int kt = 0; kt < ntiles; ++kt) {
         // queue S of the next tile: its buffer was read by the softmax of tile kt - 1, which has
         // arrived on p_bar before PV(kt - 1) was issued
         if (kt + 1 < ntiles) issue_qk(kt + 1);
         // O += P V once the rows have written P of this tile
-        mbar_wait_idle(&p_bar[kt & 1], (kt >> 1) & 1, status);
-        mbar_wait_idle(&v_bar[kt % kVStages], (kt / kVStages) & 1, status);
+        mbar_wait(&v_bar[kt % kVStages], (kt / kVStages) & 1, status);
+        mbar_wait(&p_bar[kt & 1], (kt >> 1) & 1, status);
         tc_fence_after();
         const uint64_t vd = vdesc0 + (uint64_t)(((kt % kVStages) * kTB) >> 4);
         const uint32_t p_tmem = tmem + (kt & 1) * kKeys;
@@ -1041,7 +1039,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   constexpr int kBars = kBars1 + 4 + kSStages;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kBars);
 
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = ptx::warp_index();
   const bool last_only = kFew && dm.base_mode == CAOTE_BASE_LAST_QUERY;
   const int M = kFew ? sc.Ms : dm.R, m = last_only ? 1 : dm.m;  // counted rows, and the block they are causal in
   const int nblocks = (M + kTile - 1) / kTile;
@@ -1104,7 +1102,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     }
   } else if (warp == 18) {
     // =============================== copies of Q and the statistics (one lane) ===============================
-    if (tid == kKeyThreads + 64) {
+    if (ptx::elect_one()) {
       int qb = 0;
       while (next()) {
         const float* rstat = last_only ? sc.sstat + (size_t)unit * kTile : sc.stats + (size_t)unit * sc.Mpad;
@@ -1124,24 +1122,26 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     }
   } else if (warp == 16) {
     // =============================== products (one lane) ===============================
-    if (tid == kKeyThreads) {
+    if (ptx::elect_one()) {
       constexpr uint32_t kIdesc = instr_desc(false);
       int qb = 0;
       for (int c = 0; next(); ++c) {
         const int kb = c & 1;
-        const uint32_t k_addr = smem_u32(KVs + 2 * kb * kTB);
+        const uint64_t kd0 = smem_desc(smem_u32(KVs + 2 * kb * kTB), 16, 1024);
         mbar_wait_idle(&k_full[kb], (c >> 1) & 1, status);
         for (int rb = 0; rb < nblocks; ++rb, ++qb) {
           const int buf = qb & 1, st = qb % kQStages;
           mbar_wait_idle(&q_full[st], (qb / kQStages) & 1, status);
           if (qb >= 2) mbar_wait_idle(&c_bar[buf], ((qb - 2) >> 1) & 1, status);  // its S buffers have been read
           tc_fence_after();
-          const uint32_t q_addr = smem_u32(Qst + st * kTB);
+          const uint64_t qd0 = smem_desc(smem_u32(Qst + st * kTB), 16, 1024);
 #pragma unroll
           for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
-            for (int ks = 0; ks < kSteps; ++ks)
-              umma(tmem + kk * 256 + buf * 128, desc_k_major(k_addr + kk * kTB, ks), desc_k_major(q_addr, ks), kIdesc, ks > 0);
+            for (int ks = 0; ks < kSteps; ++ks) {
+              const uint64_t off = (uint64_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4);
+              umma(tmem + kk * 256 + buf * 128, kd0 + (uint64_t)((kk * kTB) >> 4) + off, qd0 + off, kIdesc, ks > 0);
+            }
           }
           umma_commit(&s_bar[buf]);
           umma_commit(&q_done[st]);
