@@ -207,12 +207,6 @@ __device__ __forceinline__ float fast_sqrt(float x) {
   return y;
 }
 
-// k-step ks of the query operand: two boxes of 8 rows x 128 bytes, 1024 bytes apart. The product reads 16
-// rows (N = 16); rows 8..15 fall on whatever follows in shared memory and only feed unused columns.
-__device__ __forceinline__ uint64_t desc_q(uint32_t addr, int ks) {
-  return prefill::smem_desc(addr + (ks >> 2) * 1024 + (ks & 3) * 32, 16, 1024);
-}
-
 // (sum of the others, largest, its logit) of two disjoint sets of tokens -> of their union.
 __device__ __forceinline__ void top_merge(float& l, float& p, float& s, float ol, float op, float os) {
   const bool mine = s >= os;
@@ -306,7 +300,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(ctl) + 4);
   float* xword = reinterpret_cast<float*>(tmem_slot + 1);              // where the peers' "done reading" words land
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = ptx::warp_index();
   constexpr int G = kG, mode = kMode;
   constexpr bool use_base = (mode == CAOTE_BASE_ACCUM || mode == CAOTE_BASE_EXTERNAL);
   constexpr bool counted = (mode != CAOTE_BASE_EXTERNAL);
@@ -386,7 +380,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 
   if (warp == kWarpK) {
     // ================================ K copies (one lane) ================================
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       const uint64_t pol = decode::policy_evict_first();
       int ki = 0, us = 0;
       for (int k = 0; k < nk && !ctl[0]; ++k) {
@@ -416,7 +410,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     }
   } else if (warp == kWarpV) {
     // ================================ V copies (one lane) ================================
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       const uint64_t pol = decode::policy_evict_first();
       int vi = 0;
       for (int k = 0; k < nk && !ctl[0]; ++k) {
@@ -440,23 +434,27 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     }
   } else if (warp == kWarpQK) {
     // ================================ S^T products (one lane) ================================
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       constexpr uint32_t kIdQK = idesc_n16(false);
       int ki = 0, us = 0;
       for (int k = 0; k < nk && !ctl[0]; ++k) {
         const Work w = sch.at(k);
         if (!w.ok || w.T == 0) continue;
-        const uint32_t qa = smem_u32(qbuf + (us & 1) * kQBufBytes);
+        const uint64_t qd = prefill::smem_desc(smem_u32(qbuf + (us & 1) * kQBufBytes), 16, 1024);
         for (int j = 0; j < w.T; ++j) {
           const int s = ki % kKS, sb = ki % kSB;
           wait_bounded(&kfull[s], (ki / kKS) & 1, &ctl[0], status, wait_cycles, true);
           wait_bounded(&sfree[sb], ((ki / kSB) & 1) ^ 1, &ctl[0], status, wait_cycles, true);
           if (ctl[0]) break;
           prefill::tc_fence_after();
-          const uint32_t ka = smem_u32(tilesK + s * kTileBytes);
+          // (k-step ks of the tile: 32 bytes on, in the second box after four; of the query operand: two boxes of 8 rows x 128
+          // bytes, 1024 bytes apart. The product reads 16 rows (N = 16); rows 8..15 fall on whatever follows in shared memory
+          // and only feed unused columns.)
+          const uint64_t kd = prefill::smem_desc(smem_u32(tilesK + s * kTileBytes), 16, 1024);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            prefill::umma(tS + sb * 16, prefill::desc_k_major(ka, ks), desc_q(qa, ks), kIdQK, ks > 0);
+            prefill::umma(tS + sb * 16, kd + (uint64_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4),
+                          qd + (uint64_t)(((ks >> 2) * 1024 + (ks & 3) * 32) >> 4), kIdQK, ks > 0);
           prefill::umma_commit(&sfull[sb]);
           prefill::umma_commit(&kempty[s]);
           if (j == w.T - 1) prefill::umma_commit(&qfree[us & 1]);
@@ -470,9 +468,9 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     }
   } else if (warp == kWarpPV) {
     // ================================ O^T products (one lane) ================================
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       constexpr uint32_t kIdPV = idesc_n16(true);
-      const uint32_t pa = smem_u32(pbuf);
+      const uint64_t pd = prefill::smem_desc(smem_u32(pbuf), 16, 1024);
       int vi = 0;
       for (int k = 0; k < nk && !ctl[0]; ++k) {
         const Work w = sch.at(k);
@@ -483,10 +481,12 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           wait_bounded(pfull, vi & 1, &ctl[0], status, wait_cycles, false);
           if (ctl[0]) break;
           prefill::tc_fence_after();
-          const uint32_t va = smem_u32(tilesV + s * kTileBytes);
+          // (16 tokens of the tile: 2048 bytes; of P^T: 32 bytes, in the second of its two boxes after four)
+          const uint64_t vd = prefill::smem_desc(smem_u32(tilesV + s * kTileBytes), kHalfBytes, 1024);
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)  // the unit's first tile starts a new sum
-            prefill::umma(tO, prefill::desc_mn_major(va, kk), decode::desc_rows16(pa, kk), kIdPV, !(j == 0 && kk == 0));
+            prefill::umma(tO, vd + (uint64_t)(kk * 2048 >> 4), pd + (uint64_t)(((kk >> 2) * 2048 + (kk & 3) * 32) >> 4), kIdPV,
+                          !(j == 0 && kk == 0));
           prefill::umma_commit(odone);
           prefill::umma_commit(&vempty[s]);
           ++vi;
