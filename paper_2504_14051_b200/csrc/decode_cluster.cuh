@@ -453,7 +453,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           const uint64_t kd = prefill::smem_desc(smem_u32(tilesK + s * kTileBytes), 16, 1024);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            prefill::umma(tS + sb * 16, kd + (uint64_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4),
+            prefill::umma(tS + sb * 16, kd + prefill::k_major_step(ks),
                           qd + (uint64_t)(((ks >> 2) * 1024 + (ks & 3) * 32) >> 4), kIdQK, ks > 0);
           prefill::umma_commit(&sfull[sb]);
           prefill::umma_commit(&kempty[s]);
@@ -485,8 +485,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           const uint64_t vd = prefill::smem_desc(smem_u32(tilesV + s * kTileBytes), kHalfBytes, 1024);
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)  // the unit's first tile starts a new sum
-            prefill::umma(tO, vd + (uint64_t)(kk * 2048 >> 4), pd + (uint64_t)(((kk >> 2) * 2048 + (kk & 3) * 32) >> 4), kIdPV,
-                          !(j == 0 && kk == 0));
+            prefill::umma(tO, vd + prefill::mn_major_step(kk), pd + decode::rows16_step(kk), kIdPV, !(j == 0 && kk == 0));
           prefill::umma_commit(odone);
           prefill::umma_commit(&vempty[s]);
           ++vi;

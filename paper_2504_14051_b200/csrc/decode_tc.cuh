@@ -139,11 +139,9 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float x0, float x1) {
 __host__ __device__ constexpr uint32_t idesc_n16(bool a_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn_major ? 1u : 0u) << 15) | ((16u >> 3) << 17) | ((128u >> 4) << 24);
 }
-// k-step ks (16 of 128 contraction elements) of a 16-row K-major operand staged as two boxes of
+// What k-step ks (16 of 128 contraction elements) adds to the descriptor of a 16-row K-major operand staged as two boxes of
 // 16 rows x 128 bytes (128-byte swizzle): 8-row groups 1024 bytes apart, boxes 2048 bytes apart.
-__device__ __forceinline__ uint64_t desc_rows16(uint32_t addr, int ks) {
-  return prefill::smem_desc(addr + (ks >> 2) * 2048 + (ks & 3) * 32, 16, 1024);
-}
+__device__ __forceinline__ uint64_t rows16_step(int ks) { return (uint64_t)(((ks >> 2) * 2048 + (ks & 3) * 32) >> 4); }
 
 struct Entry {  // a work item a producer is feeding into its ring
   int item, unit, item0, nitems, n, t_begin, t_end;
@@ -205,7 +203,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                                                                          // [2] / [3] slots issued in ring A / B
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(ctl) + 4);
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = ptx::warp_index();
   const int G = dm.G, mode = dm.base_mode;
   const bool use_base = (mode == CAOTE_BASE_ACCUM || mode == CAOTE_BASE_EXTERNAL);
   const bool softmax_counted = (mode != CAOTE_BASE_EXTERNAL);
@@ -393,7 +391,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     }
   } else if (warp == kTcIssueWarp) {
     // ================================ issuing warp (one lane) ================================
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       constexpr uint32_t kIdQK = idesc_n16(false), kIdPV = idesc_n16(true);
       int a_cnt = 0;         // attention tiles whose S^T product has been queued
       int pv_cnt = 0;        // attention tiles whose O^T product has been queued
@@ -401,12 +399,13 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
       int qk_queued = -1;    // ring index of the last K slot whose product has been queued
       auto issue_qk = [&](int s, const Desc& d) {
         if (d.flags & kFlagFirst) ++q_items;
-        const uint32_t ka = smem_u32(tilesA + s * kTileBytes);
-        const uint32_t qa = smem_u32(qbuf + ((q_items - 1) % kQ) * kQBytes);
+        const uint64_t kd = prefill::smem_desc(smem_u32(tilesA + s * kTileBytes), 16, 1024);
+        const uint64_t qd = prefill::smem_desc(smem_u32(qbuf + ((q_items - 1) % kQ) * kQBytes), 16, 1024);
         prefill::tc_fence_after();
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks)
-          prefill::umma(tS + (a_cnt & 1) * 16, prefill::desc_k_major(ka, ks), desc_rows16(qa, ks), kIdQK, ks > 0);
+          prefill::umma(tS + (a_cnt & 1) * 16, kd + prefill::k_major_step(ks), qd + rows16_step(ks), kIdQK,
+                        ks > 0);
         prefill::umma_commit(&s_bar[a_cnt & 1]);
         prefill::umma_commit(&emptyA[s]);  // this lane's arrival on the K slot: once the product has read it
         ++a_cnt;
@@ -436,12 +435,12 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
           wait_or_stop(&p_bar[pv_cnt & 1], (pv_cnt >> 1) & 1, &ctl[0], status);
           if (ctl[0]) break;
           prefill::tc_fence_after();
-          const uint32_t va = smem_u32(tilesA + s * kTileBytes);
-          const uint32_t pa = smem_u32(pbuf + (pv_cnt & 1) * kPBytes);
+          const uint64_t vd = prefill::smem_desc(smem_u32(tilesA + s * kTileBytes), kHalfBytes, 1024);
+          const uint64_t pd = prefill::smem_desc(smem_u32(pbuf + (pv_cnt & 1) * kPBytes), 16, 1024);
           const bool first = (d.flags & kFlagFirst) != 0;
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)
-            prefill::umma(tO, prefill::desc_mn_major(va, kk), desc_rows16(pa, kk), kIdPV, !(first && kk == 0));
+            prefill::umma(tO, vd + prefill::mn_major_step(kk), pd + rows16_step(kk), kIdPV, !(first && kk == 0));
           prefill::umma_commit(&o_bar[pv_cnt & 1]);
           prefill::umma_commit(&emptyA[s]);  // this lane's arrival: once the product has read the V tile
           ++pv_cnt;

@@ -159,7 +159,7 @@ post_evict_tc_kernel(Dims dm, const __nv_bfloat16* __restrict__ q, const __nv_bf
   const int unit = blockIdx.y, b = unit / dm.Hkv;
   const int n = len[b], m = dm.m, k = n_evict[b];
   if (n <= 0 || n < m || n > dm.cap) return;
-  const int tid = threadIdx.x, warp = tid >> 5, r0 = blockIdx.x * kTile;
+  const int tid = threadIdx.x, warp = ptx::warp_index(), r0 = blockIdx.x * kTile;
   const int half = tid >> 7, r = r0 + (tid & (kTile - 1));
   const __nv_bfloat16* Ku = K + (size_t)unit * dm.cap * D;
   const __nv_bfloat16* Vu = V + (size_t)unit * dm.cap * D;
@@ -205,11 +205,11 @@ post_evict_tc_kernel(Dims dm, const __nv_bfloat16* __restrict__ q, const __nv_bf
     }
     fence_async_smem();
     __syncthreads();
-    if (tid == 0) {
+    if (warp == 0 && ptx::elect_one()) {
       tc_fence_after();
+      const uint64_t qd = smem_desc(smem_u32(Qs), 16, 1024), kd = smem_desc(smem_u32(Ks), 16, 1024);
 #pragma unroll
-      for (int ks = 0; ks < D / 16; ++ks)
-        umma(tmem, desc_k_major(smem_u32(Qs), ks), desc_k_major(smem_u32(Ks), ks), instr_desc_n(false, kTile), ks > 0);
+      for (int ks = 0; ks < D / 16; ++ks) umma(tmem, qd + k_major_step(ks), kd + k_major_step(ks), instr_desc_n(false, kTile), ks > 0);
       umma_commit(s_bar);
     }
     mbar_wait(s_bar, t & 1, status);
@@ -238,13 +238,14 @@ post_evict_tc_kernel(Dims dm, const __nv_bfloat16* __restrict__ q, const __nv_bf
     tmem_st_wait();
     tc_fence_before();
     __syncthreads();
-    if (tid == 0) {
+    if (warp == 0 && ptx::elect_one()) {
       tc_fence_after();
       constexpr uint32_t kIdesc = instr_desc_n(true, D);
+      const uint64_t vd = smem_desc(smem_u32(Vs), kHalfBytes, 1024);
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks) {
-        umma_ts(tmem + kTile, tmem + ks * 8, desc_mn_major(smem_u32(Vs), ks), kIdesc, t > 0 || ks > 0);
-        umma_ts(tmem + kTile, tmem + 64 + ks * 8, desc_mn_major(smem_u32(Vs), ks), kIdesc, true);
+        umma_ts(tmem + kTile, tmem + ks * 8, vd + mn_major_step(ks), kIdesc, t > 0 || ks > 0);
+        umma_ts(tmem + kTile, tmem + 64 + ks * 8, vd + mn_major_step(ks), kIdesc, true);
       }
       umma_commit(y_bar);
     }

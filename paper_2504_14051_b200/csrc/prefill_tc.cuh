@@ -288,16 +288,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float x0, float x1) {
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(x1), "f"(x0));
   return r;
 }
-// Descriptors of k-step ks (16 of the 128 contraction elements) of a staged tile.
-//   K-major: contraction along the 128-byte rows: 32 bytes per step inside a box, second box after 4.
-//   MN-major: contraction along the rows of the tile (16 rows = 2 groups of 8 = 2048 bytes per
-//   step); the two 64-element boxes along MN are kHalfBytes apart (leading byte offset).
-__device__ __forceinline__ uint64_t desc_k_major(uint32_t tile_addr, int ks) {
-  return smem_desc(tile_addr + (ks >> 2) * kHalfBytes + (ks & 3) * 32, 16, 1024);
-}
-__device__ __forceinline__ uint64_t desc_mn_major(uint32_t tile_addr, int ks) {
-  return smem_desc(tile_addr + ks * 2048, kHalfBytes, 1024);
-}
+// What k-step ks (16 of the 128 contraction elements) adds to the descriptor of a staged tile.
+//   K-major (leading byte offset 16): contraction along the 128-byte rows: 32 bytes per step inside a box, second box after 4.
+//   MN-major (leading byte offset kHalfBytes): contraction along the rows of the tile (16 rows = 2 groups of 8 = 2048 bytes per
+//   step); the two 64-element boxes along MN are kHalfBytes apart.
+__device__ __forceinline__ uint64_t k_major_step(int ks) { return (uint64_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4); }
+__device__ __forceinline__ uint64_t mn_major_step(int ks) { return (uint64_t)(ks * 2048 >> 4); }
 
 
 // ---- attention pass ---------------------------------------------------------------------------------
@@ -442,10 +438,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         const uint64_t kd = kdesc0 + (uint64_t)(((kt % kKStages) * kTB) >> 4);
         const uint32_t d_s = tmem + (kt & 1) * kKeys;  // S0 or S1
 #pragma unroll
-        for (int ks = 0; ks < kSteps; ++ks) {
-          const uint64_t off = (uint64_t)((((ks >> 2) * kKvHalf) + (ks & 3) * 32) >> 4);  // (boxes of Q and K are alike)
-          umma(d_s, qdesc0 + off, kd + off, kIdescS, ks > 0);
-        }
+        for (int ks = 0; ks < kSteps; ++ks) umma(d_s, qdesc0 + k_major_step(ks), kd + k_major_step(ks), kIdescS, ks > 0);
         umma_commit(&s_bar[kt & 1]);
         umma_commit(&k_free[kt % kKStages]);
       };
@@ -469,8 +462,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         umma_ts(tmem + 256, p_tmem + 64, vd, kIdescO, true);
 #pragma unroll
         for (int ks = 1; ks < 8; ++ks) {  // 16 keys = 8 packed columns per step
-          umma_ts(tmem + 256, p_tmem + ks * 8, vd + (uint64_t)((ks * 2048) >> 4), kIdescO, true);
-          umma_ts(tmem + 256, p_tmem + 64 + ks * 8, vd + (uint64_t)((ks * 2048) >> 4), kIdescO, true);
+          umma_ts(tmem + 256, p_tmem + ks * 8, vd + mn_major_step(ks), kIdescO, true);
+          umma_ts(tmem + 256, p_tmem + 64 + ks * 8, vd + mn_major_step(ks), kIdescO, true);
         }
         umma_commit(&o_bar[kt & 1]);
         umma_commit(&v_free[kt % kVStages]);
@@ -1138,10 +1131,8 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 #pragma unroll
           for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
-            for (int ks = 0; ks < kSteps; ++ks) {
-              const uint64_t off = (uint64_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4);
-              umma(tmem + kk * 256 + buf * 128, kd0 + (uint64_t)((kk * kTB) >> 4) + off, qd0 + off, kIdesc, ks > 0);
-            }
+            for (int ks = 0; ks < kSteps; ++ks)
+              umma(tmem + kk * 256 + buf * 128, kd0 + (uint64_t)((kk * kTB) >> 4) + k_major_step(ks), qd0 + k_major_step(ks), kIdesc, ks > 0);
           }
           umma_commit(&s_bar[buf]);
           umma_commit(&q_done[st]);
