@@ -230,6 +230,25 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
+// 64 consecutive columns: half a row of S.
+__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x64.b32 {"
+      "%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, "
+      "%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, "
+      "%48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
+        "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]),
+        "=f"(v[16]), "=f"(v[17]), "=f"(v[18]), "=f"(v[19]), "=f"(v[20]), "=f"(v[21]), "=f"(v[22]), "=f"(v[23]),
+        "=f"(v[24]), "=f"(v[25]), "=f"(v[26]), "=f"(v[27]), "=f"(v[28]), "=f"(v[29]), "=f"(v[30]), "=f"(v[31]),
+        "=f"(v[32]), "=f"(v[33]), "=f"(v[34]), "=f"(v[35]), "=f"(v[36]), "=f"(v[37]), "=f"(v[38]), "=f"(v[39]),
+        "=f"(v[40]), "=f"(v[41]), "=f"(v[42]), "=f"(v[43]), "=f"(v[44]), "=f"(v[45]), "=f"(v[46]), "=f"(v[47]),
+        "=f"(v[48]), "=f"(v[49]), "=f"(v[50]), "=f"(v[51]), "=f"(v[52]), "=f"(v[53]), "=f"(v[54]), "=f"(v[55]),
+        "=f"(v[56]), "=f"(v[57]), "=f"(v[58]), "=f"(v[59]), "=f"(v[60]), "=f"(v[61]), "=f"(v[62]), "=f"(v[63])
+      : "r"(taddr) : "memory");
+}
 // The same load of 16 columns without the wait, and the wait as a statement that the registers pass through: whatever reads
 // them afterwards depends on the wait, so the compiler cannot move such a read in front of it. Between the two
 // the thread may do anything that does not touch r.
@@ -354,11 +373,11 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   float* xch = reinterpret_cast<float*>(Vsm + kVStages * kTB);  // [kXchFloats]
   uint64_t* bars = reinterpret_cast<uint64_t*>(xch + kXchFloats);
   uint64_t *q_bar = &bars[0], *k_bar = &bars[1], *v_bar = k_bar + kKStages, *s_bar = v_bar + kVStages, *o_bar = s_bar + 2,
-           *p_bar = o_bar + 2, *k_free = p_bar + 2, *v_free = k_free + kKStages;
-  constexpr int kBars = 1 + 2 * (kKStages + kVStages) + 6;
+           *p_bar = o_bar + 2, *k_free = p_bar + 4, *v_free = k_free + kKStages;  // p_bar: [part][tile parity]
+  constexpr int kBars = 1 + 2 * (kKStages + kVStages) + 8;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kBars);
 
-  const int tid = threadIdx.x, warp = ptx::warp_index();
+  const int tid = threadIdx.x, lane = tid & 31, warp = ptx::warp_index();
   const int unit = blockIdx.y, row0 = blockIdx.x * kTile;
   const int b = unit / dm.Hkv;
   const int n = len[b], M = dm.R, m = dm.m;
@@ -386,8 +405,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 
   if (tid == 0) {
     for (int i = 0; i < kBars; ++i) mbar_init(&bars[i], 1);
-    mbar_init(&p_bar[0], kRowThreads);
-    mbar_init(&p_bar[1], kRowThreads);
+    for (int i = 0; i < 4; ++i) mbar_init(&p_bar[i], kRowThreads / 32);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tmem_alloc(tmem_slot, 512);
@@ -448,22 +466,20 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         // queue S of the next tile: its buffer was read by the softmax of tile kt - 1, which has
         // arrived on p_bar before PV(kt - 1) was issued
         if (kt + 1 < ntiles) issue_qk(kt + 1);
-        // O += P V once the rows have written P of this tile
+        // O += P V as the rows write P of this tile: the first 32 keys of either half, then the others
         mbar_wait(&v_bar[kt % kVStages], (kt / kVStages) & 1, status);
-        mbar_wait(&p_bar[kt & 1], (kt >> 1) & 1, status);
-        tc_fence_after();
         const uint64_t vd = vdesc0 + (uint64_t)(((kt % kVStages) * kTB) >> 4);
         const uint32_t p_tmem = tmem + (kt & 1) * kKeys;
-        if (kt % kShare == 0) {  // a new share
-          umma_ts(tmem + 256, p_tmem, vd, kIdescO, false);
-        } else {
-          umma_ts(tmem + 256, p_tmem, vd, kIdescO, true);
-        }
-        umma_ts(tmem + 256, p_tmem + 64, vd, kIdescO, true);
 #pragma unroll
-        for (int ks = 1; ks < 8; ++ks) {  // 16 keys = 8 packed columns per step
-          umma_ts(tmem + 256, p_tmem + ks * 8, vd + mn_major_step(ks), kIdescO, true);
-          umma_ts(tmem + 256, p_tmem + 64 + ks * 8, vd + mn_major_step(ks), kIdescO, true);
+        for (int part = 0; part < 2; ++part) {
+          mbar_wait(&p_bar[2 * part + (kt & 1)], (kt >> 1) & 1, status);
+          tc_fence_after();
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {  // 16 keys = 8 packed columns per step
+            const int ks = (i >> 1) * 4 + 2 * part + (i & 1);
+            umma_ts(tmem + 256, p_tmem + ks * 8, vd + mn_major_step(ks), kIdescO, ks > 0 || kt % kShare > 0);  // (a new share starts at 0)
+            umma_ts(tmem + 256, p_tmem + 64 + ks * 8, vd + mn_major_step(ks), kIdescO, true);
+          }
         }
         umma_commit(&o_bar[kt & 1]);
         umma_commit(&v_free[kt % kVStages]);
@@ -488,14 +504,19 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     const bool counted = kFew && R < M && row_counted(dm, R);
     const bool keep_top = kFew && __any_sync(0xffffffffu, counted);
 
+    if (ntiles > kShare) {  // the sum of finished shares starts at 0
+      const uint32_t zero[16] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int cc = 0; cc < D / 32; ++cc) tmem_st16u(t_o + 128 + cc * 16, zero);
+      tmem_st_wait();
+    }
     for (int kt = 0; kt < ntiles; ++kt) {
       mbar_wait(&s_bar[kt & 1], (kt >> 1) & 1, status);
       tc_fence_after();
       const int j0 = (kt0 + kt) * kKeys + half * 64;  // first key of this thread's half
       const uint32_t t_s = t_lane + (kt & 1) * kKeys + half * 64;
       float sv[64];  // raw products; masked keys become -inf
-      tmem_ld32(t_s, *reinterpret_cast<float(*)[32]>(&sv[0]));
-      tmem_ld32(t_s + 32, *reinterpret_cast<float(*)[32]>(&sv[32]));
+      tmem_ld64(t_s, sv);
       if ((kt0 + kt) * kKeys + kKeys > n - m + 1) {  // only tiles that reach into the new block (or past the length) need the mask
 #pragma unroll
         for (int i = 0; i < 64; ++i) sv[i] = (j0 + i < nvis) ? sv[i] : -INFINITY;
@@ -504,90 +525,94 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       {
         float pm[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) pm[i] = sv[i];
+        for (int i = 0; i < 8; ++i) pm[i] = fmaxf(sv[i], sv[i + 8]);
 #pragma unroll
-        for (int i = 8; i < 64; ++i) pm[i & 7] = fmaxf(pm[i & 7], sv[i]);
+        for (int i = 16; i < 64; i += 16) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) pm[e] = fmaxf(fmaxf(pm[e], sv[i + e]), sv[i + 8 + e]);
+        }
         raw_top = fmaxf(fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3])), fmaxf(fmaxf(pm[4], pm[5]), fmaxf(pm[6], pm[7])));
       }
       float mx = raw_top * scale2;
-      // the other half of the row
+      // the other half of the row (the two warps that share 32 rows meet here)
       float* xm = xch + (kt & 1) * kRowThreads;
       xm[tid] = mx;
-      asm volatile("bar.sync 1, %0;" ::"n"(kRowThreads) : "memory");
+      asm volatile("bar.sync %0, 64;" ::"r"(2 + (warp & 3)) : "memory");
       mx = fmaxf(mx, xm[tid ^ kThreads]);
       // the reference moves only when a logit exceeds it by more than 8 (p <= 256 in between)
       const bool need = mx > m_ref + 8.f;
       const bool close = kt > 0 && kt % kShare == 0;  // O holds a finished share
-      if (close || __any_sync(0xffffffffu, need)) {
-        const float corr = need ? fast_exp2(m_ref - mx) : 1.f;
-        if (need) m_ref = mx;
+      float corr = 1.f;
+      if (need) {
+        corr = fast_exp2(m_ref - mx);
+        m_ref = mx;
         l *= corr;
         if (kFew) { ptop *= corr; lrest *= corr; }
-        if (kt > 0) {
-          mbar_wait(&o_bar[(kt - 1) & 1], ((kt - 1) >> 1) & 1, status);  // O += P V of the previous tile is done
-          tc_fence_after();
-          const bool shares = kt > kShare;  // there is a sum of earlier shares
+      }
+      const float2 scale22 = make_float2(scale2, scale2), neg_ref2 = make_float2(-m_ref, -m_ref);
+      float2 ls[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      float rs[2] = {0.f, 0.f};
+      // P goes where S was: both halves of the row have read their S columns (the barrier above), and the
+      // product that read the buffer's previous P was issued before the product that formed this S
+      const uint32_t t_p = t_lane + (kt & 1) * kKeys + half * 32;  // this half's 64 keys = 32 packed columns
+      // 32 of the half's keys at a time, so that the product over the first part runs while the second is formed
+      auto numerators = [&](int part, auto top) {  // top: rs sums the numerators of all keys but the tile's largest
+        uint32_t hi[16], lo[16];  // column c = keys 2c (low half) and 2c + 1
 #pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          // P = hi + lo, hi truncated and lo rounded to bf16 (16 significant bits together); plain bit
+          // operations, so the conversion unit is left to the exponentials
+          const int i = 32 * part + 2 * c;
+          const float2 e = __ffma2_rn(make_float2(sv[i], sv[i + 1]), scale22, neg_ref2);
+          const float2 p = make_float2(fast_exp2(e.x), fast_exp2(e.y));
+          const uint32_t b0 = __float_as_uint(p.x), b1 = __float_as_uint(p.y);
+          hi[c] = __byte_perm(b0, b1, 0x7632);
+          const float2 r = __ffma2_rn(make_float2(__uint_as_float(b0 & 0xffff0000u), __uint_as_float(b1 & 0xffff0000u)),
+                                      make_float2(-1.f, -1.f), p);
+          lo[c] = __byte_perm(__float_as_uint(r.x) + 0x8000u, __float_as_uint(r.y) + 0x8000u, 0x7632);  // rounded
+          ls[c & 1] = __fadd2_rn(ls[c & 1], p);
+          if constexpr (decltype(top)::value) {
+            if (sv[i] != raw_top) rs[c & 1] += p.x;
+            if (sv[i + 1] != raw_top) rs[c & 1] += p.y;
+          }
+        }
+        tmem_st16u(t_p + 16 * part, hi);
+        tmem_st16u(t_p + 64 + 16 * part, lo);
+      };
+      auto form = [&](int part) {
+        if (kFew && keep_top) numerators(part, std::true_type{});
+        else numerators(part, std::false_type{});
+      };
+      form(0);
+      // O += P V of the previous tile has finished by now, or nearly: O is rescaled, a finished share moved, before the first
+      // product of this tile is queued
+      if (kt > 0 && (close || __any_sync(0xffffffffu, need))) {
+        mbar_wait(&o_bar[(kt - 1) & 1], ((kt - 1) >> 1) & 1, status);
+        tc_fence_after();
+        // (rolled loops: this code is seldom run, and has to be fetched every time)
+        if (close) {
+#pragma unroll 1
           for (int cc = 0; cc < D / 32; ++cc) {
             uint32_t v[16], w[16];
             tmem_ld16_issue(t_o + cc * 16, v);
-            if (shares) tmem_ld16_issue(t_o + 128 + cc * 16, w);
+            tmem_ld16_issue(t_o + 128 + cc * 16, w);
             tmem_ld16_wait(v);
-            if (shares) tmem_ld16_wait(w);
+            tmem_ld16_wait(w);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float x = __uint_as_float(v[i]), y = shares ? __uint_as_float(w[i]) : 0.f;
-              v[i] = __float_as_uint(x * corr);
-              w[i] = __float_as_uint((close ? x + y : y) * corr);
-            }
-            if (!close) tmem_st16u(t_o + cc * 16, v);
-            if (close || shares) tmem_st16u(t_o + 128 + cc * 16, w);
+            for (int i = 0; i < 16; ++i) w[i] = __float_as_uint((__uint_as_float(v[i]) + __uint_as_float(w[i])) * corr);
+            tmem_st16u(t_o + 128 + cc * 16, w);
           }
-          tmem_st_wait();
-        }
-      }
-      {
-        const float neg_ref = -m_ref;
-        float ls[4] = {0.f, 0.f, 0.f, 0.f}, rs[4] = {0.f, 0.f, 0.f, 0.f};
-        uint32_t hi[32], lo[32];  // column c = keys 2c (low half) and 2c + 1
-        auto numerators = [&](auto top) {  // top: rs sums the numerators of all keys but the tile's largest
+        } else {
+#pragma unroll 1
+          for (int cc = 0; cc < (kt > kShare ? D / 16 : D / 32); ++cc) {  // O, and the sum of earlier shares if there is one
+            const uint32_t at = t_o + (cc / (D / 32)) * 128 + (cc % (D / 32)) * 16;
+            uint32_t v[16];
+            tmem_ld16_issue(at, v);
+            tmem_ld16_wait(v);
 #pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            // P = hi + lo, hi truncated and lo rounded to bf16 (16 significant bits together); plain bit
-            // operations, so the conversion unit is left to the exponentials
-            const float p0 = fast_exp2(fmaf(sv[2 * c], scale2, neg_ref));
-            const float p1 = fast_exp2(fmaf(sv[2 * c + 1], scale2, neg_ref));
-            const uint32_t b0 = __float_as_uint(p0), b1 = __float_as_uint(p1);
-            hi[c] = __byte_perm(b0, b1, 0x7632);
-            const float r0 = p0 - __uint_as_float(b0 & 0xffff0000u), r1 = p1 - __uint_as_float(b1 & 0xffff0000u);
-            lo[c] = __byte_perm(__float_as_uint(r0) + 0x8000u, __float_as_uint(r1) + 0x8000u, 0x7632);  // rounded
-            ls[c & 3] += p0 + p1;
-            if constexpr (decltype(top)::value) {
-              if (sv[2 * c] != raw_top) rs[c & 3] += p0;
-              if (sv[2 * c + 1] != raw_top) rs[c & 3] += p1;
-            }
+            for (int i = 0; i < 16; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * corr);
+            tmem_st16u(at, v);
           }
-        };
-        if (kFew && keep_top) numerators(std::true_type{});
-        else numerators(std::false_type{});
-        // P goes where S was: both halves of the row have read their S columns (the barrier above), and the
-        // product that read the buffer's previous P was issued before the product that formed this S
-        const uint32_t t_p = t_lane + (kt & 1) * kKeys + half * 32;  // this half's 64 keys = 32 packed columns
-        tmem_st32u(t_p, hi);
-        tmem_st32u(t_p + 64, lo);
-        tmem_st_wait();
-        const float lt = (ls[0] + ls[1]) + (ls[2] + ls[3]);
-        l += lt;
-        if (kFew && keep_top) {
-          // one copy of the tile's largest numerator stays apart, any other copies join the rest (their number from the
-          // two sums: pt is the largest of 64 terms, so the sums' rounding is far below half of it)
-          const float pt = fast_exp2(fmaf(raw_top, scale2, neg_ref)), rt = (rs[0] + rs[1]) + (rs[2] + rs[3]);
-          float r = rt + (pt > 0.f ? rintf((lt - rt) / pt) - 1.f : 0.f) * pt;
-          const bool bigger = raw_top > smax;
-          r += bigger ? ptop : pt;
-          lrest += r;
-          ptop = bigger ? pt : ptop;
-          smax = bigger ? raw_top : smax;
         }
       }
       const int n_valid = min(kKeys, n - (kt0 + kt) * kKeys);
@@ -600,10 +625,30 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
           for (int c = 0; c < D / 8; ++c)
             *reinterpret_cast<uint4*>(vt + (c >> 3) * kKvHalf + tid * 128 + (((c & 7) ^ (tid & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
         }
+        fence_async_smem();
       }
-      fence_async_smem();
-      tc_fence_before();
-      mbar_arrive(&p_bar[kt & 1]);
+      auto hand_over = [&](int part) {
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&p_bar[2 * part + (kt & 1)]);
+      };
+      hand_over(0);
+      form(1);
+      hand_over(1);
+      const float lt = (ls[0].x + ls[0].y) + (ls[1].x + ls[1].y);
+      l += lt;
+      if (kFew && keep_top) {
+        // one copy of the tile's largest numerator stays apart, any other copies join the rest (their number from the
+        // two sums: pt is the largest of 64 terms, so the sums' rounding is far below half of it)
+        const float pt = fast_exp2(fmaf(raw_top, scale2, -m_ref)), rt = rs[0] + rs[1];
+        float r = rt + (pt > 0.f ? rintf((lt - rt) / pt) - 1.f : 0.f) * pt;
+        const bool bigger = raw_top > smax;
+        r += bigger ? ptop : pt;
+        lrest += r;
+        ptop = bigger ? pt : ptop;
+        smax = bigger ? raw_top : smax;
+      }
     }
     mbar_wait(&o_bar[(ntiles - 1) & 1], ((ntiles - 1) >> 1) & 1, status);
     tc_fence_after();
@@ -704,7 +749,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   if (nsp > 1 && warp < 8) {
     // ---- merge: o = sum_s o_s 2^(stat_s - stat), stat = log2 sum_s 2^stat_s; a warp per row, lane = D / 32 channels ----
     constexpr int CPL = D / 32;
-    const int rp = (kTile + nsp - 1) / nsp, lane = tid & 31;
+    const int rp = (kTile + nsp - 1) / nsp;
     const float4* rst = reinterpret_cast<const float4*>(xch);  // [split][row]: statistic, largest product, the others' share
     float cs[CPL];
 #pragma unroll
