@@ -57,7 +57,7 @@ post_evict_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
   const bool have_stat = (tag == kStatPerHead && m == 1) || tag == kStatPerRow;
   float stat2 = 0.f;  // alpha = 2^(log2(e) * scale * <q, k> - stat2)
   if (have_stat && row_ok)
-    stat2 = (tag == kStatPerHead) ? stats[(size_t)unit * kHeadStatFloats + g] : stats[(size_t)unit * prefill_stride + r];
+    stat2 = (tag == kStatPerHead) ? stats[(size_t)unit * kHeadStatFloats + g] : -stats[(size_t)unit * prefill_stride + r];  // (the row blocks leave it negated)
   // pass over the keys: running maximum and sum of exp of this row's logits, two keys per lane and tile
   float mx = -INFINITY, l = 0.f;
   for (int kt = 0; kt < (have_stat ? 0 : n); kt += kKeys) {
@@ -126,7 +126,7 @@ post_evict_kernel(Dims dm, const T* __restrict__ q, const T* __restrict__ K, con
 // unless the workspace header says so. It is the attention pass over the evicted rows with a reference that is already
 // known, so a CTA takes 128 query rows of a unit (two threads per row) and walks the unit's evicted slots 128 at a time:
 // their K and V rows are gathered into swizzled tiles by plain loads, S = Q K_E^T and Y += P V_E (P as two bf16 parts) run
-// on tcgen05, and the weights 2^(s - stat) are formed in between. What bounds it is the chain of one tile (gather, product,
+// on tcgen05, and the weights 2^(s + stat) are formed in between. What bounds it is the chain of one tile (gather, product,
 // exponentials, product, write-out): 16 units x 896 rows x 128 evictions, 82 us on the CUDA cores (a CTA per 16 rows) -> 25 between events.
 // grid = (ceil(R / 128), units), 256 threads; TMEM columns: S / P [0, 128), Y [128, 128 + D).
 constexpr int kTcThreads = 256;
@@ -176,7 +176,7 @@ post_evict_tc_kernel(Dims dm, const __nv_bfloat16* __restrict__ q, const __nv_bf
     if (r0 + rr < dm.R) v = *reinterpret_cast<const uint4*>(q + ((size_t)unit * dm.R + r0 + rr) * D + 8 * c);
     *reinterpret_cast<uint4*>(Qs + ptx::tile_off(rr, c)) = v;
   }
-  const float stat = (r < dm.R) ? stats[(size_t)unit * stat_stride + r] : INFINITY;  // (rows beyond R: weights 0)
+  const float stat = (r < dm.R) ? stats[(size_t)unit * stat_stride + r] : -INFINITY;  // (negated there; rows beyond R: weights 0)
   const int n_vis = (r < dm.R) ? n - m + (r % m) + 1 : 0;
   const float scale2 = dm.scale * 1.4426950408889634f;
   tc_fence_before();
@@ -222,8 +222,8 @@ post_evict_tc_kernel(Dims dm, const __nv_bfloat16* __restrict__ q, const __nv_bf
     for (int c = 0; c < 32; ++c) {
       const int2 jj = *reinterpret_cast<const int2*>(js + half * 64 + 2 * c);
       const bool v0 = jj.x >= 0 && jj.x < n_vis, v1 = jj.y >= 0 && jj.y < n_vis;
-      const float p0 = v0 ? fast_exp2(fmaf(sv[2 * c], scale2, -stat)) : 0.f;
-      const float p1 = v1 ? fast_exp2(fmaf(sv[2 * c + 1], scale2, -stat)) : 0.f;
+      const float p0 = v0 ? fast_exp2(fmaf(sv[2 * c], scale2, stat)) : 0.f;
+      const float p1 = v1 ? fast_exp2(fmaf(sv[2 * c + 1], scale2, stat)) : 0.f;
       gone += (v0 ? 1 : 0) + (v1 ? 1 : 0);
       const uint32_t b0 = __float_as_uint(p0), b1 = __float_as_uint(p1);
       hi[c] = __byte_perm(b0, b1, 0x7632);

@@ -60,7 +60,7 @@ constexpr int kThreads = 128;
 constexpr long long kWaitCycles = 2000000000LL;
 
 struct Scratch {
-  float* stats;  // [units][Mpad]: log2-domain softmax reference + log2(sum of 2^(s - ref)): alpha = 2^(s - stats)
+  float* stats;  // [units][Mpad]: minus (log2-domain softmax reference + log2(sum of 2^(s - ref))): alpha = 2^(s + stats)
   float* sstat;  // [units][kTile] LAST_QUERY: the counted rows' statistics side by side (else null)
   float* crest;  // [units][kTile] few: share of all tokens but the counted row's top one (else null)
   float* xpart;  // [units][row blocks][nsplit][D] per CTA of the attention pass: the sum of its counted output rows
@@ -710,7 +710,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         xch[5 * kRowThreads + (warp & 3) * D + half * (D / 2) + cc * 32 + (tid & 31)] = ov[cc][0];  // (lane l has channel l)
       }
       if (R < M && half == 0) {
-        const float stat = m_ref + __log2f(l);
+        const float stat = -(m_ref + __log2f(l));
         sc.stats[(size_t)unit * sc.Mpad + R] = stat;
         if (kFew && in_x) {
           if (sc.sstat) sc.sstat[(size_t)unit * kTile + counted_index(dm, R)] = stat;
@@ -792,7 +792,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
       if constexpr (CPL == 4) *reinterpret_cast<float4*>(orow) = make_float4(acc[0], acc[1], acc[2], acc[3]);
       else *reinterpret_cast<float2*>(orow) = make_float2(acc[0], acc[1]);
       if (lane == 0) {
-        const float stat = mx + __log2f(tot);
+        const float stat = -(mx + __log2f(tot));
         sc.stats[(size_t)unit * sc.Mpad + R] = stat;
         if (kFew && in_x) {
           const int q = counted_index(dm, R);
@@ -984,27 +984,24 @@ __device__ __forceinline__ float2 poly_exp2x2(float2 x) {
                      __int_as_float(__float_as_int(p.y) + (__float_as_int(t.y) << 23)));
 }
 
-// Adds to a key's running sum the attention weights 2^(s * scale2 - statistic) of 16 rows (v: the logits of the
+// Adds to a key's running sum the attention weights 2^(s * scale2 + statistic) of 16 rows (v: the logits of the
 // key against these rows, st: the rows' statistics). plain: no row is masked. Of every eight exponentials six go to
 // the special-function unit and two to the polynomial.
 __device__ __forceinline__ void score_piece16(const uint32_t (&v)[16], const float4 (&st)[4], float scale2, bool plain,
                                               int R0, int M, int m, int need, float2 (&hacc)[2], float& hmasked) {
   if (plain) {
+    const float2 sc2 = make_float2(scale2, scale2);
+    auto arg = [&](int i, float s0, float s1) {
+      return __ffma2_rn(make_float2(__uint_as_float(v[i]), __uint_as_float(v[i + 1])), sc2, make_float2(s0, s1));
+    };
 #pragma unroll
     for (int i = 0; i < 16; i += 8) {
       const float4 ra = st[i / 4], rb = st[i / 4 + 1];
-      const float a0 = fast_exp2(fmaf(__uint_as_float(v[i]), scale2, -ra.x));
-      const float a1 = fast_exp2(fmaf(__uint_as_float(v[i + 1]), scale2, -ra.y));
-      const float a2 = fast_exp2(fmaf(__uint_as_float(v[i + 2]), scale2, -ra.z));
-      const float a3 = fast_exp2(fmaf(__uint_as_float(v[i + 3]), scale2, -ra.w));
-      const float a4 = fast_exp2(fmaf(__uint_as_float(v[i + 4]), scale2, -rb.x));
-      const float a5 = fast_exp2(fmaf(__uint_as_float(v[i + 5]), scale2, -rb.y));
-      const float2 a67 = poly_exp2x2(make_float2(fmaf(__uint_as_float(v[i + 6]), scale2, -rb.z),
-                                                 fmaf(__uint_as_float(v[i + 7]), scale2, -rb.w)));
-      hacc[0] = __fadd2_rn(hacc[0], make_float2(a0, a1));
-      hacc[1] = __fadd2_rn(hacc[1], make_float2(a2, a3));
-      hacc[0] = __fadd2_rn(hacc[0], make_float2(a4, a5));
-      hacc[1] = __fadd2_rn(hacc[1], a67);
+      const float2 e0 = arg(i, ra.x, ra.y), e1 = arg(i + 2, ra.z, ra.w), e2 = arg(i + 4, rb.x, rb.y);
+      hacc[0] = __fadd2_rn(hacc[0], make_float2(fast_exp2(e0.x), fast_exp2(e0.y)));
+      hacc[1] = __fadd2_rn(hacc[1], make_float2(fast_exp2(e1.x), fast_exp2(e1.y)));
+      hacc[0] = __fadd2_rn(hacc[0], make_float2(fast_exp2(e2.x), fast_exp2(e2.y)));
+      hacc[1] = __fadd2_rn(hacc[1], poly_exp2x2(arg(i + 6, rb.z, rb.w)));
     }
   } else {
     // row R sees key j iff j <= n - m + (R % m), i.e. iff (R % m) >= need; R % m is carried along instead of
@@ -1015,7 +1012,7 @@ __device__ __forceinline__ void score_piece16(const uint32_t (&v)[16], const flo
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       const bool vis = (R0 + i < M) && (rm >= need);
-      const float a = fast_exp2(fmaf(__uint_as_float(v[i]), scale2, -stf[i]));
+      const float a = fast_exp2(fmaf(__uint_as_float(v[i]), scale2, stf[i]));
       hmasked += vis ? a : 0.f;
       if (++rm == m) rm = 0;
     }
@@ -1033,7 +1030,7 @@ __device__ __forceinline__ void score_piece16_few(const uint32_t (&v)[16], const
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const bool row = R0 + i < M;
-    const float a = (row && rm >= need) ? fast_exp2(fmaf(__uint_as_float(v[i]), scale2, -stf[i])) : 0.f;
+    const float a = (row && rm >= need) ? fast_exp2(fmaf(__uint_as_float(v[i]), scale2, stf[i])) : 0.f;
     h += a;
     rest += row ? (a > 0.5f ? crest[i] : 1.f - a) : 0.f;
     if (++rm == m) rm = 0;
