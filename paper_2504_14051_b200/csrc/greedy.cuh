@@ -4,21 +4,26 @@
 // A pick moves the output X = Y / H (Y = sum_j h_j v_j, H = sum_j h_j) by exactly the score of the token it evicts, and by
 // the triangle inequality no distance || X - v_j || changes by more than that. So the distances of all tokens are formed
 // once (a "build"), and from then on a token's distance is known to within the drift, the sum of the scores evicted since
-// it was last formed. A pick forms again only the distances of the tokens that can be the minimum: those whose lower bound
-// is not above the smallest upper bound, usually one to three. The pick is the same as if all distances had been formed
-// again (the same arithmetic on the same state, compared by (score bits, position, slot)); the bounds carry margins of 1e-5
-// for the rounding of scores and 5e-7 || X || per pick for that of X.
+// it was last formed. A pick forms again only the distances of the tokens that can be the minimum: in the order of their
+// lower bounds until the next one is above the smallest score found, usually one. The pick is the same as if all distances had
+// been formed again (the same arithmetic on the same state, compared by (score bits, position, slot)); the bounds carry margins
+// of 2e-5 for the rounding of scores and 5e-7 || X || per pick for that of X.
 //
 // Likewise only the tokens with small scores at the build can be picked: the `active` ones, found by a radix search, with as
 // many of their value rows in shared memory as fit. A pick whose score comes within the drift of the others' smallest score
 // is not taken but starts another build; the first pick after a build is always safe.
 //
 // A thread-block cluster per unit: all CTAs share the two sweeps over the unit's rows (Y, and the distances of a build); the
-// picks are a chain of reductions and run on eight warps of one CTA (two barriers per pick), the others wait at the cluster
-// barrier. 8 units of 4 224 tokens, 128 picks: 709 us with every distance formed at every pick (clusters of 8, rows in shared
-// memory, a cluster barrier per pick) -> 146 us, 22 of them the sweeps and the search. What is left is the latency of a
-// few hundred dependent instructions per pick. Measured for the picks: sixteen warps, active tokens in registers (up to
-// four per thread, loops unrolled) 175; four warps 181; every warp with its own bound and one barrier per pick 200 - 211.
+// picks are one chain of dependent instructions and run on one warp of one CTA, the others wait at the cluster barrier. The
+// warp keeps Y and X in registers and w / (1 - w), which all grow together as H falls, from an earlier pick while that has not
+// moved a bound by 5e-4. What bounds a pick is the number of its instructions: one warp alone runs straight-line code at about
+// four cycles each.
+// 8 units of 4 224 tokens, 128 picks: 709 us with every distance formed at every pick (clusters of 8, rows in shared
+// memory, a cluster barrier per pick) -> 149 us on eight warps with two barriers per pick -> 113, of which the sweeps and the
+// search are 12. Eight lanes per candidate on one warp, a division per token, upper bounds in a pass of their own: 149 (a pick
+// 1 830 cycles: bounds 292, exact score 1 020, though one round per pick); the same without the divisions 137. Earlier
+// still: sixteen warps, active tokens in registers, loops unrolled 175; four warps 181; every warp with its own bound and one
+// barrier per pick 200 - 211.
 #pragma once
 
 #include "common.cuh"
@@ -29,9 +34,9 @@ namespace greedy {
 
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
-constexpr int kPickWarps = 8;            // warps that run the picks (a pick is a few hundred instructions on every one of them)
-constexpr int kPickThreads = 32 * kPickWarps;
-constexpr int kList = 3 * kPickThreads;  // active tokens
+constexpr int kPer = 8;                  // active tokens per lane of the warp that runs the picks
+constexpr int kList = 32 * kPer;         // active tokens, at most
+constexpr int kWant = kList - 64;        // and what the search asks for, at most
 constexpr int kMaxTokens = 24576;        // two floats per token in shared memory
 constexpr int kMaxC = 8;
 
@@ -51,28 +56,6 @@ __device__ __forceinline__ float approx_sqrt(float x) {  // 1 ulp
   float y;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-
-// A candidate of a pick: score bits, position, slot and number in the list of active tokens, weight (as bits).
-struct __align__(16) Cand {
-  unsigned v, p, si, h;
-};
-constexpr unsigned kNoCand = 0x7fffu;  // slot of no token (slots are below kMaxTokens)
-__device__ __forceinline__ bool before(const Cand& a, const Cand& b) {
-  return a.v < b.v || (a.v == b.v && (a.p < b.p || (a.p == b.p && (a.si & 0x7fffu) < (b.si & 0x7fffu))));
-}
-
-// The lane that holds the warp's first candidate.
-__device__ __forceinline__ int first_of(const Cand& c) {
-  const unsigned v1 = __reduce_min_sync(0xffffffffu, c.v);
-  unsigned m = __ballot_sync(0xffffffffu, c.v == v1);
-  if (m & (m - 1u)) {  // a tie, or no candidate at all
-    const unsigned p1 = __reduce_min_sync(0xffffffffu, c.v == v1 ? c.p : 0xffffffffu);
-    const bool eq = c.v == v1 && c.p == p1;
-    const unsigned s1 = __reduce_min_sync(0xffffffffu, eq ? c.si & 0x7fffu : 0xffffu);
-    m = __ballot_sync(0xffffffffu, eq && (c.si & 0x7fffu) == s1);
-  }
-  return __ffs((int)m) - 1;
 }
 
 // 16 bytes of a row against the same channels of -X (nx: 16-byte aligned), packed fp32 pairs.
@@ -120,13 +103,12 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
   __shared__ float s_H;
   __shared__ int s_ctl;                                 // after a round of picks: picks done, -1: all
   __shared__ int act[kList];                            // the active tokens: slot,
-  __shared__ float th[kList], ta[kList], tr[kList];     // weight (< 0 once evicted), distance + drift when it was formed, w / (1 - w),
+  __shared__ __align__(16) float th[kList], ta[kList];  // weight (< 0: evicted, or no token), distance + drift when it was formed,
   __shared__ unsigned tp[kList];                        // position
   __shared__ unsigned hist[256];
   __shared__ int s_digit, s_below, s_incl, s_na;
-  __shared__ unsigned s_min[kWarps], s_ub[kPickWarps];
+  __shared__ unsigned s_min[kWarps];
   __shared__ int s_cnt[kWarps];
-  __shared__ Cand s_cand[kPickWarps];
 
   const int C = (int)ptx::cluster_nctarank(), rank = (int)ptx::cluster_ctarank();
   const int unit = (int)ptx::cluster_id_x(), b = unit / Hkv, hd = unit % Hkv;
@@ -228,10 +210,8 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
     ptx::cluster_sync_all();
 
     if (rank == 0) {
-      // ---- the active tokens: the smallest (score, position, slot) keys, `want` of them and at most what fills up the
-      //      threads' last round ----
-      const int present = n - t, rem = k - t, want = min(present, min(rem + 32, kList - kPickThreads)),
-                most = (want + kPickThreads - 1) / kPickThreads * kPickThreads;
+      // ---- the active tokens: the smallest (score, position, slot) keys, `want` of them, and at most as many as the list holds ----
+      const int present = n - t, rem = k - t, want = min(present, min(rem + 32, kWant));
       unsigned kb = 0u, kp = 0u, ks = 0u;  // the largest key that is taken
       int below = 0;
       for (int pass = 0;; ++pass) {  // eight bits at a time: four passes over the score, four the position, two the slot
@@ -284,7 +264,7 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
         else if (pass < 8) kp |= digit;
         else ks |= digit;
         below = s_below;
-        if (s_incl <= most || pass == 9) {
+        if (s_incl <= kList || pass == 9) {
           const unsigned ones = (1u << shift) - 1u;
           if (pass < 4) { kb |= ones; kp = 0xffffffffu; ks = 0xffffffffu; }
           else if (pass < 8) { kp |= ones; ks = 0xffffffffu; }
@@ -318,13 +298,13 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
         if (lane == 0) s_min[warp] = m;
       }
       __syncthreads();
-      const int na = min(s_na, kList), nu = (na + kPickThreads - 1) / kPickThreads;
+      const int na = min(s_na, kList);
       dmin = __uint_as_float(__reduce_min_sync(0xffffffffu, s_min[lane & (kWarps - 1)]));
       const float tau = __uint_as_float(min(kb, 0x7f800000u)), inv_dmin = 1.f / dmin;  // (0 where there are no others)
-      for (int i = tid; i < na; i += kThreads) {
-        const int j = act[i];
-        th[i] = hs[j];
-        ta[i] = ds[j];
+      for (int i = tid; i < kList; i += kThreads) {
+        const int j = i < na ? act[i] : 0;
+        th[i] = i < na ? hs[j] : -1.f;
+        ta[i] = i < na && hs[j] > 0.f ? ds[j] : INFINITY;  // (no bound: it would be visited after all others)
         tp[i] = (unsigned)(pu ? pu[j] : j);
       }
       for (int idx = tid; idx < min(na, rows_smem) * (D / E); idx += kThreads)
@@ -335,88 +315,136 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
       xn = sqrtf(warp_sum(xn));
       __syncthreads();
 
-      // ================= picks =================
-      // (the loops over a thread's tokens stay rolled: almost always there is one round, and a few warps run straight-line
-      // code no faster than it is fetched)
-      float drift = 0.f;
-      bool fresh = true;
-      while (warp < kPickWarps && t < k) {
-        // ---- the smallest upper bound ----
-        float ub = INFINITY;
-#pragma unroll 1
-        for (int i = tid; i < na; i += kPickThreads) {
-          const float h = th[i], r = ratio_of(h, H);
-          tr[i] = r;
-          if (h >= 0.f) ub = fminf(ub, r * (ta[i] + drift) * 1.00001f);
+      // ================= picks: one warp =================
+      // Lane l looks after the tokens kPer l .. kPer l + 7 of the list and after CPL channels of Y and X, in registers. A pick
+      // visits the tokens in the order of their lower bounds, the smallest first, forms the score of each, and ends when the
+      // next bound is above the smallest score so far: two rounds, mostly. The number in the list stands in the low bits of a
+      // bound, so one reduction over the warp gives both, and the next round's is the smallest key above this one.
+      if (warp == 0) {
+        float r[kPer], hm = 0.f;  // w / (1 - w) at an earlier H, times 0.99998: a lower bound, since it grows as H falls
+        int zeros = 0;            // tokens of weight 0
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+          const float h = th[kPer * lane + u];
+          r[u] = 1.f;
+          hm = fmaxf(hm, h);
+          zeros += h == 0.f ? 1 : 0;
         }
-        ub = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(ub)));
-        if (lane == 0) s_ub[warp] = __float_as_uint(ub);
-        asm volatile("bar.sync 1, %0;" ::"n"(kPickThreads) : "memory");
-        ub = __uint_as_float(__reduce_min_sync(0xffffffffu, s_ub[lane & (kPickWarps - 1)]));
-        // ---- exact scores of the tokens that can be the minimum ----
-        Cand best{0xffffffffu, 0xffffffffu, kNoCand, 0u};
-#pragma unroll 1
-        for (int u = 0; u < nu; ++u) {
-          const int i0 = warp * 32 + u * kPickThreads, mi = i0 + lane;
-          const bool mine = mi < na && th[mi] >= 0.f && !(tr[mi] * fmaxf(ta[mi] - drift, 0.f) * 0.99999f > ub);
-          unsigned mask = __ballot_sync(0xffffffffu, mine);
-#pragma unroll 1
-          while (mask) {  // four tokens at a time, eight lanes each
-            const unsigned m1 = mask & (mask - 1u), m2 = m1 & (m1 - 1u), m3 = m2 & (m2 - 1u);
-            const unsigned ms = sub == 0 ? mask : (sub == 1 ? m1 : (sub == 2 ? m2 : m3));
-            const int idx = i0 + (ms ? __ffs((int)ms) - 1 : 0), j = act[idx];
-            const float r = tr[idx], h = th[idx];
-            const unsigned p = tp[idx];
-            const uint4* row = reinterpret_cast<const uint4*>(idx < rows_smem ? rows + (size_t)idx * D : Vu + (size_t)j * D);
-            float a[NCH];
+        hm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(hm)));
+        zeros = __reduce_add_sync(0xffffffffu, zeros);
+        float y[CPL], x[CPL];  // Y, -X
 #pragma unroll
-            for (int i = 0; i < NCH; ++i)
-              a[i] = sq_dist16<T>(row[l8 + 8 * i], reinterpret_cast<const float4*>(nX) + (l8 + 8 * i) * (E / 4));
+        for (int c = 0; c < CPL; ++c) {
+          y[c] = Ys[lane * CPL + c];
+          x[c] = nX[lane * CPL + c];
+        }
+        const bool all_here = na <= rows_smem;
+        auto channels = [&](int i, float (&v)[CPL]) {  // this lane's of token i (two loads: the one from shared memory is compiled as such)
+          struct __align__(CPL * sizeof(T)) Piece { T e[CPL]; };
+          const Piece q = all_here || i < rows_smem ? reinterpret_cast<const Piece*>(rows + (size_t)i * D)[lane]
+                                                    : reinterpret_cast<const Piece*>(Vu + (size_t)act[i] * D)[lane];
 #pragma unroll
-            for (int i = 1; i < NCH; ++i) a[0] += a[i];
-            a[0] += __shfl_xor_sync(0xffffffffu, a[0], 4);
-            a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
-            a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
-            if (ms && l8 == 0) {
-              const float d = approx_sqrt(a[0]);
-              const Cand c{__float_as_uint(r == 0.f ? 0.f : r * d), p, (unsigned)j | ((unsigned)idx << 16), __float_as_uint(h)};
-              if (before(c, best)) best = c;
-              ta[idx] = d + drift;
+          for (int c = 0; c < CPL; ++c) v[c] = to_float(q.e[c]);
+        };
+        float drift = 0.f, rest0 = -1.f;  // rest0: H - hm when r was formed, < 0: not yet
+        bool fresh = true;
+        while (t < k) {
+          const float rest = H - hm, grown = __fdividef(rest0, rest);  // (what r has grown by since, at most)
+          if (!(grown > 0.f && grown < 1.0005f && rest >= 0.05f * H)) {
+#pragma unroll
+            for (int u = 0; u < kPer; ++u) {
+              const float h = th[kPer * lane + u];
+              r[u] = h > 0.f ? 0.99998f * ratio_of(h, H) : 1.f;
             }
-            mask = m3 & (m3 - 1u);
+            rest0 = rest;
           }
+          int key[kPer];
+          {
+            const float4 a0 = reinterpret_cast<const float4*>(ta)[2 * lane], a1 = reinterpret_cast<const float4*>(ta)[2 * lane + 1];
+            const float av[kPer] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+            for (int u = 0; u < kPer; u += 2) {
+              const float2 lb = __fmul2_rn(__fadd2_rn(make_float2(av[u], av[u + 1]), make_float2(-drift, -drift)), make_float2(r[u], r[u + 1]));
+              key[u] = (__float_as_int(lb.x) & ~(kList - 1)) | (kPer * lane + u);  // (as signed numbers in the order of the bounds;
+              key[u + 1] = (__float_as_int(lb.y) & ~(kList - 1)) | (kPer * lane + u + 1);  // below 0 in any order, all of them first)
+            }
+          }
+          int best_v = 0x7fffffff, bi = -1;  // the smallest score so far (its bits) and whose it is
+          auto take = [&](int i, int v) {
+            if (bi < 0 || v < best_v || (v == best_v && (tp[i] < tp[bi] || (tp[i] == tp[bi] && act[i] < act[bi])))) {
+              best_v = v;
+              bi = i;
+            }
+          };
+          if (zeros > 0) {  // tokens of weight 0 score 0 whatever their distance (they have no bound in the list): the oldest of them
+            int mine = -1;
+#pragma unroll 1
+            for (int i = kPer * lane; i < kPer * lane + kPer; ++i)
+              if (th[i] == 0.f && (mine < 0 || tp[i] < tp[mine] || (tp[i] == tp[mine] && act[i] < act[mine]))) mine = i;
+            const unsigned p1 = __reduce_min_sync(0xffffffffu, mine >= 0 ? tp[mine] : 0xffffffffu);
+            const bool old = mine >= 0 && tp[mine] == p1;
+            const unsigned s1 = __reduce_min_sync(0xffffffffu, old ? (unsigned)act[mine] : 0xffffffffu);
+            const unsigned m = __ballot_sync(0xffffffffu, old && (unsigned)act[mine] == s1);
+            take(__shfl_sync(0xffffffffu, mine, __ffs((int)m) - 1), 0);
+          }
+          for (unsigned from = 0x80000000u;;) {  // the smallest key not below `from`
+            unsigned w = (unsigned)key[0] - from;
+#pragma unroll
+            for (int u = 1; u < kPer; ++u) w = min(w, (unsigned)key[u] - from);
+            const int next = (int)(__reduce_min_sync(0xffffffffu, w) + from);
+            if (next < (int)from || (next & ~(kList - 1)) > best_v) break;
+            const int i = next & (kList - 1);
+            const float h = th[i];
+            if (h >= 0.f) {
+              float v[CPL], q = 0.f;
+              channels(i, v);
+#pragma unroll
+              for (int c = 0; c < CPL; ++c) {
+                const float df = v[c] + x[c];
+                q = fmaf(df, df, q);
+              }
+#pragma unroll
+              for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+              const float d = approx_sqrt(q), ro = ratio_of(h, H);
+              take(i, __float_as_int(ro == 0.f ? 0.f : ro * d));
+              if (lane == 0 && h > 0.f) ta[i] = d + drift;
+            }
+            if (next == 0x7fffffff) break;
+            from = (unsigned)next + 1u;
+          }
+          if (bi < 0) {         // no active token is left
+            if (fresh) t = k;   // (cannot happen with k < n)
+            break;
+          }
+          const float sc = __int_as_float(best_v);
+          if (!fresh && !(sc <= tau * (1.f - drift * inv_dmin) * 0.99999f)) break;  // another token may be smaller: build again
+          // ---- evict: Y -= h_e v_e, H -= h_e ----
+          const float he = th[bi];
+          float v[CPL];
+          channels(bi, v);
+          H -= he;
+          const float inv_H = (H > 0.f) ? __fdividef(1.f, H) : 0.f;
+#pragma unroll
+          for (int c = 0; c < CPL; ++c) {
+            y[c] -= he * v[c];
+            x[c] = -(y[c] * inv_H);
+          }
+          zeros -= he == 0.f ? 1 : 0;
+          __syncwarp();  // (th has been read)
+          if (lane == 0) {
+            const int e = act[bi];
+            ta[bi] = INFINITY;
+            th[bi] = -1.f;
+            hs[e] = -1.f;
+            if (order_out) order_out[(size_t)unit * max_evict + t] = e;
+          }
+          __syncwarp();
+          drift += sc * 1.0001f + 5e-7f * (xn + drift);
+          fresh = false;
+          ++t;
         }
-        if (lane == first_of(best)) s_cand[warp] = best;
-        asm volatile("bar.sync 1, %0;" ::"n"(kPickThreads) : "memory");
-        Cand win = s_cand[lane & (kPickWarps - 1)];
-        {
-          Cand mineonly = win;
-          if (lane >= kPickWarps) mineonly = Cand{0xffffffffu, 0xffffffffu, kNoCand, 0u};
-          const int wl = first_of(mineonly);
-          win.v = __shfl_sync(0xffffffffu, win.v, wl);
-          win.si = __shfl_sync(0xffffffffu, win.si, wl);
-          win.h = __shfl_sync(0xffffffffu, win.h, wl);
-        }
-        const int e = (int)(win.si & 0x7fffu), ei = (int)(win.si >> 16);
-        const float he = __uint_as_float(win.h), sc = __uint_as_float(win.v);
-        if (e == (int)kNoCand) { t = k; break; }  // (cannot happen with k < n; the same in every thread)
-        if (!fresh && !(sc <= tau * (1.f - drift * inv_dmin) * 0.99999f)) break;  // another token may be smaller: build again
-        // ---- evict e: Y -= h_e v_e, H -= h_e (X is read again after the next barrier) ----
-        H -= he;
-        if (tid < D) {
-          const T* row = ei < rows_smem ? rows + (size_t)ei * D : Vu + (size_t)e * D;
-          const float y = Ys[tid] - he * to_float(row[tid]);
-          Ys[tid] = y;
-          nX[tid] = -(y * ((H > 0.f) ? __fdividef(1.f, H) : 0.f));
-        }
-        if (ei % kPickThreads == tid) {
-          th[ei] = -1.f;
-          hs[e] = -1.f;
-          if (order_out) order_out[(size_t)unit * max_evict + t] = e;
-        }
-        drift += sc * 1.0001f + 5e-7f * (xn + drift);
-        fresh = false;
-        ++t;
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) Ys[lane * CPL + c] = y[c];
       }
       __syncthreads();
       if (tid == 0) {

@@ -174,3 +174,31 @@ def test_greedy_when_bounds_are_loose_or_tie(case, dtype, d):
         rem = [j for j in range(n) if j not in gone]
         hr, Vr, pr = h[0, 0, rem].numpy(), f32(V)[0, 0][rem], pos[0, 0, rem].numpy()
         follow([rem.index(j) for j in og[k - 12:]], hr, Vr, pr, 12)
+
+
+@pytest.mark.parametrize("n,k", [(2, 1), (9, 8), (191, 190), (193, 64), (255, 40), (257, 225), (330, 329)])
+@pytest.mark.parametrize("dtype,d", [(torch.bfloat16, 128), (torch.bfloat16, 64), (torch.float32, 128)])
+def test_greedy_around_the_length_of_the_list_of_active_tokens(n, k, dtype, d):
+    """192 are asked for and 256 fit; a fifth of the weights is 0, tokens without a bound."""
+    g = torch.Generator(device="cpu").manual_seed(n * 31 + k)
+    cap = n + 3
+    V = torch.randn((1, 1, cap, d), generator=g).to(dtype)
+    h = torch.randn((1, 1, cap), generator=g).exp()
+    none = torch.randperm(n, generator=g)[:n // 5]
+    h[:, :, none] = 0.0
+    pos = torch.randperm(cap, generator=g).to(torch.int32).view(1, 1, cap)
+    p = P.make_params(1, 1, 1, d, cap, 1, dtype, 1.0, "external")
+    ws = P.alloc_workspace(p, DEV)
+    ev = torch.full((1, 1, k), -1, dtype=torch.int32, device=DEV)
+    order, ne = torch.full_like(ev, -1), torch.zeros((1,), dtype=torch.int32, device=DEV)
+    lens = torch.tensor([n], dtype=torch.int32)
+    P.caote_select_evict_greedy(p, V.to(DEV), h.to(DEV), lens.to(DEV), (lens - k).to(DEV), pos.to(DEV), ev, order, ne, ws)
+    assert P.caote_read_status(ws) == 0 and ne.item() == k
+    og = order[0, 0].cpu().tolist()
+    assert sorted(og) == ev[0, 0].cpu().tolist() and len(set(og)) == k and 0 <= min(og) and max(og) < n
+    first = sorted(none.tolist(), key=lambda j: int(pos[0, 0, j]))[:k]
+    assert og[:len(first)] == first  # scores of exactly 0: the oldest first
+    rem = [j for j in range(n) if j not in set(first)]
+    more = [rem.index(j) for j in og[len(first):]][:24]
+    if more:
+        follow(more, h[0, 0, rem].numpy(), f32(V)[0, 0][rem], pos[0, 0, rem].numpy(), len(more))
