@@ -26,6 +26,8 @@
 // barrier per pick 200 - 211.
 #pragma once
 
+#include <cfloat>
+
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -57,6 +59,10 @@ __device__ __forceinline__ float approx_sqrt(float x) {  // 1 ulp
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+
+// A distance (and the drift) as a bound keeps it: finite, also where it overflows or is no number. A token's lower bound is then
+// a number: 0, as its score, when its share of the weights underflows to 0, however far it lies.
+__device__ __forceinline__ float bound_of(float dist) { return fminf(dist, FLT_MAX); }
 
 // 16 bytes of a row against the same channels of -X (nx: 16-byte aligned), packed fp32 pairs.
 template <typename T>
@@ -304,7 +310,7 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
       for (int i = tid; i < kList; i += kThreads) {
         const int j = i < na ? act[i] : 0;
         th[i] = i < na ? hs[j] : -1.f;
-        ta[i] = i < na && hs[j] > 0.f ? ds[j] : INFINITY;  // (no bound: it would be visited after all others)
+        ta[i] = i < na && hs[j] > 0.f ? bound_of(ds[j]) : INFINITY;  // (no bound: it would be visited after all others)
         tp[i] = (unsigned)(pu ? pu[j] : j);
       }
       for (int idx = tid; idx < min(na, rows_smem) * (D / E); idx += kThreads)
@@ -354,7 +360,7 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
 #pragma unroll
             for (int u = 0; u < kPer; ++u) {
               const float h = th[kPer * lane + u];
-              r[u] = h > 0.f ? 0.99998f * ratio_of(h, H) : 1.f;
+              r[u] = h > 0.f ? fminf(0.99998f * ratio_of(h, H), FLT_MAX) : 1.f;
             }
             rest0 = rest;
           }
@@ -407,7 +413,7 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
               for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
               const float d = approx_sqrt(q), ro = ratio_of(h, H);
               take(i, __float_as_int(ro == 0.f ? 0.f : ro * d));
-              if (lane == 0 && h > 0.f) ta[i] = d + drift;
+              if (lane == 0 && h > 0.f) ta[i] = bound_of(d + drift);
             }
             if (next == 0x7fffffff) break;
             from = (unsigned)next + 1u;

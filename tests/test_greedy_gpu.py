@@ -202,3 +202,34 @@ def test_greedy_around_the_length_of_the_list_of_active_tokens(n, k, dtype, d):
     more = [rem.index(j) for j in og[len(first):]][:24]
     if more:
         follow(more, h[0, 0, rem].numpy(), f32(V)[0, 0][rem], pos[0, 0, rem].numpy(), len(more))
+
+
+@pytest.mark.parametrize("kind,k", [("far_light_token", 1), ("far_light_token", 40), ("nan_light_token", 40), ("infinite_weight", 40),
+                                    ("sum_overflows", 40), ("sum_overflows", 300)])
+def test_greedy_scores_of_exactly_0_come_first_whatever_the_distance(kind, k):
+    """w / (1 - w) of 0 scores 0, also where the distance overflows, is no number or X is none; equal scores: the oldest first."""
+    n, d = 600, 128
+    g = torch.Generator(device="cpu").manual_seed(k)
+    V = torch.randn((1, 1, n, d), generator=g)
+    h = torch.rand((1, 1, n), generator=g) + 0.5
+    pos = torch.randperm(n, generator=g).to(torch.int32).view(1, 1, n)
+    if kind.endswith("light_token"):  # the smallest positive weight over a sum of about 600: 0
+        light = [9] if k == 1 else list(range(9, 9 + k))
+        V[0, 0, light, 3] = 1e20 if kind == "far_light_token" else float("nan")
+        h[0, 0, light] = 1e-45
+    elif kind == "infinite_weight":  # (the heavy token itself has the largest score)
+        light = [j for j in range(n) if j != 7]
+        h[0, 0, 7] = float("inf")
+    else:
+        light = list(range(n))
+        h *= 1e37
+    p = P.make_params(1, 1, 1, d, n, 1, torch.float32, 1.0, "external")
+    ws = P.alloc_workspace(p, DEV)
+    ev = torch.full((1, 1, k), -1, dtype=torch.int32, device=DEV)
+    order, ne = torch.full_like(ev, -1), torch.zeros((1,), dtype=torch.int32, device=DEV)
+    lens = torch.tensor([n], dtype=torch.int32)
+    P.caote_select_evict_greedy(p, V.to(DEV), h.to(DEV), lens.to(DEV), (lens - k).to(DEV), pos.to(DEV), ev, order, ne, ws)
+    assert P.caote_read_status(ws) == 0 and ne.item() == k
+    og = order[0, 0].cpu().tolist()
+    assert og == sorted(light, key=lambda j: int(pos[0, 0, j]))[:k]
+    assert ev[0, 0].cpu().tolist() == sorted(og)
