@@ -6,8 +6,9 @@
 // once (a "build"), and from then on a token's distance is known to within the drift, the sum of the scores evicted since
 // it was last formed. A pick forms again only the distances of the tokens that can be the minimum: in the order of their
 // lower bounds until the next one is above the smallest score found, usually one. The pick is the same as if all distances had
-// been formed again (the same arithmetic on the same state, compared by (score bits, position, slot)); the bounds carry margins
-// of 2e-5 for the rounding of scores and 5e-7 || X || per pick for that of X.
+// been formed again in the picks' own arithmetic (a warp's 32 lanes per row, also where all warps share the work; compared by
+// (score bits, position, slot)). The builds' sums, eight lanes per row, only make bounds; the bounds carry margins of 2e-5 for the
+// rounding of scores and 5e-7 || X || per pick for that of X.
 //
 // Likewise only the tokens with small scores at the build can be picked: the `active` ones, found by a radix search, with as
 // many of their value rows in shared memory as fit. A pick whose score comes within the drift of the others' smallest score
@@ -18,6 +19,14 @@
 // warp keeps Y and X in registers and w / (1 - w), which all grow together as H falls, from an earlier pick while that has not
 // moved a bound by 5e-4. What bounds a pick is the number of its instructions: one warp alone runs straight-line code at about
 // four cycles each.
+//
+// Where bounds do not tell the tokens apart a pick would walk through the list one token after the other; after kAlone of them all
+// warps form the other scores at once. 8 units of 4 224 tokens, 128 picks, us (eight warps and 768 active tokens, as it once
+// was; one warp; now): log-normal weights 156, 129, 128; equal weights 323, 365, 296; equal weights and 64 different rows
+// 783, 5 540, 868; equal rows 4 300, 21 360, 4 270. 900 tokens, 300 of them with weights of 1e-41, 60 picks: 107, 1 303, 221.
+// The list holds 256 tokens where it held 768, so long evictions build more often, and are faster all the same: log-normal
+// weights, 512 picks 780 -> 553, 2 048 picks 4 270 -> 2 820; equal weights, 1 600 picks 8 540 -> 5 300. What is slower for it is
+// long evictions among few different rows of equal weights, where a build lasts only a few picks: 64 rows, 1 600 picks 18.2 -> 23.4 ms.
 // 8 units of 4 224 tokens, 128 picks: 709 us with every distance formed at every pick (clusters of 8, rows in shared
 // memory, a cluster barrier per pick) -> 149 us on eight warps with two barriers per pick -> 113, of which the sweeps and the
 // search are 12. Eight lanes per candidate on one warp, a division per token, upper bounds in a pass of their own: 149 (a pick
@@ -39,6 +48,9 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kPer = 8;                  // active tokens per lane of the warp that runs the picks
 constexpr int kList = 32 * kPer;         // active tokens, at most
 constexpr int kWant = kList - 64;        // and what the search asks for, at most
+// Scores that the warp of the picks forms alone: 1: 145 us, 2: 135, log-normal weights; 2: 300, 6: 365, equal ones (128 picks, 4 224 tokens).
+constexpr int kAlone = 2;
+static_assert(kList == 16 * kWarps, "");
 constexpr int kMaxTokens = 24576;        // two floats per token in shared memory
 constexpr int kMaxC = 8;
 
@@ -64,6 +76,27 @@ __device__ __forceinline__ float approx_sqrt(float x) {  // 1 ulp
 // a number: 0, as its score, when its share of the weights underflows to 0, however far it lies.
 __device__ __forceinline__ float bound_of(float dist) { return fminf(dist, FLT_MAX); }
 
+// A token in the order of picks: score bits, position, slot; and its number in the list of active tokens.
+struct __align__(16) Cand {
+  unsigned v, p, s;
+  int i;
+};
+__device__ __forceinline__ bool before(const Cand& a, const Cand& b) {
+  return a.v < b.v || (a.v == b.v && (a.p < b.p || (a.p == b.p && a.s < b.s)));
+}
+// The lane that holds the warp's first token.
+__device__ __forceinline__ int first_of(const Cand& c) {
+  const unsigned v = __reduce_min_sync(0xffffffffu, c.v);
+  unsigned m = __ballot_sync(0xffffffffu, c.v == v);
+  if (m & (m - 1u)) {  // a tie, or no token at all
+    const unsigned p = __reduce_min_sync(0xffffffffu, c.v == v ? c.p : 0xffffffffu);
+    const bool eq = c.v == v && c.p == p;
+    const unsigned s = __reduce_min_sync(0xffffffffu, eq ? c.s : 0xffffffffu);
+    m = __ballot_sync(0xffffffffu, eq && c.s == s);
+  }
+  return __ffs((int)m) - 1;
+}
+
 // 16 bytes of a row against the same channels of -X (nx: 16-byte aligned), packed fp32 pairs.
 template <typename T>
 __device__ __forceinline__ float sq_dist16(uint4 raw, const float4* nx) {
@@ -88,6 +121,118 @@ __device__ __forceinline__ float sq_dist16(uint4 raw, const float4* nx) {
   return a.x + a.y;
 }
 
+// A lane's channels when a warp shares a row.
+template <typename T, int D>
+struct __align__(D / 32 * sizeof(T)) LanePiece { T e[D / 32]; };
+
+// The scores of the tokens of `mask` among the warp's 16 of the list, four at a time with eight lanes each, and the first of them:
+// to the last bit what a warp per token gives (a lane adds up the parts of four of its lanes in the order of their exchange).
+template <typename T, int D>
+__device__ __forceinline__ void scores_of(unsigned mask, const T* rows, int rows_smem, const T* Vu, const int* act, const float* th, float* ta,
+                                          const unsigned* tp, const float* nX, float H, float drift, Cand* out) {
+  constexpr int CPL = D / 32;
+  using Piece = LanePiece<T, D>;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane >> 3, l8 = lane & 7;
+  Cand best{0xffffffffu, 0xffffffffu, 0xffffffffu, -1};
+#pragma unroll 1
+  while (mask) {
+    const unsigned m1 = mask & (mask - 1u), m2 = m1 & (m1 - 1u), m3 = m2 & (m2 - 1u);
+    const unsigned ms = sub == 0 ? mask : (sub == 1 ? m1 : (sub == 2 ? m2 : m3));
+    const int i = 16 * warp + (ms ? __ffs((int)ms) - 1 : 0);  // (a token of the list either way: its first ones are there, or mask is 0)
+    const Piece* row = reinterpret_cast<const Piece*>(i < rows_smem ? rows + (size_t)i * D : Vu + (size_t)act[i] * D);
+    Piece v[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = row[l8 + 8 * c];
+    float q[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      q[c] = 0.f;
+#pragma unroll
+      for (int e = 0; e < CPL; ++e) {
+        const float df = to_float(v[c].e[e]) + nX[(l8 + 8 * c) * CPL + e];
+        q[c] = fmaf(df, df, q[c]);
+      }
+    }
+    float a = (q[0] + q[2]) + (q[1] + q[3]);
+    a += __shfl_xor_sync(0xffffffffu, a, 4);
+    a += __shfl_xor_sync(0xffffffffu, a, 2);
+    a += __shfl_xor_sync(0xffffffffu, a, 1);
+    if (ms && l8 == 0) {
+      const float h = th[i], d = approx_sqrt(a), ro = ratio_of(h, H);
+      const Cand c{__float_as_uint(ro == 0.f ? 0.f : ro * d), tp[i], (unsigned)act[i], i};
+      if (before(c, best)) best = c;
+      if (h > 0.f) ta[i] = bound_of(d + drift);
+    }
+    mask = m3 & (m3 - 1u);
+  }
+  if (lane == first_of(best)) out[warp] = best;
+}
+
+// This warp's part of sum_j h_j v_j and (at [D]) sum_j h_j over the rows r0 .. r1. (The two sweeps are calls: compiled as a part of the
+// kernel their loads were spread out differently with every change of the picks, up to 8 % of a sweep.)
+template <typename T, int D>
+__device__ __noinline__ void sum_rows(const T* __restrict__ Vu, const float* __restrict__ hu, int r0, int r1, float* part) {
+  constexpr int CPL = D / 32;  // channels per lane when a warp shares a row
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float hsum = 0.f, y[CPL];
+#pragma unroll
+  for (int c = 0; c < CPL; ++c) y[c] = 0.f;
+  constexpr int kFly = 8;  // rows in flight per warp
+  for (int j0 = r0 + warp; j0 < r1; j0 += kFly * kWarps) {
+    float hj[kFly], v[kFly][CPL];
+#pragma unroll
+    for (int u = 0; u < kFly; ++u) {
+      const int j = j0 + u * kWarps;
+      hj[u] = (j < r1) ? fmaxf(hu[j], 0.f) : 0.f;
+      const T* p = Vu + (size_t)min(j, r1 - 1) * D + lane * CPL;
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) v[u][c] = to_float(p[c]);
+    }
+#pragma unroll
+    for (int u = 0; u < kFly; ++u) {
+      hsum += hj[u];
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) y[c] = fmaf(hj[u], v[u][c], y[c]);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < CPL; ++c) part[lane * CPL + c] = y[c];
+  if (lane == 0) part[D] = hsum;  // (every lane added the same weights)
+}
+// The distances of the rows r0 .. r1 to X, to rank 0's array of them (its address in the cluster: ds0).
+template <typename T, int D>
+__device__ __noinline__ void distances(const T* __restrict__ Vu, int r0, int r1, const float* nX, uint32_t ds0) {
+  constexpr int E = 16 / (int)sizeof(T);  // elements per 16-byte piece
+  constexpr int NCH = D / 8 / E;          // pieces per lane when eight lanes share a row: pieces l8, l8 + 8, ...
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane >> 3, l8 = lane & 7;
+  float4 x[NCH][E / 4];
+#pragma unroll
+  for (int i = 0; i < NCH; ++i)
+#pragma unroll
+    for (int e = 0; e < E / 4; ++e) x[i][e] = reinterpret_cast<const float4*>(nX)[(l8 + 8 * i) * (E / 4) + e];
+  constexpr int kPasses = 8 / NCH;  // passes of four rows per warp in flight
+  for (int j0 = r0 + 4 * warp; j0 < r1; j0 += 4 * kWarps * kPasses) {
+    uint4 raw[kPasses][NCH];
+#pragma unroll
+    for (int u = 0; u < kPasses; ++u) {
+      const int j = min(j0 + u * 4 * kWarps + sub, r1 - 1);
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) raw[u][i] = reinterpret_cast<const uint4*>(Vu + (size_t)j * D)[l8 + 8 * i];
+    }
+#pragma unroll
+    for (int u = 0; u < kPasses; ++u) {
+      const int j = j0 + u * 4 * kWarps + sub;
+      float a = 0.f;
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) a += sq_dist16<T>(raw[u][i], x[i]);
+      a += __shfl_xor_sync(0xffffffffu, a, 4);
+      a += __shfl_xor_sync(0xffffffffu, a, 2);
+      a += __shfl_xor_sync(0xffffffffu, a, 1);
+      if (l8 == 0 && j < r1) ptx::st_dsmem_f32(ds0 + 4 * j, approx_sqrt(a));
+    }
+  }
+}
+
 // grid = units x C CTAs in clusters of C; rows_smem: value rows that fit behind the two arrays of `cap` floats.
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -96,7 +241,6 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
                       int* __restrict__ evict_idx, int* __restrict__ order_out, int max_evict, int* __restrict__ n_evict,
                       int* status) {
   constexpr int E = 16 / (int)sizeof(T);  // elements per 16-byte piece
-  constexpr int NCH = D / 8 / E;          // pieces per lane when eight lanes share a row: pieces l8, l8 + 8, ...
   constexpr int CPL = D / 32;             // channels per lane when a warp shares a row
   ptx::pdl_wait();
   ptx::pdl_trigger();
@@ -111,6 +255,10 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
   __shared__ int act[kList];                            // the active tokens: slot,
   __shared__ __align__(16) float th[kList], ta[kList];  // weight (< 0: evicted, or no token), distance + drift when it was formed,
   __shared__ unsigned tp[kList];                        // position
+  __shared__ Cand s_cand[kWarps];                       // where all warps form scores: the first of a warp's tokens,
+  __shared__ unsigned short s_want[kWarps];             // ... for which of its 16 they are formed, as bits
+  __shared__ float s_drift, s_sum;                      // ... at which drift and H
+  __shared__ int s_go;                                  // ... 0: the picks have ended
   __shared__ unsigned hist[256];
   __shared__ int s_digit, s_below, s_incl, s_na;
   __shared__ unsigned s_min[kWarps];
@@ -118,7 +266,7 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
 
   const int C = (int)ptx::cluster_nctarank(), rank = (int)ptx::cluster_ctarank();
   const int unit = (int)ptx::cluster_id_x(), b = unit / Hkv, hd = unit % Hkv;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sub = lane >> 3, l8 = lane & 7;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = len[b];
   int bud = budget[b];
   if (bud < 1) bud = 1;
@@ -139,30 +287,7 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
   {
     if (rank == 0)
       for (int j = tid; j < n; j += kThreads) hs[j] = fmaxf(hu[j], 0.f);
-    float hsum = 0.f, y[CPL];
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) y[c] = 0.f;
-    constexpr int kFly = 8;  // rows in flight per warp
-    for (int j0 = r0 + warp; j0 < r1; j0 += kFly * kWarps) {
-      float hj[kFly], v[kFly][CPL];
-#pragma unroll
-      for (int u = 0; u < kFly; ++u) {
-        const int j = j0 + u * kWarps;
-        hj[u] = (j < r1) ? fmaxf(hu[j], 0.f) : 0.f;
-        const T* p = Vu + (size_t)min(j, r1 - 1) * D + lane * CPL;
-#pragma unroll
-        for (int c = 0; c < CPL; ++c) v[u][c] = to_float(p[c]);
-      }
-#pragma unroll
-      for (int u = 0; u < kFly; ++u) {
-        hsum += hj[u];
-#pragma unroll
-        for (int c = 0; c < CPL; ++c) y[c] = fmaf(hj[u], v[u][c], y[c]);
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) wpart[warp][lane * CPL + c] = y[c];
-    if (lane == 0) wpart[warp][D] = hsum;  // (every lane added the same weights)
+    sum_rows<T, D>(Vu, hu, r0, r1, wpart[warp]);
     __syncthreads();
     if (tid <= D) {
       float t = 0.f;
@@ -186,32 +311,7 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
       const float inv_H = (H > 0.f) ? __fdividef(1.f, H) : 0.f;
       if (tid < D) nX[tid] = -(ptx::ld_dsmem_f32(ptx::map_to_rank(ptx::smem_u32(Ys + tid), 0)) * inv_H);
       __syncthreads();
-      float4 x[NCH][E / 4];
-#pragma unroll
-      for (int i = 0; i < NCH; ++i)
-#pragma unroll
-        for (int e = 0; e < E / 4; ++e) x[i][e] = reinterpret_cast<const float4*>(nX)[(l8 + 8 * i) * (E / 4) + e];
-      constexpr int kPasses = 8 / NCH;  // passes of four rows per warp in flight
-      for (int j0 = r0 + 4 * warp; j0 < r1; j0 += 4 * kWarps * kPasses) {
-        uint4 raw[kPasses][NCH];
-#pragma unroll
-        for (int u = 0; u < kPasses; ++u) {
-          const int j = min(j0 + u * 4 * kWarps + sub, r1 - 1);
-#pragma unroll
-          for (int i = 0; i < NCH; ++i) raw[u][i] = reinterpret_cast<const uint4*>(Vu + (size_t)j * D)[l8 + 8 * i];
-        }
-#pragma unroll
-        for (int u = 0; u < kPasses; ++u) {
-          const int j = j0 + u * 4 * kWarps + sub;
-          float a = 0.f;
-#pragma unroll
-          for (int i = 0; i < NCH; ++i) a += sq_dist16<T>(raw[u][i], x[i]);
-          a += __shfl_xor_sync(0xffffffffu, a, 4);
-          a += __shfl_xor_sync(0xffffffffu, a, 2);
-          a += __shfl_xor_sync(0xffffffffu, a, 1);
-          if (l8 == 0 && j < r1) ptx::st_dsmem_f32(ptx::map_to_rank(ptx::smem_u32(ds + j), 0), approx_sqrt(a));
-        }
-      }
+      distances<T, D>(Vu, r0, r1, nX, ptx::map_to_rank(ptx::smem_u32(ds), 0));
     }
     ptx::cluster_sync_all();
 
@@ -321,6 +421,8 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
       xn = sqrtf(warp_sum(xn));
       __syncthreads();
 
+      const bool all_here = na <= rows_smem;
+      using Piece = LanePiece<T, D>;
       // ================= picks: one warp =================
       // Lane l looks after the tokens kPer l .. kPer l + 7 of the list and after CPL channels of Y and X, in registers. A pick
       // visits the tokens in the order of their lower bounds, the smallest first, forms the score of each, and ends when the
@@ -344,9 +446,7 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
           y[c] = Ys[lane * CPL + c];
           x[c] = nX[lane * CPL + c];
         }
-        const bool all_here = na <= rows_smem;
         auto channels = [&](int i, float (&v)[CPL]) {  // this lane's of token i (two loads: the one from shared memory is compiled as such)
-          struct __align__(CPL * sizeof(T)) Piece { T e[CPL]; };
           const Piece q = all_here || i < rows_smem ? reinterpret_cast<const Piece*>(rows + (size_t)i * D)[lane]
                                                     : reinterpret_cast<const Piece*>(Vu + (size_t)act[i] * D)[lane];
 #pragma unroll
@@ -355,8 +455,8 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
         float drift = 0.f, rest0 = -1.f;  // rest0: H - hm when r was formed, < 0: not yet
         bool fresh = true;
         while (t < k) {
-          const float rest = H - hm, grown = __fdividef(rest0, rest);  // (what r has grown by since, at most)
-          if (!(grown > 0.f && grown < 1.0005f && rest >= 0.05f * H)) {
+          const float rest = H - hm;  // (what r has grown by since: rest0 / rest, at most)
+          if (!(rest0 > 0.f && rest0 < 1.0005f * rest && rest >= 0.05f * H)) {
 #pragma unroll
             for (int u = 0; u < kPer; ++u) {
               const float h = th[kPer * lane + u];
@@ -376,10 +476,14 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
             }
           }
           int best_v = 0x7fffffff, bi = -1;  // the smallest score so far (its bits) and whose it is
+          float he = 0.f, ve[CPL];           // its weight and channels
+          auto first = [&](int i, int v) { return bi < 0 || v < best_v || (v == best_v && (tp[i] < tp[bi] || (tp[i] == tp[bi] && act[i] < act[bi]))); };
           auto take = [&](int i, int v) {
-            if (bi < 0 || v < best_v || (v == best_v && (tp[i] < tp[bi] || (tp[i] == tp[bi] && act[i] < act[bi])))) {
+            if (first(i, v)) {
               best_v = v;
               bi = i;
+              he = th[i];
+              channels(i, ve);
             }
           };
           if (zeros > 0) {  // tokens of weight 0 score 0 whatever their distance (they have no bound in the list): the oldest of them
@@ -393,12 +497,35 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
             const unsigned m = __ballot_sync(0xffffffffu, old && (unsigned)act[mine] == s1);
             take(__shfl_sync(0xffffffffu, mine, __ffs((int)m) - 1), 0);
           }
+          int alone = 0;
           for (unsigned from = 0x80000000u;;) {  // the smallest key not below `from`
             unsigned w = (unsigned)key[0] - from;
 #pragma unroll
             for (int u = 1; u < kPer; ++u) w = min(w, (unsigned)key[u] - from);
             const int next = (int)(__reduce_min_sync(0xffffffffu, w) + from);
             if (next < (int)from || (next & ~(kList - 1)) > best_v) break;
+            if (__builtin_expect(++alone > kAlone, 0)) {  // bounds that do not tell the tokens apart: all that may still be the one, by all warps
+              unsigned mine = 0u;
+#pragma unroll
+              for (int u = 0; u < kPer; ++u)
+                mine |= key[u] >= next && (key[u] & ~(kList - 1)) <= best_v && th[kPer * lane + u] >= 0.f ? 1u << u : 0u;
+              const unsigned above = __shfl_down_sync(0xffffffffu, mine, 1);
+              if ((lane & 1) == 0) s_want[lane >> 1] = (unsigned short)(mine | (above << kPer));
+#pragma unroll
+              for (int c = 0; c < CPL; ++c) nX[lane * CPL + c] = x[c];
+              if (lane == 0) {
+                s_drift = drift;
+                s_sum = H;
+                s_go = 1;
+              }
+              asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");
+              scores_of<T, D>(s_want[0], rows, rows_smem, Vu, act, th, ta, tp, nX, H, drift, s_cand);
+              asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
+              const Cand c = s_cand[lane & (kWarps - 1)];
+              const int l1 = first_of(c), i1 = __shfl_sync(0xffffffffu, c.i, l1), v1 = __shfl_sync(0xffffffffu, (int)c.v, l1);
+              if (i1 >= 0) take(i1, v1);
+              break;
+            }
             const int i = next & (kList - 1);
             const float h = th[i];
             if (h >= 0.f) {
@@ -412,7 +539,14 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
 #pragma unroll
               for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
               const float d = approx_sqrt(q), ro = ratio_of(h, H);
-              take(i, __float_as_int(ro == 0.f ? 0.f : ro * d));
+              const int sv = __float_as_int(ro == 0.f ? 0.f : ro * d);
+              if (first(i, sv)) {
+                best_v = sv;
+                bi = i;
+                he = h;
+#pragma unroll
+                for (int c = 0; c < CPL; ++c) ve[c] = v[c];
+              }
               if (lane == 0 && h > 0.f) ta[i] = bound_of(d + drift);
             }
             if (next == 0x7fffffff) break;
@@ -425,14 +559,11 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
           const float sc = __int_as_float(best_v);
           if (!fresh && !(sc <= tau * (1.f - drift * inv_dmin) * 0.99999f)) break;  // another token may be smaller: build again
           // ---- evict: Y -= h_e v_e, H -= h_e ----
-          const float he = th[bi];
-          float v[CPL];
-          channels(bi, v);
           H -= he;
           const float inv_H = (H > 0.f) ? __fdividef(1.f, H) : 0.f;
 #pragma unroll
           for (int c = 0; c < CPL; ++c) {
-            y[c] -= he * v[c];
+            y[c] -= he * ve[c];
             x[c] = -(y[c] * inv_H);
           }
           zeros -= he == 0.f ? 1 : 0;
@@ -451,6 +582,15 @@ greedy_cluster_kernel(int Hkv, int cap, int rows_smem, const T* __restrict__ V, 
         }
 #pragma unroll
         for (int c = 0; c < CPL; ++c) Ys[lane * CPL + c] = y[c];
+        if (lane == 0) s_go = 0;
+        asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");
+      } else {
+        while (true) {  // (the warp that runs the picks ends it: the same barriers in the same order on both sides)
+          asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");
+          if (s_go == 0) break;
+          scores_of<T, D>(s_want[warp], rows, rows_smem, Vu, act, th, ta, tp, nX, s_sum, s_drift, s_cand);
+          asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
+        }
       }
       __syncthreads();
       if (tid == 0) {

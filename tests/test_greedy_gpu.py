@@ -233,3 +233,57 @@ def test_greedy_scores_of_exactly_0_come_first_whatever_the_distance(kind, k):
     og = order[0, 0].cpu().tolist()
     assert og == sorted(light, key=lambda j: int(pos[0, 0, j]))[:k]
     assert ev[0, 0].cpu().tolist() == sorted(og)
+
+
+def few_rows(n, k, kind, dtype, d, seed, distinct=64):
+    """A greedy eviction from n tokens whose value rows are `distinct` different ones; weights equal, log-normal or half of them subnormal."""
+    g = torch.Generator(device="cpu").manual_seed(seed)
+    which = torch.randint(0, distinct, (n,), generator=g)
+    V = torch.randn((distinct, d), generator=g).to(dtype)[which].view(1, 1, n, d).contiguous()
+    h = torch.full((1, 1, n), 0.5) if kind == "equal" else torch.randn((1, 1, n), generator=g).exp()
+    if kind == "subnormal":
+        h = torch.where(torch.rand((1, 1, n), generator=g) < 0.5, (which % 7 + 3).view(1, 1, n) * 1e-42, h)
+    pos = torch.randperm(n, generator=g).to(torch.int32).view(1, 1, n)
+    p = P.make_params(1, 1, 1, d, n, 1, dtype, 1.0, "external")
+    ws = P.alloc_workspace(p, DEV)
+    ev = torch.full((1, 1, k), -1, dtype=torch.int32, device=DEV)
+    order, ne = torch.full_like(ev, -1), torch.zeros((1,), dtype=torch.int32, device=DEV)
+    lens = torch.tensor([n], dtype=torch.int32)
+    args = (p, V.to(DEV), h.to(DEV), lens.to(DEV), (lens - k).to(DEV), pos.to(DEV), ev, order, ne, ws)
+    return which.tolist(), h[0, 0], f32(V)[0, 0], pos[0, 0], args
+
+
+@pytest.mark.parametrize("n,k,kind", [(300, 299, "equal"), (4224, 96, "equal"), (700, 400, "subnormal"), (20000, 40, "equal")])
+@pytest.mark.parametrize("dtype,d", [(torch.bfloat16, 128), (torch.bfloat16, 64), (torch.float32, 128)])
+def test_greedy_when_many_tokens_compete_for_every_pick(n, k, kind, dtype, d):
+    """All warps form scores, to the bit those of one warp: tokens of the same row and weight leave in the order of their positions."""
+    which, h, V, pos, args = few_rows(n, k, kind, dtype, d, n + d)
+    P.caote_select_evict_greedy(*args)
+    assert P.caote_read_status(args[-1]) == 0
+    og = args[7][0, 0].cpu().tolist()
+    assert sorted(og) == args[6][0, 0].cpu().tolist() and len(set(og)) == k and 0 <= min(og) and max(og) < n
+    same = {}
+    for j in sorted(range(n), key=lambda j: int(pos[j])):
+        same.setdefault((which[j], float(h[j])), []).append(j)
+    for t, j in enumerate(og):
+        oldest = same[which[j], float(h[j])].pop(0)
+        assert j == oldest, f"pick {t}: slot {j} leaves before slot {oldest}, an older one of the same row and weight"
+    if kind == "equal":
+        follow(og[:12], h.numpy(), V, pos.numpy(), 12)
+
+
+def test_greedy_cost_of_tokens_that_compete():
+    """Equal weights and few different rows cost more builds and shared scores, not a walk through the list for every pick: at 4 224
+    tokens and 128 picks 7 times the time of log-normal weights and different rows (51 times with the walk)."""
+    def device_ms(distinct, kind):
+        args = few_rows(4224, 128, kind, torch.bfloat16, 128, 2, distinct)[-1]
+        times = []
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            P.caote_select_evict_greedy(*args)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        return sorted(times)[2]
+    assert device_ms(64, "equal") < 20 * device_ms(4224, "log-normal")
