@@ -489,7 +489,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     // =============================== two threads per query row ===============================
     // Thread t and thread t + 128 share row t of the block: each owns 64 of a tile's 128 keys (and 64
     // of the 128 output channels when O is rescaled or written out). They agree on the softmax
-    // reference through a two-float exchange in shared memory and one barrier of the row threads.
+    // reference through a two-float exchange in shared memory and a barrier of the two warps that share the rows.
     const int rowl = tid & (kThreads - 1), half = tid >> 7;
     const int R = row0 + rowl;
     const int nvis = (R < M) ? n - m + (R % m) + 1 : n;  // keys this row sees (causal inside the block)
@@ -534,10 +534,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         raw_top = fmaxf(fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3])), fmaxf(fmaxf(pm[4], pm[5]), fmaxf(pm[6], pm[7])));
       }
       float mx = raw_top * scale2;
-      // the other half of the row (the two warps that share 32 rows meet here)
+      // the other half of the row (the two warps that share 32 rows meet here; each writes P over columns of S that the other has
+      // read, hence the fences)
       float* xm = xch + (kt & 1) * kRowThreads;
       xm[tid] = mx;
+      tc_fence_before();
       asm volatile("bar.sync %0, 64;" ::"r"(2 + (warp & 3)) : "memory");
+      tc_fence_after();
       mx = fmaxf(mx, xm[tid ^ kThreads]);
       // the reference moves only when a logit exceeds it by more than 8 (p <= 256 in between)
       const bool need = mx > m_ref + 8.f;

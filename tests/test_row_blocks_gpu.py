@@ -7,7 +7,7 @@ import oracle
 import paper_2504_14051_b200 as P
 
 from test_gpu_parity import dominant_case, make_case, run_score
-from parity import assert_close, check_scores_and_o, f32, oracle_for
+from parity import assert_close, check_scores_and_o, f32, oracle_for, sub_problem
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -242,3 +242,42 @@ def test_carried_sums_beside_the_attention_pass(d):
         return outs + [cache.base, cache.scores, cache.K, cache.V, cache.pos, cache.lens]
     for a, b in zip(run(False), run(True)):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("mode", ["last_query", "chunk_sum", "accum"])
+@pytest.mark.parametrize("case", [
+    # B, Hq, Hkv, d, cap, m, n, key tiles per CTA
+    (1, 1, 1, 128, 18448, 128, 18433, 19),  # 145 tiles in 8 splits; one counted row under last_query
+    (1, 8, 1, 64, 18448, 16, 18433, 19),
+    (1, 16, 1, 128, 18448, 1, 18433, 19),   # one query, 16 heads per group: few counted rows in every mode
+    (38, 2, 2, 128, 2440, 128, 2400, 19),   # enough row blocks that none is split
+    (38, 2, 2, 64, 2440, 128, 2400, 19),
+])
+def test_row_blocks_with_logits_that_grow_along_the_keys(case, mode):
+    """Keys far above all that came before them in tiles 3, 8, 11, 16 and the last one of a CTA's share: the softmax reference
+    moves before a share of the output is closed, on the tile that closes it, and with earlier shares set aside; for one row of
+    a warp, for several, and for the counted rows. Two runs give the same bits."""
+    B, Hq, Hkv, d, cap, m, n, tiles = case
+    G = Hq // Hkv
+    q, K, V, lens_t = make_case(60 + d + m, B, Hq, Hkv, d, cap, m, torch.bfloat16, [n] * B)
+    units = [(0, 0)] if B == 1 else [(0, 1), (37, 0)]
+    rows = [(0, 0), (G // 2, m // 2), (G - 1, m - 1)]  # head of the group, query: the last one is counted in every mode
+    for b, h in units:
+        for first in range(0, (n + 127) // 128, 3 * tiles):  # the first CTA's share, and every third
+            for i, t in enumerate((3, 8, 11, 16, 18)):  # log2 of the weights: about 22 more from one to the next
+                for g, r in (rows if i % 2 else rows[2:]):
+                    j = (first + t) * 128 + 5 + 7 * g
+                    if j < n - m:
+                        K[b, h, j] = (q[b, h * G + g, r].float() * (1.3 * (i + 1) * (128 / d) ** 0.5)).to(K.dtype)
+    base = None
+    if mode == "accum":
+        base = (torch.rand((B, Hkv, cap), generator=torch.Generator().manual_seed(6)) * 2.0).to(DEV)
+    base_in = None if base is None else base.clone()
+    _, _, o, scores = run_score(q, K, V, lens_t, m, mode, base)
+    qs, Ks, Vs, ls, bs = sub_problem(q, K, V, lens_t, base_in, units, Hkv, G)
+    r = oracle_for(qs, Ks, Vs, ls, scale=d ** -0.5, n_new=m, base_mode=mode, base=bs)
+    check_scores_and_o(r, torch.stack([scores[b, h:h + 1] for b, h in units]), torch.stack([o[b, h * G:(h + 1) * G] for b, h in units]),
+                       ls, f"{case} {mode}")
+    base2 = None if base_in is None else base_in.clone()
+    _, _, o2, scores2 = run_score(q, K, V, lens_t, m, mode, base2)
+    assert torch.equal(o, o2) and torch.equal(scores[:, :, :n], scores2[:, :, :n])
