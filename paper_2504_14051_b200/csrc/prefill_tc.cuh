@@ -1251,7 +1251,9 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         }
         piece(vb, sb, crs + 48, plain, R0 + 48);
         __syncwarp();
-        if (lane == 0) mbar_arrive(&st_free[ss]);  // ... and is done with the block's statistics
+        // ... and is done with the block's statistics (no fence: their place is filled again eight blocks later, by a copy that waits
+        // for products which wait for all warps to be four blocks further on)
+        if (lane == 0) mbar_arrive(&st_free[ss]);
       }
       h += (hacc[0].x + hacc[0].y) + (hacc[1].x + hacc[1].y);
 
@@ -1277,6 +1279,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         }
       }
       const float hb = kAccum ? Xs[kb * (D + 4) + D] : 0.f;
+      fence_async_smem();  // (the rows have been read before the copy that follows the arrival writes there)
       __syncwarp();
       if (lane == 0) mbar_arrive(&v_free[kb]);  // (and with X)
       if (rhalf) {

@@ -281,3 +281,24 @@ def test_row_blocks_with_logits_that_grow_along_the_keys(case, mode):
     base2 = None if base_in is None else base_in.clone()
     _, _, o2, scores2 = run_score(q, K, V, lens_t, m, mode, base2)
     assert torch.equal(o, o2) and torch.equal(scores[:, :, :n], scores2[:, :, :n])
+
+
+@pytest.mark.parametrize("mode,d", [("chunk_sum", 64), ("accum", 64), ("chunk_sum", 128)])
+def test_scores_of_many_equal_calls_have_the_same_bits(mode, d):
+    """Value tiles are handed back to the copies only when every row has been read: 2 500 calls of eight items per CTA each."""
+    B, Hq, Hkv, m, n = 7, 28, 4, 128, 10444
+    g = torch.Generator(device=DEV).manual_seed(1)
+    q, K, V = (torch.randn(s, generator=g, device=DEV).to(torch.bfloat16) for s in ((B, Hq, m, d), (B, Hkv, n, d), (B, Hkv, n, d)))
+    base = torch.rand((B, Hkv, n), generator=g, device=DEV)
+    lens = torch.full((B,), n, dtype=torch.int32, device=DEV)
+    p = P.make_params(B, Hq, Hkv, d, n, m, torch.bfloat16, d ** -0.5, mode)
+    ws = P.alloc_workspace(p, DEV)
+    o, scores = torch.zeros(q.shape, device=DEV), torch.zeros((B, Hkv, n), device=DEV)
+    first, differ, carried = None, torch.zeros((), dtype=torch.int64, device=DEV), torch.empty_like(base)
+    for _ in range(2500 if (mode, d) == ("chunk_sum", 64) else 500):
+        carried.copy_(base)
+        P.caote_score(p, q, K, V, lens, carried if mode == "accum" else None, o, scores, ws)
+        if first is None:
+            first = scores.clone()
+        differ += (scores != first).sum()
+    assert differ.item() == 0 and P.caote_read_status(ws) == 0
