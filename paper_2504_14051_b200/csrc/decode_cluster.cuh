@@ -804,6 +804,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             prefill::tmem_st32u(tStash + lane_base + j * kRowCols + half * 32, rw);
           }
           prefill::tmem_st_wait();
+          if (use_base) fence_async_smem();  // (the rows have gone through registers into TMEM; the base score may still be on its way)
           __syncwarp();
           if (lane == 0) mbar_arrive(&vempty[vs]);
         }

@@ -381,3 +381,22 @@ def test_a_wait_that_runs_out_is_reported_and_the_library_stays_usable():
     assert P.caote_read_status(ws) == 0
     r = oracle_for(q, K, V, lens_t, scale=d ** -0.5, n_new=1, base_mode="last_query")
     check_scores_and_o(r, scores, o, lens_t, "after a timed-out call")
+
+
+@pytest.mark.parametrize("sizes", [(32, 32, 8, 128, 3000), (8, 8, 2, 64, 9000)])
+def test_carried_scores_of_many_equal_calls_have_the_same_bits(sizes):
+    """Single queries with accumulated scores: a tile's base scores are read before its place is handed back to the copies."""
+    B, Hq, Hkv, d, n = sizes
+    q, K, V, lens = make_case(3, B, Hq, Hkv, d, n, 1, torch.bfloat16, [n] * B)
+    base = torch.rand((B, Hkv, n), generator=torch.Generator().manual_seed(4)).to(DEV)
+    p = P.make_params(B, Hq, Hkv, d, n, 1, torch.bfloat16, d ** -0.5, "accum")
+    ws = P.alloc_workspace(p, DEV)
+    o, scores, carried = torch.zeros(q.shape, device=DEV), torch.zeros((B, Hkv, n), device=DEV), torch.empty_like(base)
+    first, differ = None, torch.zeros((), dtype=torch.int64, device=DEV)
+    for _ in range(600):
+        carried.copy_(base)
+        P.caote_score(p, q, K, V, lens, carried, o, scores, ws)
+        if first is None:
+            first = (scores.clone(), carried.clone())
+        differ += (scores != first[0]).sum() + (carried != first[1]).sum()
+    assert differ.item() == 0 and P.caote_read_status(ws) == 0
