@@ -144,6 +144,7 @@ sum_errors_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_c
   bool late = false;
   int i = 0, started = min(kStages, boxes);  // the box that is read, copies started (lane 0)
   auto next = [&]() {  // the stage has been read: the box that takes its place
+    ptx::fence_async_smem();  // (by every lane: nothing else keeps the copy behind loads that are still on their way)
     __syncwarp();
     if (lane == 0 && !late && i + kStages < boxes) {
       load(i + kStages);

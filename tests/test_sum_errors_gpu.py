@@ -107,3 +107,20 @@ def test_a_pass_whose_waits_run_out_reports_it_and_leaves_nothing_behind(Hq):
     r = oracle.score(f32(q), f32(K), f32(V), lens_t.cpu().numpy(), scale=d ** -0.5, n_new=1, base_mode="last_query", agg_mode="sum_errors")
     for b, n in enumerate(lens):
         assert_close(f32(scores)[b, :, :n], r["scores"][b, :, :n], f"[b={b}]")
+
+
+@pytest.mark.parametrize("sizes", [(2, 64, 8, 128, 9000), (16, 16, 8, 64, 4000), (4, 8, 8, 128, 9000)])
+def test_scores_of_many_equal_calls_have_the_same_bits(sizes):
+    """A warp's boxes are read before the copy that takes their place starts."""
+    B, Hq, Hkv, d, n = sizes
+    q, K, V, lens = make_case(5, B, Hq, Hkv, d, n, 1, torch.bfloat16, [n] * B)
+    p = P.make_params(B, Hq, Hkv, d, n, 1, torch.bfloat16, d ** -0.5, "last_query")
+    ws = P.alloc_workspace(p, DEV)
+    o, scores = torch.zeros(q.shape, device=DEV), torch.zeros((B, Hkv, n), device=DEV)
+    first, differ = None, torch.zeros((), dtype=torch.int64, device=DEV)
+    for _ in range(600):
+        P.caote_score_sum_errors(p, q, K, V, lens, o, scores, ws)
+        if first is None:
+            first = scores.clone()
+        differ += (scores != first).sum()
+    assert differ.item() == 0 and P.caote_read_status(ws) == 0
