@@ -22,9 +22,11 @@ CASES = [
     (2, 6, 2, 64, 96, 5, [90, 17], [60, 3], torch.float32),              # most of a short sequence goes
     (3, 32, 8, 128, 4224, 1, [4129, 515, 2000], [4096, 512, 2000], torch.bfloat16),  # several tiles per unit
     (1, 12, 2, 128, 700, 33, [640], [500], torch.bfloat16),              # ragged block, 6 heads per group
+    (2, 16, 1, 128, 304, 1, [290, 130], [250, 129], torch.bfloat16),     # one query, 16 heads per group: the row blocks' statistics
+    (1, 24, 2, 64, 1400, 1, [1333], [1200], torch.bfloat16),             # 12 heads per group, several key splits
 ]
 # cases whose scoring call runs on the tensor-core kernels and so leaves the rows' statistics in the workspace
-LEAVES_STATS = {0, 1, 3, 5, 6}
+LEAVES_STATS = {0, 1, 3, 5, 6, 7, 8}
 
 
 @pytest.mark.parametrize("case", CASES)
@@ -77,6 +79,26 @@ def test_post_evict_output_matches_oracle(case):
     got3 = f32(o3)
     for b in range(B):
         assert_close(got3[b], ref[b], f"{case} o_post from the workspace statistics [b={b}]")
+
+
+def test_statistics_per_row_with_an_output_off_a_16_byte_boundary():
+    """A block's output that starts 4 bytes behind a boundary goes through the any-shape kernel, which reads the same statistics."""
+    B, Hq, Hkv, d, cap, m, n, k = 1, 8, 2, 128, 520, 64, 500, 100
+    q, K, V, lens_t = make_case(78, B, Hq, Hkv, d, cap, m, torch.bfloat16, [n])
+    p = P.make_params(B, Hq, Hkv, d, cap, m, torch.bfloat16, d ** -0.5, "chunk_sum")
+    ws = P.alloc_workspace(p, DEV)
+    o = torch.zeros(q.shape, dtype=torch.float32, device=DEV)
+    P.caote_score(p, q, K, V, lens_t, None, o, torch.zeros((B, Hkv, cap), dtype=torch.float32, device=DEV), ws)
+    ev = torch.arange(7, 7 + k, dtype=torch.int32, device=DEV).expand(B, Hkv, k).contiguous()
+    ne = torch.tensor([k], dtype=torch.int32, device=DEV)
+    o1 = torch.empty(o.numel() + 1, device=DEV)[1:].view(o.shape)
+    o1.copy_(o)
+    K1 = torch.full_like(K, float("nan"))  # only the evicted rows may be read: the statistics stand in for a pass over K
+    K1[:, :, 7:7 + k] = K[:, :, 7:7 + k]
+    P.caote_post_evict_output_ws(p, q, K1, V, lens_t, ev, ne, o1, o1, ws)
+    assert P.caote_read_status(ws) == 0
+    ref = oracle.post_evict_output(f32(q), f32(K), f32(V), [n], [[ev[0, h].cpu().numpy() for h in range(Hkv)]], scale=d ** -0.5, n_new=m)
+    assert_close(f32(o1), ref, "output off a boundary")
 
 
 def test_statistics_of_another_scoring_path_are_not_used():
