@@ -196,9 +196,10 @@ CAOTE_API int caote_select_evict(const caote_params_t* params, const float* scor
  *   evict_idx[u, 0..k) out: the evicted slots in ascending order (what caote_compact takes);
  *   order[u, 0..k) out, nullable: the same slots in the order they were evicted;  n_evict[b] = k out.
  * capacity <= 24576 (the unit's weights and distances stay in shared memory), else CAOTE_ERR_UNSUPPORTED.
- * Cost: two sweeps over the unit's value rows (its output, the distances of all tokens), one more whenever the bounds on the
- * tokens looked at no longer settle a pick (many hundreds of evictions, or weights that hold nearly all of the sum), and per
- * eviction the rows of the few tokens that can be the minimum. */
+ * Cost: two sweeps over the unit's value rows (its output, the distances of all tokens), one more whenever the tokens looked at
+ * (192, at most 256) no longer settle a pick: after some 160 to 190 evictions, sooner where scores lie close together (equal
+ * weights: every 20 to 30) or one token holds nearly all of the sum; and per eviction the rows of the tokens that can be the
+ * minimum: one or two, up to all of those looked at where rows and weights repeat. */
 CAOTE_API int caote_select_evict_greedy(const caote_params_t* params, const void* V, const float* h,
                               const int32_t* len, const int32_t* budget, const int32_t* pos,
                               int32_t* evict_idx, int32_t* order, int32_t max_evict, int32_t* n_evict,

@@ -14,9 +14,9 @@ namespace caote {
 // [256, ...)          per-call scratch, carved by the entry point that uses it
 constexpr size_t kHeaderBytes = 256;
 // Word kStatTagIndex of the workspace header says which softmax statistics the last scoring call left at
-// workspace + kHeaderBytes for the post-eviction output to reuse (reference + log2(sum) of the log2-domain
-// logits): per query head of a unit ([units][kHeadStatFloats], single-query kernels), per query row of a unit
-// ([units][padded rows], tensor-core prefill kernels), or none.
+// workspace + kHeaderBytes for the post-eviction output to reuse, from reference + log2(sum) of the log2-domain
+// logits: that value per query head of a unit ([units][kHeadStatFloats], single-query kernels), minus that value per
+// query row of a unit ([units][padded rows], row-block kernels), or none.
 constexpr int kStatTagIndex = 8;
 constexpr int kStatNone = 0, kStatPerHead = 1, kStatPerRow = 2;
 // Per query head the record is three rows of 8 floats per unit: the log-sum-exp, the largest logit, and the share of

@@ -74,10 +74,9 @@ __device__ __forceinline__ void fence_async_all() { asm volatile("fence.proxy.as
 
 // ---- one lane of a warp ------------------------------------------------------------------------------------
 // True in one lane of a fully converged warp. What a single lane has to do (products, copies) stands behind this and not
-// behind `lane == 0`: the compiler then knows that one lane is active and keeps operands in uniform registers, where
-// tcgen05 and TMA instructions take them from, instead of moving every one of them there first. Beside warps that keep
-// the scheduler busy that is the difference between a product every 64 cycles, the tensor pipe's own rate for
-// M 128 x N 128 x K 16, and one every 81 (24 products beside eight warps of softmax arithmetic: 1 538 cycles, 1 939).
+// behind `lane == 0`. Measured: 24 products (M 128 x N 128 x K 16) beside eight warps of softmax arithmetic take 1 538 cycles,
+// 64 each, which is the tensor pipe's own rate, and 1 939 from `lane == 0`; alone 1 538 either way. The likely cause: where the
+// compiler knows that one lane is active it can keep operands in uniform registers and need not move each of them there.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile(
